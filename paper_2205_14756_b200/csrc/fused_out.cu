@@ -59,7 +59,7 @@ constexpr int O_STAGING = 4 * O_STAGING_WARP;
 constexpr int O_BAR_BYTES = 512;
 constexpr int O_SMEM_FIXED = O_STAGING + O_BAR_BYTES + 1024;  // besides the rows of M, the ring and the residual blocks
 constexpr int O_SMEM_LIMIT = 226 * 1024;                     // dynamic shared memory of a CTA (1 KB of the 227 left to static data)
-static_assert(24 * O_MAX_STAGES + 16 + 16 + 8 + 8 + 8 + 4 * 8 <= O_BAR_BYTES, "barrier block");
+static_assert(24 * O_MAX_STAGES + 16 + 16 + 8 + 8 + 8 + 4 * 8 + 8 <= O_BAR_BYTES, "barrier block");
 
 __device__ int g_fused_timeout_flag = 0;
 
@@ -265,6 +265,7 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
   const uint32_t peer_res_bar = res_bar + 8;             // the peer's rows of M landed (leader only)
   const uint32_t tmem_slot = peer_res_bar + 8;
   const uint32_t resid_bar = tmem_slot + 8;              // [epilogue warp] RES: the warp's residual block landed
+  const uint32_t mfree_bar = resid_bar + 32;             // the MMAs of an image are complete: its rows of M may be replaced (commit, both CTAs)
   __shared__ int abort_flag;
   __shared__ uint32_t tmem_base_sh;
 
@@ -286,6 +287,7 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
     for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar + 8 * a, 1); mbar_init(tempty_bar + 8 * a, 2 * 4); }
     mbar_init(res_bar, 1);
     mbar_init(peer_res_bar, 1);
+    mbar_init(mfree_bar, 1);
     if (RES)
       for (int w = 0; w < 4; ++w) mbar_init(resid_bar + 8 * w, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -311,16 +313,18 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
     if (lane == 0) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tmM) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tmQ) : "memory");
-      uint32_t local = 0, s = 0, ph = 0;  // ring slot and the parity of its current use
+      uint32_t s = 0, ph = 0, mfree_ph = 0;  // ring slot and the parity of its current use
       int cur_b = -1;
       bool ok = true;
-      for (int tile = tile_first; ok && tile < tile_end; ++tile, ++local) {
+      for (int tile = tile_first; ok && tile < tile_end; ++tile) {
         const int b = tile / p.tiles_per_image, nt = tile % p.tiles_per_image;
         if (b != cur_b) {
-          if (cur_b >= 0) {  // every MMA that reads the previous image's rows of M must be complete
-            const uint32_t last = local - 1;
-            ok = mbar_wait_cluster(tfull_bar + 8 * (last & 1), (last >> 1) & 1, &abort_flag);
+          if (cur_b >= 0) {
+            // Every MMA that reads the previous image's rows of M must be complete.  The accumulators' barriers cannot tell:
+            // with few heads the ring lets the copies run several tiles ahead, and a parity two phases back looks complete.
+            ok = mbar_wait_cluster(mfree_bar, mfree_ph, &abort_flag);
             if (!ok) break;
+            mfree_ph ^= 1;
           }
           cur_b = b;
           mbar_expect_tx(res_bar, (uint32_t)(p.kslices * O_A_SLICE));
@@ -393,6 +397,7 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
           if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1; }
         }
         if (ok) umma2_commit_both(tfull_bar + 8 * acc);
+        if (ok && tile + 1 < tile_end && (tile + 1) / p.tiles_per_image != b) umma2_commit_both(mfree_bar);
       }
     }
   } else if (warp < 2 + O_XWARPS) {

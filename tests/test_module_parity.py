@@ -263,3 +263,15 @@ def test_bounded_wait_gives_up_and_leaves_the_context_usable():
 def test_no_kernel_wait_timed_out():
     """Every device-side wait in the library is bounded; none of the runs above may have hit its limit."""
     assert binding.msla_debug_wait_timeouts() == 0
+
+
+# Few heads and many images: the copies of the fused apply + projection kernel run several tiles ahead of its MMAs, across
+# image boundaries, where the folded weights in shared memory are replaced.
+@pytest.mark.parametrize("B,C,H,W,heads,d", [(40, 64, 40, 40, 2, 32), (24, 32, 48, 32, 1, 32), (30, 64, 48, 40, 4, 16)])
+def test_many_images_with_few_heads(B, C, H, W, heads, d):
+    s = inputs.ModuleShape("images", "bf16", B, C, H, W, heads, d, seed=45)
+    t = inputs.module_inputs(s)
+    ref = _ref(s, t)
+    for _ in range(3):
+        util.assert_close(util.run_module(s, t), ref, "bf16", "many images", block=util.MODULE_BLOCK)
+    assert binding.msla_debug_wait_timeouts() == 0
