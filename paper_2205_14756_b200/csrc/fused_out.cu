@@ -570,8 +570,8 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
 
 }  // namespace
 
-bool fused_out_bf16_supported(int Ht, int d, int Cout, int N) {
-  return (d == 16 || d == 32) && Ht >= 1 && Ht * d <= O_MAX_KS * OKS && Cout >= 1 && Cout <= 2 * OM && Cout % 8 == 0 && N >= 8 && N % 8 == 0;
+bool fused_out_bf16_supported(int Ht, int d, int Cout) {
+  return (d == 16 || d == 32) && Ht >= 1 && Ht * d <= O_MAX_KS * OKS && Cout >= 1 && Cout <= 2 * OM && Cout % 8 == 0;
 }
 
 // Scratch: M [B][Cout][Ht*d] bf16, then ks [B][Ht][d] fp32 (256-byte aligned).
@@ -580,8 +580,8 @@ size_t fused_out_scratch_bytes(int B, int Ht, int d, int Cout) { return fused_ou
 
 // y[b][m][n] = sum_h sum_c w[m][h*d + c] * att[b][h][n][c] + bias[m], att = Eq. 3 applied to query head h with the
 // state of (b, h) = sum over s < S of partial[(b * Ht + h) * S + s] ([d][d+1] fp32 each: KV, then the key sum in
-// column d).  q: planar bf16 query matrices [N][d], head h of image b at q + b*q_sb + h*q_sh (elements); y: NCHW
-// [B, Cout, N].
+// column d).  q: planar bf16 query matrices [N][d], head h of image b at q + b*q_sb + h*q_sh (elements); y (and
+// residual): [B, Cout, N] with rows ldy elements apart.
 namespace {
 template <int D, bool RES, bool F16>
 msla_status_t launch_fused(dim3 grid, int smem, cudaStream_t st, const CUtensorMap& tmM, const CUtensorMap& tmQ, const CUtensorMap& tmO,
@@ -603,9 +603,9 @@ msla_status_t launch_fused_for(int d, bool res, dim3 grid, int smem, cudaStream_
 // f16: queries, weights, bias, residual and output are IEEE binary16 instead of bfloat16; M, the key sums and eps are
 // scaled by the power of two just above 1 / N (N tokens' sums would leave binary16's range otherwise).
 msla_status_t run_fused_out_bf16(const void* q, long long q_sb, long long q_sh, const float* partial, int S, void* scratch,
-                                 const void* w, const void* bias, const void* residual, void* y, int B, int Ht, int d, int N, int Cout,
+                                 const void* w, const void* bias, const void* residual, void* y, int ldy, int B, int Ht, int d, int N, int Cout,
                                  float eps, cudaStream_t st, bool f16) {
-  if (!fused_out_bf16_supported(Ht, d, Cout, N) || q_sb % 8 != 0 || q_sh % 8 != 0)
+  if (!fused_out_bf16_supported(Ht, d, Cout) || ldy % 8 != 0 || q_sb % 8 != 0 || q_sh % 8 != 0)
     return fail(MSLA_ERR_UNSUPPORTED, "fused apply + projection: %d heads of %d channels, %d output channels, %d tokens", Ht, d, Cout, N);
   if (S < 1 || S > 8 * FOLD_RUNS) return fail(MSLA_ERR_UNSUPPORTED, "fused apply + projection: %d partial states per head (1 .. %d)", S, 8 * FOLD_RUNS);
   const int K = Ht * d;
@@ -624,7 +624,7 @@ msla_status_t run_fused_out_bf16(const void* q, long long q_sb, long long q_sh, 
     const cuuint64_t sQ[3] = {(cuuint64_t)d * 2, (cuuint64_t)q_sh * 2, (cuuint64_t)q_sb * 2};
     const cuuint32_t bQ[4] = {(cuuint32_t)d, (cuuint32_t)ot, 1, 1};
     const cuuint64_t dO[3] = {(cuuint64_t)N, (cuuint64_t)Cout, (cuuint64_t)B};
-    const cuuint64_t sO[2] = {(cuuint64_t)N * 2, (cuuint64_t)Cout * N * 2};
+    const cuuint64_t sO[2] = {(cuuint64_t)ldy * 2, (cuuint64_t)Cout * ldy * 2};
     const cuuint32_t bO[3] = {64, 32, 1};
     if (!tma_make_map_bf16(&tmM, M, 3, dM, sM, bM, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !tma_make_map_bf16(&tmQ, q, 4, dQ, sQ, bQ, d == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B) ||

@@ -210,7 +210,7 @@ __device__ __forceinline__ void drain_accumulator(const GemmParams& p, const CUt
       }
     } else if (row_ok) {
 #pragma unroll
-      for (int v = 0; v < 4; ++v) {  // 4 x (8 columns = 16 bytes); N is a multiple of 8
+      for (int v = 0; v < 4; ++v) {  // 4 x (8 columns = 16 bytes) of a plane
         const int n = n0 + v * 8;
         if (n < p.N) {
           bf16* dst = p.group ? obase + (((long long)(n >> gs) * p.M + m) << gs) + (n & (p.group - 1))
@@ -576,15 +576,15 @@ msla_status_t launch(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUten
 
 }  // namespace
 
-bool project_in_bf16_supported(int C, int Cout, int N, int d) {
-  return C % 8 == 0 && Cout % 8 == 0 && N % 8 == 0 && (d == 16 || d == 32) && Cout % d == 0;
+bool project_in_bf16_supported(int C, int Cout, int ldx, int d) {
+  return C % 8 == 0 && Cout % 8 == 0 && ldx % 8 == 0 && (d == 16 || d == 32) && Cout % d == 0;
 }
 
-// y[b][o / d][n][o % d] = sum_c w[o][c] * x[b][c][n];  x NCHW [B, C, N], y planar with batch stride y_sb.
-msla_status_t run_project_in_bf16(const void* x, const void* w, void* y, int B, int C, int Cout, int N, int d,
+// y[b][o / d][n][o % d] = sum_c w[o][c] * x[b][c][n];  x [B, C, N] with rows ldx elements apart, y planar with batch stride y_sb.
+msla_status_t run_project_in_bf16(const void* x, int ldx, const void* w, void* y, int B, int C, int Cout, int N, int d,
                                   long long y_sb, cudaStream_t st, bool f16) {
   CUtensorMap tmA, tmB;
-  if (!make_map(&tmA, x, (uint64_t)N, (uint64_t)C, (uint64_t)B, (uint64_t)N * 2, (uint64_t)C * N * 2, 64, BK) ||
+  if (!make_map(&tmA, x, (uint64_t)N, (uint64_t)C, (uint64_t)B, (uint64_t)ldx * 2, (uint64_t)C * ldx * 2, 64, BK) ||
       !make_map(&tmB, w, (uint64_t)C, (uint64_t)Cout, 1, (uint64_t)C * 2, (uint64_t)C * Cout * 2, BK, BN))
     return fail(MSLA_ERR_CUDA, "cuTensorMapEncodeTiled failed for the input projection");
   GemmParams p{};
@@ -607,10 +607,11 @@ msla_status_t run_project_in_bf16(const void* x, const void* w, void* y, int B, 
   return f16 ? launch<true, false, 0, true>(tmA, tmB, tmO, p, st) : launch<true>(tmA, tmB, tmO, p, st);
 }
 
-bool project_out_bf16_supported(int Cin, int Cout, int N) { return Cin % 8 == 0 && N % 8 == 0 && Cout >= 1; }
+bool project_out_bf16_supported(int Cin, int Cout, int ldy) { return Cin % 8 == 0 && ldy % 8 == 0 && Cout >= 1; }
 
-// y[b][m][n] = sum_j w[m][j] * a[b][n][j] + bias[m];  a token-major [B, N, Cin], y NCHW [B, Cout, N].
-msla_status_t run_project_out_bf16(const void* a, const void* w, const void* bias, const void* residual, void* y, int B, int Cin,
+// y[b][m][n] = sum_j w[m][j] * a[b][n][j] + bias[m];  a token-major [B, N, Cin], y (and residual) [B, Cout, N] with rows ldy
+// elements apart.
+msla_status_t run_project_out_bf16(const void* a, const void* w, const void* bias, const void* residual, void* y, int ldy, int B, int Cin,
                                    int Cout, int N, cudaStream_t st, bool f16) {
   CUtensorMap tmA, tmB;
   if (!make_map(&tmA, w, (uint64_t)Cin, (uint64_t)Cout, 1, (uint64_t)Cin * 2, (uint64_t)Cin * Cout * 2, BK, BM) ||
@@ -619,13 +620,13 @@ msla_status_t run_project_out_bf16(const void* a, const void* w, const void* bia
   GemmParams p{};
   p.M = Cout; p.N = N; p.K = Cin; p.batches = B;
   p.m_tiles = (Cout + BM - 1) / BM; p.n_tiles = (N + BN - 1) / BN;
-  p.out_batch_stride = (long long)Cout * N; p.ld_out = N; p.group = 0; p.bias_per_row = 1; p.n_fastest = 0;
+  p.out_batch_stride = (long long)Cout * ldy; p.ld_out = ldy; p.group = 0; p.bias_per_row = 1; p.n_fastest = 0;
   p.bias = (const bf16*)bias; p.out = (bf16*)y;
   CUtensorMap tmO;  // NCHW output as [batch][channel][token]; blocks of 32 channels x 32 tokens
   {
     p.tma_store = 1;
     const cuuint64_t dims[3] = {(cuuint64_t)N, (cuuint64_t)Cout, (cuuint64_t)B};
-    const cuuint64_t strides[2] = {(cuuint64_t)N * 2, (cuuint64_t)Cout * N * 2};
+    const cuuint64_t strides[2] = {(cuuint64_t)ldy * 2, (cuuint64_t)Cout * ldy * 2};
     const cuuint32_t box[3] = {32, 32, 1};
     if (!tma_make_map_bf16(&tmO, y, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B))
       return fail(MSLA_ERR_CUDA, "cuTensorMapEncodeTiled failed for the output projection's output");
@@ -635,16 +636,16 @@ msla_status_t run_project_out_bf16(const void* a, const void* w, const void* bia
   return residual ? launch<false, false, 2>(tmA, tmB, tmO, p, st) : launch<false>(tmA, tmB, tmO, p, st);
 }
 
-bool project_out_planar_bf16_supported(int Cin, int Cout, int N) { return Cin % 64 == 0 && N % 8 == 0 && Cout >= 1; }
+bool project_out_planar_bf16_supported(int Cin, int Cout) { return Cin % 64 == 0 && Cout >= 1; }
 
 // Same product with the attention output kept planar: a[b][j / 64][n][j % 64] (one [N][64] plane per pair of heads).
-msla_status_t run_project_out_planar_bf16(const void* a, const void* w, const void* bias, const void* residual, void* y, int B,
+msla_status_t run_project_out_planar_bf16(const void* a, const void* w, const void* bias, const void* residual, void* y, int ldy, int B,
                                           int Cin, int Cout, int N, cudaStream_t st, bool f16) {
   CUtensorMap tmA, tmB, tmO;
   const int planes = Cin / 64;
   {
     const cuuint64_t dO[3] = {(cuuint64_t)N, (cuuint64_t)Cout, (cuuint64_t)B};
-    const cuuint64_t sO[2] = {(cuuint64_t)N * 2, (cuuint64_t)Cout * N * 2};
+    const cuuint64_t sO[2] = {(cuuint64_t)ldy * 2, (cuuint64_t)Cout * ldy * 2};
     const cuuint32_t bO[3] = {32, 32, 1};
     if (!make_map(&tmA, w, (uint64_t)Cin, (uint64_t)Cout, 1, (uint64_t)Cin * 2, (uint64_t)Cin * Cout * 2, BK, BM) ||
         !make_map(&tmB, a, 64, (uint64_t)N, (uint64_t)B * planes, 128, (uint64_t)N * 128, BK, BN) ||
@@ -654,7 +655,7 @@ msla_status_t run_project_out_planar_bf16(const void* a, const void* w, const vo
   GemmParams p{};
   p.M = Cout; p.N = N; p.K = Cin; p.batches = B;
   p.m_tiles = (Cout + BM - 1) / BM; p.n_tiles = (N + BN - 1) / BN;
-  p.out_batch_stride = (long long)Cout * N; p.ld_out = N; p.group = 0; p.bias_per_row = 1; p.n_fastest = 0;
+  p.out_batch_stride = (long long)Cout * ldy; p.ld_out = ldy; p.group = 0; p.bias_per_row = 1; p.n_fastest = 0;
   p.bias = (const bf16*)bias; p.out = (bf16*)y;
   p.tma_store = 1; p.planes_per_batch = planes;
   p.residual = (const bf16*)residual;
@@ -663,19 +664,17 @@ msla_status_t run_project_out_planar_bf16(const void* a, const void* w, const vo
 }
 
 // ---- the two linear layers of the FFN with a depthwise convolution (Section 3.1, Fig. 2 left)
-bool ffn_bf16_supported(int C, int Ch, int Cout, int N) {
-  return C % 8 == 0 && Ch % 64 == 0 && Cout % 8 == 0 && N % 8 == 0;
-}
+bool ffn_bf16_supported(int C, int Ch, int Cout) { return C % 8 == 0 && Ch % 64 == 0 && Cout % 8 == 0; }
 
-// First layer: h[b][o / 32][n][o % 32] = act(sum_c w1[o][c] * x[b][c][n] + b1[o]); x NCHW, h planes of 32 channels
+// First layer: h[b][o / 32][n][o % 32] = act(sum_c w1[o][c] * x[b][c][n] + b1[o]); x rows ldx apart, h planes of 32 channels
 // (dense 2 KB per 32 tokens for the epilogue's TMA stores: half-line stores into 64-channel planes cost this GEMM 2x).
-msla_status_t run_ffn_expand_bf16(const void* x, const void* w1, const void* b1, void* h, int B, int C, int Ch, int N, int act,
+msla_status_t run_ffn_expand_bf16(const void* x, int ldx, const void* w1, const void* b1, void* h, int B, int C, int Ch, int N, int act,
                                   cudaStream_t st, bool f16) {
   CUtensorMap tmA, tmB, tmO;
   const cuuint64_t dims[3] = {32, (cuuint64_t)N, (cuuint64_t)B * (Ch / 32)};
   const cuuint64_t strides[2] = {64, (cuuint64_t)N * 64};
   const cuuint32_t box[3] = {32, 32, 1};
-  if (!make_map(&tmA, x, (uint64_t)N, (uint64_t)C, (uint64_t)B, (uint64_t)N * 2, (uint64_t)C * N * 2, 64, BK) ||
+  if (!make_map(&tmA, x, (uint64_t)N, (uint64_t)C, (uint64_t)B, (uint64_t)ldx * 2, (uint64_t)C * ldx * 2, 64, BK) ||
       !make_map(&tmB, w1, (uint64_t)C, (uint64_t)Ch, 1, (uint64_t)C * 2, (uint64_t)C * Ch * 2, BK, BN) ||
       !tma_make_map_bf16(&tmO, h, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B))
     return fail(MSLA_ERR_CUDA, "cuTensorMapEncodeTiled failed for the FFN's first layer");
@@ -691,13 +690,13 @@ msla_status_t run_ffn_expand_bf16(const void* x, const void* w1, const void* b1,
   return f16 ? launch<true, false, 1, true>(tmA, tmB, tmO, p, st) : launch<true, false, 1>(tmA, tmB, tmO, p, st);
 }
 
-// Second layer: y[b][m][n] = sum_j w2[m][j] * g[b][j / 64][n][j % 64] + b2[m] (+ residual[b][m][n]); g planes of 64 channels, y NCHW.
-msla_status_t run_ffn_project_bf16(const void* g, const void* w2, const void* b2, const void* residual, void* y, int B, int Ch,
+// Second layer: y[b][m][n] = sum_j w2[m][j] * g[b][j / 64][n][j % 64] + b2[m] (+ residual[b][m][n]); g planes of 64 channels, rows of y and residual ldy apart.
+msla_status_t run_ffn_project_bf16(const void* g, const void* w2, const void* b2, const void* residual, void* y, int ldy, int B, int Ch,
                                    int Cout, int N, cudaStream_t st, bool f16) {
   CUtensorMap tmA, tmB, tmO;
   const int planes = Ch / 64;
   const cuuint64_t dO[3] = {(cuuint64_t)N, (cuuint64_t)Cout, (cuuint64_t)B};
-  const cuuint64_t sO[2] = {(cuuint64_t)N * 2, (cuuint64_t)Cout * N * 2};
+  const cuuint64_t sO[2] = {(cuuint64_t)ldy * 2, (cuuint64_t)Cout * ldy * 2};
   const cuuint32_t bO[3] = {32, 32, 1};
   if (!make_map(&tmA, w2, (uint64_t)Ch, (uint64_t)Cout, 1, (uint64_t)Ch * 2, (uint64_t)Ch * Cout * 2, BK, BM) ||
       !make_map(&tmB, g, 64, (uint64_t)N, (uint64_t)B * planes, 128, (uint64_t)N * 128, BK, BN) ||
@@ -706,7 +705,7 @@ msla_status_t run_ffn_project_bf16(const void* g, const void* w2, const void* b2
   GemmParams p{};
   p.M = Cout; p.N = N; p.K = Ch; p.batches = B;
   p.m_tiles = (Cout + BM - 1) / BM; p.n_tiles = (N + BN - 1) / BN;
-  p.out_batch_stride = (long long)Cout * N; p.ld_out = N; p.group = 0; p.bias_per_row = 1; p.n_fastest = 0;
+  p.out_batch_stride = (long long)Cout * ldy; p.ld_out = ldy; p.group = 0; p.bias_per_row = 1; p.n_fastest = 0;
   p.bias = (const bf16*)b2; p.out = (bf16*)y;
   p.tma_store = 1; p.planes_per_batch = planes;
   p.residual = (const bf16*)residual;

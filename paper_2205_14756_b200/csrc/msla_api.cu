@@ -265,6 +265,11 @@ struct ForwardPlan {
   int Cp, N;
   int S;              // branches: the projected tokens and S - 1 aggregated copies
   size_t wpad2_off;   // embedded taps of the second aggregated branch
+  // 16-bit storage: the projections read x and write out as rows of `pitch` elements; where H*W is no multiple of 8 those
+  // are padded copies in the workspace (repack.cu), otherwise the caller's tensors
+  int pitch;
+  size_t xpad_off, ypad_off;
+  bool padded() const { return pitch != N; }
 };
 
 static msla_status_t validate_desc(const msla_desc* d, ForwardPlan* plan) {
@@ -280,7 +285,7 @@ static msla_status_t validate_desc(const msla_desc* d, ForwardPlan* plan) {
   if (d->n_scales == 3 && d->agg_kernel2 != 5 && d->agg_kernel2 != 3)
     return fail(MSLA_ERR_UNSUPPORTED, "agg_kernel2 = %d; 5x5 and 3x3 aggregation are supported", d->agg_kernel2);
   if (d->d != 16 && d->d != 32) return fail(MSLA_ERR_UNSUPPORTED, "d = %d; only 16 and 32 are supported", d->d);
-  if ((long long)d->H * d->W > 0x7fffffffLL) return fail(MSLA_ERR_UNSUPPORTED, "H*W exceeds 2^31-1");
+  if ((long long)d->H * d->W > 0x7ffffff8LL) return fail(MSLA_ERR_UNSUPPORTED, "H*W exceeds 2^31-8");
   if (d->C % 8 != 0 || d->C_out % 8 != 0) return fail(MSLA_ERR_UNSUPPORTED, "C and C_out must be multiples of 8");
   const int S = d->n_scales;
   if ((long long)d->B * S * d->heads > 65535 || d->B > 65535) return fail(MSLA_ERR_UNSUPPORTED, "B*n_scales*heads exceeds 65535");
@@ -294,12 +299,16 @@ static msla_status_t validate_desc(const msla_desc* d, ForwardPlan* plan) {
   plan->att_off = align_up(tokens * 3 * S * plan->Cp * e, 256);
   // the attention output's region doubles as scratch of the fused apply + projection kernel, which writes no attention output
   size_t att_bytes = tokens * S * plan->Cp * e;
-  const size_t fused_scratch = fused_out_bf16_supported(S * d->heads, d->d, d->C_out, plan->N) ? fused_out_scratch_bytes(d->B, S * d->heads, d->d, d->C_out) : 0;
+  const size_t fused_scratch = fused_out_bf16_supported(S * d->heads, d->d, d->C_out) ? fused_out_scratch_bytes(d->B, S * d->heads, d->d, d->C_out) : 0;
   if (att_bytes < fused_scratch) att_bytes = fused_scratch;
   plan->core_off = plan->att_off + align_up(att_bytes, 256);
   plan->wpad_off = plan->core_off + plan->core.bytes;
   plan->wpad2_off = plan->wpad_off + (d->agg_kernel == 3 ? align_up((size_t)3 * plan->Cp * 25 * e, 256) : 0);
-  plan->bytes = plan->wpad2_off + (S == 3 && d->agg_kernel2 == 3 ? align_up((size_t)3 * plan->Cp * 25 * e, 256) : 0);
+  plan->xpad_off = plan->wpad2_off + (S == 3 && d->agg_kernel2 == 3 ? align_up((size_t)3 * plan->Cp * 25 * e, 256) : 0);
+  plan->pitch = d->dtype == MSLA_F32 ? plan->N : (int)align_up((size_t)plan->N, 8);
+  plan->ypad_off = plan->xpad_off + (plan->padded() ? align_up((size_t)d->B * d->C * plan->pitch * e, 256) : 0);
+  // (bands of such an image may be ragged where the whole is not, so the output's copy depends on the row length)
+  plan->bytes = plan->ypad_off + (d->dtype != MSLA_F32 && d->W % 8 != 0 ? align_up((size_t)d->B * d->C_out * plan->pitch * e, 256) : 0);
   return MSLA_OK;
 }
 
@@ -310,10 +319,10 @@ static void launch_gemm(const T* A, const T* W, const T* bias, T* D, generic::Ge
   count_launches(1);
 }
 
-// y planar: y[b*y_sb + ((o/d)*N + n)*d + o%d]
-static msla_status_t run_project_in(msla_dtype_t dt, const void* x, const void* w, void* y, int B,
+// y planar: y[b*y_sb + ((o/d)*N + n)*d + o%d]; rows of x are ldx elements apart (N where the plain kernels run)
+static msla_status_t run_project_in(msla_dtype_t dt, const void* x, int ldx, const void* w, void* y, int B,
                                     int C, int Cout, int N, int d, long long y_sb, cudaStream_t st) {
-  if (dt != MSLA_F32 && project_in_bf16_supported(C, Cout, N, d)) return run_project_in_bf16(x, w, y, B, C, Cout, N, d, y_sb, st, dt == MSLA_F16);
+  if (dt != MSLA_F32 && project_in_bf16_supported(C, Cout, ldx, d)) return run_project_in_bf16(x, ldx, w, y, B, C, Cout, N, d, y_sb, st, dt == MSLA_F16);
   generic::GemmArgs g{(long long)C * N, 1, N, y_sb, d, 1, (long long)N * d, N, Cout, C, d};
   if (dt == MSLA_F32) launch_gemm<float>((const float*)x, (const float*)w, nullptr, (float*)y, g, B, st);
   else if (dt == MSLA_F16) launch_gemm<__half>((const __half*)x, (const __half*)w, nullptr, (__half*)y, g, B, st);
@@ -322,9 +331,9 @@ static msla_status_t run_project_in(msla_dtype_t dt, const void* x, const void* 
 }
 
 static msla_status_t run_project_out(msla_dtype_t dt, const void* a, const void* w, const void* bias,
-                                     void* y, int B, int Cin, int Cout, int N, cudaStream_t st, const void* residual = nullptr) {
-  if (dt != MSLA_F32 && project_out_bf16_supported(Cin, Cout, N))
-    return run_project_out_bf16(a, w, bias, residual, y, B, Cin, Cout, N, st, dt == MSLA_F16);
+                                     void* y, int ldy, int B, int Cin, int Cout, int N, cudaStream_t st, const void* residual = nullptr) {
+  if (dt != MSLA_F32 && project_out_bf16_supported(Cin, Cout, ldy))
+    return run_project_out_bf16(a, w, bias, residual, y, ldy, B, Cin, Cout, N, st, dt == MSLA_F16);
   generic::GemmArgs g{(long long)N * Cin, Cin, 1, (long long)Cout * N, 1, N, 0, N, Cout, Cin, Cout, 0, residual};
   if (dt == MSLA_F32) launch_gemm<float>((const float*)a, (const float*)w, (const float*)bias, (float*)y, g, B, st);
   else if (dt == MSLA_F16) launch_gemm<__half>((const __half*)a, (const __half*)w, (const __half*)bias, (__half*)y, g, B, st);
@@ -410,9 +419,10 @@ static msla_status_t record(void* const* events, int i, cudaStream_t st) {
 }
 
 // host_io: x and out are host pointers staged through the tail of the workspace.
-// residual: nullptr, or a device tensor shaped like out that the output projection adds (the block's first residual connection).
+// add_x: the output projection adds x (the block's first residual connection; C_out == C).
+// out_padded: receives the address of the padded copy of out where there is one (else of out itself).
 static msla_status_t forward_impl(const msla_desc* desc, const void* x, const msla_weights* w, void* out,
-                                  cudaStream_t st, void* const* events, bool host_io, const void* residual = nullptr) {
+                                  cudaStream_t st, void* const* events, bool host_io, bool add_x = false, const void** out_padded = nullptr) {
   ForwardPlan p;
   msla_status_t s = validate_desc(desc, &p);
   if (s != MSLA_OK) return s;
@@ -455,8 +465,16 @@ static msla_status_t forward_impl(const msla_desc* desc, const void* x, const ms
   char* ms = ws + p.ms_off;
   char* att = ws + p.att_off;  // [B, N, 2C'] token-major head concat
   if ((s = record(events, 0, st)) != MSLA_OK) return s;
+  void* y_dev = out_dev;
+  if (p.padded()) {
+    if ((s = run_pad_rows(x_dev, ws + p.xpad_off, (long long)desc->B * desc->C, N, p.pitch, st)) != MSLA_OK) return s;
+    x_dev = ws + p.xpad_off;
+    y_dev = ws + p.ypad_off;
+  }
+  const void* residual = add_x ? x_dev : nullptr;
+  if (out_padded) *out_padded = y_dev;
   // 1. QKV projection into the scale-0 planes
-  s = run_project_in(desc->dtype, x_dev, w->w_qkv, ms, desc->B, desc->C, 3 * Cp, N, d, ms_sb, st);
+  s = run_project_in(desc->dtype, x_dev, p.pitch, w->w_qkv, ms, desc->B, desc->C, 3 * Cp, N, d, ms_sb, st);
   if (s != MSLA_OK) return s;
   if ((s = record(events, 1, st)) != MSLA_OK) return s;
   // 2. aggregation of every scale-0 plane into the matching scale-1 plane
@@ -468,11 +486,11 @@ static msla_status_t forward_impl(const msla_desc* desc, const void* x, const ms
   // take it (dense 128-byte rows for the apply kernel's stores and the GEMM's tile loads),
   // otherwise token-major [N][2C'].
   const bool f16 = desc->dtype == MSLA_F16;
-  const bool att_planar = desc->dtype != MSLA_F32 && d == 32 && Ht % 2 == 0 && project_out_planar_bf16_supported(S * Cp, desc->C_out, N);
+  const bool att_planar = desc->dtype != MSLA_F32 && d == 32 && Ht % 2 == 0 && project_out_planar_bf16_supported(S * Cp, desc->C_out);
   const HeadView ov = att_planar ? HeadView{(long long)N * ld_att, (long long)N * 2 * d, 2 * d, 1}
                                  : HeadView{(long long)N * ld_att, d, ld_att, 0};
   // Steps 4 and 5 run as one kernel when it takes the shape: the head concat then stays in shared memory.
-  const bool fused = desc->dtype != MSLA_F32 && fused_out_bf16_supported(Ht, d, desc->C_out, N);
+  const bool fused = desc->dtype != MSLA_F32 && fused_out_bf16_supported(Ht, d, desc->C_out);
   s = run_core(desc->dtype, ms, ms + (size_t)N * d * e, ms + (size_t)2 * N * d * e, att, in, ov, desc->B, Ht, N, d, desc->eps, p.core,
                ws + p.core_off, st, events ? (cudaEvent_t)events[3] : nullptr, fused ? CORE_STATE : CORE_ALL);
   if (s != MSLA_OK) return s;
@@ -480,11 +498,12 @@ static msla_status_t forward_impl(const msla_desc* desc, const void* x, const ms
   // 5. output projection back to NCHW
   if (fused)
     s = run_fused_out_bf16(ms, ms_sb, 3LL * N * d, reinterpret_cast<const float*>(ws + p.core_off + p.core.partial_off), p.core.S, att, w->w_proj,
-                           w->b_proj, residual, out_dev, desc->B, Ht, d, N, desc->C_out, desc->eps, st, f16);
+                           w->b_proj, residual, y_dev, p.pitch, desc->B, Ht, d, N, desc->C_out, desc->eps, st, f16);
   else
-    s = att_planar ? run_project_out_planar_bf16(att, w->w_proj, w->b_proj, residual, out_dev, desc->B, S * Cp, desc->C_out, N, st, f16)
-                   : run_project_out(desc->dtype, att, w->w_proj, w->b_proj, out_dev, desc->B, S * Cp, desc->C_out, N, st, residual);
+    s = att_planar ? run_project_out_planar_bf16(att, w->w_proj, w->b_proj, residual, y_dev, p.pitch, desc->B, S * Cp, desc->C_out, N, st, f16)
+                   : run_project_out(desc->dtype, att, w->w_proj, w->b_proj, y_dev, p.pitch, desc->B, S * Cp, desc->C_out, N, st, residual);
   if (s != MSLA_OK) return s;
+  if (p.padded() && (s = run_unpad_rows(y_dev, out_dev, (long long)desc->B * desc->C_out, N, p.pitch, st)) != MSLA_OK) return s;
   if ((s = record(events, 5, st)) != MSLA_OK) return s;
   if (host_io) {
     const cudaError_t ce = cudaMemcpyAsync(out, out_dev, ob, cudaMemcpyDeviceToHost, st);
@@ -545,7 +564,11 @@ static msla_status_t band_states_impl(const msla_desc* desc, const void* x, cons
   const int Cp = p.Cp, N = p.N, d = desc->d;
   const long long ms_sb = 3LL * p.S * Cp * N;
   char* ms = ws + p.ms_off;
-  s = run_project_in(desc->dtype, x, w->w_qkv, ms, desc->B, desc->C, 3 * Cp, N, d, ms_sb, st);
+  if (p.padded()) {
+    if ((s = run_pad_rows(x, ws + p.xpad_off, (long long)desc->B * desc->C, N, p.pitch, st)) != MSLA_OK) return s;
+    x = ws + p.xpad_off;
+  }
+  s = run_project_in(desc->dtype, x, p.pitch, w->w_qkv, ms, desc->B, desc->C, 3 * Cp, N, d, ms_sb, st);
   if (s != MSLA_OK) return s;
   if ((s = run_branches(desc, w, p, ms, ms_sb, st)) != MSLA_OK) return s;
   const HeadView in{ms_sb, 3LL * N * d, d};
@@ -590,18 +613,26 @@ static msla_status_t band_output_impl(const msla_desc* desc, const msla_weights*
   count_launches(1);
   if ((s = check_launch("sum of the bands' states")) != MSLA_OK) return s;
   const char* q = ms + (size_t)b.tok_off * d * e;
-  if (desc->dtype != MSLA_F32 && fused_out_bf16_supported(Ht, d, desc->C_out, Nb))
-    return run_fused_out_bf16(q, ms_sb, 3LL * N * d, state, 1, att, w->w_proj, w->b_proj, nullptr, out, desc->B, Ht, d, Nb, desc->C_out, desc->eps, st,
-                              desc->dtype == MSLA_F16);
-  const HeadView in{ms_sb, 3LL * N * d, d};
-  const bool att_planar = desc->dtype != MSLA_F32 && d == 32 && Ht % 2 == 0 && project_out_planar_bf16_supported(p.S * Cp, desc->C_out, Nb);
-  const HeadView ov = att_planar ? HeadView{(long long)Nb * ld_att, (long long)Nb * 2 * d, 2 * d, 1}
-                                 : HeadView{(long long)Nb * ld_att, d, ld_att, 0};
-  s = run_core(desc->dtype, q, q + (size_t)N * d * e, q + (size_t)2 * N * d * e, att, in, ov, desc->B, Ht, Nb, d, desc->eps, b.core,
-               ws + p.core_off, st, nullptr, CORE_APPLY);
-  if (s != MSLA_OK) return s;
-  return att_planar ? run_project_out_planar_bf16(att, w->w_proj, w->b_proj, nullptr, out, desc->B, p.S * Cp, desc->C_out, Nb, st, desc->dtype == MSLA_F16)
-                    : run_project_out(desc->dtype, att, w->w_proj, w->b_proj, out, desc->B, p.S * Cp, desc->C_out, Nb, st);
+  const bool f16 = desc->dtype == MSLA_F16;
+  // a band whose token count is no multiple of 8 leaves through the padded copy (reserved for the band with its halo)
+  const int pitch = desc->dtype == MSLA_F32 ? Nb : (int)align_up((size_t)Nb, 8);
+  const bool padded = pitch != Nb;
+  void* y = padded ? ws + p.ypad_off : out;
+  if (desc->dtype != MSLA_F32 && fused_out_bf16_supported(Ht, d, desc->C_out)) {
+    s = run_fused_out_bf16(q, ms_sb, 3LL * N * d, state, 1, att, w->w_proj, w->b_proj, nullptr, y, pitch, desc->B, Ht, d, Nb, desc->C_out, desc->eps, st, f16);
+  } else {
+    const HeadView in{ms_sb, 3LL * N * d, d};
+    const bool att_planar = desc->dtype != MSLA_F32 && d == 32 && Ht % 2 == 0 && project_out_planar_bf16_supported(p.S * Cp, desc->C_out);
+    const HeadView ov = att_planar ? HeadView{(long long)Nb * ld_att, (long long)Nb * 2 * d, 2 * d, 1}
+                                   : HeadView{(long long)Nb * ld_att, d, ld_att, 0};
+    s = run_core(desc->dtype, q, q + (size_t)N * d * e, q + (size_t)2 * N * d * e, att, in, ov, desc->B, Ht, Nb, d, desc->eps, b.core,
+                 ws + p.core_off, st, nullptr, CORE_APPLY);
+    if (s != MSLA_OK) return s;
+    s = att_planar ? run_project_out_planar_bf16(att, w->w_proj, w->b_proj, nullptr, y, pitch, desc->B, p.S * Cp, desc->C_out, Nb, st, f16)
+                   : run_project_out(desc->dtype, att, w->w_proj, w->b_proj, y, pitch, desc->B, p.S * Cp, desc->C_out, Nb, st);
+  }
+  if (s != MSLA_OK || !padded) return s;
+  return run_unpad_rows(y, out, (long long)desc->B * desc->C_out, Nb, pitch, st);
 }
 
 // ---------------------------------------------------------- FFN with a depthwise convolution
@@ -609,6 +640,9 @@ struct FfnPlan {
   size_t h_off, g_off, bytes;
   int N;
   bool tuned;  // bf16 / fp16 tensor-core path with the hidden tensor as planes of 64 channels
+  int pitch;   // tuned: elements between rows of x and out; padded copies in the workspace where that is not H*W
+  size_t xpad_off, ypad_off;
+  bool padded() const { return pitch != N; }
 };
 
 static msla_status_t validate_ffn(const msla_ffn_desc* d, FfnPlan* plan) {
@@ -621,21 +655,25 @@ static msla_status_t validate_ffn(const msla_ffn_desc* d, FfnPlan* plan) {
     return fail(MSLA_ERR_INVALID_ARG, "unknown activation %d", (int)d->act);
   if (d->dw_kernel != 3) return fail(MSLA_ERR_UNSUPPORTED, "dw_kernel = %d; only the 3x3 depthwise convolution is supported", d->dw_kernel);
   if (d->residual && d->C_out != d->C) return fail(MSLA_ERR_INVALID_ARG, "the residual connection needs C_out == C (%d, %d)", d->C_out, d->C);
-  if ((long long)d->H * d->W > 0x7fffffffLL) return fail(MSLA_ERR_UNSUPPORTED, "H*W exceeds 2^31-1");
+  if ((long long)d->H * d->W > 0x7ffffff8LL) return fail(MSLA_ERR_UNSUPPORTED, "H*W exceeds 2^31-8");
   if (d->C % 8 != 0 || d->C_hidden % 8 != 0 || d->C_out % 8 != 0) return fail(MSLA_ERR_UNSUPPORTED, "C, C_hidden and C_out must be multiples of 8");
   if (d->B > 65535) return fail(MSLA_ERR_UNSUPPORTED, "B exceeds 65535");
   plan->N = d->H * d->W;
-  plan->tuned = d->dtype != MSLA_F32 && ffn_bf16_supported(d->C, d->C_hidden, d->C_out, plan->N) &&
+  plan->tuned = d->dtype != MSLA_F32 && ffn_bf16_supported(d->C, d->C_hidden, d->C_out) &&
                 (long long)d->B * (d->C_hidden / 64) <= 65535;
   const size_t hid = align_up((size_t)d->B * d->C_hidden * plan->N * elem_size(d->dtype), 256);
   plan->h_off = 0;
   plan->g_off = hid;
-  plan->bytes = 2 * hid;
+  plan->pitch = plan->tuned ? (int)align_up((size_t)plan->N, 8) : plan->N;
+  plan->xpad_off = 2 * hid;
+  plan->ypad_off = plan->xpad_off + (plan->padded() ? align_up((size_t)d->B * d->C * plan->pitch * 2, 256) : 0);
+  plan->bytes = plan->ypad_off + (plan->padded() ? align_up((size_t)d->B * d->C_out * plan->pitch * 2, 256) : 0);
   return MSLA_OK;
 }
 
+// x_padded: a copy of x with rows of the plan's pitch that the caller already has, or nullptr.
 static msla_status_t ffn_impl(const msla_ffn_desc* desc, const void* x, const msla_ffn_weights* w, void* out, bool residual,
-                              cudaStream_t st) {
+                              cudaStream_t st, const void* x_padded = nullptr) {
   FfnPlan p;
   msla_status_t s = validate_ffn(desc, &p);
   if (s != MSLA_OK) return s;
@@ -655,16 +693,25 @@ static msla_status_t ffn_impl(const msla_ffn_desc* desc, const void* x, const ms
   char* ws = (char*)desc->workspace;
   void* h = ws + p.h_off;
   void* g = ws + p.g_off;
-  const void* res = residual ? x : nullptr;
   if (p.tuned) {
     const bool f16 = desc->dtype == MSLA_F16;
-    if ((s = run_ffn_expand_bf16(x, w->w1, w->b1, h, B, C, Ch, N, act, st, f16)) != MSLA_OK) return s;
+    void* y = out;
+    if (p.padded()) {
+      if (!x_padded) {
+        if ((s = run_pad_rows(x, ws + p.xpad_off, (long long)B * C, N, p.pitch, st)) != MSLA_OK) return s;
+        x_padded = ws + p.xpad_off;
+      }
+      x = x_padded;
+      y = ws + p.ypad_off;
+    }
+    if ((s = run_ffn_expand_bf16(x, p.pitch, w->w1, w->b1, h, B, C, Ch, N, act, st, f16)) != MSLA_OK) return s;
     if ((s = run_ffn_dw3x3_bf16(h, w->w_dw, w->b_dw, g, B, Ch, desc->H, desc->W, act, st, f16)) != MSLA_OK) return s;
-    return run_ffn_project_bf16(g, w->w2, w->b2, res, out, B, Ch, Co, N, st, f16);
+    if ((s = run_ffn_project_bf16(g, w->w2, w->b2, residual ? x : nullptr, y, p.pitch, B, Ch, Co, N, st, f16)) != MSLA_OK) return s;
+    return p.padded() ? run_unpad_rows(y, out, (long long)B * Co, N, p.pitch, st) : MSLA_OK;
   }
   // plain kernels, hidden tensor NCHW
   generic::GemmArgs g1{(long long)C * N, 1, N, (long long)Ch * N, 1, N, 0, N, Ch, C, Ch, act, nullptr};
-  generic::GemmArgs g2{(long long)Ch * N, 1, N, (long long)Co * N, 1, N, 0, N, Co, Ch, Co, 0, res};
+  generic::GemmArgs g2{(long long)Ch * N, 1, N, (long long)Co * N, 1, N, 0, N, Co, Ch, Co, 0, residual ? x : nullptr};
   const long long total = (long long)B * Ch * N;
   auto plain = [&](auto* tag) {
     using T = std::remove_pointer_t<decltype(tag)>;
@@ -698,8 +745,9 @@ static msla_status_t block_impl(const msla_desc* attn, const msla_weights* aw, c
       (attn->workspace && overlaps(y, bytes, attn->workspace, ap.bytes)) || (ffn->workspace && overlaps(y, bytes, ffn->workspace, fp.bytes)))
     return fail(MSLA_ERR_INVALID_ARG, "y overlaps x, out or a workspace");
   // y = MSLA(x) + x: the output projection's epilogue adds the residual
-  if ((s = forward_impl(attn, x, aw, y, st, nullptr, false, x)) != MSLA_OK) return s;
-  return ffn_impl(ffn, y, fw, out, true, st);
+  const void* y_padded = nullptr;
+  if ((s = forward_impl(attn, x, aw, y, st, nullptr, false, true, &y_padded)) != MSLA_OK) return s;
+  return ffn_impl(ffn, y, fw, out, true, st, ap.padded() ? y_padded : nullptr);
 }
 
 }  // namespace msla
@@ -791,7 +839,7 @@ msla_status_t msla_evit_block(const msla_desc* attn, const msla_weights* aw, con
 int msla_forward_fuses_apply(const msla_desc* desc) {
   ForwardPlan p;
   if (validate_desc(desc, &p) != MSLA_OK) return -1;
-  return desc->dtype == MSLA_BF16 && fused_out_bf16_supported(p.S * desc->heads, desc->d, desc->C_out, p.N) ? 1 : 0;
+  return desc->dtype == MSLA_BF16 && fused_out_bf16_supported(p.S * desc->heads, desc->d, desc->C_out) ? 1 : 0;
 }
 
 unsigned long long msla_kernel_launches(void) { return g_launches; }
@@ -817,7 +865,7 @@ msla_status_t msla_project_in(msla_dtype_t dtype, const void* x, const void* w, 
   if (!aligned16(x) || !aligned16(w) || !aligned16(y)) return fail(MSLA_ERR_ALIGNMENT, "pointers must be 16-byte aligned");
   msla_status_t s = check_arch();
   if (s != MSLA_OK) return s;
-  return run_project_in(dtype, x, w, y, B, C, Cout, N, d, (long long)Cout * N, (cudaStream_t)stream);
+  return run_project_in(dtype, x, N, w, y, B, C, Cout, N, d, (long long)Cout * N, (cudaStream_t)stream);
 }
 
 msla_status_t msla_aggregate(msla_dtype_t dtype, const void* t, const void* w_dw, const void* w_pw, void* y, int B, int H, int W, int Ch, int d, void* stream) {
@@ -844,7 +892,7 @@ msla_status_t msla_project_out(msla_dtype_t dtype, const void* a, const void* w,
   if (!aligned16(a) || !aligned16(w) || !aligned16(y) || (bias && !aligned16(bias))) return fail(MSLA_ERR_ALIGNMENT, "pointers must be 16-byte aligned");
   msla_status_t s = check_arch();
   if (s != MSLA_OK) return s;
-  return run_project_out(dtype, a, w, bias, y, B, Cin, Cout, N, (cudaStream_t)stream);
+  return run_project_out(dtype, a, w, bias, y, N, B, Cin, Cout, N, (cudaStream_t)stream);
 }
 
 const char* msla_status_string(msla_status_t s) {

@@ -104,35 +104,36 @@ msla_status_t run_core_bf16(const void* q, const void* k, const void* v, void* o
 // FFN with a depthwise convolution (gemm_tcgen05.cu, ffn_dw_bf16.cu): bf16; the hidden tensor is planes of 32 channels
 // [B][Ch / 32][N][32] after the first layer, planes of 64 channels [B][Ch / 64][N][64] after the depthwise convolution.
 // act: 0 none, 1 ReLU, 2 hard-swish.
-bool ffn_bf16_supported(int C, int Ch, int Cout, int N);
-msla_status_t run_ffn_expand_bf16(const void* x, const void* w1, const void* b1, void* h, int B, int C, int Ch, int N, int act,
+bool ffn_bf16_supported(int C, int Ch, int Cout);
+// ldx, ldy: elements between rows (tokens of one channel) of x, and of y and the residual; multiples of 8, as tensor maps need.
+msla_status_t run_ffn_expand_bf16(const void* x, int ldx, const void* w1, const void* b1, void* h, int B, int C, int Ch, int N, int act,
                                   cudaStream_t st, bool f16 = false);
 msla_status_t run_ffn_dw3x3_bf16(const void* h, const void* w_dw, const void* b_dw, void* g, int B, int Ch, int H, int W, int act,
                                  cudaStream_t st, bool f16 = false);
-msla_status_t run_ffn_project_bf16(const void* g, const void* w2, const void* b2, const void* residual, void* y, int B, int Ch,
+msla_status_t run_ffn_project_bf16(const void* g, const void* w2, const void* b2, const void* residual, void* y, int ldy, int B, int Ch,
                                    int Cout, int N, cudaStream_t st, bool f16 = false);
 
 // Apply step and output projection as one GEMM per image (fused_out.cu): bf16, d in {16, 32}, at most 512 attention
 // channels and 256 output channels.  q: planar query matrices [N][d], head h of image b at q + b*q_sb + h*q_sh
 // (elements).
-bool fused_out_bf16_supported(int Ht, int d, int Cout, int N);
+bool fused_out_bf16_supported(int Ht, int d, int Cout);
 size_t fused_out_scratch_bytes(int B, int Ht, int d, int Cout);
 msla_status_t run_fused_out_bf16(const void* q, long long q_sb, long long q_sh, const float* partial, int S, void* scratch,
-                                 const void* w, const void* bias, const void* residual, void* y, int B, int Ht, int d, int N, int Cout,
+                                 const void* w, const void* bias, const void* residual, void* y, int ldy, int B, int Ht, int d, int N, int Cout,
                                  float eps, cudaStream_t st, bool f16 = false);
 int fused_timeout_flag();
 int dw_timeout_flag();
 
 // bf16 projections on tcgen05 tensor cores (gemm_tcgen05.cu).
-bool project_in_bf16_supported(int C, int Cout, int N, int d);
-msla_status_t run_project_in_bf16(const void* x, const void* w, void* y, int B, int C, int Cout, int N, int d,
+bool project_in_bf16_supported(int C, int Cout, int ldx, int d);
+msla_status_t run_project_in_bf16(const void* x, int ldx, const void* w, void* y, int B, int C, int Cout, int N, int d,
                                   long long y_batch_stride, cudaStream_t st, bool f16 = false);
-bool project_out_bf16_supported(int Cin, int Cout, int N);
+bool project_out_bf16_supported(int Cin, int Cout, int ldy);
 // residual: nullptr, or a tensor shaped like y that is added to it
-msla_status_t run_project_out_bf16(const void* a, const void* w, const void* bias, const void* residual, void* y, int B, int Cin,
+msla_status_t run_project_out_bf16(const void* a, const void* w, const void* bias, const void* residual, void* y, int ldy, int B, int Cin,
                                    int Cout, int N, cudaStream_t st, bool f16 = false);
-bool project_out_planar_bf16_supported(int Cin, int Cout, int N);
-msla_status_t run_project_out_planar_bf16(const void* a, const void* w, const void* bias, const void* residual, void* y, int B,
+bool project_out_planar_bf16_supported(int Cin, int Cout);
+msla_status_t run_project_out_planar_bf16(const void* a, const void* w, const void* bias, const void* residual, void* y, int ldy, int B,
                                           int Cin, int Cout, int N, cudaStream_t st, bool f16 = false);
 int gemm_timeout_flag();
 int run_wait_selftest(long long limit_cycles, int* scratch, cudaStream_t st);
@@ -144,5 +145,9 @@ msla_status_t run_aggregate_bf16(const void* src, long long src_planes_total, in
                                  const void* w_pw, void* dst, long long dst_sb, int B, int H, int W, int Ch, int d,
                                  cudaStream_t st, bool f16 = false);
 int agg_timeout_flag();
+
+// Rows of n 16-bit elements to and from rows `pitch` (a multiple of 8) elements apart (repack.cu).
+msla_status_t run_pad_rows(const void* src, void* dst, long long rows, int n, int pitch, cudaStream_t st);
+msla_status_t run_unpad_rows(const void* src, void* dst, long long rows, int n, int pitch, cudaStream_t st);
 
 }  // namespace msla
