@@ -160,85 +160,144 @@ template <bool F16> __device__ __forceinline__ uint32_t pack16(float lo, float h
 
 // ---------------------------------------------------------------------------
 // Second level of the state reduction (Eq. 3) and the fold of the state into the projection weights.
-// Grid (B * Ht, chunks): a CTA takes one head and `da` = d / chunks of its key channels a, i.e. `da` consecutive rows of the
-// head's state.  partial: [B*Ht][S][d*(d+1)] fp32, entry [a][c], column d = key sum.
-//   ks[bh][a]            = sum_s partial[bh][s][a][d]
-//   M[b][m][hh*d + a]    = sum_c w[m][hh*d + c] * (sum_s partial[bh][s][a][c])        (bf16, row stride K), all m < Cout
-// Fixed summation order: the S partial states are cut into FOLD_RUNS runs of consecutive indices, each run is summed in
-// index order by its own thread, and the run sums are added in run order.  A thread issues all loads of its run
-// (<= 8 vectors of 16 bytes) before the first add, so the kernel pays one round trip to memory, not S.
+// Grid (B * Ht, D / DA): a CTA takes one head and DA of its key channels a, i.e. DA consecutive rows of the head's state.
+// partial: [B*Ht][S][D*(D+1)] fp32, entry [a][c], column D = key sum.
+//   ks[bh][a]            = sum_s partial[bh][s][a][D]
+//   M[b][m][hh*D + a]    = sum_c w[m][hh*D + c] * (sum_s partial[bh][s][a][c])        (16 bit, row stride K), all m < Cout
+// Fixed summation order: the S partial states are cut into RUNS runs of consecutive indices, each run is summed in index
+// order by its own thread with eight 16-byte loads in flight, and the run sums are added in run order.
+// The product runs on mma.sync with output channels as rows, key channels as columns and c along the contraction.  The
+// weights are 16-bit already; the fp32 state is cut into PIECES 16-bit pieces (bf16: three, which hold all 24 bits; fp16:
+// two, 22 bits of a value that is rounded to 11).  Contraction slots and columns are assigned so that a lane loads 16
+// consecutive bytes of a weight row (8 for D = 16) and, where the CTA has whole rows of M (DA = D), stores as many.
+// Latency bounds it with few heads (one memory round trip, two barriers), the write of M with many.  Against the version
+// that did the product on the fp32 pipes with 1024 threads per CTA: 1024 heads (64 images, S = 1) 73.4 -> 13.7 us, 256
+// heads 22.9 -> 6.4 us, 16 heads (S = 37) 7.0 -> 4.3 us.
 // ---------------------------------------------------------------------------
-constexpr int FOLD_THREADS = 1024;
-constexpr int FOLD_RUNS = 8;       // S <= 64: at most 8 partial states per run
-constexpr int FOLD_RUN_BYTES = FOLD_RUNS * 32 * 33 * 4, FOLD_ST_BYTES = 32 * 33 * 4;
-constexpr int FOLD_SMEM = FOLD_RUN_BYTES + FOLD_ST_BYTES + 256 * 32 * 2;  // + the head's [Cout <= 256][d <= 32] weight columns
+template <int D, int DA> struct FoldShape {
+  static constexpr int RUNS = DA == 8 ? 8 : DA * D >= 1024 ? 1 : 4;
+  static constexpr int NV = DA * (D + 1) / 4;                       // 16-byte vectors of the CTA's rows of a state
+  static constexpr int THREADS = (NV * RUNS + 31) / 32 * 32;        // 288, 544, 544 for D = 32 and DA = 32, 16, 8; 288 for D = 16
+};
+
+template <bool F16>
+__device__ __forceinline__ void fold_mma(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  if constexpr (F16)
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+  else
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
 // F16: M and ks are multiplied by `scale`, a power of two near 1 / N (the output kernel scales eps alike, so Eq. 3's quotient is
 // unchanged): sums over N tokens then stay inside binary16's range.
-template <bool F16>
-__global__ void __launch_bounds__(FOLD_THREADS)
+template <int D, int DA, bool F16>
+__global__ void __launch_bounds__(FoldShape<D, DA>::THREADS, DA == D ? 4 : 1)
 state_fold_kernel(const float* __restrict__ partial, int S, const bf16* __restrict__ w, bf16* __restrict__ M, float* __restrict__ ks,
-                  int Ht, int d, int Cout, int K, int da, float scale) {
-  extern __shared__ __align__(16) unsigned char fold_smem[];
-  float4 (*run_sum)[32 * 33 / 4] = reinterpret_cast<float4 (*)[32 * 33 / 4]>(fold_smem);
-  float* st = reinterpret_cast<float*>(fold_smem + FOLD_RUN_BYTES);
-  uint4* wtile = reinterpret_cast<uint4*>(fold_smem + FOLD_RUN_BYTES + FOLD_ST_BYTES);  // the head's columns of w: [Cout][d] bf16
+                  int Ht, int Cout, int K, float scale) {
+  constexpr int RUNS = FoldShape<D, DA>::RUNS, NV = FoldShape<D, DA>::NV, THREADS = FoldShape<D, DA>::THREADS;
+  constexpr int D1 = D + 1, NE4 = D * D1 / 4, WARPS = THREADS / 32;
+  constexpr int KS = D / 16, NT = DA / 8, PIECES = F16 ? 2 : 3;
+  __shared__ float4 run_sum[RUNS][NV];
+  __shared__ uint32_t rounded[PIECES][DA][D / 2 + 1];  // pairs of neighbouring c
+  float* st = reinterpret_cast<float*>(run_sum[0]);
   pdl_launch_dependents();
-  const int bh = blockIdx.x, b = bh / Ht, hh = bh % Ht;
-  // the projection weights do not come from the previous kernel: staged while it drains
-  for (int i = threadIdx.x; i < Cout * (d / 8); i += FOLD_THREADS) {
-    const int m = i / (d / 8), c8 = i - m * (d / 8);
-    wtile[i] = __ldg(reinterpret_cast<const uint4*>(w + (long long)m * K + hh * d) + c8);  // 16-byte aligned: K and d are multiples of 8
-  }
-  pdl_wait();  // the partial states come from the previous kernel
-  const int d1 = d + 1, ne = d * d1;
-  const int a0 = blockIdx.y * da;
-  const int nq4 = da * d1 / 4;  // this CTA's rows of the state, in 16-byte vectors (da * d1 is a multiple of 4)
-  const float4* sp = reinterpret_cast<const float4*>(partial + (long long)bh * S * ne + a0 * d1);
-  const int ne4 = ne / 4;
-  for (int item = threadIdx.x; item < FOLD_RUNS * nq4; item += FOLD_THREADS) {
-    const int j = item / nq4, e = item - j * nq4;
-    const int s0 = S * j / FOLD_RUNS, s1 = S * (j + 1) / FOLD_RUNS;
-    float4 t[8];
+  const int bh = blockIdx.x, b = bh / Ht, hh = bh % Ht, a0 = blockIdx.y * DA;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+  // A fragments of 16 output channels: lane (g, t) holds c = t*D/4 .. + D/4 - 1 of rows g and g + 8
+  auto load_weights = [&](int m0, uint32_t (&x)[2][D / 8]) {
 #pragma unroll
-    for (int u = 0; u < 8; ++u) t[u] = s0 + u < s1 ? __ldg(sp + (long long)(s0 + u) * ne4 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 v = t[0];
+    for (int r = 0; r < 2; ++r) {
+      const bf16* src = w + (long long)(m0 + g + 8 * r) * K + hh * D + t * (D / 4);
+      const bool ok = m0 + g + 8 * r < Cout;
+      if constexpr (D == 32) {
+        const uint4 v = ok ? __ldg(reinterpret_cast<const uint4*>(src)) : make_uint4(0u, 0u, 0u, 0u);
+        x[r][0] = v.x; x[r][1] = v.y; x[r][2] = v.z; x[r][3] = v.w;
+      } else {
+        const uint2 v = ok ? __ldg(reinterpret_cast<const uint2*>(src)) : make_uint2(0u, 0u);
+        x[r][0] = v.x; x[r][1] = v.y;
+      }
+    }
+  };
+  uint32_t x[2][D / 8];
+  load_weights(16 * warp, x);  // the projection weights do not come from the previous kernel: fetched while it drains
+  pdl_wait();                  // the partial states do
+  const float4* sp = reinterpret_cast<const float4*>(partial + (long long)bh * S * (D * D1) + a0 * D1);
+  if (tid < RUNS * NV) {
+    const int j = tid / NV, e = tid - j * NV;
+    const int s0 = S * j / RUNS, s1 = S * (j + 1) / RUNS;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s = s0; s < s1; s += 8) {
+      float4 q[8];
 #pragma unroll
-    for (int u = 1; u < 8; ++u) { v.x += t[u].x; v.y += t[u].y; v.z += t[u].z; v.w += t[u].w; }
+      for (int u = 0; u < 8; ++u) q[u] = s + u < s1 ? __ldg(sp + (long long)(s + u) * NE4 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) { v.x += q[u].x; v.y += q[u].y; v.z += q[u].z; v.w += q[u].w; }
+    }
     run_sum[j][e] = v;
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < nq4; e += FOLD_THREADS) {
-    float4 v = run_sum[0][e];
+  if (RUNS > 1) {
+    if (tid < NV) {
+      float4 v = run_sum[0][tid];
 #pragma unroll
-    for (int j = 1; j < FOLD_RUNS; ++j) { const float4 r = run_sum[j][e]; v.x += r.x; v.y += r.y; v.z += r.z; v.w += r.w; }
-    reinterpret_cast<float4*>(st)[e] = v;  // st[al * d1 + c], al = a - a0
+      for (int j = 1; j < RUNS; ++j) { const float4 r = run_sum[j][tid]; v.x += r.x; v.y += r.y; v.z += r.z; v.w += r.w; }
+      run_sum[0][tid] = v;  // st[al * D1 + c], al = a - a0
+    }
+    __syncthreads();
+  }
+  if (tid < DA) ks[(long long)bh * D + a0 + tid] = F16 ? st[tid * D1 + D] * scale : st[tid * D1 + D];
+  for (int i = tid; i < DA * D / 2; i += THREADS) {
+    const int al = i / (D / 2), c2 = i - al * (D / 2);
+    float v0 = st[al * D1 + 2 * c2], v1 = st[al * D1 + 2 * c2 + 1];
+    if (F16) { v0 *= scale; v1 *= scale; }
+#pragma unroll
+    for (int k = 0; k < PIECES; ++k) {
+      const uint32_t word = pack16<F16>(v0, v1);
+      rounded[k][al][c2] = word;
+      v0 -= lo16<F16>(word); v1 -= hi16<F16>(word);
+    }
   }
   __syncthreads();
-  for (int al = threadIdx.x; al < da; al += FOLD_THREADS) ks[(long long)bh * d + a0 + al] = F16 ? st[al * d1 + d] * scale : st[al * d1 + d];
-  // M: a thread keeps key channel al = threadIdx.x % da (FOLD_THREADS is a multiple of da), i.e. one row of the state,
-  // in registers and walks the output channels m = threadIdx.x / da, + FOLD_THREADS / da, ...
-  const int al = threadIdx.x % da;
-  float srow[32];
+  // B fragments: column g of tile j is key channel al(j), contraction slots of step i: c = t*D/4 + 4*i + {0 .. 3}; read when
+  // they are needed (held for the whole loop they cost 48 registers, and two of four CTAs per SM)
+  const uint32_t pieces = smem_u32(&rounded[0][0][0]) + (uint32_t)((DA == D ? (g >> 1) * (D / 4) + (g & 1) : g) * (D / 2 + 1) + t * (D / 8)) * 4u;
+  for (int m0 = 16 * warp; m0 < Cout; m0 += 16 * WARPS) {
+    if (m0 != 16 * warp) load_weights(m0, x);
+    float acc[NT][4];
 #pragma unroll
-  for (int c = 0; c < 32; ++c) srow[c] = c < d ? st[al * d1 + c] : 0.f;
-  for (int m = threadIdx.x / da; m < Cout; m += FOLD_THREADS / da) {
-    const uint4* wr = wtile + m * (d / 8);
-    uint4 wv[4];
+    for (int j = 0; j < NT; ++j) {
 #pragma unroll
-    for (int c8 = 0; c8 < 4; ++c8) wv[c8] = c8 < d / 8 ? wr[c8] : make_uint4(0u, 0u, 0u, 0u);
-    float acc = 0.f;
+      for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
 #pragma unroll
-    for (int c8 = 0; c8 < 4; ++c8) {
-      const uint32_t word[4] = {wv[c8].x, wv[c8].y, wv[c8].z, wv[c8].w};
+      for (int k = PIECES - 1; k >= 0; --k)  // small pieces first
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {  // channels beyond d carry zeros on both sides
-        acc = fmaf(lo16<F16>(word[e]), srow[8 * c8 + 2 * e], acc);
-        acc = fmaf(hi16<F16>(word[e]), srow[8 * c8 + 2 * e + 1], acc);
+        for (int i = 0; i < KS; ++i) {
+          const uint32_t A[4] = {x[0][2 * i], x[1][2 * i], x[0][2 * i + 1], x[1][2 * i + 1]};
+          const uint32_t at = pieces + (uint32_t)((k * DA + (DA == D ? 2 : 8) * j) * (D / 2 + 1) + 2 * i) * 4u;
+          uint32_t b0, b1;
+          asm volatile("ld.shared.u32 %0, [%1];" : "=r"(b0) : "r"(at));
+          asm volatile("ld.shared.u32 %0, [%1];" : "=r"(b1) : "r"(at + 4));
+          fold_mma<F16>(acc[j], A, b0, b1);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int m = m0 + g + 8 * r;
+      if (m >= Cout) continue;
+      bf16* row = M + ((long long)b * Cout + m) * K + hh * D + a0;
+      if constexpr (DA == D) {
+        uint32_t o[NT];
+#pragma unroll
+        for (int j = 0; j < NT; ++j) o[j] = pack16<F16>(acc[j][2 * r], acc[j][2 * r + 1]);
+        if constexpr (D == 32) *reinterpret_cast<uint4*>(row + 8 * t) = make_uint4(o[0], o[1], o[2], o[3]);
+        else *reinterpret_cast<uint2*>(row + 4 * t) = make_uint2(o[0], o[1]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < NT; ++j) *reinterpret_cast<uint32_t*>(row + 8 * j + 2 * t) = pack16<F16>(acc[j][2 * r], acc[j][2 * r + 1]);
       }
     }
-    bf16* mp = M + ((long long)b * Cout + m) * K + hh * d + a0 + al;
-    if constexpr (F16) *reinterpret_cast<__half*>(mp) = __float2half_rn(acc * scale);
-    else *mp = __float2bfloat16_rn(acc);
   }
 }
 
@@ -592,6 +651,18 @@ msla_status_t launch_fused(dim3 grid, int smem, cudaStream_t st, const CUtensorM
   launch_pdl_cluster2(fused_out_kernel<D, RES, F16>, grid, dim3(O_THREADS), (size_t)smem, st, tmM, tmQ, tmO, tmR, p);
   return MSLA_OK;
 }
+template <int D, bool F16>
+msla_status_t launch_fold(const float* partial, int S, const void* w, bf16* M, float* ks, int B, int Ht, int Cout, float scale, cudaStream_t st) {
+  // few heads: a head's key channels are shared out, to about one CTA per SM
+  const int heads = B * Ht, sms = device_sm_count(), K = Ht * D;
+  if (D == 32 && 4 * heads <= sms)
+    launch_pdl(state_fold_kernel<D, 8, F16>, dim3(heads, D / 8), dim3(FoldShape<D, 8>::THREADS), 0, st, partial, S, (const bf16*)w, M, ks, Ht, Cout, K, scale);
+  else if (2 * heads <= sms)
+    launch_pdl(state_fold_kernel<D, D / 2, F16>, dim3(heads, 2), dim3(FoldShape<D, D / 2>::THREADS), 0, st, partial, S, (const bf16*)w, M, ks, Ht, Cout, K, scale);
+  else
+    launch_pdl(state_fold_kernel<D, D, F16>, dim3(heads), dim3(FoldShape<D, D>::THREADS), 0, st, partial, S, (const bf16*)w, M, ks, Ht, Cout, K, scale);
+  return check_launch("sum of the partial states");
+}
 template <bool F16>
 msla_status_t launch_fused_for(int d, bool res, dim3 grid, int smem, cudaStream_t st, const CUtensorMap& tmM, const CUtensorMap& tmQ,
                                const CUtensorMap& tmO, const CUtensorMap& tmR, const OutParams& p) {
@@ -607,7 +678,7 @@ msla_status_t run_fused_out_bf16(const void* q, long long q_sb, long long q_sh, 
                                  float eps, cudaStream_t st, bool f16) {
   if (!fused_out_bf16_supported(Ht, d, Cout) || ldy % 8 != 0 || q_sb % 8 != 0 || q_sh % 8 != 0)
     return fail(MSLA_ERR_UNSUPPORTED, "fused apply + projection: %d heads of %d channels, %d output channels, %d tokens", Ht, d, Cout, N);
-  if (S < 1 || S > 8 * FOLD_RUNS) return fail(MSLA_ERR_UNSUPPORTED, "fused apply + projection: %d partial states per head (1 .. %d)", S, 8 * FOLD_RUNS);
+  if (S < 1) return fail(MSLA_ERR_UNSUPPORTED, "fused apply + projection: %d partial states per head", S);
   const int K = Ht * d;
   // 256-token tiles per pair of CTAs; 128-token tiles for problems so small that half the pairs would have nothing
   // to do (the larger tile is the more efficient one as soon as every pair has work)
@@ -653,16 +724,9 @@ msla_status_t run_fused_out_bf16(const void* q, long long q_sb, long long q_sh, 
   long long pairs = sms / 2;
   if (pairs > tiles) pairs = tiles;
   if (pairs < 1) pairs = 1;
-  // about one CTA per SM: few heads -> up to eight CTAs per head, each with a share of the head's key channels
-  // (a share's rows of the state, da * (d + 1) floats, must stay a whole number of 16-byte vectors: da >= 4)
-  int fold_chunks = sms / (B * Ht);
-  fold_chunks = (fold_chunks >= 8 && d == 32) ? 8 : fold_chunks >= 4 ? 4 : (fold_chunks >= 2 ? 2 : 1);
-  static std::atomic<unsigned long long> attr_fold{0}, attr_fold16{0};
-  msla_status_t s = f16 ? ensure_smem_attr(attr_fold16, state_fold_kernel<true>, FOLD_SMEM) : ensure_smem_attr(attr_fold, state_fold_kernel<false>, FOLD_SMEM);
+  msla_status_t s = d == 32 ? (f16 ? launch_fold<32, true>(partial, S, w, M, ks, B, Ht, Cout, scale, st) : launch_fold<32, false>(partial, S, w, M, ks, B, Ht, Cout, scale, st))
+                            : (f16 ? launch_fold<16, true>(partial, S, w, M, ks, B, Ht, Cout, scale, st) : launch_fold<16, false>(partial, S, w, M, ks, B, Ht, Cout, scale, st));
   if (s != MSLA_OK) return s;
-  const dim3 fold_grid((unsigned)(B * Ht), (unsigned)fold_chunks);
-  if (f16) launch_pdl(state_fold_kernel<true>, fold_grid, dim3(FOLD_THREADS), FOLD_SMEM, st, partial, S, (const bf16*)w, M, ks, Ht, d, Cout, K, d / fold_chunks, scale);
-  else launch_pdl(state_fold_kernel<false>, fold_grid, dim3(FOLD_THREADS), FOLD_SMEM, st, partial, S, (const bf16*)w, M, ks, Ht, d, Cout, K, d / fold_chunks, scale);
   const dim3 grid((unsigned)(2 * pairs));
   s = f16 ? launch_fused_for<true>(d, residual != nullptr, grid, smem, st, tmM, tmQ, tmO, tmR, p)
           : launch_fused_for<false>(d, residual != nullptr, grid, smem, st, tmM, tmQ, tmO, tmR, p);
