@@ -121,18 +121,24 @@ static msla_status_t run_core_generic(const T* q, const T* k, const T* v, T* out
   float* state = reinterpret_cast<float*>(ws + p.state_off);
   int launches = 0;
   if (phases & CORE_STATE) {
-    generic::kv_partial_kernel<T><<<dim3((unsigned)BH, p.S), 256, 0, st>>>(k, v, partial, in, heads, N, d, p.S, p.chunk);
+    const dim3 grid((unsigned)BH, p.S);
+    if (d == 32) launch_pdl(generic::kv_partial_kernel<T, 32>, grid, dim3(128), 0, st, k, v, partial, in, heads, N, p.S, p.chunk);
+    else launch_pdl(generic::kv_partial_kernel<T, 16>, grid, dim3(128), 0, st, k, v, partial, in, heads, N, p.S, p.chunk);
     ++launches;
   }
-  if (phases & CORE_COMBINE) {
+  // a single partial state is the state: nothing to add when the apply step follows here
+  const bool one = p.S == 1 && (phases & CORE_STATE) && (phases & CORE_APPLY);
+  if ((phases & CORE_COMBINE) && !one) {
     const long long total = BH * p.ne;
-    generic::kv_combine_kernel<<<(unsigned)ceil_div_ll(total, 256), 256, 0, st>>>(partial, state, p.S, p.ne, total);
+    launch_pdl(generic::kv_combine_kernel, dim3((unsigned)ceil_div_ll(total, 256)), dim3(256), 0, st, partial, state, p.S, p.ne, total);
     ++launches;
   }
   if (mid) cudaEventRecord(mid, st);
   if (phases & CORE_APPLY) {
-    generic::apply_kernel<T><<<dim3((unsigned)ceil_div_ll(N, 128), (unsigned)BH), 128, 0, st>>>(
-        q, state, out, in, ov, heads, N, d, eps);
+    const dim3 grid((unsigned)ceil_div_ll(N, 128), (unsigned)BH);
+    const float* sum = one ? partial : state;
+    if (d == 32) launch_pdl(generic::apply_kernel<T, 32>, grid, dim3(128), 0, st, q, sum, out, in, ov, heads, N, eps);
+    else launch_pdl(generic::apply_kernel<T, 16>, grid, dim3(128), 0, st, q, sum, out, in, ov, heads, N, eps);
     ++launches;
   }
   count_launches(launches);
@@ -312,11 +318,22 @@ static msla_status_t validate_desc(const msla_desc* d, ForwardPlan* plan) {
   return MSLA_OK;
 }
 
+template <typename T, int BM, int BN, int BK, int TM>
+static void launch_gemm_tile(const T* A, const T* W, const T* bias, T* D, generic::GemmArgs g, int B, bool vec, cudaStream_t st) {
+  dim3 grid((unsigned)ceil_div_ll(g.M, BM), (unsigned)ceil_div_ll(g.Nc, BN), (unsigned)B);
+  launch_pdl(generic::gemm_kernel<T, BM, BN, BK, TM>, grid, dim3((BM / TM) * (BN / 4)), 0, st, A, W, bias, D, g, vec);
+  count_launches(1);
+}
+
+// The largest tile that still gives every SM about two CTAs: a larger one feeds more multiply-adds per shared-memory load,
+// a smaller one shortens the serial chain of a small problem.
 template <typename T>
 static void launch_gemm(const T* A, const T* W, const T* bias, T* D, generic::GemmArgs g, int B, cudaStream_t st) {
-  dim3 grid((unsigned)ceil_div_ll(g.M, 64), (unsigned)ceil_div_ll(g.Nc, 64), (unsigned)B);
-  generic::gemm_kernel<T><<<grid, 256, 0, st>>>(A, W, bias, D, g);
-  count_launches(1);
+  const bool vec = g.sDm == 1 ? g.sDn % 4 == 0 && g.sDg % 4 == 0 && g.sDb % 4 == 0 : g.sDm % 4 == 0 && g.sDg % 4 == 0 && g.sDb % 4 == 0;
+  const long long sms = device_sm_count();
+  if ((long long)B * ceil_div_ll(g.M, 128) * ceil_div_ll(g.Nc, 64) >= 2 * sms) launch_gemm_tile<T, 128, 64, 16, 8>(A, W, bias, D, g, B, vec, st);
+  else if ((long long)B * ceil_div_ll(g.M, 64) * ceil_div_ll(g.Nc, 64) >= 2 * sms) launch_gemm_tile<T, 64, 64, 16, 4>(A, W, bias, D, g, B, vec, st);
+  else launch_gemm_tile<T, 32, 32, 32, 4>(A, W, bias, D, g, B, vec, st);
 }
 
 // y planar: y[b*y_sb + ((o/d)*N + n)*d + o%d]; rows of x are ldx elements apart (N where the plain kernels run)
@@ -341,45 +358,53 @@ static msla_status_t run_project_out(msla_dtype_t dt, const void* a, const void*
   return check_launch("output projection");
 }
 
+template <typename T, int D, int TH, int TW>
+static msla_status_t launch_aggregate_tile(const T* src, const T* w_dw, const T* w_pw, T* dst, int B, int H, int W, int groups, long long src_sb, long long dst_sb,
+                                           cudaStream_t st) {
+  constexpr int smem = generic::aggregate_smem<D, TH, TW>();
+  static std::atomic<unsigned long long> attr_done{0};
+  const msla_status_t s = ensure_smem_attr(attr_done, generic::aggregate_kernel<T, D, TH, TW>, smem);
+  if (s != MSLA_OK) return s;
+  const dim3 grid((unsigned)(ceil_div_ll(W, TW) * ceil_div_ll(H, TH)), (unsigned)groups, (unsigned)B);
+  launch_pdl(generic::aggregate_kernel<T, D, TH, TW>, grid, dim3(TH * TW * D / 32), smem, st, src, w_dw, w_pw, dst, H, W, src_sb, dst_sb);
+  count_launches(1);
+  return check_launch("token aggregation");
+}
+// 16 x 16 pixels re-read the halo least (1.56 loads per pixel against 2.25); 8 x 8 where that leaves SMs without a tile
+template <typename T, int D>
+static msla_status_t launch_aggregate(const T* src, const T* w_dw, const T* w_pw, T* dst, int B, int H, int W, int groups, long long src_sb, long long dst_sb,
+                                      cudaStream_t st) {
+  if (ceil_div_ll(W, 16) * ceil_div_ll(H, 16) * groups * B >= device_sm_count())
+    return launch_aggregate_tile<T, D, 16, 16>(src, w_dw, w_pw, dst, B, H, W, groups, src_sb, dst_sb, st);
+  return launch_aggregate_tile<T, D, 8, 8>(src, w_dw, w_pw, dst, B, H, W, groups, src_sb, dst_sb, st);
+}
+template <typename T>
+static msla_status_t run_aggregate_plain(const void* src, const void* w_dw, const void* w_pw, void* dst, int B, int H, int W, int groups, int d, long long src_sb,
+                                         long long dst_sb, cudaStream_t st) {
+  if (d == 32) return launch_aggregate<T, 32>((const T*)src, (const T*)w_dw, (const T*)w_pw, (T*)dst, B, H, W, groups, src_sb, dst_sb, st);
+  return launch_aggregate<T, 16>((const T*)src, (const T*)w_dw, (const T*)w_pw, (T*)dst, B, H, W, groups, src_sb, dst_sb, st);
+}
+
 // src, dst planar [B, Ch/d, H*W, d] with batch strides src_sb, dst_sb (elements)
 static msla_status_t run_aggregate(msla_dtype_t dt, const void* src, const void* w_dw, const void* w_pw,
                                    void* dst, int B, int H, int W, int Ch, int d, long long src_sb,
                                    long long dst_sb, cudaStream_t st) {
+  if (dt == MSLA_F32) return run_aggregate_plain<float>(src, w_dw, w_pw, dst, B, H, W, Ch / d, d, src_sb, dst_sb, st);
   const long long plane = (long long)H * W * d;
   const bool f16 = dt == MSLA_F16;
-  if (dt != MSLA_F32 && src_sb % plane == 0 && dst_sb % plane == 0) {
-    if (aggregate_bf16_supported(H, W, Ch, d))
-      return run_aggregate_bf16(src, (long long)B * (src_sb / plane), (int)(src_sb / plane), w_dw, w_pw, dst, dst_sb, B, H, W, Ch, d, st, f16);
-    if (d == 16 && Ch > 16 && aggregate_bf16_supported(H, W, Ch - 16, d)) {
-      // odd number of 16-channel groups: the tuned kernel takes them in pairs, the plain one the last group
-      msla_status_t s = run_aggregate_bf16(src, (long long)B * (src_sb / plane), (int)(src_sb / plane), w_dw, w_pw, dst, dst_sb, B, H, W, Ch - 16, d, st, f16);
-      if (s != MSLA_OK) return s;
-      dim3 grid1((unsigned)(ceil_div_ll(W, 8) * ceil_div_ll(H, 8)), 1u, (unsigned)B);
-      auto last_group = [&](auto* tag) {
-        using T = std::remove_pointer_t<decltype(tag)>;
-        generic::aggregate_kernel<T><<<grid1, 256, 0, st>>>((const T*)src + (long long)(Ch / 16 - 1) * plane, (const T*)w_dw + (long long)(Ch - 16) * 25,
-                                                            (const T*)w_pw + (long long)(Ch - 16) * 16, (T*)dst + (long long)(Ch / 16 - 1) * plane, H, W, d,
-                                                            src_sb, dst_sb);
-      };
-      if (f16) last_group((__half*)nullptr);
-      else last_group((__nv_bfloat16*)nullptr);
-      count_launches(1);
-      return check_launch("token aggregation (last group)");
-    }
+  int done = 0;  // channels the tensor-core kernel takes: all, or with an odd number of 16-channel groups all but the last
+  if (src_sb % plane == 0 && dst_sb % plane == 0) {
+    if (aggregate_bf16_supported(H, W, Ch, d)) done = Ch;
+    else if (d == 16 && Ch > 16 && aggregate_bf16_supported(H, W, Ch - 16, d)) done = Ch - 16;
   }
-  dim3 grid((unsigned)(ceil_div_ll(W, 8) * ceil_div_ll(H, 8)), (unsigned)(Ch / d), (unsigned)B);
-  if (dt == MSLA_F32)
-    generic::aggregate_kernel<float><<<grid, 256, 0, st>>>((const float*)src, (const float*)w_dw, (const float*)w_pw,
-                                                           (float*)dst, H, W, d, src_sb, dst_sb);
-  else if (dt == MSLA_F16)
-    generic::aggregate_kernel<__half><<<grid, 256, 0, st>>>((const __half*)src, (const __half*)w_dw, (const __half*)w_pw,
-                                                            (__half*)dst, H, W, d, src_sb, dst_sb);
-  else
-    generic::aggregate_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>((const __nv_bfloat16*)src, (const __nv_bfloat16*)w_dw,
-                                                                   (const __nv_bfloat16*)w_pw, (__nv_bfloat16*)dst, H, W, d,
-                                                                   src_sb, dst_sb);
-  count_launches(1);
-  return check_launch("token aggregation");
+  if (done) {
+    const msla_status_t s = run_aggregate_bf16(src, (long long)B * (src_sb / plane), (int)(src_sb / plane), w_dw, w_pw, dst, dst_sb, B, H, W, done, d, st, f16);
+    if (s != MSLA_OK || done == Ch) return s;
+  }
+  const size_t first = (size_t)(done / d) * plane * 2;
+  const void *wd = (const char*)w_dw + (size_t)done * 25 * 2, *wp = (const char*)w_pw + (size_t)done * d * 2;
+  if (f16) return run_aggregate_plain<__half>((const char*)src + first, wd, wp, (char*)dst + first, B, H, W, (Ch - done) / d, d, src_sb, dst_sb, st);
+  return run_aggregate_plain<__nv_bfloat16>((const char*)src + first, wd, wp, (char*)dst + first, B, H, W, (Ch - done) / d, d, src_sb, dst_sb, st);
 }
 
 // The aggregation kernels are 5x5.  A 3x3 depthwise filter (another of Section 3.1's small kernels) is the same
