@@ -234,7 +234,7 @@ kv_combine_bf16path_kernel(const float* __restrict__ partial, float* __restrict_
   const int e = (int)(idx % ne);
   const float* p = partial + bh * S * ne + e;
   float acc = 0.f;
-  for (int s = 0; s < S; ++s) acc += p[(long long)s * ne];
+  for (int s = 0; s < S; ++s) acc += __uint_as_float(ld_dep32(p + (long long)s * ne));
   state[idx] = acc;
 }
 
@@ -321,7 +321,7 @@ apply_mma_kernel(const bf16* __restrict__ q, const float* __restrict__ state, bf
         for (int r = 0; r < 2; ++r) {
           const int a0 = CPT * t + 4 * ks + 2 * r;
           const int c = j < NT ? (g >> 1) * CPT + 2 * j + (g & 1) : D;
-          const float v0 = st[a0 * (D + 1) + c] * state_scale, v1 = st[(a0 + 1) * (D + 1) + c] * state_scale;
+          const float v0 = __uint_as_float(ld_dep32(st + a0 * (D + 1) + c)) * state_scale, v1 = __uint_as_float(ld_dep32(st + (a0 + 1) * (D + 1) + c)) * state_scale;
           bhi[ks][j][r] = pack16<F16>(v0, v1);
           blo[ks][j][r] = pack16<F16>(v0 - round16<F16>(v0), v1 - round16<F16>(v1));
         }

@@ -231,7 +231,7 @@ state_fold_kernel(const float* __restrict__ partial, int S, const bf16* __restri
     for (int s = s0; s < s1; s += 8) {
       float4 q[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) q[u] = s + u < s1 ? __ldg(sp + (long long)(s + u) * NE4 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int u = 0; u < 8; ++u) q[u] = s + u < s1 ? ld_dep128f(sp + (long long)(s + u) * NE4 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int u = 0; u < 8; ++u) { v.x += q[u].x; v.y += q[u].y; v.z += q[u].z; v.w += q[u].w; }
     }
@@ -488,7 +488,7 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
         const float4* ksp = reinterpret_cast<const float4*>(p.ks + ((long long)b * p.Ht + min(h, p.Ht - 1)) * D);
 #pragma unroll
         for (int a4 = 0; a4 < D / 4; ++a4) {
-          const float4 v = __ldg(ksp + a4);
+          const float4 v = ld_dep128f(ksp + a4);
           kk[4 * a4] = v.x; kk[4 * a4 + 1] = v.y; kk[4 * a4 + 2] = v.z; kk[4 * a4 + 3] = v.w;
         }
         ok = mbar_wait(full_bar + 8 * cs, cph, &abort_flag);

@@ -142,7 +142,7 @@ __device__ __forceinline__ void drain_accumulator(const GemmParams& p, const CUt
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
       const int n = ncol0 + c * 32 + v * 8;
-      rs[c & 1][v] = (res_row && n < p.N) ? __ldg(reinterpret_cast<const uint4*>(res_row + n)) : make_uint4(0u, 0u, 0u, 0u);
+      rs[c & 1][v] = (res_row && n < p.N) ? *reinterpret_cast<const uint4*>(res_row + n) : make_uint4(0u, 0u, 0u, 0u);
     }
   };
   if (EPI == 2) load_residual(0);

@@ -5,7 +5,7 @@
 //
 // What bounds them is how many multiply-adds a shared-memory access feeds: every inner loop works on a register tile
 // (4 x 4 to 8 x 4 outputs) read in 16-byte pieces.  Module [1, 192, 64, 128], d = 32, fp32: 333 us per forward with one or
-// two shared-memory loads per multiply-add, F32_NEW us now; [1, 64, 16, 16], d = 16 (all latency): 71 -> F32_SMALL us.
+// two shared-memory loads per multiply-add, 176 us now; [1, 64, 16, 16], d = 16 (all latency): 71 -> 21 us.
 #pragma once
 
 #include "msla_common.cuh"
@@ -46,6 +46,24 @@ template <typename T> __device__ __forceinline__ float4 load4(const T* p) {
     return make_float4(to_f32(e[0]), to_f32(e[1]), to_f32(e[2]), to_f32(e[3]));
   }
 }
+// The same, and one element, of a tensor that an earlier kernel of the stream may have written.
+template <typename T> __device__ __forceinline__ float4 load4_dep(const T* p) {
+  if constexpr (sizeof(T) == 4) {
+    return ld_dep128f(p);
+  } else {
+    const uint2 v = ld_dep64(p);
+    const T* e = reinterpret_cast<const T*>(&v);
+    return make_float4(to_f32(e[0]), to_f32(e[1]), to_f32(e[2]), to_f32(e[3]));
+  }
+}
+template <typename T> __device__ __forceinline__ float load1_dep(const T* p) {
+  if constexpr (sizeof(T) == 4) {
+    return __uint_as_float(ld_dep32(p));
+  } else {
+    const unsigned short v = (unsigned short)ld_dep16(p);
+    return to_f32(*reinterpret_cast<const T*>(&v));
+  }
+}
 template <typename T> __device__ __forceinline__ void store4(T* p, const float (&v)[4]) {
   if constexpr (sizeof(T) == 4) {
     *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
@@ -58,16 +76,23 @@ template <typename T> __device__ __forceinline__ void store4(T* p, const float (
   }
 }
 
-// Tile BM x BN, a thread owns TM x 4 outputs (TM / 4 runs of four consecutive tokens, four consecutive channels); the next
-// BK-slice of both operands is fetched into registers while the current one is multiplied.  Threads run along whichever
-// output index is contiguous in memory.  vec: four consecutive outputs along that index are an aligned vector.
-template <typename T, int BM, int BN, int BK, int TM>
-__global__ void __launch_bounds__((BM / TM) * (BN / 4))
+// Tile BM x BN, a thread owns TM x TN outputs (TM / 4 runs of four consecutive tokens, TN / 4 runs of four consecutive
+// channels); the next BK-slice of both operands is fetched into registers while the current one is multiplied.  Threads run
+// along whichever output index is contiguous in memory.  vec: four consecutive outputs along that index are an aligned vector.
+// Instruction issue bounds it: packed multiply-adds (two tokens) and four elements per load leave 25 instructions per k for
+// 32 multiply-adds; 8192 x 576 x 192 runs in 45 us = 40 TFLOP/s (58 us with scalar ones; 8 x 8 outputs per thread: slower,
+// too few warps).
+// MODE: how a slice of A is fetched, four consecutive elements at a time where rows allow it.
+enum GemmFetch { FETCH_K4, FETCH_M4, FETCH_M1 };  // k contiguous; tokens contiguous, aligned rows; tokens contiguous, ragged rows
+template <typename T, int BM, int BN, int BK, int TM, int TN, int MODE>
+__global__ void __launch_bounds__((BM / TM) * (BN / TN))
 gemm_kernel(const T* __restrict__ A, const T* __restrict__ Wt, const T* __restrict__ bias,
             T* __restrict__ D, GemmArgs g, bool vec) {
-  constexpr int TX = BM / TM, THREADS = TX * (BN / 4);
-  constexpr int LA = BM * BK / THREADS, LW = BN * BK / THREADS;
-  static_assert(BM * BK % THREADS == 0 && BN * BK % THREADS == 0 && TM % 4 == 0, "tile shape");
+  constexpr int TX = BM / TM, TY = BN / TN, THREADS = TX * TY;
+  constexpr int VA = MODE == FETCH_M1 ? 1 : 4;                          // elements per load
+  constexpr int LA = BM * BK / THREADS / VA, LW = BN * BK / THREADS / 4;
+  constexpr int KV = BK / 4, MV = BM / VA;
+  static_assert(LA >= 1 && LW >= 1 && THREADS % KV == 0 && THREADS % MV == 0 && TM % 4 == 0 && TN % 4 == 0, "tile shape");
   __shared__ __align__(16) float As[2][BK][BM + 4];
   __shared__ __align__(16) float Ws[2][BK][BN + 4];
   pdl_launch_dependents();
@@ -75,39 +100,50 @@ gemm_kernel(const T* __restrict__ A, const T* __restrict__ Wt, const T* __restri
   const long long m0 = (long long)blockIdx.x * BM;
   const int n0 = blockIdx.y * BN;
   const int b = blockIdx.z;
-  const bool a_m_contig = (g.sAm == 1);
   const bool d_m_contig = (g.sDm == 1);
-  const int tm = d_m_contig ? tid % TX : tid / (BN / 4), tn = d_m_contig ? tid / TX : tid % (BN / 4);
-  const T* Ab = A + (long long)b * g.sAb;
-  float ra[LA], rw[LW];
-  auto fetch_w = [&](int k0) {
+  const int tm = d_m_contig ? tid % TX : tid / TY, tn = d_m_contig ? tid / TX : tid % TY;
+  // this thread's loads of a slice: load i adds am_step tokens and ak_step channels
+  constexpr int am_step = MODE == FETCH_K4 ? THREADS / KV : 0, ak_step = MODE == FETCH_K4 ? 0 : THREADS / MV;
+  const int am = MODE == FETCH_K4 ? tid / KV : tid % MV * VA, ak = MODE == FETCH_K4 ? tid % KV * 4 : tid / MV;
+  const T* pa = A + (long long)b * g.sAb + (m0 + am) * g.sAm + (long long)ak * g.sAk;
+  const long long stepA = am_step * g.sAm + ak_step * g.sAk, sliceA = (long long)BK * g.sAk;
+  const int wn = tid / KV, wk = tid % KV * 4;
+  const T* pw = Wt + (long long)(n0 + wn) * g.K + wk;
+  const int stepW = THREADS / KV * g.K;
+  const int m_left = (int)min((long long)BM, g.M - m0), n_left = g.Nc - n0;
+  float ra[LA][VA], rw[LW][4];
+  auto fetch_w = [&](int k0) {  // K is a multiple of 8: a vector exists whole or not at all
 #pragma unroll
-    for (int i = 0; i < LW; ++i) {
-      const int e = tid + i * THREADS, k = e % BK, n = e / BK;
-      rw[i] = n0 + n < g.Nc && k0 + k < g.K ? to_f32(__ldg(Wt + (long long)(n0 + n) * g.K + k0 + k)) : 0.f;
-    }
+    for (int i = 0; i < LW; ++i)
+      *reinterpret_cast<float4*>(rw[i]) = wn + i * (THREADS / KV) < n_left && k0 + wk < g.K ? load4(pw + (long long)i * stepW) : make_float4(0.f, 0.f, 0.f, 0.f);
+    pw += BK;
   };
-  auto fetch_a = [&](int k0) {
+  auto fetch_a = [&](int k0) {  // FETCH_M4: rows are a multiple of four tokens
+    const T* q = pa;
 #pragma unroll
-    for (int i = 0; i < LA; ++i) {
-      const int e = tid + i * THREADS, m = a_m_contig ? e % BM : e / BK, k = a_m_contig ? e / BM : e % BK;
-      ra[i] = m0 + m < g.M && k0 + k < g.K ? to_f32(Ab[(m0 + m) * g.sAm + (long long)(k0 + k) * g.sAk]) : 0.f;
+    for (int i = 0; i < LA; ++i, q += stepA) {
+      const bool ok = am + i * am_step < m_left && k0 + ak + i * ak_step < g.K;
+      if constexpr (VA == 4) *reinterpret_cast<float4*>(ra[i]) = ok ? load4_dep(q) : make_float4(0.f, 0.f, 0.f, 0.f);
+      else ra[i][0] = ok ? load1_dep(q) : 0.f;
     }
+    pa += sliceA;
   };
   auto put = [&](int buf) {
 #pragma unroll
     for (int i = 0; i < LA; ++i) {
-      const int e = tid + i * THREADS;
-      if (a_m_contig) As[buf][e / BM][e % BM] = ra[i];
-      else As[buf][e % BK][e / BK] = ra[i];
+      if constexpr (MODE == FETCH_M4) {
+        *reinterpret_cast<float4*>(&As[buf][ak + i * ak_step][am]) = *reinterpret_cast<const float4*>(ra[i]);
+      } else {
+#pragma unroll
+        for (int v = 0; v < VA; ++v) As[buf][ak + i * ak_step + v][am + i * am_step] = ra[i][v];
+      }
     }
 #pragma unroll
-    for (int i = 0; i < LW; ++i) {
-      const int e = tid + i * THREADS;
-      Ws[buf][e % BK][e / BK] = rw[i];
-    }
+    for (int i = 0; i < LW; ++i)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) Ws[buf][wk + v][wn + i * (THREADS / KV)] = rw[i][v];
   };
-  float acc[TM][4] = {};
+  unsigned long long acc2[TM / 2][TN] = {};  // pairs of tokens
   fetch_w(0);
   pdl_wait();  // the weights do not come from the previous kernel
   fetch_a(0);
@@ -119,53 +155,63 @@ gemm_kernel(const T* __restrict__ A, const T* __restrict__ Wt, const T* __restri
     if (more) { fetch_w(k0 + BK); fetch_a(k0 + BK); }
 #pragma unroll
     for (int k = 0; k < BK; ++k) {
-      float a[TM];
+      ulonglong2 a[TM / 4];
+      float w[TN];
 #pragma unroll
-      for (int r = 0; r < TM / 4; ++r) {
-        const float4 v = *reinterpret_cast<const float4*>(&As[buf][k][r * (TX * 4) + tm * 4]);
-        a[4 * r] = v.x; a[4 * r + 1] = v.y; a[4 * r + 2] = v.z; a[4 * r + 3] = v.w;
-      }
-      const float4 w = *reinterpret_cast<const float4*>(&Ws[buf][k][tn * 4]);
+      for (int r = 0; r < TM / 4; ++r) a[r] = *reinterpret_cast<const ulonglong2*>(&As[buf][k][r * (TX * 4) + tm * 4]);
 #pragma unroll
-      for (int i = 0; i < TM; ++i) {
-        acc[i][0] = fmaf(a[i], w.x, acc[i][0]);
-        acc[i][1] = fmaf(a[i], w.y, acc[i][1]);
-        acc[i][2] = fmaf(a[i], w.z, acc[i][2]);
-        acc[i][3] = fmaf(a[i], w.w, acc[i][3]);
+      for (int r = 0; r < TN / 4; ++r) *reinterpret_cast<float4*>(w + 4 * r) = *reinterpret_cast<const float4*>(&Ws[buf][k][r * (TY * 4) + tn * 4]);
+#pragma unroll
+      for (int j = 0; j < TN; ++j) {
+        unsigned long long ww;
+        asm("mov.b64 %0, {%1, %1};" : "=l"(ww) : "f"(w[j]));
+#pragma unroll
+        for (int i = 0; i < TM / 4; ++i) {
+          asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc2[2 * i][j]) : "l"(a[i].x), "l"(ww));
+          asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc2[2 * i + 1][j]) : "l"(a[i].y), "l"(ww));
+        }
       }
     }
     if (more) put(buf ^ 1);  // last read before the previous barrier
     __syncthreads();
   }
+  float acc[TM][TN];
+#pragma unroll
+  for (int i = 0; i < TM / 2; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[2 * i][j]), "=f"(acc[2 * i + 1][j]) : "l"(acc2[i][j]));
   T* Db = D + (long long)b * g.sDb;
   const T* Rb = static_cast<const T*>(g.residual) + (g.residual ? (long long)b * g.sDb : 0);
-  const int n = n0 + tn * 4;  // Nc is a multiple of 8: all four channels exist or none does
-  if (n >= g.Nc) return;
-  float bv[4];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) bv[j] = bias ? to_f32(bias[n + j]) : 0.f;
-  const long long at_n = (long long)(n / g.group) * g.sDg + (long long)(n % g.group) * g.sDn;  // four channels share a plane
+  for (int c = 0; c < TN / 4; ++c) {
+    const int n = n0 + c * (TY * 4) + tn * 4;  // Nc is a multiple of 8: all four channels exist or none does
+    if (n >= g.Nc) continue;
+    float bv[4];
 #pragma unroll
-  for (int r = 0; r < TM / 4; ++r) {
-    const long long m = m0 + r * (TX * 4) + tm * 4;
+    for (int j = 0; j < 4; ++j) bv[j] = bias ? to_f32(bias[n + j]) : 0.f;
+    const long long at_n = (long long)(n / g.group) * g.sDg + (long long)(n % g.group) * g.sDn;  // four channels share a plane
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {  // a vector: four tokens of channel n + u, or four channels of token m + u
-      float v[4];
+    for (int r = 0; r < TM / 4; ++r) {
+      const long long m = m0 + r * (TX * 4) + tm * 4;
 #pragma unroll
-      for (int e = 0; e < 4; ++e) v[e] = act_f32(d_m_contig ? acc[4 * r + e][u] + bv[u] : acc[4 * r + u][e] + bv[e], g.act);
-      const long long at = at_n + (d_m_contig ? m * g.sDm + u * g.sDn : (m + u) * g.sDm);
-      const int count = d_m_contig ? (int)min(4LL, g.M - m) : (m + u < g.M ? 4 : 0);
-      const long long step = d_m_contig ? g.sDm : g.sDn;
-      if (vec && count == 4) {
-        if (g.residual) {
-          const float4 x = load4(Rb + at);
-          v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
+      for (int u = 0; u < 4; ++u) {  // a vector: four tokens of channel n + u, or four channels of token m + u
+        float v[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = act_f32(d_m_contig ? acc[4 * r + e][4 * c + u] + bv[u] : acc[4 * r + u][4 * c + e] + bv[e], g.act);
+        const long long at = at_n + (d_m_contig ? m * g.sDm + u * g.sDn : (m + u) * g.sDm);
+        const int count = d_m_contig ? (int)min(4LL, g.M - m) : (m + u < g.M ? 4 : 0);
+        const long long step = d_m_contig ? g.sDm : g.sDn;
+        if (vec && count == 4) {
+          if (g.residual) {
+            const float4 x = load4_dep(Rb + at);
+            v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
+          }
+          store4(Db + at, v);
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (e < count) Db[at + e * step] = from_f32<T>(g.residual ? v[e] + to_f32(Rb[at + e * step]) : v[e]);
         }
-        store4(Db + at, v);
-      } else {
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-          if (e < count) Db[at + e * step] = from_f32<T>(g.residual ? v[e] + to_f32(Rb[at + e * step]) : v[e]);
       }
     }
   }
@@ -216,88 +262,90 @@ embed_taps_kernel(const T* __restrict__ w3, T* __restrict__ w5, long long total)
 // on planar activations [B, groups, H*W, D].  One CTA = one tile of TH x TW pixels of
 // one group.  src(b, g, n, i) = src[b*src_sb + (g*H*W + n)*D + i]; dst likewise with dst_sb.
 // A lane keeps one channel (D = 16: the half-warps take different pixels): the depthwise step slides down a strip of
-// four pixel columns and eight rows with five rows of sums in registers (8 shared-memory loads per 100 multiply-adds), the
-// 1x1 step holds the channel's D weights in registers and reads the depthwise results as broadcast 16-byte pieces.
+// four pixel columns and SH rows with five rows of sums in registers (8 shared-memory loads per 100 multiply-adds), the
+// 1x1 step holds the channel's D weights in registers and reads the depthwise results, which replace the staged tile in
+// shared memory, as broadcast 16-byte pieces.
 // ---------------------------------------------------------------------------
-template <typename T, int D, int TH, int TW>
-__global__ void __launch_bounds__(TH * TW * D / 32)
+template <typename T, int D, int TH, int TW, int SH>
+__global__ void __launch_bounds__(TH * TW * D / (4 * SH))
 aggregate_kernel(const T* __restrict__ src, const T* __restrict__ w_dw, const T* __restrict__ w_pw,
                  T* __restrict__ dst, int H, int W, long long src_sb, long long dst_sb) {
-  constexpr int THREADS = TH * TW * D / 32;  // a strip of 32 pixels per lane
+  constexpr int PX = 4 * SH, THREADS = TH * TW * D / PX;  // a strip of PX pixels per lane
   constexpr int HW_ = TW + 4, HH = TH + 4, CV = D / 4;
-  static_assert(TH % 8 == 0 && TW % 4 == 0, "strips of 4 x 8 pixels");
+  static_assert(TH % SH == 0 && TW % 4 == 0, "strips of 4 x SH pixels");
   extern __shared__ __align__(16) float agg_smem[];
-  float* tile = agg_smem;                  // [HH][HW_][D]
-  float* dwo = agg_smem + HH * HW_ * D;    // [TH * TW][D]
+  float* tile = agg_smem;  // [HH][HW_][D], then the depthwise results [TH * TW][D]
   pdl_launch_dependents();
   const int tid = threadIdx.x;
   const int tiles_x = (W + TW - 1) / TW;
   const int x0 = (blockIdx.x % tiles_x) * TW, y0 = (blockIdx.x / tiles_x) * TH;
   const int ch0 = blockIdx.y * D;
   const int b = blockIdx.z;
-  const int c = tid % D, strip = tid / D;  // strips: row-major over (TH / 8) x (TW / 4)
-  float taps[25], pw[D];
-#pragma unroll
-  for (int i = 0; i < D; i += 4) {
-    const float4 v = load4(w_pw + (long long)(ch0 + c) * D + i);
-    pw[i] = v.x; pw[i + 1] = v.y; pw[i + 2] = v.z; pw[i + 3] = v.w;
-  }
-  pdl_wait();  // the 1x1 weights do not come from the previous kernel; the taps may (a 3x3 filter embedded in 5x5)
+  const int c = tid % D, strip = tid / D;  // strips: row-major over (TH / SH) x (TW / 4)
+  float taps[25];
+  pdl_wait();  // the planes come from the previous kernel, and the taps may (a 3x3 filter embedded in 5x5)
 #pragma unroll
   for (int i = 0; i < 25; ++i) taps[i] = to_f32(__ldg(w_dw + (long long)(ch0 + c) * 25 + i));
   const T* sb = src + (long long)b * src_sb + (long long)blockIdx.y * H * W * D;
+#pragma unroll 8
   for (int e = tid; e < HH * HW_ * CV; e += THREADS) {
     const int cv = e % CV, p = e / CV;
     const int yy = y0 + p / HW_ - 2, xx = x0 + p % HW_ - 2;
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (yy >= 0 && yy < H && xx >= 0 && xx < W) v = load4(sb + ((long long)yy * W + xx) * D + cv * 4);
+    if (yy >= 0 && yy < H && xx >= 0 && xx < W) v = load4_dep(sb + ((long long)yy * W + xx) * D + cv * 4);
     *reinterpret_cast<float4*>(tile + p * D + cv * 4) = v;
   }
   __syncthreads();
+  const int sx = (strip % (TW / 4)) * 4, sy = strip / (TW / 4) * SH;
+  float acc[SH][4];
   {
-    const int sx = (strip % (TW / 4)) * 4, sy = strip / (TW / 4) * 8;
     const float* t0 = tile + (sy * HW_ + sx) * D + c;
-    float acc[5][4];
 #pragma unroll
-    for (int r = 0; r < 12; ++r) {  // staged row r feeds output rows r - 4 .. r of the strip
+    for (int r = 0; r < SH + 4; ++r) {  // staged row r feeds output rows r - 4 .. r of the strip
       float in[8];
 #pragma unroll
       for (int x = 0; x < 8; ++x) in[x] = t0[(r * HW_ + x) * D];
 #pragma unroll
       for (int dy = 0; dy < 5; ++dy) {
         const int o = r - dy;
-        if (o < 0 || o >= 8) continue;
-        float (&a)[4] = acc[o % 5];
+        if (o < 0 || o >= SH) continue;
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
-          float v = dy == 0 ? 0.f : a[x];
+          float v = dy == 0 ? 0.f : acc[o][x];
 #pragma unroll
           for (int dx = 0; dx < 5; ++dx) v = fmaf(taps[dy * 5 + dx], in[x + dx], v);
-          a[x] = v;
+          acc[o][x] = v;
         }
-      }
-      if (r >= 4) {
-#pragma unroll
-        for (int x = 0; x < 4; ++x) dwo[((sy + r - 4) * TW + sx + x) * D + c] = acc[(r - 4) % 5][x];
       }
     }
   }
+  float pw[D];
+#pragma unroll
+  for (int i = 0; i < D; i += 4) {
+    const float4 v = load4(w_pw + (long long)(ch0 + c) * D + i);
+    pw[i] = v.x; pw[i + 1] = v.y; pw[i + 2] = v.z; pw[i + 3] = v.w;
+  }
+  __syncthreads();  // the staged tile has been read
+#pragma unroll
+  for (int o = 0; o < SH; ++o)
+#pragma unroll
+    for (int x = 0; x < 4; ++x) tile[((sy + o) * TW + sx + x) * D + c] = acc[o][x];
   __syncthreads();
   T* db = dst + (long long)b * dst_sb + (long long)blockIdx.y * H * W * D;
 #pragma unroll 2
-  for (int i = 0; i < 32; ++i) {
+  for (int i = 0; i < PX; ++i) {
     const int p = strip + i * (THREADS / D);
     const int yy = y0 + p / TW, xx = x0 + p % TW;
     float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll
     for (int k = 0; k < D; k += 4) {
-      const float4 v = *reinterpret_cast<const float4*>(dwo + p * D + k);
+      const float4 v = *reinterpret_cast<const float4*>(tile + p * D + k);
       a0 = fmaf(pw[k], v.x, a0); a1 = fmaf(pw[k + 1], v.y, a1); a2 = fmaf(pw[k + 2], v.z, a2); a3 = fmaf(pw[k + 3], v.w, a3);
     }
     if (yy < H && xx < W) db[((long long)yy * W + xx) * D + c] = from_f32<T>((a0 + a1) + (a2 + a3));
   }
 }
-template <int D, int TH, int TW> constexpr int aggregate_smem() { return ((TH + 4) * (TW + 4) + TH * TW) * D * 4; }
+template <int D, int TH, int TW> constexpr int aggregate_smem() { return (TH + 4) * (TW + 4) * D * 4; }
 
 // ---------------------------------------------------------------------------
 // KV-state reduction, first level (Eq. 3): for one (batch, head) and one chunk
@@ -333,8 +381,8 @@ kv_partial_kernel(const T* __restrict__ k, const T* __restrict__ v, float* __res
       const int e = lane + 32 * i, n = n0 + e / CV;
       const bool ok = n < n_end;
       const long long off = base + (long long)(ok ? n : n_begin) * kv.ld + e % CV * 4;
-      rk[i] = ok ? load4(k + off) : make_float4(0.f, 0.f, 0.f, 0.f);
-      rv[i] = ok ? load4(v + off) : make_float4(0.f, 0.f, 0.f, 0.f);
+      rk[i] = ok ? load4_dep(k + off) : make_float4(0.f, 0.f, 0.f, 0.f);
+      rv[i] = ok ? load4_dep(v + off) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   };
   int n0 = n_begin + warp * TT;
@@ -394,7 +442,7 @@ kv_combine_kernel(const float* __restrict__ partial, float* __restrict__ state, 
   const int e = (int)(idx % ne);
   const float* p = partial + bh * S * ne + e;
   float acc = 0.f;
-  for (int s = 0; s < S; ++s) acc += p[(long long)s * ne];
+  for (int s = 0; s < S; ++s) acc += load1_dep(p + (long long)s * ne);
   state[idx] = acc;
 }
 
@@ -412,49 +460,61 @@ band_state_sum_kernel(const float* __restrict__ states, float* __restrict__ stat
 // ---------------------------------------------------------------------------
 // Apply step (Eq. 3): out[i,c] = relu(q[i]) . KV[:,c] / (relu(q[i]) . ks + eps),
 // written at channel offset head*D of the output view (head concat).
-// One thread per token with its D sums in registers; state [BH][D*(D+1)] fp32 staged in shared memory with rows of
-// D + 4 floats, read as broadcast 16-byte pieces (one per four multiply-adds).
+// A CTA takes 512 / (D / 4) tokens of one head, a thread four of them and four channels: per four key channels eight
+// 16-byte shared-memory loads for 80 multiply-adds (the normaliser's among them, formed by every thread of a token).
 // ---------------------------------------------------------------------------
+template <int D> constexpr int APPLY_TOKENS = 4 * 128 / (D / 4);
 template <typename T, int D>
 __global__ void __launch_bounds__(128)
 apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* __restrict__ out,
              HeadView qv, HeadView ov, int heads, int N, float eps) {
-  constexpr int D1 = D + 1, P = D + 4;
-  __shared__ __align__(16) float st[D * P];
+  constexpr int D1 = D + 1, CV = D / 4, TG = 128 / CV, TOK = APPLY_TOKENS<D>, P = D + 4;
+  __shared__ __align__(16) float st[D * P];    // rows of the state: D values, then the key sum
+  __shared__ __align__(16) float qs[TOK * P];
   pdl_launch_dependents();
   pdl_wait();
   const int bh = blockIdx.y;
   const int b = bh / heads, h = bh % heads;
-  for (int e = threadIdx.x; e < D * D1; e += 128) st[e / D1 * P + e % D1] = state[(long long)bh * D * D1 + e];
-  const int n = blockIdx.x * 128 + threadIdx.x;
-  const T* qp = q + (long long)b * qv.batch + (long long)h * qv.head + (long long)min(n, N - 1) * qv.ld;
-  float qr[D];
+  const int n0 = blockIdx.x * TOK, tid = threadIdx.x;
+  const T* qp = q + (long long)b * qv.batch + (long long)h * qv.head;
+#pragma unroll
+  for (int i = 0; i < TOK * CV / 128; ++i) {
+    const int e = tid + i * 128, n = e / CV, cv = e % CV;
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (n0 + n < N) x = load4_dep(qp + (long long)(n0 + n) * qv.ld + cv * 4);
+    *reinterpret_cast<float4*>(qs + n * P + cv * 4) = make_float4(fmaxf(x.x, 0.f), fmaxf(x.y, 0.f), fmaxf(x.z, 0.f), fmaxf(x.w, 0.f));
+  }
+  for (int e = tid; e < D * D1; e += 128) st[e / D1 * P + e % D1] = load1_dep(state + (long long)bh * D * D1 + e);
+  __syncthreads();
+  const int tn = tid % CV, tm = tid / CV;
+  float num[4][4] = {}, den[4] = {};
 #pragma unroll
   for (int a = 0; a < D; a += 4) {
-    const float4 x = load4(qp + a);
-    qr[a] = fmaxf(x.x, 0.f); qr[a + 1] = fmaxf(x.y, 0.f); qr[a + 2] = fmaxf(x.z, 0.f); qr[a + 3] = fmaxf(x.w, 0.f);
-  }
-  __syncthreads();
-  if (n >= N) return;
-  T* op = out + (long long)b * ov.batch + (long long)h * ov.head + (long long)n * ov.ld;
-  float den = 0.f, num[D];
+    float w[4][4], ks[4], x[4][4];
 #pragma unroll
-  for (int c = 0; c < D; ++c) num[c] = 0.f;
-#pragma unroll
-  for (int a = 0; a < D; ++a) {
-#pragma unroll
-    for (int c = 0; c < D; c += 4) {
-      const float4 x = *reinterpret_cast<const float4*>(st + a * P + c);
-      num[c] = fmaf(qr[a], x.x, num[c]); num[c + 1] = fmaf(qr[a], x.y, num[c + 1]);
-      num[c + 2] = fmaf(qr[a], x.z, num[c + 2]); num[c + 3] = fmaf(qr[a], x.w, num[c + 3]);
+    for (int k = 0; k < 4; ++k) {
+      *reinterpret_cast<float4*>(w[k]) = *reinterpret_cast<const float4*>(st + (a + k) * P + tn * 4);
+      ks[k] = st[(a + k) * P + D];
     }
-    den = fmaf(qr[a], st[a * P + D], den);
-  }
-  const float inv = 1.f / (den + eps);
 #pragma unroll
-  for (int c = 0; c < D; c += 4) {
-    const float o[4] = {num[c] * inv, num[c + 1] * inv, num[c + 2] * inv, num[c + 3] * inv};
-    store4(op + c, o);
+    for (int i = 0; i < 4; ++i) *reinterpret_cast<float4*>(x[i]) = *reinterpret_cast<const float4*>(qs + (tm + i * TG) * P + a);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        den[i] = fmaf(x[i][k], ks[k], den[i]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) num[i][j] = fmaf(x[i][k], w[k][j], num[i][j]);
+      }
+  }
+  T* op = out + (long long)b * ov.batch + (long long)h * ov.head + tn * 4;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int n = n0 + tm + i * TG;
+    if (n >= N) continue;
+    const float inv = 1.f / (den[i] + eps);
+    const float o[4] = {num[i][0] * inv, num[i][1] * inv, num[i][2] * inv, num[i][3] * inv};
+    store4(op + (long long)n * ov.ld, o);
   }
 }
 

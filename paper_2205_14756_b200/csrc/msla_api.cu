@@ -135,7 +135,7 @@ static msla_status_t run_core_generic(const T* q, const T* k, const T* v, T* out
   }
   if (mid) cudaEventRecord(mid, st);
   if (phases & CORE_APPLY) {
-    const dim3 grid((unsigned)ceil_div_ll(N, 128), (unsigned)BH);
+    const dim3 grid((unsigned)ceil_div_ll(N, d == 32 ? generic::APPLY_TOKENS<32> : generic::APPLY_TOKENS<16>), (unsigned)BH);
     const float* sum = one ? partial : state;
     if (d == 32) launch_pdl(generic::apply_kernel<T, 32>, grid, dim3(128), 0, st, q, sum, out, in, ov, heads, N, eps);
     else launch_pdl(generic::apply_kernel<T, 16>, grid, dim3(128), 0, st, q, sum, out, in, ov, heads, N, eps);
@@ -318,10 +318,13 @@ static msla_status_t validate_desc(const msla_desc* d, ForwardPlan* plan) {
   return MSLA_OK;
 }
 
-template <typename T, int BM, int BN, int BK, int TM>
+template <typename T, int BM, int BN, int BK, int TM, int TN>
 static void launch_gemm_tile(const T* A, const T* W, const T* bias, T* D, generic::GemmArgs g, int B, bool vec, cudaStream_t st) {
   dim3 grid((unsigned)ceil_div_ll(g.M, BM), (unsigned)ceil_div_ll(g.Nc, BN), (unsigned)B);
-  launch_pdl(generic::gemm_kernel<T, BM, BN, BK, TM>, grid, dim3((BM / TM) * (BN / 4)), 0, st, A, W, bias, D, g, vec);
+  const dim3 block((BM / TM) * (BN / TN));
+  if (g.sAk == 1) launch_pdl(generic::gemm_kernel<T, BM, BN, BK, TM, TN, generic::FETCH_K4>, grid, block, 0, st, A, W, bias, D, g, vec);
+  else if (g.M % 4 == 0) launch_pdl(generic::gemm_kernel<T, BM, BN, BK, TM, TN, generic::FETCH_M4>, grid, block, 0, st, A, W, bias, D, g, vec);
+  else launch_pdl(generic::gemm_kernel<T, BM, BN, BK, TM, TN, generic::FETCH_M1>, grid, block, 0, st, A, W, bias, D, g, vec);
   count_launches(1);
 }
 
@@ -331,9 +334,9 @@ template <typename T>
 static void launch_gemm(const T* A, const T* W, const T* bias, T* D, generic::GemmArgs g, int B, cudaStream_t st) {
   const bool vec = g.sDm == 1 ? g.sDn % 4 == 0 && g.sDg % 4 == 0 && g.sDb % 4 == 0 : g.sDm % 4 == 0 && g.sDg % 4 == 0 && g.sDb % 4 == 0;
   const long long sms = device_sm_count();
-  if ((long long)B * ceil_div_ll(g.M, 128) * ceil_div_ll(g.Nc, 64) >= 2 * sms) launch_gemm_tile<T, 128, 64, 16, 8>(A, W, bias, D, g, B, vec, st);
-  else if ((long long)B * ceil_div_ll(g.M, 64) * ceil_div_ll(g.Nc, 64) >= 2 * sms) launch_gemm_tile<T, 64, 64, 16, 4>(A, W, bias, D, g, B, vec, st);
-  else launch_gemm_tile<T, 32, 32, 32, 4>(A, W, bias, D, g, B, vec, st);
+  if ((long long)B * ceil_div_ll(g.M, 128) * ceil_div_ll(g.Nc, 64) >= 2 * sms) launch_gemm_tile<T, 128, 64, 16, 8, 4>(A, W, bias, D, g, B, vec, st);
+  else if ((long long)B * ceil_div_ll(g.M, 64) * ceil_div_ll(g.Nc, 64) >= 2 * sms) launch_gemm_tile<T, 64, 64, 16, 8, 4>(A, W, bias, D, g, B, vec, st);
+  else launch_gemm_tile<T, 32, 32, 32, 4, 4>(A, W, bias, D, g, B, vec, st);
 }
 
 // y planar: y[b*y_sb + ((o/d)*N + n)*d + o%d]; rows of x are ldx elements apart (N where the plain kernels run)
@@ -358,25 +361,25 @@ static msla_status_t run_project_out(msla_dtype_t dt, const void* a, const void*
   return check_launch("output projection");
 }
 
-template <typename T, int D, int TH, int TW>
+template <typename T, int D, int TH, int TW, int SH>
 static msla_status_t launch_aggregate_tile(const T* src, const T* w_dw, const T* w_pw, T* dst, int B, int H, int W, int groups, long long src_sb, long long dst_sb,
                                            cudaStream_t st) {
   constexpr int smem = generic::aggregate_smem<D, TH, TW>();
   static std::atomic<unsigned long long> attr_done{0};
-  const msla_status_t s = ensure_smem_attr(attr_done, generic::aggregate_kernel<T, D, TH, TW>, smem);
+  const msla_status_t s = ensure_smem_attr(attr_done, generic::aggregate_kernel<T, D, TH, TW, SH>, smem);
   if (s != MSLA_OK) return s;
   const dim3 grid((unsigned)(ceil_div_ll(W, TW) * ceil_div_ll(H, TH)), (unsigned)groups, (unsigned)B);
-  launch_pdl(generic::aggregate_kernel<T, D, TH, TW>, grid, dim3(TH * TW * D / 32), smem, st, src, w_dw, w_pw, dst, H, W, src_sb, dst_sb);
+  launch_pdl(generic::aggregate_kernel<T, D, TH, TW, SH>, grid, dim3(TH * TW * D / (4 * SH)), smem, st, src, w_dw, w_pw, dst, H, W, src_sb, dst_sb);
   count_launches(1);
   return check_launch("token aggregation");
 }
-// 16 x 16 pixels re-read the halo least (1.56 loads per pixel against 2.25); 8 x 8 where that leaves SMs without a tile
+// larger tiles re-read the halo less; 8 x 8 pixels where they leave SMs without a tile
 template <typename T, int D>
 static msla_status_t launch_aggregate(const T* src, const T* w_dw, const T* w_pw, T* dst, int B, int H, int W, int groups, long long src_sb, long long dst_sb,
                                       cudaStream_t st) {
   if (ceil_div_ll(W, 16) * ceil_div_ll(H, 16) * groups * B >= device_sm_count())
-    return launch_aggregate_tile<T, D, 16, 16>(src, w_dw, w_pw, dst, B, H, W, groups, src_sb, dst_sb, st);
-  return launch_aggregate_tile<T, D, 8, 8>(src, w_dw, w_pw, dst, B, H, W, groups, src_sb, dst_sb, st);
+    return launch_aggregate_tile<T, D, 16, 16, 8>(src, w_dw, w_pw, dst, B, H, W, groups, src_sb, dst_sb, st);
+  return launch_aggregate_tile<T, D, 8, 8, 4>(src, w_dw, w_pw, dst, B, H, W, groups, src_sb, dst_sb, st);
 }
 template <typename T>
 static msla_status_t run_aggregate_plain(const void* src, const void* w_dw, const void* w_pw, void* dst, int B, int H, int W, int groups, int d, long long src_sb,

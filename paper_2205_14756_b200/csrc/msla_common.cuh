@@ -45,6 +45,31 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // one has started (it still waits in pdl_wait for this kernel's completion).
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Loads of data that an earlier kernel of the stream wrote, in kernels that may have become resident while it ran.  They are
+// ordered after pdl_wait() (both are volatile) and are plain loads: the read-only path (__ldg, and what the compiler makes of
+// const __restrict__ pointers) is for data that does not change during the kernel's life, which includes the time before the
+// wait.  A sector written partly by this SM and partly by another was seen stale there.
+__device__ __forceinline__ uint32_t ld_dep32(const void* p) {
+  uint32_t r;
+  asm volatile("ld.global.u32 %0, [%1];" : "=r"(r) : "l"(p));
+  return r;
+}
+__device__ __forceinline__ uint32_t ld_dep16(const void* p) {
+  unsigned short r;
+  asm volatile("ld.global.u16 %0, [%1];" : "=h"(r) : "l"(p));
+  return r;
+}
+__device__ __forceinline__ uint2 ld_dep64(const void* p) {
+  uint2 r;
+  asm volatile("ld.global.v2.u32 {%0,%1}, [%2];" : "=r"(r.x), "=r"(r.y) : "l"(p));
+  return r;
+}
+__device__ __forceinline__ float4 ld_dep128f(const void* p) {
+  float4 r;
+  asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w) : "l"(p));
+  return r;
+}
+
 __host__ __device__ __forceinline__ long long ceil_div_ll(long long a, long long b) {
   return (a + b - 1) / b;
 }

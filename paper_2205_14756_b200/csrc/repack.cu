@@ -21,8 +21,8 @@ __device__ __forceinline__ uint4 load8(const unsigned short* __restrict__ src, l
   uint32_t w[5];
 #pragma unroll
   for (int i = 0; i < 5; ++i) {
-    if (2 * i + 1 < left && (i < 4 || odd)) w[i] = __ldg(words + i);
-    else if (2 * i < left && (i < 4 || odd)) w[i] = __ldg(src + (s & ~1LL) + 2 * i);
+    if (2 * i + 1 < left && (i < 4 || odd)) w[i] = ld_dep32(words + i);
+    else if (2 * i < left && (i < 4 || odd)) w[i] = ld_dep16(src + (s & ~1LL) + 2 * i);
     else w[i] = 0u;
   }
   if (!odd) return make_uint4(w[0], w[1], w[2], w[3]);
@@ -57,7 +57,7 @@ unpad_rows_kernel(const unsigned short* __restrict__ src, unsigned short* __rest
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
     if (col == n) { col = 0; ++row; }
-    v[e] = f + e < total ? __ldg(src + row * pitch + col) : (unsigned short)0;
+    v[e] = f + e < total ? (unsigned short)ld_dep16(src + row * pitch + col) : (unsigned short)0;
     ++col;
   }
   if (f + 8 <= total) {

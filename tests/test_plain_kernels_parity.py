@@ -1,0 +1,30 @@
+"""The kernels on the fp32 pipes at the sizes where a tile, a fetch mode or a dispatch rule changes (GPU against the oracle)."""
+import pytest
+
+import __graft_entry__  # noqa: F401
+import oracle
+import util
+from paper_2205_14756_b200 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+# 128 x 64, 64 x 64 and 32 x 32 GEMM tiles; rows that are and are not a multiple of four tokens; K that is no multiple of a
+# slice (24, 72 channels); aggregation tiles of 16 x 16 and 8 x 8 pixels with ragged edges; one and several partial states
+@pytest.mark.parametrize("B,C,H,W,heads,d", [(2, 192, 65, 127, 6, 32), (1, 96, 64, 96, 3, 32), (3, 72, 33, 31, 4, 16), (1, 24, 5, 3, 2, 32),
+                                             (2, 64, 17, 16, 4, 16), (9, 32, 48, 33, 2, 16)])
+def test_module_f32_tiles(B, C, H, W, heads, d):
+    s = inputs.ModuleShape("f32_tiles", "f32", B, C, H, W, heads, d, seed=71)
+    t = inputs.module_inputs(s)
+    ref = oracle.msla_forward(t["x"], t["w_qkv"], t["w_dw"], t["w_pw"], t["w_proj"], heads=heads, d=d, eps=s.eps)
+    util.assert_close(util.run_module(s, t), ref, "f32", "fp32 module")
+
+
+# the plain GEMM with bias, activation and residual, on vectors and on ragged rows; fp32 and a 16-bit width the tensor-core
+# kernels do not take (hidden width no multiple of 64)
+@pytest.mark.parametrize("dtype,B,C,H,W,Ch", [("f32", 2, 40, 9, 13, 72), ("f32", 1, 64, 48, 64, 256), ("bf16", 1, 48, 9, 7, 72), ("f16", 2, 32, 16, 16, 40)])
+def test_ffn_on_the_plain_kernels(dtype, B, C, H, W, Ch):
+    s = inputs.FfnShape("plain_ffn", dtype, B, C, H, W, Ch, C, seed=72)
+    t = inputs.ffn_inputs(s)
+    ref = oracle.ffn_dwconv(t["x"], t["w1"], t["w_dw"], t["w2"], t["b1"], t["b_dw"], t["b2"], act="hardswish", residual=True)
+    util.assert_close(util.run_ffn(s, t, "hardswish", True), ref, dtype, "FFN on the plain kernels")
