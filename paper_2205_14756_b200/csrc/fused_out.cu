@@ -164,8 +164,9 @@ template <bool F16> __device__ __forceinline__ uint32_t pack16(float lo, float h
 // partial: [B*Ht][S][D*(D+1)] fp32, entry [a][c], column D = key sum.
 //   ks[bh][a]            = sum_s partial[bh][s][a][D]
 //   M[b][m][hh*D + a]    = sum_c w[m][hh*D + c] * (sum_s partial[bh][s][a][c])        (16 bit, row stride K), all m < Cout
-// Fixed summation order: the S partial states are cut into RUNS runs of consecutive indices, each run is summed in index
-// order by its own thread with eight 16-byte loads in flight, and the run sums are added in run order.
+// Fixed summation order, the same for every DA: the S partial states are cut into eight runs of consecutive indices, each run
+// is summed in index order (eight 16-byte loads in flight) and the run sums are added in run order.  With few heads every run
+// has threads of its own, otherwise a thread sums FOLD_RUNS / GROUPS of them.
 // The product runs on mma.sync with output channels as rows, key channels as columns and c along the contraction.  The
 // weights are 16-bit already; the fp32 state is cut into PIECES 16-bit pieces (bf16: three, which hold all 24 bits; fp16:
 // two, 22 bits of a value that is rounded to 11).  Contraction slots and columns are assigned so that a lane loads 16
@@ -174,10 +175,11 @@ template <bool F16> __device__ __forceinline__ uint32_t pack16(float lo, float h
 // that did the product on the fp32 pipes with 1024 threads per CTA: 1024 heads (64 images, S = 1) 73.4 -> 13.7 us, 256
 // heads 22.9 -> 6.4 us, 16 heads (S = 37) 7.0 -> 4.3 us.
 // ---------------------------------------------------------------------------
+constexpr int FOLD_RUNS = 8;
 template <int D, int DA> struct FoldShape {
-  static constexpr int RUNS = DA == 8 ? 8 : DA * D >= 1024 ? 1 : 4;
+  static constexpr int GROUPS = DA == 8 ? 8 : DA * D >= 1024 ? 1 : 4;  // threads that share the runs of a vector
   static constexpr int NV = DA * (D + 1) / 4;                       // 16-byte vectors of the CTA's rows of a state
-  static constexpr int THREADS = (NV * RUNS + 31) / 32 * 32;        // 288, 544, 544 for D = 32 and DA = 32, 16, 8; 288 for D = 16
+  static constexpr int THREADS = (NV * GROUPS + 31) / 32 * 32;        // 288, 544, 544 for D = 32 and DA = 32, 16, 8; 288 for D = 16
 };
 
 template <bool F16>
@@ -196,10 +198,10 @@ template <int D, int DA, bool F16>
 __global__ void __launch_bounds__(FoldShape<D, DA>::THREADS, DA == D ? 4 : 1)
 state_fold_kernel(const float* __restrict__ partial, int S, const bf16* __restrict__ w, bf16* __restrict__ M, float* __restrict__ ks,
                   int Ht, int Cout, int K, float scale) {
-  constexpr int RUNS = FoldShape<D, DA>::RUNS, NV = FoldShape<D, DA>::NV, THREADS = FoldShape<D, DA>::THREADS;
+  constexpr int GROUPS = FoldShape<D, DA>::GROUPS, NV = FoldShape<D, DA>::NV, THREADS = FoldShape<D, DA>::THREADS;
   constexpr int D1 = D + 1, NE4 = D * D1 / 4, WARPS = THREADS / 32;
   constexpr int KS = D / 16, NT = DA / 8, PIECES = F16 ? 2 : 3;
-  __shared__ float4 run_sum[RUNS][NV];
+  __shared__ float4 run_sum[GROUPS == 1 ? 1 : FOLD_RUNS][NV];
   __shared__ uint32_t rounded[PIECES][DA][D / 2 + 1];  // pairs of neighbouring c
   float* st = reinterpret_cast<float*>(run_sum[0]);
   pdl_launch_dependents();
@@ -224,25 +226,40 @@ state_fold_kernel(const float* __restrict__ partial, int S, const bf16* __restri
   load_weights(16 * warp, x);  // the projection weights do not come from the previous kernel: fetched while it drains
   pdl_wait();                  // the partial states do
   const float4* sp = reinterpret_cast<const float4*>(partial + (long long)bh * S * (D * D1) + a0 * D1);
-  if (tid < RUNS * NV) {
-    const int j = tid / NV, e = tid - j * NV;
-    const int s0 = S * j / RUNS, s1 = S * (j + 1) / RUNS;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s = s0; s < s1; s += 8) {
+  auto add = [](float4& v, const float4& x) { v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w; };
+  if (tid < GROUPS * NV) {
+    const int group = tid / NV, e = tid - group * NV;
+    float4 total = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (GROUPS == 1 && S <= 8) {  // a run has one partial state or none
       float4 q[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) q[u] = s + u < s1 ? ld_dep128f(sp + (long long)(s + u) * NE4 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int u = 0; u < 8; ++u) q[u] = u < S ? ld_dep128f(sp + (long long)u * NE4 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int u = 0; u < 8; ++u) { v.x += q[u].x; v.y += q[u].y; v.z += q[u].z; v.w += q[u].w; }
+      for (int u = 0; u < 8; ++u) add(total, q[u]);
+    } else {
+#pragma unroll 1
+      for (int j = group * (FOLD_RUNS / GROUPS); j < (group + 1) * (FOLD_RUNS / GROUPS); ++j) {
+        const int s0 = S * j / FOLD_RUNS, s1 = S * (j + 1) / FOLD_RUNS;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int s = s0; s < s1; s += 8) {
+          float4 q[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) q[u] = s + u < s1 ? ld_dep128f(sp + (long long)(s + u) * NE4 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int u = 0; u < 8; ++u) add(v, q[u]);
+        }
+        if (GROUPS == 1) add(total, v);
+        else run_sum[j][e] = v;
+      }
     }
-    run_sum[j][e] = v;
+    if (GROUPS == 1) run_sum[0][e] = total;
   }
   __syncthreads();
-  if (RUNS > 1) {
+  if (GROUPS > 1) {
     if (tid < NV) {
       float4 v = run_sum[0][tid];
 #pragma unroll
-      for (int j = 1; j < RUNS; ++j) { const float4 r = run_sum[j][tid]; v.x += r.x; v.y += r.y; v.z += r.z; v.w += r.w; }
+      for (int j = 1; j < FOLD_RUNS; ++j) add(v, run_sum[j][tid]);
       run_sum[0][tid] = v;  // st[al * D1 + c], al = a - a0
     }
     __syncthreads();

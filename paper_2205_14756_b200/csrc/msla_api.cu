@@ -278,7 +278,9 @@ struct ForwardPlan {
   bool padded() const { return pitch != N; }
 };
 
-static msla_status_t validate_desc(const msla_desc* d, ForwardPlan* plan) {
+// core_B: images the split of the token reduction is planned for, where a call is a part of a batch (0: desc->B); its sums
+// are then those of the whole batch, bit for bit.
+static msla_status_t validate_desc(const msla_desc* d, ForwardPlan* plan, int core_B = 0) {
   if (!d) return fail(MSLA_ERR_INVALID_ARG, "null descriptor");
   if (d->struct_size != sizeof(msla_desc)) return fail(MSLA_ERR_INVALID_ARG, "desc.struct_size = %u, expected %zu", d->struct_size, sizeof(msla_desc));
   if (!known_dtype(d->dtype)) return fail(MSLA_ERR_INVALID_ARG, "unknown dtype %d", (int)d->dtype);
@@ -300,7 +302,7 @@ static msla_status_t validate_desc(const msla_desc* d, ForwardPlan* plan) {
   plan->N = d->H * d->W;
   const size_t e = elem_size(d->dtype);
   const size_t tokens = (size_t)d->B * plan->N;
-  plan->core = make_core_plan((long long)d->B * S * d->heads, plan->N, d->d);
+  plan->core = make_core_plan((long long)(core_B ? core_B : d->B) * S * d->heads, plan->N, d->d);
   plan->ms_off = 0;
   plan->att_off = align_up(tokens * 3 * S * plan->Cp * e, 256);
   // the attention output's region doubles as scratch of the fused apply + projection kernel, which writes no attention output
@@ -446,28 +448,26 @@ static msla_status_t record(void* const* events, int i, cudaStream_t st) {
   return MSLA_OK;
 }
 
-// host_io: x and out are host pointers staged through the tail of the workspace.
 // add_x: the output projection adds x (the block's first residual connection; C_out == C).
 // out_padded: receives the address of the padded copy of out where there is one (else of out itself).
 static msla_status_t forward_impl(const msla_desc* desc, const void* x, const msla_weights* w, void* out,
-                                  cudaStream_t st, void* const* events, bool host_io, bool add_x = false, const void** out_padded = nullptr) {
+                                  cudaStream_t st, void* const* events, bool add_x = false, const void** out_padded = nullptr, int core_B = 0) {
   ForwardPlan p;
-  msla_status_t s = validate_desc(desc, &p);
+  msla_status_t s = validate_desc(desc, &p, core_B);
   if (s != MSLA_OK) return s;
   if (!x || !out || !w) return fail(MSLA_ERR_INVALID_ARG, "null x, out or weights");
   if (!w->w_qkv || !w->w_dw || !w->w_pw || !w->w_proj) return fail(MSLA_ERR_INVALID_ARG, "null weight pointer");
   if (p.S == 3 && (!w->w_dw2 || !w->w_pw2)) return fail(MSLA_ERR_INVALID_ARG, "three branches need w_dw2 and w_pw2");
-  const void* ptrs[] = {host_io ? nullptr : x, host_io ? nullptr : out, w->w_qkv, w->w_dw, w->w_pw, w->w_proj, w->b_proj, desc->workspace,
+  const void* ptrs[] = {x, out, w->w_qkv, w->w_dw, w->w_pw, w->w_proj, w->b_proj, desc->workspace,
                         p.S == 3 ? w->w_dw2 : nullptr, p.S == 3 ? w->w_pw2 : nullptr};
   for (const void* ptr : ptrs)
     if (ptr && !aligned16(ptr)) return fail(MSLA_ERR_ALIGNMENT, "all device pointers must be 16-byte aligned");
   const size_t e = elem_size(desc->dtype);
   const size_t xb = (size_t)desc->B * desc->C * p.N * e, ob = (size_t)desc->B * desc->C_out * p.N * e;
-  const size_t need = p.bytes + (host_io ? align_up(xb, 256) + align_up(ob, 256) : 0);
-  if (!desc->workspace || desc->workspace_bytes < need)
-    return fail(MSLA_ERR_WORKSPACE, "workspace of %zu bytes needed, %zu given", need, desc->workspace ? desc->workspace_bytes : (size_t)0);
+  if (!desc->workspace || desc->workspace_bytes < p.bytes)
+    return fail(MSLA_ERR_WORKSPACE, "workspace of %zu bytes needed, %zu given", p.bytes, desc->workspace ? desc->workspace_bytes : (size_t)0);
   if (overlaps(out, ob, x, xb)) return fail(MSLA_ERR_INVALID_ARG, "out overlaps x");
-  if (!host_io && (overlaps(out, ob, desc->workspace, need) || overlaps(x, xb, desc->workspace, need)))
+  if (overlaps(out, ob, desc->workspace, p.bytes) || overlaps(x, xb, desc->workspace, p.bytes))
     return fail(MSLA_ERR_INVALID_ARG, "workspace overlaps x or out");
   s = check_arch();
   if (s != MSLA_OK) return s;
@@ -475,15 +475,6 @@ static msla_status_t forward_impl(const msla_desc* desc, const void* x, const ms
   char* ws = (char*)desc->workspace;
   const void* x_dev = x;
   void* out_dev = out;
-  if (host_io) {
-    x_dev = ws + p.bytes;
-    out_dev = ws + p.bytes + align_up(xb, 256);
-    const cudaError_t ce = cudaMemcpyAsync((void*)x_dev, x, xb, cudaMemcpyHostToDevice, st);
-    if (ce != cudaSuccess) {
-      cudaGetLastError();
-      return fail(MSLA_ERR_CUDA, "host-to-device copy of x: %s", cudaGetErrorString(ce));
-    }
-  }
   const int Cp = p.Cp, N = p.N, d = desc->d, heads = desc->heads;
   const int S = p.S, Ht = S * heads;
   const long long ld_att = (long long)S * Cp;
@@ -533,12 +524,100 @@ static msla_status_t forward_impl(const msla_desc* desc, const void* x, const ms
   if (s != MSLA_OK) return s;
   if (p.padded() && (s = run_unpad_rows(y_dev, out_dev, (long long)desc->B * desc->C_out, N, p.pitch, st)) != MSLA_OK) return s;
   if ((s = record(events, 5, st)) != MSLA_OK) return s;
-  if (host_io) {
-    const cudaError_t ce = cudaMemcpyAsync(out, out_dev, ob, cudaMemcpyDeviceToHost, st);
-    if (ce != cudaSuccess) {
+  return MSLA_OK;
+}
+
+// ------------------------------------------------------------ host buffers
+// The two copy streams of a thread on one device, created on first use and destroyed with the thread.  Calls of one thread
+// on several streams share them, ordered by events like any other work.
+struct CopyLanes {
+  int dev = -1;
+  cudaStream_t in = nullptr, out = nullptr;
+  cudaEvent_t arrived = nullptr, done = nullptr;
+  bool create(int device) {
+    if (dev == device) return true;
+    release();
+    if (cudaStreamCreateWithFlags(&in, cudaStreamNonBlocking) != cudaSuccess || cudaStreamCreateWithFlags(&out, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&arrived, cudaEventDisableTiming) != cudaSuccess || cudaEventCreateWithFlags(&done, cudaEventDisableTiming) != cudaSuccess) {
       cudaGetLastError();
-      return fail(MSLA_ERR_CUDA, "device-to-host copy of out: %s", cudaGetErrorString(ce));
+      release();
+      return false;
     }
+    dev = device;
+    return true;
+  }
+  void release() {  // work already submitted still completes
+    if (in) cudaStreamDestroy(in);
+    if (out) cudaStreamDestroy(out);
+    if (arrived) cudaEventDestroy(arrived);
+    if (done) cudaEventDestroy(done);
+    in = out = nullptr; arrived = done = nullptr; dev = -1;
+  }
+  ~CopyLanes() { release(); }
+};
+
+// A batch goes through in parts of whole images: the copy to the device of one part, the forward of the part before it and the
+// copy back of the one before that run at the same time (the link is full duplex, and the copies, not the kernels, are what
+// takes the time).  Nothing flows back before the first part is through, and nothing in after the last, so those are small
+// (HOST_PART_BYTES); a copy has a fixed cost of 5 to 10 us, so the parts between them grow.  [16, 256, 64, 64] bf16, 33.5 MB each way
+// (628 us one way, 724 both at once): 1400 us with all copies on one stream, 1130 us in equal parts of 2 MB, 1010 us so.  On a capturing stream, and for a single part, everything stays on the caller's stream.
+constexpr size_t HOST_PART_BYTES = 4 << 20;
+
+static msla_status_t forward_host_impl(const msla_desc* desc, const void* x, const msla_weights* w, void* out, cudaStream_t st) {
+  ForwardPlan p;
+  msla_status_t s = validate_desc(desc, &p);
+  if (s != MSLA_OK) return s;
+  if (!x || !out || !w) return fail(MSLA_ERR_INVALID_ARG, "null x, out or weights");
+  if (desc->workspace && !aligned16(desc->workspace)) return fail(MSLA_ERR_ALIGNMENT, "all device pointers must be 16-byte aligned");
+  const size_t e = elem_size(desc->dtype);
+  const size_t xi = (size_t)desc->C * p.N * e, oi = (size_t)desc->C_out * p.N * e;  // bytes per image
+  const size_t xb = desc->B * xi, ob = desc->B * oi;
+  const size_t need = p.bytes + align_up(xb, 256) + align_up(ob, 256);
+  if (!desc->workspace || desc->workspace_bytes < need)
+    return fail(MSLA_ERR_WORKSPACE, "workspace of %zu bytes needed, %zu given", need, desc->workspace ? desc->workspace_bytes : (size_t)0);
+  if (overlaps(out, ob, x, xb)) return fail(MSLA_ERR_INVALID_ARG, "out overlaps x");
+  if ((s = check_arch()) != MSLA_OK) return s;
+  char* x_dev = (char*)desc->workspace + p.bytes;
+  char* out_dev = x_dev + align_up(xb, 256);
+
+  // images per part: whole multiples of 16 bytes, so that every part of the staging buffers is aligned
+  int step = (int)((HOST_PART_BYTES + (xi < oi ? oi : xi) - 1) / (xi < oi ? oi : xi));
+  while (step < desc->B && ((step * xi) % 16 || (step * oi) % 16)) ++step;
+  thread_local CopyLanes lanes;
+  int dev = -1;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  const bool overlap = step < desc->B && cudaStreamIsCapturing(st, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone &&
+                       cudaGetDevice(&dev) == cudaSuccess && lanes.create(dev);
+  cudaGetLastError();
+  cudaError_t ce = cudaSuccess;
+  auto ok = [&](cudaError_t r) {
+    if (ce == cudaSuccess) ce = r;
+    return ce == cudaSuccess;
+  };
+  if (overlap && ok(cudaEventRecord(lanes.done, st))) ok(cudaStreamWaitEvent(lanes.in, lanes.done, 0));  // the staging buffers are free by then
+  msla_desc part = *desc;
+  part.B = 0;
+  for (int b = 0; b < desc->B && ce == cudaSuccess; b += part.B) {
+    const int left = desc->B - b;
+    int n = part.B + step;                                              // one step more than the part before,
+    if (n > 4 * step) n = 4 * step;                                     // up to four steps,
+    if (n > (left + 1) / 2) n = ((left + 1) / 2 + step - 1) / step * step;  // and at most half of what is left
+    part.B = !overlap || n > left ? left : n;
+    const char* xs = (const char*)x + b * xi;
+    if (!ok(cudaMemcpyAsync(x_dev + b * xi, xs, part.B * xi, cudaMemcpyHostToDevice, overlap ? lanes.in : st))) break;
+    if (overlap && (!ok(cudaEventRecord(lanes.arrived, lanes.in)) || !ok(cudaStreamWaitEvent(st, lanes.arrived, 0)))) break;
+    if ((s = forward_impl(&part, x_dev + b * xi, w, out_dev + b * oi, st, nullptr, false, nullptr, desc->B)) != MSLA_OK) break;
+    if (overlap && (!ok(cudaEventRecord(lanes.done, st)) || !ok(cudaStreamWaitEvent(lanes.out, lanes.done, 0)))) break;
+    ok(cudaMemcpyAsync((char*)out + b * oi, out_dev + b * oi, part.B * oi, cudaMemcpyDeviceToHost, overlap ? lanes.out : st));
+  }
+  if (overlap) {  // also after an error: the caller's stream orders everything that was submitted
+    if (cudaEventRecord(lanes.arrived, lanes.in) == cudaSuccess) ok(cudaStreamWaitEvent(st, lanes.arrived, 0));
+    if (cudaEventRecord(lanes.done, lanes.out) == cudaSuccess) ok(cudaStreamWaitEvent(st, lanes.done, 0));
+  }
+  if (s != MSLA_OK) return s;
+  if (ce != cudaSuccess) {
+    cudaGetLastError();
+    return fail(MSLA_ERR_CUDA, "copies between host and device: %s", cudaGetErrorString(ce));
   }
   return MSLA_OK;
 }
@@ -774,7 +853,7 @@ static msla_status_t block_impl(const msla_desc* attn, const msla_weights* aw, c
     return fail(MSLA_ERR_INVALID_ARG, "y overlaps x, out or a workspace");
   // y = MSLA(x) + x: the output projection's epilogue adds the residual
   const void* y_padded = nullptr;
-  if ((s = forward_impl(attn, x, aw, y, st, nullptr, false, true, &y_padded)) != MSLA_OK) return s;
+  if ((s = forward_impl(attn, x, aw, y, st, nullptr, true, &y_padded)) != MSLA_OK) return s;
   return ffn_impl(ffn, y, fw, out, true, st, ap.padded() ? y_padded : nullptr);
 }
 
@@ -817,7 +896,7 @@ size_t msla_forward_workspace_bytes(const msla_desc* desc) {
 }
 
 msla_status_t msla_forward(const msla_desc* desc, const void* x, const msla_weights* w, void* out, void* stream) {
-  return forward_impl(desc, x, w, out, (cudaStream_t)stream, nullptr, false);
+  return forward_impl(desc, x, w, out, (cudaStream_t)stream, nullptr);
 }
 
 msla_status_t msla_forward_profiled(const msla_desc* desc, const void* x, const msla_weights* w, void* out,
@@ -825,7 +904,7 @@ msla_status_t msla_forward_profiled(const msla_desc* desc, const void* x, const 
   if (!events || n_events != 6) return fail(MSLA_ERR_INVALID_ARG, "events must hold exactly 6 cudaEvent_t handles");
   for (int i = 0; i < 6; ++i)
     if (!events[i]) return fail(MSLA_ERR_INVALID_ARG, "events[%d] is null", i);
-  return forward_impl(desc, x, w, out, (cudaStream_t)stream, events, false);
+  return forward_impl(desc, x, w, out, (cudaStream_t)stream, events);
 }
 
 size_t msla_forward_host_workspace_bytes(const msla_desc* desc) {
@@ -836,7 +915,7 @@ size_t msla_forward_host_workspace_bytes(const msla_desc* desc) {
 }
 
 msla_status_t msla_forward_host(const msla_desc* desc, const void* x_host, const msla_weights* w, void* out_host, void* stream) {
-  return forward_impl(desc, x_host, w, out_host, (cudaStream_t)stream, nullptr, true);
+  return forward_host_impl(desc, x_host, w, out_host, (cudaStream_t)stream);
 }
 
 msla_status_t msla_band_states(const msla_desc* desc, const void* x_band, const msla_weights* w, int halo_top, int halo_bottom,

@@ -275,3 +275,31 @@ def test_many_images_with_few_heads(B, C, H, W, heads, d):
     for _ in range(3):
         util.assert_close(util.run_module(s, t), ref, "bf16", "many images", block=util.MODULE_BLOCK)
     assert binding.msla_debug_wait_timeouts() == 0
+
+
+# Host buffers large enough to go through in parts of whole images (copies overlapped with the kernels): equal bit for bit to
+# the call on device tensors, also when calls follow one another on one workspace and when the last part is a small one.
+@pytest.mark.parametrize("dtype,B,C,H,W,heads,d", [("bf16", 7, 64, 64, 96, 2, 32), ("f32", 5, 32, 96, 65, 2, 16), ("f16", 9, 64, 57, 71, 4, 16)])
+def test_forward_host_in_parts(dtype, B, C, H, W, heads, d):
+    dt = util.TORCH_DTYPE[dtype]
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    rnd = lambda *shape: (torch.randn(*shape, generator=gen, device="cuda") * shape[-1] ** -0.5).to(dt)
+    weights = [rnd(3 * heads * d, C), rnd(3 * heads * d, 5, 5), rnd(3 * heads * d, d), rnd(C, 2 * heads * d)]
+    w = binding.make_weights(*weights)
+    d0 = binding.make_desc(B, C, H, W, heads, d, C, util.CODE[dtype])
+    ws = torch.empty(binding.msla_forward_host_workspace_bytes(d0), dtype=torch.uint8, device="cuda")
+    desc = binding.make_desc(B, C, H, W, heads, d, C, util.CODE[dtype], workspace=ws)
+    xs = [torch.randn(B, C, H, W, generator=gen, device="cuda").to(dt) for _ in range(2)]
+    refs = []
+    for x in xs:
+        out = torch.empty_like(x)
+        binding.msla_forward(desc, x, w, out)
+        refs.append(out.cpu())
+    hx = [x.cpu().pin_memory() for x in xs]
+    ho = [torch.empty_like(x).pin_memory() for x in hx]
+    for _ in range(2):
+        for i in range(2):
+            binding.msla_forward_host(desc, hx[i], w, ho[i])
+    torch.cuda.synchronize()
+    for i in range(2):
+        assert torch.equal(ho[i], refs[i])
