@@ -257,10 +257,17 @@ kv_combine_bf16path_kernel(const float* __restrict__ partial, float* __restrict_
 // state_scale: the state (numerator and denominator columns alike) and eps are multiplied by it before they are cut
 // into 16-bit pieces; the quotient of Eq. 3 does not change.  1 for bf16 (its exponent range is fp32's); for fp16 a
 // power of two near 1/N, so that sums over N tokens fit the format.
-template <int D, int NWARPS, int STAGES, int U, bool PAIR, bool F16>
+// PLANES: the queries lie in channel-blocked planes [token / 8][D][8] (PlanesView); a warp copies them as they lie and
+// ldmatrix.trans makes the fragments.
+struct PlanesView {
+  const unsigned char *q0, *q1;      // see PlanesQueries (msla_host.h)
+  long long plane_bytes, tok_bytes;  // bytes of a plane; offset of the first token inside it
+  int heads, B;                      // heads per scale
+};
+template <int D, int NWARPS, int STAGES, int U, bool PAIR, bool F16, bool PLANES = false>
 __global__ void __launch_bounds__(NWARPS * 32)
 apply_mma_kernel(const bf16* __restrict__ q, const float* __restrict__ state, bf16* __restrict__ out,
-                 HeadView qv, HeadView ov, int heads, int N, float eps, int tok_per_cta, float state_scale) {
+                 HeadView qv, HeadView ov, int heads, int N, float eps, int tok_per_cta, float state_scale, PlanesView pv) {
   constexpr int KS = D / 16;   // MMA steps over the channel contraction
   constexpr int NT = D / 8;    // output tiles, + 1 for the denominator
   constexpr int CPT = D / 4;   // channels per lane per token
@@ -287,10 +294,28 @@ apply_mma_kernel(const bf16* __restrict__ q, const float* __restrict__ state, bf
   constexpr int TS = 16 * U;
   const int groups = (n_end - n_begin + TS - 1) / TS;
   const int my_groups = groups > wslot ? (groups - wslot + NW - 1) / NW : 0;
-  const uint32_t ring = smem_u32(fifo) + warp * (STAGES * STAGEB) + lane * LB;
+  constexpr int OCTET = D * 16;  // bytes of eight tokens of a plane
+  static_assert(STAGEB == TS * D * 2, "a stage holds TS tokens in either layout");
+  const uint32_t ring = smem_u32(fifo) + warp * (STAGES * STAGEB) + (PLANES ? 0 : lane * LB);
+  const unsigned char* plane = nullptr;
+  if constexpr (PLANES) {
+    const int sc = h / pv.heads, hd = h - sc * pv.heads;
+    plane = (sc == 0 ? pv.q0 + ((long long)b * pv.heads + hd) * 3 * pv.plane_bytes
+                     : pv.q1 + (((long long)(sc - 1) * pv.B + b) * pv.heads + hd) * pv.plane_bytes) + pv.tok_bytes;
+  }
 
   auto issue = [&](int it) {
     const uint32_t dst = ring + (it % STAGES) * STAGEB;
+    if constexpr (PLANES) {
+      const int first = n_begin + (wslot + it * NW) * TS;
+#pragma unroll
+      for (int i = 0; i < STAGEB / 512; ++i) {
+        const int off = (i * 32 + lane) * 16, n = first + off / OCTET * 8;
+        const bool ok = n < n_end;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + off), "l"(plane + (ok ? (long long)first * (D * 2) + off : 0)), "r"(ok ? 16 : 0) : "memory");
+      }
+      return;
+    }
     const int n0 = n_begin + (wslot + it * NW) * TS + g;
 #pragma unroll
     for (int u = 0; u < 2 * U; ++u) {  // u even: token g of tile u/2, odd: token g+8
@@ -319,7 +344,7 @@ apply_mma_kernel(const bf16* __restrict__ q, const float* __restrict__ state, bf
       for (int j = 0; j <= NT; ++j)
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-          const int a0 = CPT * t + 4 * ks + 2 * r;
+          const int a0 = PLANES ? 16 * ks + 2 * t + 8 * r : CPT * t + 4 * ks + 2 * r;
           const int c = j < NT ? (g >> 1) * CPT + 2 * j + (g & 1) : D;
           const float v0 = __uint_as_float(ld_dep32(st + a0 * (D + 1) + c)) * state_scale, v1 = __uint_as_float(ld_dep32(st + (a0 + 1) * (D + 1) + c)) * state_scale;
           bhi[ks][j][r] = pack16<F16>(v0, v1);
@@ -334,9 +359,17 @@ apply_mma_kernel(const bf16* __restrict__ q, const float* __restrict__ state, bf
     const uint32_t src = ring + (it % STAGES) * STAGEB;
     const int n0 = n_begin + (wslot + it * NW) * TS;
     uint32_t qa[U][WQ], qb[U][WQ];
+    if constexpr (PLANES) __syncwarp();  // the other lanes' copies
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      if constexpr (LB == 16) {
+      if constexpr (PLANES) {  // A fragments of 16 tokens: (octet 2u, channels 8cb ..), (octet 2u + 1, ..)
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) {
+          uint32_t r[4];
+          ldsm_x4_trans(r, src + (2 * u + ((lane >> 3) & 1)) * OCTET + (2 * ks + (lane >> 4)) * 128 + (lane & 7) * 16);
+          qa[u][2 * ks] = r[0]; qb[u][2 * ks] = r[1]; qa[u][2 * ks + 1] = r[2]; qb[u][2 * ks + 1] = r[3];
+        }
+      } else if constexpr (LB == 16) {
         lds128(qa[u], src + (2 * u) * 32 * LB);
         lds128(qb[u], src + (2 * u + 1) * 32 * LB);
       } else {
@@ -381,6 +414,7 @@ apply_mma_kernel(const bf16* __restrict__ q, const float* __restrict__ state, bf
       if (na < n_end) stg(out + obase + (long long)na * ov.ld, oa);
       if (nb < n_end) stg(out + obase + (long long)nb * ov.ld, ob);
     }
+    if constexpr (PLANES) __syncwarp();  // the stage may be overwritten
   }
   cp_async_wait<0>();
 }
@@ -416,11 +450,11 @@ msla_status_t launch_core(const bf16* q, const bf16* k, const bf16* v, bf16* out
     if (ov.pair) {  // heads is even here, so a pair never straddles two images
       const int tok_per_cta = p.apply_tokens / 2;
       launch_pdl(apply_mma_kernel<D, AP_WARPS, AP_STAGES, AP_U, true, F16>, dim3((unsigned)ceil_div_ll(N, tok_per_cta), (unsigned)(BH / 2)),
-                 dim3(AP_WARPS * 32), 0, st, q, state, out, in, ov, heads, N, eps, tok_per_cta, state_scale);
+                 dim3(AP_WARPS * 32), 0, st, q, state, out, in, ov, heads, N, eps, tok_per_cta, state_scale, PlanesView{});
     } else {
       const int tok_per_cta = p.apply_tokens;
       launch_pdl(apply_mma_kernel<D, AP_WARPS, AP_STAGES, AP_U, false, F16>, dim3((unsigned)ceil_div_ll(N, tok_per_cta), (unsigned)BH),
-                 dim3(AP_WARPS * 32), 0, st, q, state, out, in, ov, heads, N, eps, tok_per_cta, state_scale);
+                 dim3(AP_WARPS * 32), 0, st, q, state, out, in, ov, heads, N, eps, tok_per_cta, state_scale, PlanesView{});
     }
     ++launches;
   }
@@ -428,7 +462,32 @@ msla_status_t launch_core(const bf16* q, const bf16* k, const bf16* v, bf16* out
   return check_launch(F16 ? "attention core kernels (fp16)" : "attention core kernels (bf16)");
 }
 
+template <int D, bool F16>
+msla_status_t launch_apply_planes(const PlanesView& pv, const float* state, bf16* out, HeadView ov, int B, int Ht, int N, float eps, float state_scale, cudaStream_t st) {
+  constexpr int AP_WARPS = 4, AP_STAGES = 4, AP_U = 2;
+  const long long BH = (long long)B * Ht;
+  const int tok = make_core_plan(BH, N, D).apply_tokens;
+  if (ov.pair)
+    launch_pdl(apply_mma_kernel<D, AP_WARPS, AP_STAGES, AP_U, true, F16, true>, dim3((unsigned)ceil_div_ll(N, tok / 2), (unsigned)(BH / 2)), dim3(AP_WARPS * 32), 0, st,
+               nullptr, state, out, HeadView{}, ov, Ht, N, eps, tok / 2, state_scale, pv);
+  else
+    launch_pdl(apply_mma_kernel<D, AP_WARPS, AP_STAGES, AP_U, false, F16, true>, dim3((unsigned)ceil_div_ll(N, tok), (unsigned)BH), dim3(AP_WARPS * 32), 0, st,
+               nullptr, state, out, HeadView{}, ov, Ht, N, eps, tok, state_scale, pv);
+  count_launches(1);
+  return check_launch("apply step on channel-blocked planes");
+}
+
 }  // namespace
+
+msla_status_t run_apply_planes(const PlanesQueries& q, const float* state, void* att, HeadView ov, int B, int Ht, int N, int d, float eps,
+                               long long sum_tokens, cudaStream_t st, bool f16) {
+  const PlanesView pv{(const unsigned char*)q.q0, (const unsigned char*)q.q1, q.plane_tokens * d * 2, q.first_token * d * 2, q.heads, B};
+  float scale = 1.f;  // fp16 pieces of the state must fit the format: a sum over N tokens is scaled by the power of two just above 1/N
+  if (f16) for (long long n = 1; n < sum_tokens; n *= 2) scale *= 0.5f;
+  bf16* out = (bf16*)att;
+  if (d == 32) return f16 ? launch_apply_planes<32, true>(pv, state, out, ov, B, Ht, N, eps * scale, scale, st) : launch_apply_planes<32, false>(pv, state, out, ov, B, Ht, N, eps, scale, st);
+  return f16 ? launch_apply_planes<16, true>(pv, state, out, ov, B, Ht, N, eps * scale, scale, st) : launch_apply_planes<16, false>(pv, state, out, ov, B, Ht, N, eps, scale, st);
+}
 
 msla_status_t run_core_bf16(const void* q, const void* k, const void* v, void* out, HeadView in, HeadView ov, int B,
                             int heads, int N, int d, float eps, const CorePlan& p, void* ws, cudaStream_t st,

@@ -32,6 +32,11 @@
 //                  (RES kernels: the same block of a residual tensor, fetched by TMA into a block of its own one
 //                  block ahead of its use, is added before the conversion: the residual connection around the module)
 //   Two accumulator sets (2 x 256 TMEM columns) let the drain of a tile overlap the next.
+// Queries come in one of two layouts: planes [token][d] (above), or (PL) channel-blocked planes [token / 8][d][8], where eight
+// tokens of one channel are 16 contiguous bytes.  PL kernels fetch a head's 128 tokens by one bulk copy (contiguous in the
+// plane); a transform warp takes 32 tokens through ldmatrix.trans, which gives a lane the same two channels of every channel
+// octet for four tokens, the four lanes of a token add their parts of the normaliser, and stmatrix.trans puts the scaled queries
+// back; the MMA reads them as they lie (tokens contiguous: an MN-major operand of 8 x 8 core matrices without swizzle).
 // No TMA load is multicast: each CTA loads its own operands; only tcgen05.commit signals
 // both CTAs' barriers.  Every mbarrier wait is bounded as in the GEMM.
 #include <cuda.h>
@@ -64,6 +69,9 @@ static_assert(24 * O_MAX_STAGES + 16 + 16 + 8 + 8 + 8 + 4 * 8 + 8 <= O_BAR_BYTES
 __device__ int g_fused_timeout_flag = 0;
 
 struct OutParams {
+  const unsigned char *q0, *q1;      // PL: see PlanesQueries (msla_host.h)
+  long long plane_bytes, tok_bytes;  // PL: bytes of a plane; offset of the first token inside it
+  int heads;                         // PL: heads per scale
   const float* ks;   // [B][Ht][d] key sums
   const bf16* bias;  // [Cout] or nullptr
   const bf16* residual;  // RES kernels: [B][Cout][N], added to the output (the residual connection around the module)
@@ -126,6 +134,14 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
 __device__ __forceinline__ uint64_t make_desc_kmajor(uint32_t addr, uint32_t sbo16, uint64_t mode) {
   return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)sbo16 << 32) | (1ull << 46) | (mode << 61);
 }
+// Descriptor of an MN-major operand without swizzle: core matrices of 8 k x 8 tokens (16-byte rows, 128 contiguous bytes);
+// lbo16 = distance between groups of 8 k, sbo16 = between groups of 8 tokens, in 16-byte units.
+__device__ __forceinline__ uint64_t make_desc_octets(uint32_t addr, uint32_t lbo16, uint32_t sbo16) {
+  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)lbo16 << 16) | ((uint64_t)sbo16 << 32) | (1ull << 46);
+}
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
 __device__ __forceinline__ void umma2_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
@@ -164,6 +180,9 @@ template <bool F16> __device__ __forceinline__ uint32_t pack16(float lo, float h
 // partial: [B*Ht][S][D*(D+1)] fp32, entry [a][c], column D = key sum.
 //   ks[bh][a]            = sum_s partial[bh][s][a][D]
 //   M[b][m][hh*D + a]    = sum_c w[m][hh*D + c] * (sum_s partial[bh][s][a][c])        (16 bit, row stride K), all m < Cout
+// SLOTS: the partial states are the slots that the aggregation's CTAs wrote (msla_host.h, AggStatePlan): a contiguous run of
+// them, and those of aggregated scales still lack the grouped 1x1 of the values, S[a][c] = sum_c' Wv[c][c'] (sum_s ..)[a][c'].
+// With M == nullptr the states go to state_out [B*Ht][D][D+1] instead.
 // Fixed summation order, the same for every DA: the S partial states are cut into eight runs of consecutive indices, each run
 // is summed in index order (eight 16-byte loads in flight) and the run sums are added in run order.  With few heads every run
 // has threads of its own, otherwise a thread sums FOLD_RUNS / GROUPS of them.
@@ -194,18 +213,35 @@ __device__ __forceinline__ void fold_mma(float (&c)[4], const uint32_t (&a)[4], 
 
 // F16: M and ks are multiplied by `scale`, a power of two near 1 / N (the output kernel scales eps alike, so Eq. 3's quotient is
 // unchanged): sums over N tokens then stay inside binary16's range.
-template <int D, int DA, bool F16>
+struct FoldParams {
+  const float* partial;      // [B*Ht][S][D][D+1]
+  int S;
+  const float* slots[2];     // SLOTS: per aggregated branch (the first also carries scale 0)
+  const bf16* w_pw[2];       // SLOTS: the branches' grouped 1x1 weights
+  int slot_floats, grid, kv_cost;  // SLOTS: of the aggregation
+  long long tiles, cost;
+  const bf16* w;             // projection weights [Cout][K]
+  bf16* M;
+  float *ks, *state_out;
+  int B, heads, Ht, Cout, K;
+  float scale;
+};
+template <int D, int DA, bool F16, bool SLOTS>
 __global__ void __launch_bounds__(FoldShape<D, DA>::THREADS, DA == D ? 4 : 1)
-state_fold_kernel(const float* __restrict__ partial, int S, const bf16* __restrict__ w, bf16* __restrict__ M, float* __restrict__ ks,
-                  int Ht, int Cout, int K, float scale) {
+state_fold_kernel(FoldParams p) {
   constexpr int GROUPS = FoldShape<D, DA>::GROUPS, NV = FoldShape<D, DA>::NV, THREADS = FoldShape<D, DA>::THREADS;
   constexpr int D1 = D + 1, NE4 = D * D1 / 4, WARPS = THREADS / 32;
   constexpr int KS = D / 16, NT = DA / 8, PIECES = F16 ? 2 : 3;
   __shared__ float4 run_sum[GROUPS == 1 ? 1 : FOLD_RUNS][NV];
   __shared__ uint32_t rounded[PIECES][DA][D / 2 + 1];  // pairs of neighbouring c
+  __shared__ float wv[SLOTS ? D : 1][D + 1];           // SLOTS: Wv transposed, [c'][c]
   float* st = reinterpret_cast<float*>(run_sum[0]);
   pdl_launch_dependents();
+  const int Ht = p.Ht, Cout = p.Cout, K = p.K;
+  const float scale = p.scale;
+  const bf16* w = p.w;
   const int bh = blockIdx.x, b = bh / Ht, hh = bh % Ht, a0 = blockIdx.y * DA;
+  const int branch = SLOTS ? hh / p.heads : 0, h = SLOTS ? hh - branch * p.heads : 0;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
   // A fragments of 16 output channels: lane (g, t) holds c = t*D/4 .. + D/4 - 1 of rows g and g + 8
   auto load_weights = [&](int m0, uint32_t (&x)[2][D / 8]) {
@@ -223,9 +259,30 @@ state_fold_kernel(const float* __restrict__ partial, int S, const bf16* __restri
     }
   };
   uint32_t x[2][D / 8];
-  load_weights(16 * warp, x);  // the projection weights do not come from the previous kernel: fetched while it drains
-  pdl_wait();                  // the partial states do
-  const float4* sp = reinterpret_cast<const float4*>(partial + (long long)bh * S * (D * D1) + a0 * D1);
+  // the weights do not come from the previous kernel: fetched while it drains; the partial states do
+  if (p.M) load_weights(16 * warp, x);
+  if (SLOTS && branch > 0) {
+    const bf16* src = (branch == 2 ? p.w_pw[1] : p.w_pw[0]) + (long long)(3 * h + 2) * D * D;
+    for (int i = tid; i < D * D / 2; i += THREADS) {
+      const uint32_t v = __ldg(reinterpret_cast<const uint32_t*>(src) + i);
+      const int c = i / (D / 2), k = i % (D / 2) * 2;
+      wv[k][c] = lo16<F16>(v);
+      wv[k + 1][c] = hi16<F16>(v);
+    }
+  }
+  pdl_wait();
+  int S = p.S;
+  long long stride4 = NE4;
+  const float* first = p.partial + (long long)bh * S * (D * D1);
+  if constexpr (SLOTS) {
+    constexpr int HPB = 32 / D;  // heads per slot
+    const long long seg = (long long)(h / HPB) * p.B + b;
+    const long long c0 = agg_state_cta_of(p.cost, p.kv_cost, seg * p.tiles, p.grid), c1 = agg_state_cta_of(p.cost, p.kv_cost, (seg + 1) * p.tiles - 1, p.grid);
+    S = (int)(c1 - c0) + 1;
+    stride4 = p.slot_floats / 4;
+    first = (branch == 2 ? p.slots[1] : p.slots[0]) + (seg + c0) * p.slot_floats + ((h % HPB) * 2 + (branch > 0 ? 1 : 0)) * (D * D1);
+  }
+  const float4* sp = reinterpret_cast<const float4*>(first + a0 * D1);
   auto add = [](float4& v, const float4& x) { v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w; };
   if (tid < GROUPS * NV) {
     const int group = tid / NV, e = tid - group * NV;
@@ -233,7 +290,7 @@ state_fold_kernel(const float* __restrict__ partial, int S, const bf16* __restri
     if (GROUPS == 1 && S <= 8) {  // a run has one partial state or none
       float4 q[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) q[u] = u < S ? ld_dep128f(sp + (long long)u * NE4 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int u = 0; u < 8; ++u) q[u] = u < S ? ld_dep128f(sp + u * stride4 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int u = 0; u < 8; ++u) add(total, q[u]);
     } else {
@@ -244,7 +301,7 @@ state_fold_kernel(const float* __restrict__ partial, int S, const bf16* __restri
         for (int s = s0; s < s1; s += 8) {
           float4 q[8];
 #pragma unroll
-          for (int u = 0; u < 8; ++u) q[u] = s + u < s1 ? ld_dep128f(sp + (long long)(s + u) * NE4 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int u = 0; u < 8; ++u) q[u] = s + u < s1 ? ld_dep128f(sp + (s + u) * stride4 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
           for (int u = 0; u < 8; ++u) add(v, q[u]);
         }
@@ -264,7 +321,32 @@ state_fold_kernel(const float* __restrict__ partial, int S, const bf16* __restri
     }
     __syncthreads();
   }
-  if (tid < DA) ks[(long long)bh * D + a0 + tid] = F16 ? st[tid * D1 + D] * scale : st[tid * D1 + D];
+  if (SLOTS && branch > 0) {  // the grouped 1x1 of the values: an entry of the CTA's rows per thread and round
+    constexpr int PER = (DA * D + THREADS - 1) / THREADS;
+    float mixed[PER];
+#pragma unroll
+    for (int r = 0; r < PER; ++r) {
+      const int i = tid + r * THREADS, al = i / D, c = i % D;
+      float v = 0.f;
+      if (i < DA * D) {
+#pragma unroll
+        for (int k = 0; k < D; ++k) v = fmaf(wv[k][c], st[al * D1 + k], v);
+      }
+      mixed[r] = v;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < PER; ++r) {
+      const int i = tid + r * THREADS;
+      if (i < DA * D) st[i / D * D1 + i % D] = mixed[r];
+    }
+    __syncthreads();
+  }
+  if (!p.M) {
+    for (int i = tid; i < DA * D1; i += THREADS) p.state_out[(long long)bh * (D * D1) + a0 * D1 + i] = st[i];
+    return;
+  }
+  if (tid < DA) p.ks[(long long)bh * D + a0 + tid] = F16 ? st[tid * D1 + D] * scale : st[tid * D1 + D];
   for (int i = tid; i < DA * D / 2; i += THREADS) {
     const int al = i / (D / 2), c2 = i - al * (D / 2);
     float v0 = st[al * D1 + 2 * c2], v1 = st[al * D1 + 2 * c2 + 1];
@@ -303,7 +385,7 @@ state_fold_kernel(const float* __restrict__ partial, int S, const bf16* __restri
     for (int r = 0; r < 2; ++r) {
       const int m = m0 + g + 8 * r;
       if (m >= Cout) continue;
-      bf16* row = M + ((long long)b * Cout + m) * K + hh * D + a0;
+      bf16* row = p.M + ((long long)b * Cout + m) * K + hh * D + a0;
       if constexpr (DA == D) {
         uint32_t o[NT];
 #pragma unroll
@@ -318,7 +400,7 @@ state_fold_kernel(const float* __restrict__ partial, int S, const bf16* __restri
   }
 }
 
-template <int D, bool RES, bool F16>
+template <int D, bool RES, bool F16, bool PL>
 __global__ void __launch_bounds__(O_THREADS, 1)
 fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant__ CUtensorMap tmQ,
                  const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmR, OutParams p) {
@@ -327,7 +409,8 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
   const uint32_t a_base = smem_base;                                  // resident rows of M: kslices x 16 KB
   constexpr int SLICE = OT * D * 2;                                    // one head's queries of this CTA's (up to) 128 tokens
   constexpr int SLOT = 2 * SLICE;                                      // ring slot: two consecutive heads
-  constexpr int ROWB = D * 2;                                          // bytes per token row = the swizzle span
+  constexpr int ROWB = D * 2;                                          // bytes per token row = the swizzle span (not PL)
+  constexpr int OCTET = D * 16;                                        // PL: bytes of eight tokens
   const uint32_t ring = a_base + (uint32_t)p.kslices * O_A_SLICE;
   const uint32_t staging = ring + (uint32_t)p.stages * SLOT;
   const uint32_t resbuf = staging + O_STAGING;           // RES: one 32-channel x 64-token block of the residual per epilogue warp
@@ -388,7 +471,7 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
     // ------------------------------------------------------------ TMA producer (each CTA for itself)
     if (lane == 0) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tmM) : "memory");
-      asm volatile("prefetch.tensormap [%0];" ::"l"(&tmQ) : "memory");
+      if (!PL) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmQ) : "memory");
       uint32_t s = 0, ph = 0, mfree_ph = 0;  // ring slot and the parity of its current use
       int cur_b = -1;
       bool ok = true;
@@ -412,9 +495,25 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
           ok = mbar_wait_cluster(empty_bar + 8 * s, ph ^ 1, &abort_flag);
           if (!ok) break;
           const bool two = h + 1 < p.Ht;  // an odd head count leaves the last slot half used
-          mbar_expect_tx(full_bar + 8 * s, (uint32_t)((two ? 2 : 1) * p.ot * ROWB));
-          tma_load_4d(ring + s * SLOT, &tmQ, full_bar + 8 * s, 0, n0, h, b);  // rows past the last token are filled with zeros
-          if (two) tma_load_4d(ring + s * SLOT + SLICE, &tmQ, full_bar + 8 * s, 0, n0, h + 1, b);
+          if constexpr (PL) {
+            // tokens past the last one are not copied: their accumulator columns are never stored
+            const uint32_t bytes = (uint32_t)max(0, min(p.ot, p.N - n0)) * (D * 2);
+            auto query = [&](int hq) -> const unsigned char* {
+              const int sc = hq / p.heads, hd = hq - sc * p.heads;
+              const unsigned char* plane = sc == 0 ? p.q0 + ((long long)b * p.heads + hd) * 3 * p.plane_bytes
+                                                   : p.q1 + (((long long)(sc - 1) * p.B + b) * p.heads + hd) * p.plane_bytes;
+              return plane + p.tok_bytes + (long long)n0 * (D * 2);
+            };
+            mbar_expect_tx(full_bar + 8 * s, (two ? 2u : 1u) * bytes);
+            if (bytes) {
+              bulk_load(ring + s * SLOT, query(h), bytes, full_bar + 8 * s);
+              if (two) bulk_load(ring + s * SLOT + SLICE, query(h + 1), bytes, full_bar + 8 * s);
+            }
+          } else {
+            mbar_expect_tx(full_bar + 8 * s, (uint32_t)((two ? 2 : 1) * p.ot * ROWB));
+            tma_load_4d(ring + s * SLOT, &tmQ, full_bar + 8 * s, 0, n0, h, b);  // rows past the last token are filled with zeros
+            if (two) tma_load_4d(ring + s * SLOT + SLICE, &tmQ, full_bar + 8 * s, 0, n0, h + 1, b);
+          }
           if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1; }
         }
       }
@@ -422,13 +521,13 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (leader) / M hand-shake (peer)
     if (lane == 0) {
-      // instruction descriptor: D = f32, A = B = bf16, both K-major, N = 256, M = 256 (pair)
-      const uint32_t idesc = (1u << 4) | (F16 ? 0u : ((1u << 7) | (1u << 10))) | ((uint32_t)((2 * p.ot) >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
+      // instruction descriptor: D = f32, A = B = bf16, both K-major (PL: B MN-major), N = 256, M = 256 (pair)
+      const uint32_t idesc = (1u << 4) | (F16 ? 0u : ((1u << 7) | (1u << 10))) | (PL ? 1u << 16 : 0u) | ((uint32_t)((2 * p.ot) >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
       const uint32_t peer_res_remote = map_to_cta(peer_res_bar, 0);
       uint32_t local = 0, res_ph = 0, s = 0, ph = 0;  // s, ph: ring slot and the parity of its current use
       // Matrix descriptors: the high words are constants; the low words carry the start address in 16-byte units
       // (A: the 128B-swizzled rows of M; B: the slice, K-major, the swizzle span being the token row).
-      const uint64_t a_hi = make_desc(0, 1, 1024 >> 4), b_hi = make_desc_kmajor(0, (8 * ROWB) >> 4, D == 32 ? 4ull : 6ull);
+      const uint64_t a_hi = make_desc(0, 1, 1024 >> 4), b_hi = PL ? make_desc_octets(0, 128 >> 4, OCTET >> 4) : make_desc_kmajor(0, (8 * ROWB) >> 4, D == 32 ? 4ull : 6ull);
       const uint32_t a_lo0 = (a_base & 0x3FFFFu) >> 4, b_lo0 = (ring & 0x3FFFFu) >> 4;
       int cur_b = -1;
       bool ok = true;
@@ -464,7 +563,7 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
             if (h + j >= p.Ht) break;
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk) {
-              umma2_bf16(d_tmem, a_hi | a_lo, b_hi | (b_lo + (uint32_t)(j * (SLICE >> 4) + 2 * kk)), idesc, (h > 0 || j > 0 || kk > 0) ? 1u : 0u);
+              umma2_bf16(d_tmem, a_hi | a_lo, b_hi | (b_lo + (uint32_t)(j * (SLICE >> 4) + (PL ? 16 : 2) * kk)), idesc, (h > 0 || j > 0 || kk > 0) ? 1u : 0u);
               col += 16;
               a_lo += (col & 63) ? 2u : (uint32_t)((O_A_SLICE - 96) >> 4);
             }
@@ -500,6 +599,63 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
         if (!mine) continue;
         // with 64-token tiles only the first two warps of a group own rows; past the last head there is nothing to do
         const bool has_row = (int)row < p.ot && h < p.Ht;
+        if constexpr (PL) {
+          constexpr int CB = D / 8;  // channel octets; register (o, cb) of lane (g, t) holds channels 8 cb + 2t, + 1 of token 8 o + g
+          const int t = lane & 3;
+          float2 kk[CB];  // the lane's key sums, fetched before the wait so that their latency hides behind it
+          const float2* ksp = reinterpret_cast<const float2*>(p.ks + ((long long)b * p.Ht + min(h, p.Ht - 1)) * D) + t;
+#pragma unroll
+          for (int cb = 0; cb < CB; ++cb) {
+            const uint2 v = ld_dep64(ksp + 4 * cb);
+            kk[cb] = make_float2(__uint_as_float(v.x), __uint_as_float(v.y));
+          }
+          ok = mbar_wait(full_bar + 8 * cs, cph, &abort_flag);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          if (wig * 32 >= p.ot || h >= p.Ht) {  // warp-uniform
+            if (lane == 0) mbar_arrive_cluster(ready_remote + 8 * cs);
+            continue;
+          }
+          const uint32_t base = ring + cs * SLOT + (uint32_t)(h & 1) * SLICE + (uint32_t)(wig * 4 * OCTET + lane * 16);
+          uint32_t q[4 * CB];  // q[o * CB + cb]
+#pragma unroll
+          for (int i = 0; i < CB; ++i)
+            asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                         : "=r"(q[4 * i]), "=r"(q[4 * i + 1]), "=r"(q[4 * i + 2]), "=r"(q[4 * i + 3]) : "r"(base + i * 512) : "memory");
+          float den[4];
+#pragma unroll
+          for (int o = 0; o < 4; ++o) {
+            float d0 = 0.f, d1 = 0.f;
+#pragma unroll
+            for (int cb = 0; cb < CB; ++cb) {
+              uint32_t& w = q[o * CB + cb];
+              if constexpr (F16) asm("max.f16x2 %0, %1, %2;" : "=r"(w) : "r"(w), "r"(0u));
+              else asm("max.bf16x2 %0, %1, %2;" : "=r"(w) : "r"(w), "r"(0u));
+              d0 = fmaf(lo16<F16>(w), kk[cb].x, d0);
+              d1 = fmaf(hi16<F16>(w), kk[cb].y, d1);
+            }
+            den[o] = d0 + d1;
+          }
+          // sum over the four lanes of a token; lane t ends up with octet 2 (t & 1) + (t >> 1)
+          const bool odd = t & 1, up = t & 2;
+          const float k0 = (odd ? den[2] : den[0]) + __shfl_xor_sync(0xffffffffu, odd ? den[0] : den[2], 1);
+          const float k1 = (odd ? den[3] : den[1]) + __shfl_xor_sync(0xffffffffu, odd ? den[1] : den[3], 1);
+          const float tot = (up ? k1 : k0) + __shfl_xor_sync(0xffffffffu, up ? k0 : k1, 2);
+          const float inv = __frcp_rn(tot + p.eps);
+#pragma unroll
+          for (int o = 0; o < 4; ++o) {
+            const float io = __shfl_sync(0xffffffffu, inv, (lane & ~3) | (o >> 1) | ((o & 1) << 1));
+#pragma unroll
+            for (int cb = 0; cb < CB; ++cb) {
+              uint32_t& w = q[o * CB + cb];
+              w = pack16<F16>(lo16<F16>(w) * io, hi16<F16>(w) * io);
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < CB; ++i)
+            asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(base + i * 512), "r"(q[4 * i]), "r"(q[4 * i + 1]),
+                         "r"(q[4 * i + 2]), "r"(q[4 * i + 3]) : "memory");
+        } else {
         // the head's key sums, fetched before the wait so that their latency hides behind it
         float kk[D];
         const float4* ksp = reinterpret_cast<const float4*>(p.ks + ((long long)b * p.Ht + min(h, p.Ht - 1)) * D);
@@ -536,6 +692,7 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
         for (int c = 0; c < PCS; ++c)
           asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(rbase + (((uint32_t)c ^ swz) << 4)), "r"(q[4 * c]), "r"(q[4 * c + 1]),
                        "r"(q[4 * c + 2]), "r"(q[4 * c + 3]) : "memory");
+        }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the tensor cores read what was just written
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(ready_remote + 8 * cs);
@@ -659,43 +816,63 @@ size_t fused_out_scratch_bytes(int B, int Ht, int d, int Cout) { return fused_ou
 // column d).  q: planar bf16 query matrices [N][d], head h of image b at q + b*q_sb + h*q_sh (elements); y (and
 // residual): [B, Cout, N] with rows ldy elements apart.
 namespace {
-template <int D, bool RES, bool F16>
+template <int D, bool RES, bool F16, bool PL>
 msla_status_t launch_fused(dim3 grid, int smem, cudaStream_t st, const CUtensorMap& tmM, const CUtensorMap& tmQ, const CUtensorMap& tmO,
                            const CUtensorMap& tmR, const OutParams& p) {
   static std::atomic<unsigned long long> attr_done{0};
-  const msla_status_t s = ensure_smem_attr(attr_done, fused_out_kernel<D, RES, F16>, O_SMEM_LIMIT);
+  const msla_status_t s = ensure_smem_attr(attr_done, fused_out_kernel<D, RES, F16, PL>, O_SMEM_LIMIT);
   if (s != MSLA_OK) return s;
-  launch_pdl_cluster2(fused_out_kernel<D, RES, F16>, grid, dim3(O_THREADS), (size_t)smem, st, tmM, tmQ, tmO, tmR, p);
-  return MSLA_OK;
+  launch_pdl_cluster2(fused_out_kernel<D, RES, F16, PL>, grid, dim3(O_THREADS), (size_t)smem, st, tmM, tmQ, tmO, tmR, p);
+  count_launches(1);
+  return check_launch("fused apply + output projection (tcgen05, paired CTAs)");
 }
-template <int D, bool F16>
-msla_status_t launch_fold(const float* partial, int S, const void* w, bf16* M, float* ks, int B, int Ht, int Cout, float scale, cudaStream_t st) {
-  // few heads: a head's key channels are shared out, to about one CTA per SM
-  const int heads = B * Ht, sms = device_sm_count(), K = Ht * D;
-  if (D == 32 && 4 * heads <= sms)
-    launch_pdl(state_fold_kernel<D, 8, F16>, dim3(heads, D / 8), dim3(FoldShape<D, 8>::THREADS), 0, st, partial, S, (const bf16*)w, M, ks, Ht, Cout, K, scale);
-  else if (2 * heads <= sms)
-    launch_pdl(state_fold_kernel<D, D / 2, F16>, dim3(heads, 2), dim3(FoldShape<D, D / 2>::THREADS), 0, st, partial, S, (const bf16*)w, M, ks, Ht, Cout, K, scale);
-  else
-    launch_pdl(state_fold_kernel<D, D, F16>, dim3(heads), dim3(FoldShape<D, D>::THREADS), 0, st, partial, S, (const bf16*)w, M, ks, Ht, Cout, K, scale);
-  return check_launch("sum of the partial states");
-}
-template <bool F16>
+template <bool F16, bool PL>
 msla_status_t launch_fused_for(int d, bool res, dim3 grid, int smem, cudaStream_t st, const CUtensorMap& tmM, const CUtensorMap& tmQ,
                                const CUtensorMap& tmO, const CUtensorMap& tmR, const OutParams& p) {
-  if (d == 32) return res ? launch_fused<32, true, F16>(grid, smem, st, tmM, tmQ, tmO, tmR, p) : launch_fused<32, false, F16>(grid, smem, st, tmM, tmQ, tmO, tmR, p);
-  return res ? launch_fused<16, true, F16>(grid, smem, st, tmM, tmQ, tmO, tmR, p) : launch_fused<16, false, F16>(grid, smem, st, tmM, tmQ, tmO, tmR, p);
+  if (d == 32) return res ? launch_fused<32, true, F16, PL>(grid, smem, st, tmM, tmQ, tmO, tmR, p) : launch_fused<32, false, F16, PL>(grid, smem, st, tmM, tmQ, tmO, tmR, p);
+  return res ? launch_fused<16, true, F16, PL>(grid, smem, st, tmM, tmQ, tmO, tmR, p) : launch_fused<16, false, F16, PL>(grid, smem, st, tmM, tmQ, tmO, tmR, p);
+}
+
+template <int D, bool F16, bool SLOTS>
+msla_status_t launch_fold(const FoldParams& p, cudaStream_t st) {
+  // few heads: a head's key channels are shared out, to about one CTA per SM
+  const int heads = p.B * p.Ht, sms = device_sm_count();
+  if (D == 32 && 4 * heads <= sms) launch_pdl(state_fold_kernel<D, 8, F16, SLOTS>, dim3(heads, D / 8), dim3(FoldShape<D, 8>::THREADS), 0, st, p);
+  else if (2 * heads <= sms) launch_pdl(state_fold_kernel<D, D / 2, F16, SLOTS>, dim3(heads, 2), dim3(FoldShape<D, D / 2>::THREADS), 0, st, p);
+  else launch_pdl(state_fold_kernel<D, D, F16, SLOTS>, dim3(heads), dim3(FoldShape<D, D>::THREADS), 0, st, p);
+  count_launches(1);
+  return check_launch("sum of the partial states");
+}
+msla_status_t run_fold(const FoldStates& in, FoldParams& f, int d, cudaStream_t st, bool f16) {
+  f.partial = in.partial; f.S = in.S;
+  const bool slots = in.plan.grid > 0;
+  for (int i = 0; i < 2; ++i) { f.slots[i] = in.slots[i]; f.w_pw[i] = (const bf16*)in.w_pw[i]; }
+  f.slot_floats = in.plan.slot_floats; f.grid = in.plan.grid; f.kv_cost = in.plan.kv_cost; f.tiles = in.plan.kv_tiles; f.cost = in.plan.cost;
+  if (!slots && f.S < 1) return fail(MSLA_ERR_UNSUPPORTED, "fused apply + projection: %d partial states per head", f.S);
+  if (d == 32) {
+    if (slots) return f16 ? launch_fold<32, true, true>(f, st) : launch_fold<32, false, true>(f, st);
+    return f16 ? launch_fold<32, true, false>(f, st) : launch_fold<32, false, false>(f, st);
+  }
+  if (slots) return f16 ? launch_fold<16, true, true>(f, st) : launch_fold<16, false, true>(f, st);
+  return f16 ? launch_fold<16, true, false>(f, st) : launch_fold<16, false, false>(f, st);
 }
 }  // namespace
 
+msla_status_t run_sum_states(const FoldStates& in, float* state_out, int B, int heads, int Ht, int d, cudaStream_t st, bool f16) {
+  FoldParams f{};
+  f.state_out = state_out;
+  f.B = B; f.heads = heads; f.Ht = Ht; f.scale = 1.f;
+  return run_fold(in, f, d, st, f16);
+}
+
 // f16: queries, weights, bias, residual and output are IEEE binary16 instead of bfloat16; M, the key sums and eps are
 // scaled by the power of two just above 1 / N (N tokens' sums would leave binary16's range otherwise).
-msla_status_t run_fused_out_bf16(const void* q, long long q_sb, long long q_sh, const float* partial, int S, void* scratch,
+// planes: nullptr, or the channel-blocked query planes that take the place of q.
+msla_status_t run_fused_out_bf16(const void* q, long long q_sb, long long q_sh, const PlanesQueries* planes, const FoldStates& states, void* scratch,
                                  const void* w, const void* bias, const void* residual, void* y, int ldy, int B, int Ht, int d, int N, int Cout,
                                  float eps, cudaStream_t st, bool f16) {
-  if (!fused_out_bf16_supported(Ht, d, Cout) || ldy % 8 != 0 || q_sb % 8 != 0 || q_sh % 8 != 0)
+  if (!fused_out_bf16_supported(Ht, d, Cout) || ldy % 8 != 0 || q_sb % 8 != 0 || q_sh % 8 != 0 || (planes && N % 8 != 0))
     return fail(MSLA_ERR_UNSUPPORTED, "fused apply + projection: %d heads of %d channels, %d output channels, %d tokens", Ht, d, Cout, N);
-  if (S < 1) return fail(MSLA_ERR_UNSUPPORTED, "fused apply + projection: %d partial states per head", S);
   const int K = Ht * d;
   // 256-token tiles per pair of CTAs; 128-token tiles for problems so small that half the pairs would have nothing
   // to do (the larger tile is the more efficient one as soon as every pair has work)
@@ -715,16 +892,26 @@ msla_status_t run_fused_out_bf16(const void* q, long long q_sb, long long q_sh, 
     const cuuint64_t sO[2] = {(cuuint64_t)ldy * 2, (cuuint64_t)Cout * ldy * 2};
     const cuuint32_t bO[3] = {64, 32, 1};
     if (!tma_make_map_bf16(&tmM, M, 3, dM, sM, bM, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !tma_make_map_bf16(&tmQ, q, 4, dQ, sQ, bQ, d == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B) ||
+        (!planes && !tma_make_map_bf16(&tmQ, q, 4, dQ, sQ, bQ, d == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B)) ||
         !tma_make_map_bf16(&tmO, y, 3, dO, sO, bO, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !tma_make_map_bf16(&tmR, residual ? residual : y, 3, dO, sO, bO, CU_TENSOR_MAP_SWIZZLE_128B))
       return fail(MSLA_ERR_CUDA, "cuTensorMapEncodeTiled failed for the fused apply + output projection");
+    if (planes) tmQ = tmM;  // not read
   }
-  OutParams p{};
-  p.ks = ks; p.bias = (const bf16*)bias; p.residual = (const bf16*)residual;
   float scale = 1.f;
   if (f16)
     for (long long n = 1; n < N; n <<= 1) scale *= 0.5f;
+  FoldParams f{};
+  f.w = (const bf16*)w; f.M = M; f.ks = ks;
+  f.B = B; f.heads = planes ? planes->heads : Ht; f.Ht = Ht; f.Cout = Cout; f.K = K; f.scale = scale;
+  msla_status_t s = run_fold(states, f, d, st, f16);
+  if (s != MSLA_OK) return s;
+  OutParams p{};
+  if (planes) {
+    p.q0 = (const unsigned char*)planes->q0; p.q1 = (const unsigned char*)planes->q1; p.heads = planes->heads;
+    p.plane_bytes = planes->plane_tokens * d * 2; p.tok_bytes = planes->first_token * d * 2;
+  }
+  p.ks = ks; p.bias = (const bf16*)bias; p.residual = (const bf16*)residual;
   p.B = B; p.N = N; p.Cout = Cout; p.Ht = Ht; p.d = d; p.eps = eps * scale;
   p.kslices = (K + OKS - 1) / OKS;
   p.ot = ot;
@@ -741,15 +928,10 @@ msla_status_t run_fused_out_bf16(const void* q, long long q_sb, long long q_sh, 
   long long pairs = sms / 2;
   if (pairs > tiles) pairs = tiles;
   if (pairs < 1) pairs = 1;
-  msla_status_t s = d == 32 ? (f16 ? launch_fold<32, true>(partial, S, w, M, ks, B, Ht, Cout, scale, st) : launch_fold<32, false>(partial, S, w, M, ks, B, Ht, Cout, scale, st))
-                            : (f16 ? launch_fold<16, true>(partial, S, w, M, ks, B, Ht, Cout, scale, st) : launch_fold<16, false>(partial, S, w, M, ks, B, Ht, Cout, scale, st));
-  if (s != MSLA_OK) return s;
   const dim3 grid((unsigned)(2 * pairs));
-  s = f16 ? launch_fused_for<true>(d, residual != nullptr, grid, smem, st, tmM, tmQ, tmO, tmR, p)
-          : launch_fused_for<false>(d, residual != nullptr, grid, smem, st, tmM, tmQ, tmO, tmR, p);
-  if (s != MSLA_OK) return s;
-  count_launches(2);
-  return check_launch("fused apply + output projection (tcgen05, paired CTAs)");
+  const bool res = residual != nullptr;
+  if (planes) return f16 ? launch_fused_for<true, true>(d, res, grid, smem, st, tmM, tmQ, tmO, tmR, p) : launch_fused_for<false, true>(d, res, grid, smem, st, tmM, tmQ, tmO, tmR, p);
+  return f16 ? launch_fused_for<true, false>(d, res, grid, smem, st, tmM, tmQ, tmO, tmR, p) : launch_fused_for<false, false>(d, res, grid, smem, st, tmM, tmQ, tmO, tmR, p);
 }
 
 int fused_timeout_flag() {

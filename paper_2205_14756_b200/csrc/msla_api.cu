@@ -271,12 +271,28 @@ struct ForwardPlan {
   int Cp, N;
   int S;              // branches: the projected tokens and S - 1 aggregated copies
   size_t wpad2_off;   // embedded taps of the second aggregated branch
-  // 16-bit storage: the projections read x and write out as rows of `pitch` elements; where H*W is no multiple of 8 those
-  // are padded copies in the workspace (repack.cu), otherwise the caller's tensors
+  // 16-bit storage: the projections read x and write out as rows of `pitch` elements, one per channel; where the caller's rows
+  // are not as wide those are padded copies in the workspace (repack.cu), otherwise the caller's tensors
   int pitch;
   size_t xpad_off, ypad_off;
   bool padded() const { return pitch != N; }
+  // Channel-blocked planes (see planes_path): ms holds the 3*heads projected planes per image, then the aggregated query
+  // planes branch by branch.
+  bool planes;
+  size_t q1_off, state_off, partial_bytes;  // from core_off: the partial states of branch br at (br - 1) * partial_bytes
+  AggStatePlan agg;
 };
+
+// Which layout the multi-scale tokens take between the steps: planes of token rows [N][d] and a kernel per step, or
+// channel-blocked planes (msla_host.h) with steps 2 and 3 in one kernel.  The second moves less (the aggregated keys and values
+// are never written) and spends half the shared-memory cycles on step 2, but its kernel has one CTA per SM and a longer
+// start-up, and rows that are no whole number of pixel octets would have to be padded in copies.  Whole forward, us, old / new
+// layout: [1, 256, 512, 512] 491 / 417, [1, 128, 512, 512] d = 16 309 / 254, [16, 256, 64, 64] 147 / 142, [1, 256, 128, 256] 81 / 75,
+// [8, 128, 128, 40] 63 / 61; below the line [1, 256, 128, 128] 51 / 52, [4, 256, 64, 64] 53 / 54, [64, 256, 14, 14] 79 / 80; ragged rows
+// [12, 128, 220, 134] 369 / 396.
+static bool planes_path(const msla_desc* d) {
+  return d->dtype != MSLA_F32 && d->W % 8 == 0 && d->H >= 2 && (long long)d->B * d->H * d->W * d->heads * d->d >= (5LL << 20);
+}
 
 // core_B: images the split of the token reduction is planned for, where a call is a part of a batch (0: desc->B); its sums
 // are then those of the whole batch, bit for bit.
@@ -309,11 +325,22 @@ static msla_status_t validate_desc(const msla_desc* d, ForwardPlan* plan, int co
   size_t att_bytes = tokens * S * plan->Cp * e;
   const size_t fused_scratch = fused_out_bf16_supported(S * d->heads, d->d, d->C_out) ? fused_out_scratch_bytes(d->B, S * d->heads, d->d, d->C_out) : 0;
   if (att_bytes < fused_scratch) att_bytes = fused_scratch;
+  plan->planes = planes_path(d);
+  plan->pitch = d->dtype == MSLA_F32 ? plan->N : (int)align_up((size_t)plan->N, 8);
+  size_t core_bytes = plan->core.bytes;
+  if (plan->planes) {
+    plan->agg = make_agg_state_plan(d->B, d->heads, d->H, d->W, d->d);
+    plan->q1_off = align_up(tokens * 3 * plan->Cp * e, 256);
+    plan->att_off = plan->q1_off + align_up(tokens * (S - 1) * plan->Cp * e, 256);
+    att_bytes = fused_out_bf16_supported(S * d->heads, d->d, d->C_out) ? fused_scratch : tokens * S * plan->Cp * e;
+    plan->partial_bytes = align_up(plan->agg.partial_bytes, 256);
+    plan->state_off = (S - 1) * plan->partial_bytes;
+    core_bytes = plan->state_off + align_up((size_t)d->B * S * d->heads * d->d * (d->d + 1) * sizeof(float), 256);
+  }
   plan->core_off = plan->att_off + align_up(att_bytes, 256);
-  plan->wpad_off = plan->core_off + plan->core.bytes;
+  plan->wpad_off = plan->core_off + core_bytes;
   plan->wpad2_off = plan->wpad_off + (d->agg_kernel == 3 ? align_up((size_t)3 * plan->Cp * 25 * e, 256) : 0);
   plan->xpad_off = plan->wpad2_off + (S == 3 && d->agg_kernel2 == 3 ? align_up((size_t)3 * plan->Cp * 25 * e, 256) : 0);
-  plan->pitch = d->dtype == MSLA_F32 ? plan->N : (int)align_up((size_t)plan->N, 8);
   plan->ypad_off = plan->xpad_off + (plan->padded() ? align_up((size_t)d->B * d->C * plan->pitch * e, 256) : 0);
   // (bands of such an image may be ragged where the whole is not, so the output's copy depends on the row length)
   plan->bytes = plan->ypad_off + (d->dtype != MSLA_F32 && d->W % 8 != 0 ? align_up((size_t)d->B * d->C_out * plan->pitch * e, 256) : 0);
@@ -438,6 +465,68 @@ static msla_status_t run_branches(const msla_desc* desc, const msla_weights* w, 
   return MSLA_OK;
 }
 
+static msla_status_t record(void* const* events, int i, cudaStream_t st);
+
+static FoldStates dense_states(const void* partial, int S) {
+  FoldStates in{};
+  in.partial = (const float*)partial;
+  in.S = S;
+  return in;
+}
+
+// ---- channel-blocked planes: steps 2 and 3, and what steps 4 and 5 read
+static FoldStates planes_states(const msla_desc* desc, const msla_weights* w, const ForwardPlan& p) {
+  FoldStates in{};
+  for (int br = 1; br < p.S; ++br) {
+    in.slots[br - 1] = reinterpret_cast<const float*>((const char*)desc->workspace + p.core_off + (br - 1) * p.partial_bytes);
+    in.w_pw[br - 1] = br == 1 ? w->w_pw : w->w_pw2;
+  }
+  in.plan = p.agg;
+  return in;
+}
+
+// Image rows [row_lo, row_hi) count in the states.
+static msla_status_t run_planes_branches(const msla_desc* desc, const msla_weights* w, const ForwardPlan& p, int row_lo, int row_hi, cudaStream_t st) {
+  char* ws = (char*)desc->workspace;
+  for (int br = 1; br < p.S; ++br) {
+    const msla_status_t s = run_agg_state(ws + p.ms_off, ws + p.q1_off + (size_t)(br - 1) * desc->B * p.Cp * p.pitch * 2, (float*)(ws + p.core_off + (br - 1) * p.partial_bytes),
+                                          aggregation_taps(desc, w, p, br, st), br == 1 ? w->w_pw : w->w_pw2, p.agg, desc->B, desc->heads, desc->H, desc->W,
+                                          desc->d, row_lo, row_hi, br == 1, st, desc->dtype == MSLA_F16);
+    if (s != MSLA_OK) return s;
+  }
+  return MSLA_OK;
+}
+
+// Steps 4 and 5 on `tokens` tokens of every plane from `first` on; rows of y and residual are `tokens` apart.
+static msla_status_t run_planes_rest(const msla_desc* desc, const msla_weights* w, const ForwardPlan& p, const FoldStates& in, int first, int tokens,
+                                     long long sum_tokens, const void* residual, void* y, void* const* events, cudaStream_t st) {
+  char* ws = (char*)desc->workspace;
+  const bool f16 = desc->dtype == MSLA_F16;
+  const int B = desc->B, Ht = p.S * desc->heads, d = desc->d;
+  char* att = ws + p.att_off;
+  const PlanesQueries q{ws + p.ms_off, ws + p.q1_off, desc->heads, p.pitch, first};
+  msla_status_t s = MSLA_OK;
+  if (fused_out_bf16_supported(Ht, d, desc->C_out)) {
+    if (events && ((s = record(events, 3, st)) != MSLA_OK || (s = record(events, 4, st)) != MSLA_OK)) return s;
+    return run_fused_out_bf16(nullptr, 0, 0, &q, in, att, w->w_proj, w->b_proj, residual, y, tokens, B, Ht, d, tokens, desc->C_out, desc->eps, st, f16);
+  }
+  // attention output: one [N][2d] plane per pair of heads where the projection takes it, otherwise token-major
+  const float* state = in.partial;
+  if (in.plan.grid > 0) {
+    float* sum = reinterpret_cast<float*>(ws + p.core_off + p.state_off);
+    if ((s = run_sum_states(in, sum, B, desc->heads, Ht, d, st, f16)) != MSLA_OK) return s;
+    state = sum;
+  }
+  if ((s = record(events, 3, st)) != MSLA_OK) return s;
+  const long long ld_att = (long long)p.S * p.Cp;
+  const bool paired = d == 32 && Ht % 2 == 0 && project_out_planar_bf16_supported(p.S * p.Cp, desc->C_out);
+  const HeadView ov = paired ? HeadView{(long long)tokens * ld_att, (long long)tokens * 2 * d, 2 * d, 1} : HeadView{(long long)tokens * ld_att, d, ld_att, 0};
+  if ((s = run_apply_planes(q, state, att, ov, B, Ht, tokens, d, desc->eps, sum_tokens, st, f16)) != MSLA_OK) return s;
+  if ((s = record(events, 4, st)) != MSLA_OK) return s;
+  return paired ? run_project_out_planar_bf16(att, w->w_proj, w->b_proj, residual, y, tokens, B, p.S * p.Cp, desc->C_out, tokens, st, f16)
+                : run_project_out(desc->dtype, att, w->w_proj, w->b_proj, y, tokens, B, p.S * p.Cp, desc->C_out, tokens, st, residual);
+}
+
 static msla_status_t record(void* const* events, int i, cudaStream_t st) {
   if (!events) return MSLA_OK;
   const cudaError_t e = cudaEventRecord((cudaEvent_t)events[i], st);
@@ -492,6 +581,15 @@ static msla_status_t forward_impl(const msla_desc* desc, const void* x, const ms
   }
   const void* residual = add_x ? x_dev : nullptr;
   if (out_padded) *out_padded = y_dev;
+  if (p.planes) {
+    // 1. QKV projection; 2 + 3. aggregation and the states of all scales; 4 + 5. apply and output projection
+    if ((s = run_project_planes(x_dev, w->w_qkv, ms, desc->B, desc->C, 3 * Cp, p.pitch, d, 3LL * Cp * p.pitch, st, desc->dtype == MSLA_F16)) != MSLA_OK) return s;
+    if ((s = record(events, 1, st)) != MSLA_OK) return s;
+    if ((s = run_planes_branches(desc, w, p, 0, desc->H, st)) != MSLA_OK) return s;
+    if ((s = record(events, 2, st)) != MSLA_OK) return s;
+    if ((s = run_planes_rest(desc, w, p, planes_states(desc, w, p), 0, p.pitch, N, residual, y_dev, events, st)) != MSLA_OK) return s;
+    return record(events, 5, st);
+  }
   // 1. QKV projection into the scale-0 planes
   s = run_project_in(desc->dtype, x_dev, p.pitch, w->w_qkv, ms, desc->B, desc->C, 3 * Cp, N, d, ms_sb, st);
   if (s != MSLA_OK) return s;
@@ -516,8 +614,8 @@ static msla_status_t forward_impl(const msla_desc* desc, const void* x, const ms
   if ((s = record(events, 4, st)) != MSLA_OK) return s;
   // 5. output projection back to NCHW
   if (fused)
-    s = run_fused_out_bf16(ms, ms_sb, 3LL * N * d, reinterpret_cast<const float*>(ws + p.core_off + p.core.partial_off), p.core.S, att, w->w_proj,
-                           w->b_proj, residual, y_dev, p.pitch, desc->B, Ht, d, N, desc->C_out, desc->eps, st, f16);
+    s = run_fused_out_bf16(ms, ms_sb, 3LL * N * d, nullptr, dense_states(ws + p.core_off + p.core.partial_off, p.core.S), att, w->w_proj, w->b_proj,
+                            residual, y_dev, p.pitch, desc->B, Ht, d, N, desc->C_out, desc->eps, st, f16);
   else
     s = att_planar ? run_project_out_planar_bf16(att, w->w_proj, w->b_proj, residual, y_dev, p.pitch, desc->B, S * Cp, desc->C_out, N, st, f16)
                    : run_project_out(desc->dtype, att, w->w_proj, w->b_proj, y_dev, p.pitch, desc->B, S * Cp, desc->C_out, N, st, residual);
@@ -642,7 +740,7 @@ static msla_status_t validate_band(const msla_desc* desc, int halo_top, int halo
   b->Nb = (desc->H - halo_top - halo_bottom) * desc->W;
   b->tok_off = (long long)halo_top * desc->W;
   b->core = make_core_plan((long long)desc->B * b->f.S * desc->heads, b->Nb, desc->d);
-  if (b->core.bytes > b->f.core.bytes) return fail(MSLA_ERR_WORKSPACE, "band plan exceeds the forward plan");
+  if (!b->f.planes && b->core.bytes > b->f.core.bytes) return fail(MSLA_ERR_WORKSPACE, "band plan exceeds the forward plan");
   if (!desc->workspace || desc->workspace_bytes < b->f.bytes)
     return fail(MSLA_ERR_WORKSPACE, "workspace of %zu bytes needed, %zu given", b->f.bytes, desc->workspace ? desc->workspace_bytes : (size_t)0);
   if (!aligned16(desc->workspace)) return fail(MSLA_ERR_ALIGNMENT, "workspace must be 16-byte aligned");
@@ -674,6 +772,12 @@ static msla_status_t band_states_impl(const msla_desc* desc, const void* x, cons
   if (p.padded()) {
     if ((s = run_pad_rows(x, ws + p.xpad_off, (long long)desc->B * desc->C, N, p.pitch, st)) != MSLA_OK) return s;
     x = ws + p.xpad_off;
+  }
+  if (p.planes) {
+    const bool f16 = desc->dtype == MSLA_F16;
+    if ((s = run_project_planes(x, w->w_qkv, ms, desc->B, desc->C, 3 * Cp, p.pitch, d, 3LL * Cp * p.pitch, st, f16)) != MSLA_OK) return s;
+    if ((s = run_planes_branches(desc, w, p, halo_top, desc->H - halo_bottom, st)) != MSLA_OK) return s;
+    return run_sum_states(planes_states(desc, w, p), state_out, desc->B, desc->heads, p.S * desc->heads, d, st, f16);
   }
   s = run_project_in(desc->dtype, x, p.pitch, w->w_qkv, ms, desc->B, desc->C, 3 * Cp, N, d, ms_sb, st);
   if (s != MSLA_OK) return s;
@@ -715,10 +819,13 @@ static msla_status_t band_output_impl(const msla_desc* desc, const msla_weights*
   const long long ms_sb = 3LL * p.S * Cp * N, ld_att = (long long)p.S * Cp;
   char* ms = ws + p.ms_off;
   char* att = ws + p.att_off;
-  float* state = reinterpret_cast<float*>(ws + p.core_off + b.core.state_off);
+  float* state = reinterpret_cast<float*>(ws + p.core_off + (p.planes ? p.state_off : b.core.state_off));
   generic::band_state_sum_kernel<<<(unsigned)ceil_div_ll(total, 256), 256, 0, st>>>(states, state, R, total);
   count_launches(1);
   if ((s = check_launch("sum of the bands' states")) != MSLA_OK) return s;
+  if (p.planes) {
+    return run_planes_rest(desc, w, p, dense_states(state, 1), (int)b.tok_off, Nb, (long long)R * Nb, nullptr, out, nullptr, st);
+  }
   const char* q = ms + (size_t)b.tok_off * d * e;
   const bool f16 = desc->dtype == MSLA_F16;
   // a band whose token count is no multiple of 8 leaves through the padded copy (reserved for the band with its halo)
@@ -726,7 +833,7 @@ static msla_status_t band_output_impl(const msla_desc* desc, const msla_weights*
   const bool padded = pitch != Nb;
   void* y = padded ? ws + p.ypad_off : out;
   if (desc->dtype != MSLA_F32 && fused_out_bf16_supported(Ht, d, desc->C_out)) {
-    s = run_fused_out_bf16(q, ms_sb, 3LL * N * d, state, 1, att, w->w_proj, w->b_proj, nullptr, y, pitch, desc->B, Ht, d, Nb, desc->C_out, desc->eps, st, f16);
+    s = run_fused_out_bf16(q, ms_sb, 3LL * N * d, nullptr, dense_states(state, 1), att, w->w_proj, w->b_proj, nullptr, y, pitch, desc->B, Ht, d, Nb, desc->C_out, desc->eps, st, f16);
   } else {
     const HeadView in{ms_sb, 3LL * N * d, d};
     const bool att_planar = desc->dtype != MSLA_F32 && d == 32 && Ht % 2 == 0 && project_out_planar_bf16_supported(p.S * Cp, desc->C_out);
@@ -952,8 +1059,13 @@ int msla_forward_fuses_apply(const msla_desc* desc) {
 unsigned long long msla_kernel_launches(void) { return g_launches; }
 
 int msla_debug_wait_timeouts(void) {
-  const int a = gemm_timeout_flag(), b = agg_timeout_flag(), c = fused_timeout_flag(), e = dw_timeout_flag();
-  return (a < 0 || b < 0 || c < 0 || e < 0) ? -1 : (a | b | c | e);
+  int all = 0;
+  for (int (*flag)() : {gemm_timeout_flag, agg_timeout_flag, fused_timeout_flag, dw_timeout_flag, agg_state_timeout_flag, project_planes_timeout_flag}) {
+    const int v = flag();
+    if (v < 0) return -1;
+    all |= v;
+  }
+  return all;
 }
 
 int msla_debug_wait_selftest(long long limit_cycles, void* scratch, void* stream) {

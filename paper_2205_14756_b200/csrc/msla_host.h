@@ -118,9 +118,6 @@ msla_status_t run_ffn_project_bf16(const void* g, const void* w2, const void* b2
 // (elements).
 bool fused_out_bf16_supported(int Ht, int d, int Cout);
 size_t fused_out_scratch_bytes(int B, int Ht, int d, int Cout);
-msla_status_t run_fused_out_bf16(const void* q, long long q_sb, long long q_sh, const float* partial, int S, void* scratch,
-                                 const void* w, const void* bias, const void* residual, void* y, int ldy, int B, int Ht, int d, int N, int Cout,
-                                 float eps, cudaStream_t st, bool f16 = false);
 int fused_timeout_flag();
 int dw_timeout_flag();
 
@@ -149,5 +146,59 @@ int agg_timeout_flag();
 // Rows of n 16-bit elements to and from rows `pitch` (a multiple of 8) elements apart (repack.cu).
 msla_status_t run_pad_rows(const void* src, void* dst, long long rows, int n, int pitch, cudaStream_t st);
 msla_status_t run_unpad_rows(const void* src, void* dst, long long rows, int n, int pitch, cudaStream_t st);
+
+// ---- The 16-bit module path on channel-blocked planes: a plane (q, k or v of one head) is [H][W / 8][d][8], W a multiple of 8,
+// i.e. eight horizontally neighbouring pixels of one channel are 16 contiguous bytes.
+//
+// Aggregation and state sums (agg_state.cu).  The grid's CTAs take contiguous runs of tiles, of equal cost; CTA c writes the
+// part of segment s (a pair of blocks of one image: s = pair * B + image) that it summed to slot s + c (unique, because both
+// grow along the list of tiles).
+constexpr int AGG_STATE_CTAS = 148;
+struct AggStatePlan {
+  int kv_tiles_x, q_tiles_x, tiles_y, grid, slot_floats, kv_cost, q_cost;
+  long long kv_tiles, segments, kv_units, cost;
+  size_t partial_bytes;
+};
+AggStatePlan make_agg_state_plan(int B, int heads, int H, int W, int d);
+// First tile of CTA c; the CTA that has key/value tile u.
+__host__ __device__ inline long long agg_state_first_unit(long long cost, int kv_cost, int q_cost, long long kv_units, long long c, long long grid) {
+  const long long at = cost * c / grid, kv = kv_cost * kv_units;
+  return at < kv ? (at + kv_cost - 1) / kv_cost : kv_units + (at - kv + q_cost - 1) / q_cost;
+}
+__host__ __device__ inline long long agg_state_cta_of(long long cost, int kv_cost, long long u, long long grid) { return (grid * (kv_cost * u + 1) - 1) / cost; }
+// ms0: [B][3*heads] planes; q1: [B][heads] planes; rows [row_lo, row_hi) count in the states.
+msla_status_t run_agg_state(const void* ms0, void* q1, float* partial, const void* w_dw, const void* w_pw, const AggStatePlan& plan, int B,
+                            int heads, int H, int W, int d, int row_lo, int row_hi, bool with_scale0, cudaStream_t st, bool f16);
+int agg_state_timeout_flag();
+
+// Input projection into scale-0 planes (proj_planes.cu): x [B][C][Np], Np a multiple of 8.
+msla_status_t run_project_planes(const void* x, const void* w, void* y, int B, int C, int Cout, int Np, int d, long long y_sb, cudaStream_t st, bool f16);
+int project_planes_timeout_flag();
+
+// Where the partial states lie that the fold adds: [B*Ht][S][d][d+1] (slots.grid == 0), or the slots of the aggregation launches,
+// one per aggregated branch, with the grouped 1x1 weights whose value rows are still to be applied.
+struct FoldStates {
+  const float* partial;
+  int S;
+  const float* slots[2];
+  const void* w_pw[2];
+  AggStatePlan plan;
+};
+// Queries of all scales in channel-blocked planes: query head h of image b at scale 0 is plane (b*heads + h)*3 of q0, at branch s
+// plane ((s-1)*B + b)*heads + h of q1.
+struct PlanesQueries {
+  const void *q0, *q1;
+  int heads;                            // per scale
+  long long plane_tokens, first_token;  // tokens of a plane; first one used (a multiple of 8)
+};
+// Fold and fused output kernel (see above); planes: nullptr, or the query planes that take the place of q.
+msla_status_t run_fused_out_bf16(const void* q, long long q_sb, long long q_sh, const PlanesQueries* planes, const FoldStates& states, void* scratch,
+                                 const void* w, const void* bias, const void* residual, void* y, int ldy, int B, int Ht, int d, int N, int Cout,
+                                 float eps, cudaStream_t st, bool f16 = false);
+// The sum of the partial states [B*Ht][d][d+1] (planes path where steps 4 and 5 stay apart, and bands).
+msla_status_t run_sum_states(const FoldStates& in, float* state_out, int B, int heads, int Ht, int d, cudaStream_t st, bool f16);
+// The apply step on such planes; att token-major or paired planes (ov).  sum_tokens: tokens the states were summed over.
+msla_status_t run_apply_planes(const PlanesQueries& q, const float* state, void* att, HeadView ov, int B, int Ht, int N, int d, float eps,
+                               long long sum_tokens, cudaStream_t st, bool f16);
 
 }  // namespace msla

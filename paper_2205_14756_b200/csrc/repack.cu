@@ -37,7 +37,8 @@ pad_rows_kernel(const unsigned short* __restrict__ src, uint4* __restrict__ dst,
   const long long i = (long long)blockIdx.x * RP_THREADS + threadIdx.x;
   if (i >= count) return;
   const long long row = count <= 0xffffffffLL ? (uint32_t)i / (uint32_t)pieces : i / pieces;
-  dst[i] = load8(src, row * n + (i - row * pieces) * 8, total);
+  const int col = (int)(i - row * pieces) * 8;
+  dst[i] = load8(src, row * n + col, total);
 }
 
 // dst[row][0 .. n) <- src[row][0 .. n) of rows `pitch` apart; a thread writes eight consecutive elements of dst.
