@@ -257,6 +257,8 @@ kv_combine_bf16path_kernel(const float* __restrict__ partial, float* __restrict_
 // state_scale: the state (numerator and denominator columns alike) and eps are multiplied by it before they are cut
 // into 16-bit pieces; the quotient of Eq. 3 does not change.  1 for bf16 (its exponent range is fp32's); for fp16 a
 // power of two near 1/N, so that sums over N tokens fit the format.
+// state: [heads of all images][S][D][D+1], S partial states per head that every CTA adds for itself, in index order (S = 1: the
+// state).  With few of them that costs less than a kernel of its own for the sum: see launch_core.
 // PLANES: the queries lie in channel-blocked planes [token / 8][D][8] (PlanesView); a warp copies them as they lie and
 // ldmatrix.trans makes the fragments.
 struct PlanesView {
@@ -266,7 +268,7 @@ struct PlanesView {
 };
 template <int D, int NWARPS, int STAGES, int U, bool PAIR, bool F16, bool PLANES = false>
 __global__ void __launch_bounds__(NWARPS * 32)
-apply_mma_kernel(const bf16* __restrict__ q, const float* __restrict__ state, bf16* __restrict__ out,
+apply_mma_kernel(const bf16* __restrict__ q, const float* __restrict__ state, int S, bf16* __restrict__ out,
                  HeadView qv, HeadView ov, int heads, int N, float eps, int tok_per_cta, float state_scale, PlanesView pv) {
   constexpr int KS = D / 16;   // MMA steps over the channel contraction
   constexpr int NT = D / 8;    // output tiles, + 1 for the denominator
@@ -334,10 +336,9 @@ apply_mma_kernel(const bf16* __restrict__ q, const float* __restrict__ state, bf
     cp_async_commit();
   }
 
-  // state -> B fragments (bf16 hi + lo), overlapping the first copies
+  // The state's B fragments (bf16 hi + lo), overlapping the first copies
   uint32_t bhi[KS][NT + 1][2], blo[KS][NT + 1][2];
-  {
-    const float* st = state + (long long)bh * D * (D + 1);
+  auto fragments = [&](auto st) {  // st(e): entry e of the head's state
 #pragma unroll
     for (int ks = 0; ks < KS; ++ks)
 #pragma unroll
@@ -346,10 +347,41 @@ apply_mma_kernel(const bf16* __restrict__ q, const float* __restrict__ state, bf
         for (int r = 0; r < 2; ++r) {
           const int a0 = PLANES ? 16 * ks + 2 * t + 8 * r : CPT * t + 4 * ks + 2 * r;
           const int c = j < NT ? (g >> 1) * CPT + 2 * j + (g & 1) : D;
-          const float v0 = __uint_as_float(ld_dep32(st + a0 * (D + 1) + c)) * state_scale, v1 = __uint_as_float(ld_dep32(st + (a0 + 1) * (D + 1) + c)) * state_scale;
+          const float v0 = st(a0 * (D + 1) + c) * state_scale, v1 = st((a0 + 1) * (D + 1) + c) * state_scale;
           bhi[ks][j][r] = pack16<F16>(v0, v1);
           blo[ks][j][r] = pack16<F16>(v0 - round16<F16>(v0), v1 - round16<F16>(v1));
         }
+  };
+  constexpr int NE = D * (D + 1);
+  if (S == 1) {  // every lane fetches its entries: one round trip
+    const float* src = state + (long long)bh * NE;
+    fragments([&](int e) { return __uint_as_float(ld_dep32(src + e)); });
+  } else {
+    // The sums lie in the warps' last FIFO stage meanwhile, which nothing is copied into yet: with memory of their own an SM would
+    // hold a CTA less.
+    constexpr int NV = NE / 4, HPC = PAIR ? 2 : 1, CAP = NWARPS * STAGEB / 16;  // vectors that fit there
+    __shared__ float4 rest[HPC * NV > CAP ? HPC * NV - CAP : 1];
+    auto vec = [&](int i) -> float4* {
+      if (HPC * NV > CAP && i >= CAP) return rest + (i - CAP);
+      return reinterpret_cast<float4*>(fifo + (i / (STAGEB / 16)) * (STAGES * STAGEB) + (STAGES - 1) * STAGEB) + i % (STAGEB / 16);
+    };
+    const float4* src = reinterpret_cast<const float4*>(state) + (long long)(PAIR ? 2 * blockIdx.y : blockIdx.y) * S * NV;
+    for (int i = threadIdx.x; i < HPC * NV; i += NWARPS * 32) {
+      const float4* p = src + (PAIR && i >= NV ? (long long)S * NV + i - NV : i);
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int s = 0; s < S; s += 4) {
+        float4 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = s + u < S ? ld_dep128f(p + (s + u) * NV) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) { v.x += x[u].x; v.y += x[u].y; v.z += x[u].z; v.w += x[u].w; }
+      }
+      *vec(i) = v;
+    }
+    __syncthreads();
+    const int first = PAIR ? (warp & 1) * NE : 0;
+    fragments([&](int e) { e += first; return reinterpret_cast<const float*>(vec(e >> 2))[e & 3]; });
+    __syncthreads();  // every warp has its fragments: the stages may be filled
   }
 
   for (int it = 0; it < my_groups; ++it) {
@@ -436,7 +468,12 @@ msla_status_t launch_core(const bf16* q, const bf16* k, const bf16* v, bf16* out
     launch_pdl(kv_state_mma_kernel<D, KV_WARPS, KV_STAGES, F16>, dim3((unsigned)BH, p.S), dim3(KV_WARPS * 32), kv_smem, st, k, v, partial, in, heads, N, p.S, p.chunk);
     ++launches;
   }
-  if (phases & CORE_COMBINE) {
+  // A few partial states are added by every CTA of the apply step (S of 4 KB each, from L2); a kernel of its own adds them where
+  // there are more (few heads, many chunks), where the caller wants the sum, and for paired planes, whose CTAs serve two heads with
+  // half the tokens each.  Core, us, with / without that kernel: [1, 16, 4096, 32] (S = 16) 19.4 / 16.1, [32, 8, 784, 32] (S = 3) 19.0 /
+  // 17.1, [2, 24, 12000, 32] 39.3 / 38.0; [1, 10, 70844, 32] (S = 60) 52 / 61; module [2, 384, 100, 40] (paired) 58 / 60.
+  const bool direct = (phases & CORE_STATE) && (phases & CORE_APPLY) && !ov.pair && p.S <= 16;
+  if ((phases & CORE_COMBINE) && !direct) {
     const long long total = BH * p.ne;
     launch_pdl(kv_combine_bf16path_kernel, dim3((unsigned)ceil_div_ll(total, 256)), dim3(256), 0, st, partial, state, p.S, p.ne, total);
     ++launches;
@@ -447,14 +484,16 @@ msla_status_t launch_core(const bf16* q, const bf16* k, const bf16* v, bf16* out
     float state_scale = 1.f;
     if (F16) for (long long n = 1; n < N; n *= 2) state_scale *= 0.5f;
     eps *= state_scale;
+    const float* sums = direct ? partial : state;
+    const int S = direct ? p.S : 1;
     if (ov.pair) {  // heads is even here, so a pair never straddles two images
       const int tok_per_cta = p.apply_tokens / 2;
       launch_pdl(apply_mma_kernel<D, AP_WARPS, AP_STAGES, AP_U, true, F16>, dim3((unsigned)ceil_div_ll(N, tok_per_cta), (unsigned)(BH / 2)),
-                 dim3(AP_WARPS * 32), 0, st, q, state, out, in, ov, heads, N, eps, tok_per_cta, state_scale, PlanesView{});
+                 dim3(AP_WARPS * 32), 0, st, q, sums, S, out, in, ov, heads, N, eps, tok_per_cta, state_scale, PlanesView{});
     } else {
       const int tok_per_cta = p.apply_tokens;
       launch_pdl(apply_mma_kernel<D, AP_WARPS, AP_STAGES, AP_U, false, F16>, dim3((unsigned)ceil_div_ll(N, tok_per_cta), (unsigned)BH),
-                 dim3(AP_WARPS * 32), 0, st, q, state, out, in, ov, heads, N, eps, tok_per_cta, state_scale, PlanesView{});
+                 dim3(AP_WARPS * 32), 0, st, q, sums, S, out, in, ov, heads, N, eps, tok_per_cta, state_scale, PlanesView{});
     }
     ++launches;
   }
@@ -469,10 +508,10 @@ msla_status_t launch_apply_planes(const PlanesView& pv, const float* state, bf16
   const int tok = make_core_plan(BH, N, D).apply_tokens;
   if (ov.pair)
     launch_pdl(apply_mma_kernel<D, AP_WARPS, AP_STAGES, AP_U, true, F16, true>, dim3((unsigned)ceil_div_ll(N, tok / 2), (unsigned)(BH / 2)), dim3(AP_WARPS * 32), 0, st,
-               nullptr, state, out, HeadView{}, ov, Ht, N, eps, tok / 2, state_scale, pv);
+               nullptr, state, 1, out, HeadView{}, ov, Ht, N, eps, tok / 2, state_scale, pv);
   else
     launch_pdl(apply_mma_kernel<D, AP_WARPS, AP_STAGES, AP_U, false, F16, true>, dim3((unsigned)ceil_div_ll(N, tok), (unsigned)BH), dim3(AP_WARPS * 32), 0, st,
-               nullptr, state, out, HeadView{}, ov, Ht, N, eps, tok, state_scale, pv);
+               nullptr, state, 1, out, HeadView{}, ov, Ht, N, eps, tok, state_scale, pv);
   count_launches(1);
   return check_launch("apply step on channel-blocked planes");
 }

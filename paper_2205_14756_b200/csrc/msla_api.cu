@@ -100,7 +100,9 @@ CorePlan make_core_plan(long long BH, int N, int d) {
   chunk = ceil_div_ll(chunk, 64) * 64;
   p.chunk = (int)chunk;
   p.S = (int)ceil_div_ll(N, chunk);
-  long long at = ceil_div_ll(ceil_div_ll((long long)N * BH, 1184), 256) * 256;
+  // tokens per CTA of the apply step: all CTAs resident at once, about eight per SM for d = 16; about four for d = 32, where the
+  // state's fragments cost each CTA more (core [8, 16, 4096, 32], us, with CTAs for 1184 / 592: 39.3 / 37.0; d = 16 [16, 8, 9000, 16] 36.5 / 38.2)
+  long long at = ceil_div_ll(ceil_div_ll((long long)N * BH, d == 32 ? 592 : 1184), 256) * 256;
   p.apply_tokens = (int)(at < 256 ? 256 : (at > 2048 ? 2048 : at));
   p.partial_off = 0;
   p.state_off = align_up((size_t)BH * p.S * p.ne * sizeof(float), 256);
