@@ -45,9 +45,13 @@ inline bool tma_make_map_bf16(CUtensorMap* map, const void* base, int rank, cons
   k.base = base; k.rank = rank; k.swizzle = (int)swizzle;
   for (int i = 0; i < rank; ++i) { k.dims[i] = dims[i]; k.box[i] = box[i]; }
   for (int i = 0; i + 1 < rank; ++i) k.strides[i] = strides[i];
-  unsigned long long h = 1469598103934665603ull;  // FNV-1a over the key bytes
-  const unsigned char* kb = reinterpret_cast<const unsigned char*>(&k);
-  for (size_t i = 0; i < sizeof(Key); ++i) h = (h ^ kb[i]) * 1099511628211ull;
+  static_assert(sizeof(Key) % 8 == 0, "hashed in 64-bit words");
+  unsigned long long h = 1469598103934665603ull, words[sizeof(Key) / 8];  // FNV-1a over the key's words: a byte at a time took 0.2 us a map
+  memcpy(words, &k, sizeof(Key));
+  for (unsigned long long w : words) {
+    h = (h ^ w) * 1099511628211ull;
+    h ^= h >> 29;
+  }
   const int set = (int)((h >> 20) % SETS);
   for (int w = 0; w < WAYS; ++w)
     if (cache[set][w].used && memcmp(&cache[set][w].key, &k, sizeof(Key)) == 0) {
