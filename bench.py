@@ -42,6 +42,8 @@ UNIT = "tokens/s"
 STAGES = ("project_in", "aggregate", "kv_state", "apply", "project_out")
 # when the library runs steps 4 and 5 as one kernel (msla_forward_fuses_apply), they are one stage
 STAGES_FUSED = ("project_in", "aggregate", "kv_state", "apply_project")
+# 16-bit storage and many tokens: steps 2 and 3 are one kernel (the event between them falls directly after the one that ends it)
+MERGED = {"aggregate": "aggregate_kv_state"}
 FALLBACK_HBM_GBS = 6650.0
 BLOCKS = 7           # timed blocks of --steps forwards; the median block is reported
 
@@ -49,6 +51,15 @@ BLOCKS = 7           # timed blocks of --steps forwards; the median block is rep
 def workload_by_name(name: str) -> inputs.ModuleShape:
     table = {s.name: s for s in (inputs.CONFIG1, inputs.CONFIG3, inputs.CONFIG4) + inputs.CONFIG5}
     return table[name]
+
+
+def plan_stages(s: inputs.ModuleShape, fused: bool, launches: int) -> tuple:
+    """Names of the steps that one forward of `launches` kernels runs as a kernel (or more) each.  A 16-bit forward takes 5
+    launches with steps 4 and 5 fused and 6 without; one fewer means that steps 2 and 3 are fused too."""
+    names = STAGES_FUSED if fused else STAGES
+    if s.dtype != "f32" and launches == (4 if fused else 5):
+        names = tuple(MERGED.get(n, n) for n in names if n != "kv_state")
+    return names
 
 
 def stage_bytes_per_token(s: inputs.ModuleShape) -> dict:
@@ -59,6 +70,7 @@ def stage_bytes_per_token(s: inputs.ModuleShape) -> dict:
         "project_in": (C + 3 * Cp) * e,
         "aggregate": (3 * Cp + 3 * Cp) * e,
         "kv_state": 2 * 2 * Cp * e,              # K and V of both scales
+        "aggregate_kv_state": (3 * Cp + Cp) * e,  # fused: the aggregated keys and values stay on chip
         "apply": (2 * Cp + 2 * Cp) * e,          # Q of both scales in, attention out
         "project_out": (2 * Cp + Co) * e,
         "apply_project": (2 * Cp + Co) * e,      # fused: Q of both scales in, y out; the head concat stays on chip
@@ -71,6 +83,7 @@ def stage_flops_per_token(s: inputs.ModuleShape) -> dict:
         "project_in": 2 * 3 * Cp * C,
         "aggregate": 2 * (25 * 3 * Cp + 3 * Cp * d),
         "kv_state": 2 * 2 * Cp * (d + 1),
+        "aggregate_kv_state": 2 * (25 * 3 * Cp + 3 * Cp * d) + 2 * 2 * Cp * (d + 1),
         "apply": 2 * 2 * Cp * (d + 1),
         "project_out": 2 * 2 * Cp * Co,
         "apply_project": 2 * 2 * Cp * (d + 1) + 2 * 2 * Cp * Co,
@@ -89,9 +102,10 @@ def measured_peaks() -> tuple:
 
 # Sources that decide each stage's kernels: the recorded DRAM traffic of a stage stays valid while these are unchanged.
 STAGE_SOURCES = {
-    "project_in": ["gemm_tcgen05.cu", "tcgen05_util.cuh", "tma_host.h", "msla_common.cuh"],
+    "project_in": ["gemm_tcgen05.cu", "proj_planes.cu", "tcgen05_util.cuh", "tma_host.h", "msla_common.cuh"],
     "aggregate": ["agg_bf16.cu", "tma_host.h", "msla_common.cuh"],
     "kv_state": ["core_bf16.cu", "msla_common.cuh"],
+    "aggregate_kv_state": ["agg_state.cu", "tma_host.h", "msla_common.cuh"],
     "apply_project": ["fused_out.cu", "tcgen05_util.cuh", "tma_host.h", "msla_common.cuh"],
 }
 
@@ -524,12 +538,15 @@ def main() -> None:
         mdesc = binding.make_desc(ms_shape.B, ms_shape.C, ms_shape.H, ms_shape.W, ms_shape.heads, ms_shape.d, ms_shape.C_out, mcode,
                                   ms_shape.eps, workspace=mws)
         call = lambda i: binding.msla_forward(mdesc, mx, mweights, mo, stream)
-        for i in range(3):
-            call(i)
+        call(0)
+        before = binding.msla_kernel_launches()
+        call(1)
+        launches_m = binding.msla_kernel_launches() - before
+        call(2)
         ms = [m / steps for m in timed_blocks(call, blocks=blocks, steps=steps)]
         fused_m = binding.msla_forward_fuses_apply(mdesc) == 1
         bpt_m = stage_bytes_per_token(ms_shape)
-        names = STAGES_FUSED if fused_m else STAGES
+        names = plan_stages(ms_shape, fused_m, launches_m)
         mbytes = sum(bpt_m[n] for n in names) * ms_shape.B * ms_shape.N
         return {"workload": ms_shape.name, "tokens": ms_shape.B * ms_shape.N, "ms": round(med(ms), 5), "ms_min": round(min(ms), 5),
                 "ms_max": round(max(ms), 5), "tokens_per_s": ms_shape.B * ms_shape.N / (med(ms) * 1e-3),
@@ -609,10 +626,12 @@ def main() -> None:
 
     if rank == 0:
         fused = binding.msla_forward_fuses_apply(desc) == 1
-        stage_names = STAGES_FUSED if fused else STAGES
+        stage_names = plan_stages(s, fused, launches // K)
         stage_ms = {name: statistics.mean(v) for name, v in stage_acc.items()}
         if fused:  # the event between steps 4 and 5 falls directly after the one that ends step 3
             stage_ms["apply_project"] = stage_ms.pop("apply") + stage_ms.pop("project_out")
+        if "aggregate_kv_state" in stage_names:
+            stage_ms["aggregate_kv_state"] = stage_ms.pop("aggregate") + stage_ms.pop("kv_state")
         bpt, fpt = stage_bytes_per_token(s), stage_flops_per_token(s)
         peak, peak_kind = measured_peaks()
         stages = {}
@@ -637,11 +656,10 @@ def main() -> None:
                     "frac": round(achieved / peak, 4), "peak_kind": f"of {peak_kind}",
                     "traffic": recorded_traffic(dom, s.name),
                     "algorithmic_bytes_per_launch": bpt[dom] * s.B * s.N}
-        if dom == "aggregate":
-            # HBM is the roof this step is judged against.  What limits the kernel as built is the shared-memory
-            # pipe (the staged tile is turned to channel-planar there, then read as MMA operands: about 65 % busy)
-            # together with the issue rate of mma.sync (112 warp-level MMAs per 8x8 pixel block).
-            roofline["limiter"] = "shared-memory pipe (tile transposition + ldmatrix operand loads) and mma.sync issue rate"
+        if dom in ("aggregate", "aggregate_kv_state"):
+            # HBM is the roof this step is judged against.  What limits the kernels as built is the shared-memory pipe (MMA
+            # operands) together with the issue rate of mma.sync (the depthwise window as Toeplitz products).
+            roofline["limiter"] = "shared-memory pipe (operand loads) and mma.sync issue rate"
         result = {
             "metric": METRIC, "value": whole_job_value(s.B * s.N, world, ms_total, K), "unit": UNIT, "n_gpus": world, "steps": K,
             "warmup": W, "ms_per_step": ms_total / K, "ms_per_step_min": ms_lo / K, "ms_per_step_max": ms_hi / K,

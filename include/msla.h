@@ -183,8 +183,10 @@ msla_status_t msla_forward(const msla_desc* desc, const void* x, const msla_weig
  * reduction (the per-chunk partial states), events[4] directly after it, so
  * the interval of step 4 is empty and events[4]..events[5] covers the second
  * level of the state reduction (fixed-order sum of the partial states, folded
- * into the projection weights) together with apply + projection.  Everything
- * else is as for msla_forward. */
+ * into the projection weights) together with apply + projection.  With 16-bit
+ * storage, rows of a multiple of 8 pixels and many tokens steps 2 and 3 are
+ * one kernel: events[2] is recorded after it and events[3] directly after
+ * events[2].  Everything else is as for msla_forward. */
 msla_status_t msla_forward_profiled(const msla_desc* desc, const void* x, const msla_weights* weights,
                                     void* out, void* stream, void* const* events, int n_events);
 
