@@ -18,7 +18,7 @@
 //
 // One persistent CTA per SM, warp-specialised: warp 0 issues TMA, warp 1
 // issues MMAs (and owns the tensor-memory allocation), warps 2-9 drain the
-// accumulators.  Two 128x256 fp32 accumulators (all 512 TMEM columns) let the
+// accumulators.  Two 128 x (up to) 256 fp32 accumulators (all 512 TMEM columns) let the
 // epilogue of one tile overlap the MMAs of the next.  The epilogue converts to
 // bf16, stages 32x32 blocks in shared memory and writes them with TMA stores
 // (whole lines; a lane-per-row store of 16-byte pieces was twice as slow).
@@ -38,13 +38,11 @@ namespace {
 
 using bf16 = __nv_bfloat16;
 
-constexpr int BM = 128, BN = 256, BK = 64;  // CTA tile; BK = one 128-byte swizzle span of bf16
-constexpr int STAGES = 4;
+constexpr int BM = 128, BN = 256, BK = 64;  // CTA tile (BN: the widest; the kernels' TN); BK = one 128-byte swizzle span of bf16
 constexpr int A_STAGE_BYTES = BM * BK * 2;  // 16 KB
-constexpr int B_STAGE_BYTES = BN * BK * 2;  // 32 KB
-constexpr int STAGE_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
 constexpr int NUM_THREADS = 320;  // TMA warp, MMA warp, 8 epilogue warps
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 8 * 2048 + 256 + 1024;  // ring + epilogue staging + barriers + alignment slack
+constexpr int RING_BYTES = 192 * 1024;      // 4 stages of 128 x 256 tiles, 6 of 128 x 128, 8 of 128 x 64
+constexpr int SMEM_BYTES = RING_BYTES + 8 * 2048 + 256 + 1024;  // ring + epilogue staging + barriers + alignment slack
 
 // Sticky: set when any wait in any GEMM launch of this process timed out.
 __device__ int g_gemm_timeout_flag = 0;
@@ -77,8 +75,8 @@ __device__ __forceinline__ void tile_coords(const GemmParams& p, int tile, int& 
 
 constexpr int STAGING_BYTES = 8 * 2048;  // one 32-row x 64-byte block per epilogue warp
 
-// One epilogue warp's share of a finished 128x256 accumulator: TMEM lanes
-// 32*quarter .. +31 (= tile rows), columns col_half*128 .. +127, converted to
+// One epilogue warp's share of a finished 128 x TN accumulator: TMEM lanes
+// 32*quarter .. +31 (= tile rows), columns col_half*TN/2 .. +TN/2-1, converted to
 // bf16 (+ bias).  A lane owns one row, so storing straight from registers
 // scatters 16-byte pieces over 32 rows per instruction; instead each 32x32
 // block is laid out in shared memory (64-byte rows, 16-byte chunks XOR-swizzled
@@ -87,7 +85,7 @@ constexpr int STAGING_BYTES = 8 * 2048;  // one 32-row x 64-byte block per epilo
 // store map (planes of 16 channels) the lane stores its vectors directly.
 // EPI selects what else the epilogue does (compiled out of the plain projections):
 //   0  nothing
-//   1  column biases read from shared memory (bias_sm: the tile's 256 columns as fp32) and the activation
+//   1  column biases read from shared memory (bias_sm: the tile's TN columns as fp32) and the activation
 //      act(v) = v * sat(v * p.act_a + p.act_b), which is the identity for (0, 1), hard-swish for (1/6, 1/2) and ReLU
 //      for (1e30, 0); the staging block is double-buffered (NBUF = 2) so that this arithmetic overlaps the previous
 //      block's TMA store instead of lengthening the chain tmem load -> convert -> stage -> store
@@ -119,7 +117,7 @@ template <bool F16> __device__ __forceinline__ void unpack16(uint32_t w, float& 
 }
 template <bool F16> __device__ __forceinline__ constexpr uint32_t operand_format_bits() { return F16 ? 0u : ((1u << 7) | (1u << 10)); }
 
-template <int EPI, int NBUF = 1, bool F16 = false>
+template <int TN, int EPI, int NBUF = 1, bool F16 = false>
 __device__ __forceinline__ void drain_accumulator(const GemmParams& p, const CUtensorMap* tmO, uint32_t stage, int b,
                                                   int mt, int nt, uint32_t tmem_acc, int quarter, int col_half, int lane,
                                                   const float* bias_sm = nullptr) {
@@ -130,8 +128,8 @@ __device__ __forceinline__ void drain_accumulator(const GemmParams& p, const CUt
   bf16* obase = p.out + (long long)b * p.out_batch_stride;
   const float bias_row = (EPI != 1 && p.bias && p.bias_per_row && row_ok) ? (F16 ? ld16<true>(p.bias + m) : __bfloat162float(p.bias[m])) : 0.f;
   const bool bias_col = EPI != 1 && p.bias && !p.bias_per_row;
-  const int ncol0 = nt * BN + col_half * 128;
-  const uint32_t taddr = tmem_acc + col_half * 128 + ((uint32_t)(quarter * 32) << 16);
+  const int ncol0 = nt * TN + col_half * (TN / 2);
+  const uint32_t taddr = tmem_acc + col_half * (TN / 2) + ((uint32_t)(quarter * 32) << 16);
   const uint32_t sw = (uint32_t)((lane >> 1) & 3);
   uint32_t r[2][32];
   tmem_ld32(taddr, r[0]);
@@ -147,10 +145,10 @@ __device__ __forceinline__ void drain_accumulator(const GemmParams& p, const CUt
   };
   if (EPI == 2) load_residual(0);
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
+  for (int c = 0; c < TN / 64; ++c) {
     tmem_ld_wait();
-    if (c + 1 < 4) tmem_ld32(taddr + (c + 1) * 32, r[(c + 1) & 1]);  // next chunk streams in while this one is stored
-    if (EPI == 2 && c + 1 < 4) load_residual(c + 1);
+    if (c + 1 < TN / 64) tmem_ld32(taddr + (c + 1) * 32, r[(c + 1) & 1]);  // next chunk streams in while this one is stored
+    if (EPI == 2 && c + 1 < TN / 64) load_residual(c + 1);
     const uint32_t(&rc)[32] = r[c & 1];
     const int n0 = ncol0 + c * 32;
     if (n0 >= p.N) continue;  // warp-uniform
@@ -159,8 +157,8 @@ __device__ __forceinline__ void drain_accumulator(const GemmParams& p, const CUt
     for (int v = 0; v < 4; ++v) {
       float bc[8];
       if (EPI == 1 && bias_sm) {  // same address in every lane: broadcast reads
-        const float4 b0 = *reinterpret_cast<const float4*>(bias_sm + col_half * 128 + c * 32 + v * 8);
-        const float4 b1 = *reinterpret_cast<const float4*>(bias_sm + col_half * 128 + c * 32 + v * 8 + 4);
+        const float4 b0 = *reinterpret_cast<const float4*>(bias_sm + col_half * (TN / 2) + c * 32 + v * 8);
+        const float4 b1 = *reinterpret_cast<const float4*>(bias_sm + col_half * (TN / 2) + c * 32 + v * 8 + 4);
         bc[0] = b0.x; bc[1] = b0.y; bc[2] = b0.z; bc[3] = b0.w; bc[4] = b1.x; bc[5] = b1.y; bc[6] = b1.z; bc[7] = b1.w;
       } else if (EPI == 1) {      // no staged copy (the kernel whose CTAs change weight block from tile to tile)
 #pragma unroll
@@ -224,13 +222,15 @@ __device__ __forceinline__ void drain_accumulator(const GemmParams& p, const CUt
 
 // B_PLANAR (output projection with the attention output kept as one [N][64]
 // plane per pair of heads): the 64-wide k-slice kb of B is plane kb of the image.
-template <bool A_MN_MAJOR, bool B_PLANAR, int EPI, bool F16>
+template <int TN, bool A_MN_MAJOR, bool B_PLANAR, int EPI, bool F16>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 gemm_bf16_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                          const __grid_constant__ CUtensorMap tmO, GemmParams p) {
+  constexpr int STAGE_BYTES = A_STAGE_BYTES + TN * BK * 2;
+  constexpr int STAGES = RING_BYTES / STAGE_BYTES;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;  // swizzle atoms need 1024-byte alignment
-  const uint32_t staging = smem_base + STAGES * STAGE_BYTES;
+  const uint32_t staging = smem_base + RING_BYTES;
   const uint32_t bars = staging + STAGING_BYTES;
   const uint32_t full_bar = bars, empty_bar = bars + 8 * STAGES;
   const uint32_t tfull_bar = bars + 16 * STAGES, tempty_bar = tfull_bar + 16;
@@ -263,35 +263,44 @@ gemm_bf16_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
   }
   __syncthreads();
   const uint32_t tmem_base = tmem_base_sh;
-  pdl_wait();  // barriers and tensor memory are set up; the activations come from the previous kernel
-
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB) : "memory");
-      uint32_t it = 0;
+      const auto load_weights = [&](uint32_t sa, uint32_t bar, int kb, int mt, int nt) {
+        if (A_MN_MAJOR) tma_load_3d(sa + A_STAGE_BYTES, &tmB, bar, kb * BK, nt * TN, 0);
+        else            tma_load_3d(sa, &tmA, bar, kb * BK, mt * BM, 0);  // one box of 64 k x 128 rows
+      };
+      // the first stages' weights do not come from the previous kernel, the activations do
+      int b, mt, nt;
+      const int early = min(STAGES, k_iters);
+      tile_coords(p, blockIdx.x, b, mt, nt);
+      for (int kb = 0; kb < early; ++kb) {
+        mbar_expect_tx(full_bar + 8 * kb, STAGE_BYTES);
+        load_weights(smem_base + kb * STAGE_BYTES, full_bar + 8 * kb, kb, mt, nt);
+      }
+      pdl_wait();
+      int it = 0;
       bool ok = true;
       for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x) {
-        int b, mt, nt;
         tile_coords(p, tile, b, mt, nt);
         for (int kb = 0; ok && kb < k_iters; ++kb, ++it) {
-          const uint32_t s = it % STAGES, ph = (it / STAGES) & 1;
-          ok = mbar_wait(empty_bar + 8 * s, ph ^ 1, &abort_flag);
-          if (!ok) break;
+          const uint32_t s = (uint32_t)it % STAGES, ph = ((uint32_t)it / STAGES) & 1;
           const uint32_t sa = smem_base + s * STAGE_BYTES, sb = sa + A_STAGE_BYTES;
-          mbar_expect_tx(full_bar + 8 * s, STAGE_BYTES);
-          if (B_PLANAR) {    // 64 k x 128 weight rows, and one plane: 64 channels x 256 tokens
-            tma_load_3d(sa, &tmA, full_bar + 8 * s, kb * BK, mt * BM, 0);
-            tma_load_3d(sb, &tmB, full_bar + 8 * s, 0, nt * BN, b * p.planes_per_batch + kb);
+          if (it >= early) {
+            ok = mbar_wait(empty_bar + 8 * s, ph ^ 1, &abort_flag);
+            if (!ok) break;
+            mbar_expect_tx(full_bar + 8 * s, STAGE_BYTES);
+            load_weights(sa, full_bar + 8 * s, kb, mt, nt);
+          }
+          if (B_PLANAR) {           // one plane: 64 channels x TN tokens
+            tma_load_3d(sb, &tmB, full_bar + 8 * s, 0, nt * TN, b * p.planes_per_batch + kb);
+          } else if (A_MN_MAJOR) {  // two boxes of 64 tokens x 64 k
+            tma_load_3d(sa, &tmA, full_bar + 8 * s, mt * BM, kb * BK, b);
+            tma_load_3d(sa + A_STAGE_BYTES / 2, &tmA, full_bar + 8 * s, mt * BM + 64, kb * BK, b);
           } else {
-            if (A_MN_MAJOR) {  // two boxes of 64 tokens x 64 k
-              tma_load_3d(sa, &tmA, full_bar + 8 * s, mt * BM, kb * BK, b);
-              tma_load_3d(sa + A_STAGE_BYTES / 2, &tmA, full_bar + 8 * s, mt * BM + 64, kb * BK, b);
-            } else {           // one box of 64 k x 128 rows
-              tma_load_3d(sa, &tmA, full_bar + 8 * s, kb * BK, mt * BM, 0);
-            }
-            tma_load_3d(sb, &tmB, full_bar + 8 * s, kb * BK, nt * BN, A_MN_MAJOR ? 0 : b);
+            tma_load_3d(sb, &tmB, full_bar + 8 * s, kb * BK, nt * TN, b);
           }
         }
       }
@@ -299,9 +308,9 @@ gemm_bf16_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
   } else if (warp == 1) {
     // -------------------------------------------------------------- MMA issuer
     if (lane == 0) {
-      // instruction descriptor: D = f32, A = B = bf16, A major, B K-major, N = 256, M = 128
+      // instruction descriptor: D = f32, A = B = bf16, A major, B K-major, N = TN, M = 128
       const uint32_t idesc = (1u << 4) | operand_format_bits<F16>() | ((A_MN_MAJOR ? 1u : 0u) << 15) |
-                             ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+                             ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
       uint32_t it = 0, local = 0;
       bool ok = true;
       for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x, ++local) {
@@ -333,11 +342,12 @@ gemm_bf16_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
   } else {
     // ---------------------------------------------------------------- epilogue
     // Eight warps: warp%4 selects the TMEM lane quarter (a hardware rule), the
-    // other bit selects which 128 of the tile's 256 columns the warp drains.
+    // other bit selects which half of the tile's columns the warp drains.
     const int quarter = warp & 3;
     const int col_half = (warp - 2) >> 2;
     uint32_t local = 0;
     bool ok = true;
+    pdl_wait();  // residual and output may be in use by the previous kernel
     for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x, ++local) {
       int b, mt, nt;
       tile_coords(p, tile, b, mt, nt);
@@ -346,7 +356,7 @@ gemm_bf16_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
-      drain_accumulator<EPI, 1, F16>(p, &tmO, staging + (warp - 2) * 2048, b, mt, nt, tmem_base + acc * BN, quarter, col_half, lane);
+      drain_accumulator<TN, EPI, 1, F16>(p, &tmO, staging + (warp - 2) * 2048, b, mt, nt, tmem_base + acc * BN, quarter, col_half, lane);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty_bar + 8 * acc);  // this warp's share of the accumulator is drained
@@ -376,7 +386,7 @@ gemm_bf16_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
 // serialise in their L2 slices.  Here a CTA owns one block of output channels
 // for its whole life: that block of the weight matrix (<= 128 KB) is loaded
 // into shared memory once, and only activation tiles stream through a ring.
-// Used for the input projection: B = 256 weight rows resident (K <= 256), A = 128-token x tiles,
+// Used for the input projection and the FFN's first layer: B = TN weight rows resident (K <= 512), A = 128-token x tiles,
 // MN-major, 16 KB stages (5 deep).  CTA c serves weight block c % blocks and the activation
 // tiles c / blocks, c / blocks + workers, ...  Barriers, TMEM use and epilogue are as above.
 // ---------------------------------------------------------------------------
@@ -385,34 +395,34 @@ constexpr int WS_RING_BYTES = 80 * 1024;
 constexpr int WS_SMEM_BYTES = RES_BYTES + WS_RING_BYTES + STAGING_BYTES + 256 + 1024;
 constexpr int WS_MAX_STAGES = 6;
 
-template <int EPI, bool F16>
+template <int TN, int EPI, bool F16>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 gemm_bf16_stationary_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                             const __grid_constant__ CUtensorMap tmO, GemmParams p, int blocks, int workers) {
   constexpr int STREAM_BYTES = A_STAGE_BYTES;             // one k-slice of the streamed operand (the x tile)
   constexpr int NBUF = EPI == 1 ? 2 : 1;                  // staging blocks per epilogue warp
-  constexpr int RING_BYTES = WS_RING_BYTES - (NBUF - 1) * STAGING_BYTES;  // the second staging block comes out of the ring
-  constexpr int NSTAGE = RING_BYTES / STREAM_BYTES;       // 5 (4 with double-buffered staging)
-  constexpr int RES_SLICE = B_STAGE_BYTES;                // one k-slice of the resident operand (256 weight rows)
+  constexpr int STREAM_RING = WS_RING_BYTES - (NBUF - 1) * STAGING_BYTES;  // the second staging block comes out of the ring
+  constexpr int NSTAGE = STREAM_RING / STREAM_BYTES;       // 5 (4 with double-buffered staging)
+  constexpr int RES_SLICE = TN * BK * 2;                  // one k-slice of the resident operand (TN weight rows)
   extern __shared__ unsigned char smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t res_base = smem_base, ring_base = smem_base + RES_BYTES;
-  const uint32_t staging = ring_base + RING_BYTES;
+  const uint32_t staging = ring_base + STREAM_RING;
   const uint32_t bars = staging + NBUF * STAGING_BYTES;
   const uint32_t full_bar = bars, empty_bar = bars + 8 * WS_MAX_STAGES;
   const uint32_t tfull_bar = bars + 16 * WS_MAX_STAGES, tempty_bar = tfull_bar + 16;
   const uint32_t res_bar = tempty_bar + 16, tmem_slot = res_bar + 8;
   __shared__ int abort_flag;
   __shared__ uint32_t tmem_base_sh;
-  __shared__ __align__(16) float bias_sm[EPI == 1 ? BN : 4];  // the CTA's 256 column biases (weights: not the previous kernel's output)
+  __shared__ __align__(16) float bias_sm[EPI == 1 ? TN : 4];  // the CTA's column biases (weights: not the previous kernel's output)
 
   pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int k_iters = (p.K + BK - 1) / BK;
   const int blk = blockIdx.x % blocks, worker = blockIdx.x / blocks;
   if (EPI == 1) {
-    for (int i = threadIdx.x; i < BN; i += NUM_THREADS) {
-      const int n = blk * BN + i;
+    for (int i = threadIdx.x; i < TN; i += NUM_THREADS) {
+      const int n = blk * TN + i;
       bias_sm[i] = (p.bias && !p.bias_per_row && n < p.N) ? (F16 ? ld16<true>(p.bias + n) : __bfloat162float(p.bias[n])) : 0.f;
     }
   }
@@ -448,7 +458,7 @@ gemm_bf16_stationary_kernel(const __grid_constant__ CUtensorMap tmA, const __gri
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB) : "memory");
       // the resident weight block: all k-slices on one barrier
       mbar_expect_tx(res_bar, (uint32_t)(k_iters * RES_SLICE));
-      for (int kb = 0; kb < k_iters; ++kb) tma_load_3d(res_base + kb * RES_SLICE, &tmB, res_bar, kb * BK, blk * BN, 0);
+      for (int kb = 0; kb < k_iters; ++kb) tma_load_3d(res_base + kb * RES_SLICE, &tmB, res_bar, kb * BK, blk * TN, 0);
       pdl_wait();  // the streamed operand may come from the previous kernel; the weights above do not
       uint32_t it = 0;
       bool ok = true;
@@ -470,7 +480,7 @@ gemm_bf16_stationary_kernel(const __grid_constant__ CUtensorMap tmA, const __gri
     // -------------------------------------------------------------- MMA issuer
     if (lane == 0) {
       const uint32_t idesc = (1u << 4) | operand_format_bits<F16>() | (1u << 15) |
-                             ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+                             ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
       uint32_t it = 0, local = 0;
       bool ok = mbar_wait(res_bar, 0, &abort_flag);
       for (int si = worker; ok && si < stream_total; si += workers, ++local) {
@@ -511,7 +521,7 @@ gemm_bf16_stationary_kernel(const __grid_constant__ CUtensorMap tmA, const __gri
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
-      drain_accumulator<EPI, NBUF, F16>(p, &tmO, staging + (warp - 2) * 2048 * NBUF, b, mt, nt, tmem_base + acc * BN, quarter, col_half, lane, bias_sm);
+      drain_accumulator<TN, EPI, NBUF, F16>(p, &tmO, staging + (warp - 2) * 2048 * NBUF, b, mt, nt, tmem_base + acc * BN, quarter, col_half, lane, bias_sm);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty_bar + 8 * acc);
@@ -543,35 +553,97 @@ bool make_map(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, uint
   return tma_make_map_bf16(map, base, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
-template <int EPI, bool F16>
-msla_status_t launch_stationary(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmO, const GemmParams& p,
-                                int blocks, cudaStream_t st) {
+// Which tile a problem gets.  A small one is latency: 256 columns per CTA leave most SMs idle while a few load 128 KB of
+// weights and drain 128 x 256 accumulators; a large one wants few passes over the activations.  Both kernels take the
+// narrowest tile whose grid is still one wave; beyond that the stationary one minimises rounds x (columns + 64), the 64 standing
+// for what a tile costs whatever its width.  Whole call, us, 256 columns / the rule: [1, 256, 32, 32] 26.4 / 24.7 (64 columns),
+// [1, 192, 64, 128] 31.7 / 30.6 (192), f16 [8, 128, 45, 80] 52.6 / 50.4 (128), [1, 384, 32, 32] 30.4 / 25.9 (64), building block
+// f16 [4, 128, 28, 28] with 512 hidden channels 48.7 / 40.8, [1, 256, 64, 64] with 1024 58.2 / 53.9, [8, 192, 48, 48] with 768
+// 94.5 / 93.7.  64 columns everywhere: [4, 256, 64, 64] 61.0 against 52.6.
+// Rows of 257 to 512 channels fit with blocks of 128 or 64: against the streaming kernel [12, 384, 30, 30] d = 16 73.2 -> 70.5,
+// building block [3, 320, 100, 160] with 1280 328 -> 321, [1, 384, 28, 28] 47.1 -> 46.4; [8, 384, 44, 44] 81.2 -> 83.0.
+
+// Columns of a CTA's weight block (TN) in the stationary kernel for T activation tiles; 0: rows too long.
+int stationary_columns(long long T, int K, int Cout) {
+  const int sms = device_sm_count(), k_iters = (K + BK - 1) / BK;
+  if (k_iters * 128 * BK * 2 > RES_BYTES) return 0;
+  int best = 0;
+  long long best_cost = 0;
+  for (int tn : {256, 192, 128, 64}) {
+    const int blocks = (Cout + tn - 1) / tn;
+    if (k_iters * tn * BK * 2 > RES_BYTES || blocks > sms) continue;
+    const long long workers = T < sms / blocks ? T : sms / blocks, rounds = (T + workers - 1) / workers;
+    const long long cost = rounds * (tn + 64);
+    if (!best || cost < best_cost) { best = tn; best_cost = cost; }
+  }
+  return best;
+}
+
+// Columns (tokens) per tile of the streaming kernel.
+int streaming_columns(long long row_tiles, int N) {
+  for (int tn : {64, 128})
+    if (row_tiles * ((N + tn - 1) / tn) <= device_sm_count()) return tn;
+  return BN;
+}
+
+template <int TN, int EPI, bool F16>
+msla_status_t launch_stationary_tn(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmO, const GemmParams& p, cudaStream_t st) {
   static std::atomic<unsigned long long> attr_done{0};
-  const msla_status_t as = ensure_smem_attr(attr_done, gemm_bf16_stationary_kernel<EPI, F16>, WS_SMEM_BYTES);
+  const msla_status_t as = ensure_smem_attr(attr_done, gemm_bf16_stationary_kernel<TN, EPI, F16>, WS_SMEM_BYTES);
   if (as != MSLA_OK) return as;
+  const int blocks = p.n_tiles;
   const long long stream_total = (long long)p.batches * p.m_tiles;
   long long workers = device_sm_count() / blocks;
   if (workers > stream_total) workers = stream_total;
-  launch_pdl(gemm_bf16_stationary_kernel<EPI, F16>, dim3((unsigned)(workers * blocks)), dim3(NUM_THREADS), WS_SMEM_BYTES, st, tmA, tmB, tmO, p, blocks, (int)workers);
+  launch_pdl(gemm_bf16_stationary_kernel<TN, EPI, F16>, dim3((unsigned)(workers * blocks)), dim3(NUM_THREADS), WS_SMEM_BYTES, st, tmA, tmB, tmO, p, blocks, (int)workers);
   count_launches(1);
   return check_launch("projection GEMM (tcgen05, stationary weights)");
 }
 
-template <bool A_MN, bool B_PLANAR = false, int EPI = 0, bool F16 = false>
-msla_status_t launch(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmO, const GemmParams& p, cudaStream_t st) {
-  // weight-stationary kernel when the CTA's weight block fits its 128 KB of shared memory
-  const int blocks = A_MN ? p.n_tiles : p.m_tiles;
-  const int k_iters = (p.K + BK - 1) / BK;
-  if (A_MN && k_iters * B_STAGE_BYTES <= RES_BYTES && blocks <= 16 && blocks <= device_sm_count())
-    return launch_stationary<EPI, F16>(tmA, tmB, tmO, p, blocks, st);
+template <int TN, bool A_MN, bool B_PLANAR, int EPI, bool F16>
+msla_status_t launch_streaming_tn(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmO, const GemmParams& p, cudaStream_t st) {
   static std::atomic<unsigned long long> attr_done{0};
-  const msla_status_t as = ensure_smem_attr(attr_done, gemm_bf16_tcgen05_kernel<A_MN, B_PLANAR, EPI, F16>, SMEM_BYTES);
+  const msla_status_t as = ensure_smem_attr(attr_done, gemm_bf16_tcgen05_kernel<TN, A_MN, B_PLANAR, EPI, F16>, SMEM_BYTES);
   if (as != MSLA_OK) return as;
   const long long tiles = (long long)p.batches * p.m_tiles * p.n_tiles;
   const int grid = (int)(tiles < device_sm_count() ? tiles : device_sm_count());
-  launch_pdl(gemm_bf16_tcgen05_kernel<A_MN, B_PLANAR, EPI, F16>, dim3(grid), dim3(NUM_THREADS), SMEM_BYTES, st, tmA, tmB, tmO, p);
+  launch_pdl(gemm_bf16_tcgen05_kernel<TN, A_MN, B_PLANAR, EPI, F16>, dim3(grid), dim3(NUM_THREADS), SMEM_BYTES, st, tmA, tmB, tmO, p);
   count_launches(1);
   return check_launch("projection GEMM (tcgen05)");
+}
+
+template <bool A_MN, bool B_PLANAR, int EPI, bool F16>
+msla_status_t launch_streaming(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmO, const GemmParams& p, int tn, cudaStream_t st) {
+  switch (tn) {
+    case 64: return launch_streaming_tn<64, A_MN, B_PLANAR, EPI, F16>(tmA, tmB, tmO, p, st);
+    case 128: return launch_streaming_tn<128, A_MN, B_PLANAR, EPI, F16>(tmA, tmB, tmO, p, st);
+    default: return launch_streaming_tn<BN, A_MN, B_PLANAR, EPI, F16>(tmA, tmB, tmO, p, st);
+  }
+}
+
+// Activations [C][N] times weights [Cout][C]: p.n_tiles counts blocks of tn output channels.
+struct InTile { bool stationary; int tn; };
+InTile in_tile(int K, int Cout, int N, int B) {
+  const long long T = (long long)B * ((N + BM - 1) / BM);
+  const int tn = stationary_columns(T, K, Cout);
+  return tn ? InTile{true, tn} : InTile{false, streaming_columns(T, Cout)};
+}
+template <int EPI, bool F16>
+msla_status_t launch_in(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmO, const GemmParams& p, InTile t, cudaStream_t st) {
+  if (!t.stationary) return launch_streaming<true, false, EPI, F16>(tmA, tmB, tmO, p, t.tn, st);
+  switch (t.tn) {
+    case 64: return launch_stationary_tn<64, EPI, F16>(tmA, tmB, tmO, p, st);
+    case 128: return launch_stationary_tn<128, EPI, F16>(tmA, tmB, tmO, p, st);
+    case 192: return launch_stationary_tn<192, EPI, F16>(tmA, tmB, tmO, p, st);
+    default: return launch_stationary_tn<BN, EPI, F16>(tmA, tmB, tmO, p, st);
+  }
+}
+
+// Weights [Cout][K] times activations: p.n_tiles counts blocks of tn tokens.
+int columns_out(int Cout, int N, int B) { return streaming_columns((long long)B * ((Cout + BM - 1) / BM), N); }
+template <bool B_PLANAR, int EPI, bool F16>
+msla_status_t launch_out(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmO, const GemmParams& p, int tn, cudaStream_t st) {
+  return launch_streaming<false, B_PLANAR, EPI, F16>(tmA, tmB, tmO, p, tn, st);
 }
 
 }  // namespace
@@ -583,13 +655,14 @@ bool project_in_bf16_supported(int C, int Cout, int ldx, int d) {
 // y[b][o / d][n][o % d] = sum_c w[o][c] * x[b][c][n];  x [B, C, N] with rows ldx elements apart, y planar with batch stride y_sb.
 msla_status_t run_project_in_bf16(const void* x, int ldx, const void* w, void* y, int B, int C, int Cout, int N, int d,
                                   long long y_sb, cudaStream_t st, bool f16) {
+  const InTile tile = in_tile(C, Cout, N, B);
   CUtensorMap tmA, tmB;
   if (!make_map(&tmA, x, (uint64_t)N, (uint64_t)C, (uint64_t)B, (uint64_t)ldx * 2, (uint64_t)C * ldx * 2, 64, BK) ||
-      !make_map(&tmB, w, (uint64_t)C, (uint64_t)Cout, 1, (uint64_t)C * 2, (uint64_t)C * Cout * 2, BK, BN))
+      !make_map(&tmB, w, (uint64_t)C, (uint64_t)Cout, 1, (uint64_t)C * 2, (uint64_t)C * Cout * 2, BK, (uint32_t)tile.tn))
     return fail(MSLA_ERR_CUDA, "cuTensorMapEncodeTiled failed for the input projection");
   GemmParams p{};
   p.M = N; p.N = Cout; p.K = C; p.batches = B;
-  p.m_tiles = (N + BM - 1) / BM; p.n_tiles = (Cout + BN - 1) / BN;
+  p.m_tiles = (N + BM - 1) / BM; p.n_tiles = (Cout + tile.tn - 1) / tile.tn;
   p.out_batch_stride = y_sb; p.ld_out = 0; p.group = d; p.bias_per_row = 0; p.n_fastest = 1;
   p.bias = nullptr; p.out = (bf16*)y;
   // planes of 32 channels are written as 32-token x 32-channel blocks by TMA
@@ -604,7 +677,7 @@ msla_status_t run_project_in_bf16(const void* x, int ldx, const void* w, void* y
     if (!tma_make_map_bf16(&tmO, y, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B))
       return fail(MSLA_ERR_CUDA, "cuTensorMapEncodeTiled failed for the input projection's output");
   }
-  return f16 ? launch<true, false, 0, true>(tmA, tmB, tmO, p, st) : launch<true>(tmA, tmB, tmO, p, st);
+  return f16 ? launch_in<0, true>(tmA, tmB, tmO, p, tile, st) : launch_in<0, false>(tmA, tmB, tmO, p, tile, st);
 }
 
 bool project_out_bf16_supported(int Cin, int Cout, int ldy) { return Cin % 8 == 0 && ldy % 8 == 0 && Cout >= 1; }
@@ -613,13 +686,14 @@ bool project_out_bf16_supported(int Cin, int Cout, int ldy) { return Cin % 8 == 
 // elements apart.
 msla_status_t run_project_out_bf16(const void* a, const void* w, const void* bias, const void* residual, void* y, int ldy, int B, int Cin,
                                    int Cout, int N, cudaStream_t st, bool f16) {
+  const int tn = columns_out(Cout, N, B);
   CUtensorMap tmA, tmB;
   if (!make_map(&tmA, w, (uint64_t)Cin, (uint64_t)Cout, 1, (uint64_t)Cin * 2, (uint64_t)Cin * Cout * 2, BK, BM) ||
-      !make_map(&tmB, a, (uint64_t)Cin, (uint64_t)N, (uint64_t)B, (uint64_t)Cin * 2, (uint64_t)N * Cin * 2, BK, BN))
+      !make_map(&tmB, a, (uint64_t)Cin, (uint64_t)N, (uint64_t)B, (uint64_t)Cin * 2, (uint64_t)N * Cin * 2, BK, (uint32_t)tn))
     return fail(MSLA_ERR_CUDA, "cuTensorMapEncodeTiled failed for the output projection");
   GemmParams p{};
   p.M = Cout; p.N = N; p.K = Cin; p.batches = B;
-  p.m_tiles = (Cout + BM - 1) / BM; p.n_tiles = (N + BN - 1) / BN;
+  p.m_tiles = (Cout + BM - 1) / BM; p.n_tiles = (N + tn - 1) / tn;
   p.out_batch_stride = (long long)Cout * ldy; p.ld_out = ldy; p.group = 0; p.bias_per_row = 1; p.n_fastest = 0;
   p.bias = (const bf16*)bias; p.out = (bf16*)y;
   CUtensorMap tmO;  // NCHW output as [batch][channel][token]; blocks of 32 channels x 32 tokens
@@ -632,8 +706,8 @@ msla_status_t run_project_out_bf16(const void* a, const void* w, const void* bia
       return fail(MSLA_ERR_CUDA, "cuTensorMapEncodeTiled failed for the output projection's output");
   }
   p.residual = (const bf16*)residual;
-  if (f16) return residual ? launch<false, false, 2, true>(tmA, tmB, tmO, p, st) : launch<false, false, 0, true>(tmA, tmB, tmO, p, st);
-  return residual ? launch<false, false, 2>(tmA, tmB, tmO, p, st) : launch<false>(tmA, tmB, tmO, p, st);
+  if (f16) return residual ? launch_out<false, 2, true>(tmA, tmB, tmO, p, tn, st) : launch_out<false, 0, true>(tmA, tmB, tmO, p, tn, st);
+  return residual ? launch_out<false, 2, false>(tmA, tmB, tmO, p, tn, st) : launch_out<false, 0, false>(tmA, tmB, tmO, p, tn, st);
 }
 
 bool project_out_planar_bf16_supported(int Cin, int Cout) { return Cin % 64 == 0 && Cout >= 1; }
@@ -641,6 +715,7 @@ bool project_out_planar_bf16_supported(int Cin, int Cout) { return Cin % 64 == 0
 // Same product with the attention output kept planar: a[b][j / 64][n][j % 64] (one [N][64] plane per pair of heads).
 msla_status_t run_project_out_planar_bf16(const void* a, const void* w, const void* bias, const void* residual, void* y, int ldy, int B,
                                           int Cin, int Cout, int N, cudaStream_t st, bool f16) {
+  const int tn = columns_out(Cout, N, B);
   CUtensorMap tmA, tmB, tmO;
   const int planes = Cin / 64;
   {
@@ -648,19 +723,19 @@ msla_status_t run_project_out_planar_bf16(const void* a, const void* w, const vo
     const cuuint64_t sO[2] = {(cuuint64_t)ldy * 2, (cuuint64_t)Cout * ldy * 2};
     const cuuint32_t bO[3] = {32, 32, 1};
     if (!make_map(&tmA, w, (uint64_t)Cin, (uint64_t)Cout, 1, (uint64_t)Cin * 2, (uint64_t)Cin * Cout * 2, BK, BM) ||
-        !make_map(&tmB, a, 64, (uint64_t)N, (uint64_t)B * planes, 128, (uint64_t)N * 128, BK, BN) ||
+        !make_map(&tmB, a, 64, (uint64_t)N, (uint64_t)B * planes, 128, (uint64_t)N * 128, BK, (uint32_t)tn) ||
         !tma_make_map_bf16(&tmO, y, 3, dO, sO, bO, CU_TENSOR_MAP_SWIZZLE_64B))
       return fail(MSLA_ERR_CUDA, "cuTensorMapEncodeTiled failed for the output projection");
   }
   GemmParams p{};
   p.M = Cout; p.N = N; p.K = Cin; p.batches = B;
-  p.m_tiles = (Cout + BM - 1) / BM; p.n_tiles = (N + BN - 1) / BN;
+  p.m_tiles = (Cout + BM - 1) / BM; p.n_tiles = (N + tn - 1) / tn;
   p.out_batch_stride = (long long)Cout * ldy; p.ld_out = ldy; p.group = 0; p.bias_per_row = 1; p.n_fastest = 0;
   p.bias = (const bf16*)bias; p.out = (bf16*)y;
   p.tma_store = 1; p.planes_per_batch = planes;
   p.residual = (const bf16*)residual;
-  if (f16) return residual ? launch<false, true, 2, true>(tmA, tmB, tmO, p, st) : launch<false, true, 0, true>(tmA, tmB, tmO, p, st);
-  return residual ? launch<false, true, 2>(tmA, tmB, tmO, p, st) : launch<false, true>(tmA, tmB, tmO, p, st);
+  if (f16) return residual ? launch_out<true, 2, true>(tmA, tmB, tmO, p, tn, st) : launch_out<true, 0, true>(tmA, tmB, tmO, p, tn, st);
+  return residual ? launch_out<true, 2, false>(tmA, tmB, tmO, p, tn, st) : launch_out<true, 0, false>(tmA, tmB, tmO, p, tn, st);
 }
 
 // ---- the two linear layers of the FFN with a depthwise convolution (Section 3.1, Fig. 2 left)
@@ -670,46 +745,48 @@ bool ffn_bf16_supported(int C, int Ch, int Cout) { return C % 8 == 0 && Ch % 64 
 // (dense 2 KB per 32 tokens for the epilogue's TMA stores: half-line stores into 64-channel planes cost this GEMM 2x).
 msla_status_t run_ffn_expand_bf16(const void* x, int ldx, const void* w1, const void* b1, void* h, int B, int C, int Ch, int N, int act,
                                   cudaStream_t st, bool f16) {
+  const InTile tile = in_tile(C, Ch, N, B);
   CUtensorMap tmA, tmB, tmO;
   const cuuint64_t dims[3] = {32, (cuuint64_t)N, (cuuint64_t)B * (Ch / 32)};
   const cuuint64_t strides[2] = {64, (cuuint64_t)N * 64};
   const cuuint32_t box[3] = {32, 32, 1};
   if (!make_map(&tmA, x, (uint64_t)N, (uint64_t)C, (uint64_t)B, (uint64_t)ldx * 2, (uint64_t)C * ldx * 2, 64, BK) ||
-      !make_map(&tmB, w1, (uint64_t)C, (uint64_t)Ch, 1, (uint64_t)C * 2, (uint64_t)C * Ch * 2, BK, BN) ||
+      !make_map(&tmB, w1, (uint64_t)C, (uint64_t)Ch, 1, (uint64_t)C * 2, (uint64_t)C * Ch * 2, BK, (uint32_t)tile.tn) ||
       !tma_make_map_bf16(&tmO, h, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B))
     return fail(MSLA_ERR_CUDA, "cuTensorMapEncodeTiled failed for the FFN's first layer");
   GemmParams p{};
   p.M = N; p.N = Ch; p.K = C; p.batches = B;
-  p.m_tiles = (N + BM - 1) / BM; p.n_tiles = (Ch + BN - 1) / BN;
+  p.m_tiles = (N + BM - 1) / BM; p.n_tiles = (Ch + tile.tn - 1) / tile.tn;
   p.out_batch_stride = (long long)Ch * N; p.ld_out = 0; p.group = 32; p.bias_per_row = 0; p.n_fastest = 1;
   p.bias = (const bf16*)b1; p.out = (bf16*)h;
   p.tma_store = 1; p.planes_per_batch = Ch / 32; p.plane_shift = 5;
   p.act_a = act == 2 ? 1.f / 6.f : (act == 1 ? 1e30f : 0.f);  // act(v) = v * sat(v * act_a + act_b)
   p.act_b = act == 2 ? 0.5f : (act == 1 ? 0.f : 1.f);
   p.residual = nullptr;
-  return f16 ? launch<true, false, 1, true>(tmA, tmB, tmO, p, st) : launch<true, false, 1>(tmA, tmB, tmO, p, st);
+  return f16 ? launch_in<1, true>(tmA, tmB, tmO, p, tile, st) : launch_in<1, false>(tmA, tmB, tmO, p, tile, st);
 }
 
 // Second layer: y[b][m][n] = sum_j w2[m][j] * g[b][j / 64][n][j % 64] + b2[m] (+ residual[b][m][n]); g planes of 64 channels, rows of y and residual ldy apart.
 msla_status_t run_ffn_project_bf16(const void* g, const void* w2, const void* b2, const void* residual, void* y, int ldy, int B, int Ch,
                                    int Cout, int N, cudaStream_t st, bool f16) {
+  const int tn = columns_out(Cout, N, B);
   CUtensorMap tmA, tmB, tmO;
   const int planes = Ch / 64;
   const cuuint64_t dO[3] = {(cuuint64_t)N, (cuuint64_t)Cout, (cuuint64_t)B};
   const cuuint64_t sO[2] = {(cuuint64_t)ldy * 2, (cuuint64_t)Cout * ldy * 2};
   const cuuint32_t bO[3] = {32, 32, 1};
   if (!make_map(&tmA, w2, (uint64_t)Ch, (uint64_t)Cout, 1, (uint64_t)Ch * 2, (uint64_t)Ch * Cout * 2, BK, BM) ||
-      !make_map(&tmB, g, 64, (uint64_t)N, (uint64_t)B * planes, 128, (uint64_t)N * 128, BK, BN) ||
+      !make_map(&tmB, g, 64, (uint64_t)N, (uint64_t)B * planes, 128, (uint64_t)N * 128, BK, (uint32_t)tn) ||
       !tma_make_map_bf16(&tmO, y, 3, dO, sO, bO, CU_TENSOR_MAP_SWIZZLE_64B))
     return fail(MSLA_ERR_CUDA, "cuTensorMapEncodeTiled failed for the FFN's second layer");
   GemmParams p{};
   p.M = Cout; p.N = N; p.K = Ch; p.batches = B;
-  p.m_tiles = (Cout + BM - 1) / BM; p.n_tiles = (N + BN - 1) / BN;
+  p.m_tiles = (Cout + BM - 1) / BM; p.n_tiles = (N + tn - 1) / tn;
   p.out_batch_stride = (long long)Cout * ldy; p.ld_out = ldy; p.group = 0; p.bias_per_row = 1; p.n_fastest = 0;
   p.bias = (const bf16*)b2; p.out = (bf16*)y;
   p.tma_store = 1; p.planes_per_batch = planes;
   p.residual = (const bf16*)residual;
-  return f16 ? launch<false, true, 2, true>(tmA, tmB, tmO, p, st) : launch<false, true, 2>(tmA, tmB, tmO, p, st);
+  return f16 ? launch_out<true, 2, true>(tmA, tmB, tmO, p, tn, st) : launch_out<true, 2, false>(tmA, tmB, tmO, p, tn, st);
 }
 
 // Self-test of the bounded wait every kernel of the library relies on: one thread waits, with the given cycle

@@ -103,3 +103,12 @@ def test_ffn_rejects_bad_descriptors():
     w = [torch.zeros(n, device="cuda", dtype=torch.bfloat16) for n in (128 * 64, 128 * 9, 64 * 128)]
     with pytest.raises(binding.MslaError):
         binding.msla_ffn_dwconv(desc, x, binding.make_ffn_weights(*w), torch.empty_like(x))
+
+
+# The second layer's tiles of 64, 128 and 256 tokens, each with a remainder and the residual connection.
+@pytest.mark.parametrize("dtype,B,C,H,W,Ch", [("f16", 1, 40, 9, 11, 64), ("bf16", 1, 96, 60, 163, 64), ("bf16", 3, 136, 50, 130, 128)])
+def test_ffn_tiles(dtype, B, C, H, W, Ch):
+    s = inputs.FfnShape("ffn_tiles", dtype, B, C, H, W, Ch, C, seed=35)
+    t = inputs.ffn_inputs(s, True)
+    util.assert_close(util.run_ffn(s, t, "hardswish", True), _ref(t, "hardswish", True), dtype, f"{(B, C, H, W, Ch)}", block=util.MODULE_BLOCK)
+    assert binding.msla_debug_wait_timeouts() == 0

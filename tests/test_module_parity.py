@@ -303,3 +303,16 @@ def test_forward_host_in_parts(dtype, B, C, H, W, heads, d):
     torch.cuda.synchronize()
     for i in range(2):
         assert torch.equal(ho[i], refs[i])
+
+
+# The projections' kernels take 64 to 256 output columns per tile by problem size: each width, with remainders on both sides, rows
+# of up to 512 channels in the kernel that keeps its weights and longer ones in the one that streams them.
+@pytest.mark.parametrize("dtype,B,C,Cout,N", [("bf16", 1, 64, 176, 136), ("f16", 1, 72, 384, 5112), ("bf16", 1, 128, 352, 8952), ("bf16", 5, 40, 464, 7096),
+                                              ("bf16", 2, 264, 208, 1000), ("f16", 1, 512, 160, 8), ("bf16", 1, 520, 96, 264), ("bf16", 1, 520, 336, 5112)])
+def test_project_in_tiles(dtype, B, C, Cout, N):
+    test_stage_project_in(dtype, B, C, Cout, N)
+
+
+@pytest.mark.parametrize("dtype,B,Cin,Cout,N", [("bf16", 1, 136, 200, 72), ("f16", 1, 40, 96, 9480), ("bf16", 3, 24, 200, 6408), ("bf16", 2, 1032, 72, 8)])
+def test_project_out_tiles(dtype, B, Cin, Cout, N):
+    test_stage_project_out(dtype, B, Cin, Cout, N)
