@@ -120,7 +120,7 @@ template <bool F16> __device__ __forceinline__ constexpr uint32_t operand_format
 template <int TN, int EPI, int NBUF = 1, bool F16 = false>
 __device__ __forceinline__ void drain_accumulator(const GemmParams& p, const CUtensorMap* tmO, uint32_t stage, int b,
                                                   int mt, int nt, uint32_t tmem_acc, int quarter, int col_half, int lane,
-                                                  const float* bias_sm = nullptr) {
+                                                  uint32_t& stored, const float* bias_sm = nullptr) {
   const int gs = p.group == 32 ? 5 : 4;  // log2(group) when the output is planar
   const int row0 = mt * BM + quarter * 32;
   const int m = row0 + lane;
@@ -188,7 +188,8 @@ __device__ __forceinline__ void drain_accumulator(const GemmParams& p, const CUt
       }
     }
     if (p.tma_store) {
-      const uint32_t buf = stage + (NBUF == 2 ? (uint32_t)(c & 1) * 2048u : 0u);
+      // the warp's stores take the buffers in turn: `stored` counts them across tiles, of which one may have an odd number
+      const uint32_t buf = stage + (NBUF == 2 ? (stored++ & 1u) * 2048u : 0u);
       // the block stored from this buffer before must have been read out of it
       if (lane == 0) {
         if (NBUF == 2) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
@@ -345,6 +346,7 @@ gemm_bf16_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     // other bit selects which half of the tile's columns the warp drains.
     const int quarter = warp & 3;
     const int col_half = (warp - 2) >> 2;
+    uint32_t stored = 0;
     uint32_t local = 0;
     bool ok = true;
     pdl_wait();  // residual and output may be in use by the previous kernel
@@ -356,7 +358,7 @@ gemm_bf16_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
-      drain_accumulator<TN, EPI, 1, F16>(p, &tmO, staging + (warp - 2) * 2048, b, mt, nt, tmem_base + acc * BN, quarter, col_half, lane);
+      drain_accumulator<TN, EPI, 1, F16>(p, &tmO, staging + (warp - 2) * 2048, b, mt, nt, tmem_base + acc * BN, quarter, col_half, lane, stored);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty_bar + 8 * acc);  // this warp's share of the accumulator is drained
@@ -510,6 +512,7 @@ gemm_bf16_stationary_kernel(const __grid_constant__ CUtensorMap tmA, const __gri
     // ---------------------------------------------------------------- epilogue
     const int quarter = warp & 3;
     const int col_half = (warp - 2) >> 2;
+    uint32_t stored = 0;
     uint32_t local = 0;
     bool ok = true;
     pdl_wait();  // no global write before the previous kernel is done with the output buffer
@@ -521,7 +524,7 @@ gemm_bf16_stationary_kernel(const __grid_constant__ CUtensorMap tmA, const __gri
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
-      drain_accumulator<TN, EPI, NBUF, F16>(p, &tmO, staging + (warp - 2) * 2048 * NBUF, b, mt, nt, tmem_base + acc * BN, quarter, col_half, lane, bias_sm);
+      drain_accumulator<TN, EPI, NBUF, F16>(p, &tmO, staging + (warp - 2) * 2048 * NBUF, b, mt, nt, tmem_base + acc * BN, quarter, col_half, lane, stored, bias_sm);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty_bar + 8 * acc);

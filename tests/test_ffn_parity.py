@@ -105,10 +105,35 @@ def test_ffn_rejects_bad_descriptors():
         binding.msla_ffn_dwconv(desc, x, binding.make_ffn_weights(*w), torch.empty_like(x))
 
 
-# The second layer's tiles of 64, 128 and 256 tokens, each with a remainder and the residual connection.
-@pytest.mark.parametrize("dtype,B,C,H,W,Ch", [("f16", 1, 40, 9, 11, 64), ("bf16", 1, 96, 60, 163, 64), ("bf16", 3, 136, 50, 130, 128)])
+# The second layer's tiles of 64, 128 and 256 tokens, each with a remainder and the residual connection; the first layer's of 64
+# and 192 channels, several tiles to a CTA (an odd number of staged blocks per tile and warp).
+@pytest.mark.parametrize("dtype,B,C,H,W,Ch", [("f16", 1, 40, 9, 11, 64), ("bf16", 1, 96, 60, 163, 64), ("bf16", 3, 136, 50, 130, 128),
+                                             ("f16", 10, 96, 76, 77, 384), ("bf16", 8, 32, 76, 80, 64)])
 def test_ffn_tiles(dtype, B, C, H, W, Ch):
     s = inputs.FfnShape("ffn_tiles", dtype, B, C, H, W, Ch, C, seed=35)
     t = inputs.ffn_inputs(s, True)
     util.assert_close(util.run_ffn(s, t, "hardswish", True), _ref(t, "hardswish", True), dtype, f"{(B, C, H, W, Ch)}", block=util.MODULE_BLOCK)
     assert binding.msla_debug_wait_timeouts() == 0
+
+
+def test_ffn_is_bitwise_reproducible():
+    """Many tiles per CTA and an odd number of staged blocks per tile: a block must not be refilled before its store has read it."""
+    import torch
+    B, C, H, W, Ch = 40, 96, 76, 80, 384
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    rnd = lambda *shape: (torch.randn(*shape, generator=gen, device="cuda") * shape[-1] ** -0.5).half()
+    w = [rnd(Ch, C), rnd(Ch, 3, 3), rnd(C, Ch), rnd(Ch), rnd(Ch), rnd(C)]
+    weights = binding.make_ffn_weights(*w)
+    d0 = binding.make_ffn_desc(B, C, H, W, Ch, C, binding.MSLA_F16, binding.MSLA_ACT_HARDSWISH, True)
+    ws = torch.empty(binding.msla_ffn_workspace_bytes(d0), dtype=torch.uint8, device="cuda")
+    desc = binding.make_ffn_desc(B, C, H, W, Ch, C, binding.MSLA_F16, binding.MSLA_ACT_HARDSWISH, True, workspace=ws)
+    xs = [torch.randn(B, C, H, W, generator=gen, device="cuda").half() for _ in range(2)]
+    first = None
+    for _ in range(20):
+        for i in (1, 0):  # the other input in between: stale data would show
+            out = torch.empty_like(xs[i])
+            binding.msla_ffn_dwconv(desc, xs[i], weights, out)
+        torch.cuda.synchronize()
+        if first is None:
+            first = out
+        assert torch.equal(out, first)
