@@ -21,17 +21,21 @@
 //   owns 128 of the pair's 256 tokens per tile.  The unit handed from role to role is a pair of
 //   heads (two slices of d query channels in one ring slot, one set of barriers): the thread that
 //   issues the MMAs pays a wait and a commit per unit, and its serial chain is what bounds the kernel.
-//     warp 0       TMA: per head one box of 128 tokens x d channels of the head's planar [N][d]
-//                  query matrix (one contiguous 8 KB piece for d = 32; swizzle span = the row)
+//     warp 0       TMA: per unit one box of 2 heads x 128 tokens x d channels of the heads' planar [N][d]
+//                  query matrices (contiguous 8 KB pieces for d = 32; swizzle span = the row)
 //     warps 2-13   turn q into qt in place (normaliser on the fp32 pipes, one token per lane);
 //                  three groups of four warps, each taking every third slice
-//     warp 1       (leader CTA only) issues tcgen05.mma 256 x 256 x 16: A = M, B = qt, both
-//                  K-major, fp32 accumulators in both CTAs' tensor memory
+//     warp 1       loads the rows of M and the key sums; in the leader CTA issues tcgen05.mma 256 x 256 x 16: A = M,
+//                  B = qt, both K-major, fp32 accumulators in both CTAs' tensor memory
 //     warps 14-17  drain the accumulators: TMEM -> bf16 (+ bias) -> swizzled staging -> TMA
 //                  stores of 32-channel x 64-token blocks into the NCHW output
 //                  (RES kernels: the same block of a residual tensor, fetched by TMA into a block of its own one
 //                  block ahead of its use, is added before the conversion: the residual connection around the module)
 //   Two accumulator sets (2 x 256 TMEM columns) let the drain of a tile overlap the next.
+//   A small problem (one tile of 64 tokens per CTA) is the latency of this chain: six transform groups of two warps, a ring that
+//   holds every unit, one copy per unit and M requested by a warp of its own took [1, 256, 32, 32] from 24.7 to 23.8 us a
+//   forward, [1, 192, 64, 128] from 30.6 to 29.8, f16 [8, 128, 45, 80] from 50.2 to 49.4.  Waiting for M slice by slice is slower (25.1):
+//   the waits lengthen the issuing thread's chain.
 // Queries come in one of two layouts: planes [token][d] (above), or (PL) channel-blocked planes [token / 8][d][8], where eight
 // tokens of one channel are 16 contiguous bytes.  PL kernels fetch a head's 128 tokens by one bulk copy (contiguous in the
 // plane); a transform warp takes 32 tokens through ldmatrix.trans, which gives a lane the same two channels of every channel
@@ -62,9 +66,10 @@ constexpr int O_THREADS = 32 * (2 + O_XWARPS + 4);
 constexpr int O_STAGING_WARP = 32 * 128;
 constexpr int O_STAGING = 4 * O_STAGING_WARP;
 constexpr int O_BAR_BYTES = 512;
-constexpr int O_SMEM_FIXED = O_STAGING + O_BAR_BYTES + 1024;  // besides the rows of M, the ring and the residual blocks
-constexpr int O_SMEM_LIMIT = 226 * 1024;                     // dynamic shared memory of a CTA (1 KB of the 227 left to static data)
-static_assert(24 * O_MAX_STAGES + 16 + 16 + 8 + 8 + 8 + 4 * 8 + 8 <= O_BAR_BYTES, "barrier block");
+constexpr int O_KS_BYTES = O_MAX_KS * OKS * 4;  // the image's key sums
+constexpr int O_SMEM_FIXED = O_STAGING + O_BAR_BYTES + O_KS_BYTES;  // besides the rows of M, the ring and the residual blocks
+constexpr int O_SMEM_LIMIT = 227 * 1024;                     // all of it dynamic
+static_assert(24 * O_MAX_STAGES + 16 + 16 + 8 + 8 + 8 + 4 * 8 + 8 + 8 + 8 <= O_BAR_BYTES, "barrier block");
 
 __device__ int g_fused_timeout_flag = 0;
 
@@ -404,12 +409,13 @@ template <int D, bool RES, bool F16, bool PL>
 __global__ void __launch_bounds__(O_THREADS, 1)
 fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant__ CUtensorMap tmQ,
                  const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmR, OutParams p) {
-  extern __shared__ unsigned char smem_raw[];
-  const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;  // swizzle atoms need 1024-byte alignment
+  extern __shared__ __align__(1024) unsigned char smem_raw[];  // swizzle atoms need 1024-byte alignment
+  const uint32_t smem_base = smem_u32(smem_raw);
   const uint32_t a_base = smem_base;                                  // resident rows of M: kslices x 16 KB
-  constexpr int SLICE = OT * D * 2;                                    // one head's queries of this CTA's (up to) 128 tokens
-  constexpr int SLOT = 2 * SLICE;                                      // ring slot: two consecutive heads
+  const uint32_t SLICE = (uint32_t)p.ot * D * 2;                       // one head's queries of this CTA's tokens
+  const uint32_t SLOT = 2 * SLICE;                                     // ring slot: two consecutive heads
   constexpr int ROWB = D * 2;                                          // bytes per token row = the swizzle span (not PL)
+  const int xwarps = p.ot / 32;                                        // transform warps per group: one token per lane
   constexpr int OCTET = D * 16;                                        // PL: bytes of eight tokens
   const uint32_t ring = a_base + (uint32_t)p.kslices * O_A_SLICE;
   const uint32_t staging = ring + (uint32_t)p.stages * SLOT;
@@ -425,8 +431,9 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
   const uint32_t tmem_slot = peer_res_bar + 8;
   const uint32_t resid_bar = tmem_slot + 8;              // [epilogue warp] RES: the warp's residual block landed
   const uint32_t mfree_bar = resid_bar + 32;             // the MMAs of an image are complete: its rows of M may be replaced (commit, both CTAs)
-  __shared__ int abort_flag;
-  __shared__ uint32_t tmem_base_sh;
+  const uint32_t ks_bar = mfree_bar + 8;                 // the image's key sums landed (own CTA)
+  const uint32_t ks_sm = bars + O_BAR_BYTES;
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_raw + (ks_bar + 8 - smem_base));
 
   pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -437,16 +444,17 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
   const int tile_first = min(pair * tiles_per_pair, p.num_tiles), tile_end = min(tile_first + tiles_per_pair, p.num_tiles);
 
   if (threadIdx.x == 0) {
-    abort_flag = 0;
+    *abort_flag = 0;
     for (int s = 0; s < p.stages; ++s) {
       mbar_init(full_bar + 8 * s, 1);
       mbar_init(empty_bar + 8 * s, 1);
-      mbar_init(ready_bar + 8 * s, 2 * 2 * 4);  // per head the four warps of one transform group, in both CTAs
+      mbar_init(ready_bar + 8 * s, 2 * 2 * xwarps);  // per head the warps of one transform group, in both CTAs
     }
     for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar + 8 * a, 1); mbar_init(tempty_bar + 8 * a, 2 * 4); }
     mbar_init(res_bar, 1);
     mbar_init(peer_res_bar, 1);
     mbar_init(mfree_bar, 1);
+    mbar_init(ks_bar, 1);
     if (RES)
       for (int w = 0; w < 4; ++w) mbar_init(resid_bar + 8 * w, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -458,44 +466,25 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (threadIdx.x == 0) {
-    uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(tmem_slot));
-    tmem_base_sh = v;
-  }
   cluster_sync_all();  // both CTAs' barriers exist before anything arrives on them from the other CTA
-  const uint32_t tmem_base = tmem_base_sh;
+  uint32_t tmem_base;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(tmem_slot));
   pdl_wait();  // queries, states and M come from earlier kernels
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (each CTA for itself)
     if (lane == 0) {
-      asm volatile("prefetch.tensormap [%0];" ::"l"(&tmM) : "memory");
       if (!PL) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmQ) : "memory");
-      uint32_t s = 0, ph = 0, mfree_ph = 0;  // ring slot and the parity of its current use
-      int cur_b = -1;
+      uint32_t s = 0, ph = 0;  // ring slot and the parity of its current use
       bool ok = true;
       for (int tile = tile_first; ok && tile < tile_end; ++tile) {
         const int b = tile / p.tiles_per_image, nt = tile % p.tiles_per_image;
-        if (b != cur_b) {
-          if (cur_b >= 0) {
-            // Every MMA that reads the previous image's rows of M must be complete.  The accumulators' barriers cannot tell:
-            // with few heads the ring lets the copies run several tiles ahead, and a parity two phases back looks complete.
-            ok = mbar_wait_cluster(mfree_bar, mfree_ph, &abort_flag);
-            if (!ok) break;
-            mfree_ph ^= 1;
-          }
-          cur_b = b;
-          mbar_expect_tx(res_bar, (uint32_t)(p.kslices * O_A_SLICE));
-          for (int ks = 0; ks < p.kslices; ++ks)
-            tma_load_3d(a_base + ks * O_A_SLICE, &tmM, res_bar, ks * OKS, (int)rank * OM, b);
-        }
         const int n0 = nt * (2 * p.ot) + (int)rank * p.ot;
         for (int h = 0; ok && h < p.Ht; h += 2) {
-          ok = mbar_wait_cluster(empty_bar + 8 * s, ph ^ 1, &abort_flag);
+          ok = mbar_wait_cluster(empty_bar + 8 * s, ph ^ 1, abort_flag);
           if (!ok) break;
-          const bool two = h + 1 < p.Ht;  // an odd head count leaves the last slot half used
           if constexpr (PL) {
+            const bool two = h + 1 < p.Ht;  // an odd head count leaves the last slot half used
             // tokens past the last one are not copied: their accumulator columns are never stored
             const uint32_t bytes = (uint32_t)max(0, min(p.ot, p.N - n0)) * (D * 2);
             auto query = [&](int hq) -> const unsigned char* {
@@ -509,22 +498,22 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
               bulk_load(ring + s * SLOT, query(h), bytes, full_bar + 8 * s);
               if (two) bulk_load(ring + s * SLOT + SLICE, query(h + 1), bytes, full_bar + 8 * s);
             }
-          } else {
-            mbar_expect_tx(full_bar + 8 * s, (uint32_t)((two ? 2 : 1) * p.ot * ROWB));
-            tma_load_4d(ring + s * SLOT, &tmQ, full_bar + 8 * s, 0, n0, h, b);  // rows past the last token are filled with zeros
-            if (two) tma_load_4d(ring + s * SLOT + SLICE, &tmQ, full_bar + 8 * s, 0, n0, h + 1, b);
+          } else {  // one box of two heads; rows past the last token (and the head past an odd count) are filled with zeros
+            mbar_expect_tx(full_bar + 8 * s, SLOT);
+            tma_load_4d(ring + s * SLOT, &tmQ, full_bar + 8 * s, 0, n0, h, b);
           }
           if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1; }
         }
       }
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer (leader) / M hand-shake (peer)
+    // ------------------------------------------------------------ rows of M and key sums (each CTA for itself), MMA issuer (leader)
     if (lane == 0) {
+      asm volatile("prefetch.tensormap [%0];" ::"l"(&tmM) : "memory");
       // instruction descriptor: D = f32, A = B = bf16, both K-major (PL: B MN-major), N = 256, M = 256 (pair)
       const uint32_t idesc = (1u << 4) | (F16 ? 0u : ((1u << 7) | (1u << 10))) | (PL ? 1u << 16 : 0u) | ((uint32_t)((2 * p.ot) >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
       const uint32_t peer_res_remote = map_to_cta(peer_res_bar, 0);
-      uint32_t local = 0, res_ph = 0, s = 0, ph = 0;  // s, ph: ring slot and the parity of its current use
+      uint32_t local = 0, res_ph = 0, mfree_ph = 0, s = 0, ph = 0;  // s, ph: ring slot and the parity of its current use
       // Matrix descriptors: the high words are constants; the low words carry the start address in 16-byte units
       // (A: the 128B-swizzled rows of M; B: the slice, K-major, the swizzle span being the token row).
       const uint64_t a_hi = make_desc(0, 1, 1024 >> 4), b_hi = PL ? make_desc_octets(0, 128 >> 4, OCTET >> 4) : make_desc_kmajor(0, (8 * ROWB) >> 4, D == 32 ? 4ull : 6ull);
@@ -534,11 +523,22 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
       for (int tile = tile_first; ok && tile < tile_end; ++tile, ++local) {
         const int b = tile / p.tiles_per_image;
         if (b != cur_b) {
+          if (cur_b >= 0) {
+            // Every MMA that reads the previous image's rows of M must be complete (and with them every scaling that reads its key
+            // sums).  The accumulators' barriers cannot tell: a parity two phases back looks complete.
+            ok = mbar_wait_cluster(mfree_bar, mfree_ph, abort_flag);
+            if (!ok) break;
+            mfree_ph ^= 1;
+          }
           cur_b = b;
-          ok = mbar_wait(res_bar, res_ph, &abort_flag);  // own rows of M
+          mbar_expect_tx(ks_bar, (uint32_t)(p.Ht * D * 4));
+          bulk_load(ks_sm, p.ks + (long long)b * p.Ht * D, (uint32_t)(p.Ht * D * 4), ks_bar);
+          mbar_expect_tx(res_bar, (uint32_t)(p.kslices * O_A_SLICE));
+          for (int ks = 0; ks < p.kslices; ++ks) tma_load_3d(a_base + ks * O_A_SLICE, &tmM, res_bar, ks * OKS, (int)rank * OM, b);
+          ok = mbar_wait(res_bar, res_ph, abort_flag);  // own rows of M
           if (!ok) break;
           if (rank == 0) {
-            ok = mbar_wait_cluster(peer_res_bar, res_ph, &abort_flag);  // the peer's rows of M
+            ok = mbar_wait_cluster(peer_res_bar, res_ph, abort_flag);  // the peer's rows of M
             if (!ok) break;
           } else {
             mbar_arrive_cluster(peer_res_remote);
@@ -547,27 +547,26 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
         }
         if (rank != 0) continue;
         const uint32_t acc = local & 1, acc_ph = (local >> 1) & 1;
-        ok = mbar_wait_cluster(tempty_bar + 8 * acc, acc_ph ^ 1, &abort_flag);
+        ok = mbar_wait_cluster(tempty_bar + 8 * acc, acc_ph ^ 1, abort_flag);
         if (!ok) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * 256;
-        uint32_t a_lo = a_lo0;  // walks the columns of M: 32 bytes per 16 columns, 64-column slices O_A_SLICE apart
-        int col = 0;
+        uint32_t a_lo = a_lo0;  // the unit's columns of M: 32 bytes per 16 columns, 64-column slices O_A_SLICE apart
         for (int h = 0; ok && h < p.Ht; h += 2) {
-          ok = mbar_wait_cluster(ready_bar + 8 * s, ph, &abort_flag);
+          ok = mbar_wait_cluster(ready_bar + 8 * s, ph, abort_flag);
           if (!ok) break;
           tc_fence_after();
-          const uint32_t b_lo = b_lo0 + s * (uint32_t)(SLOT >> 4);
+          const uint32_t b_lo = b_lo0 + s * (SLOT >> 4);
 #pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            if (h + j >= p.Ht) break;
+          for (int kk = 0; kk < D / 16; ++kk)
+            umma2_bf16(d_tmem, a_hi | (a_lo + 2u * kk), b_hi | (b_lo + (PL ? 16u : 2u) * kk), idesc, (h > 0 || kk > 0) ? 1u : 0u);
+          if (h + 1 < p.Ht) {
 #pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk) {
-              umma2_bf16(d_tmem, a_hi | a_lo, b_hi | (b_lo + (uint32_t)(j * (SLICE >> 4) + (PL ? 16 : 2) * kk)), idesc, (h > 0 || j > 0 || kk > 0) ? 1u : 0u);
-              col += 16;
-              a_lo += (col & 63) ? 2u : (uint32_t)((O_A_SLICE - 96) >> 4);
-            }
+            for (int kk = 0; kk < D / 16; ++kk)
+              umma2_bf16(d_tmem, a_hi | (a_lo + 2u * (D / 16 + kk)), b_hi | (b_lo + (SLICE >> 4) + (PL ? 16u : 2u) * kk), idesc, 1u);
           }
+          // two heads of 32 fill a 64-column slice, two heads of 16 half of one
+          a_lo += D == 32 || (h & 2) ? (uint32_t)((O_A_SLICE - (D == 32 ? 0 : 64)) >> 4) : 4u;
           umma2_commit_both(empty_bar + 8 * s);  // both CTAs may refill the slot once these MMAs have read it
           if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1; }
         }
@@ -577,42 +576,46 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
     }
   } else if (warp < 2 + O_XWARPS) {
     // ------------------------------------------------------------ transform warps: q -> relu(q) / den, in place
-    // Group xg of four warps takes every third slice, starting with slice xg; its 128 lanes own one token
-    // row each (d channels: 64 or 32 bytes, 16-byte pieces XOR-swizzled with the row as the TMA unit
-    // wrote them and as the MMA reads them; eight consecutive rows cover all banks once).
+    // Groups of as many warps as a CTA's tile has token rows for (three groups of four, or six of two) take the slices in
+    // turn, starting with slice xg; a lane owns one token row (d channels: 64 or 32 bytes, 16-byte pieces XOR-swizzled with
+    // the row as the TMA unit wrote them and as the MMA reads them; eight consecutive rows cover all banks once).
     constexpr int PCS = D / 8;     // 16-byte pieces per token row
-    const int xw = warp - 2, xg = xw >> 2, wig = xw & 3;
+    const int xw = warp - 2, xg = xw / xwarps, wig = xw - xg * xwarps, groups = O_XWARPS / xwarps;
     const uint32_t ready_remote = map_to_cta(ready_bar, 0);
     const uint32_t row = (uint32_t)(wig * 32 + lane);
     const uint32_t swz = D == 32 ? (row >> 1) & 3u : (row >> 2) & 1u;
     const uint32_t row_off = row * ROWB;
     uint32_t s = 0, ph = 0, turn = 0;  // ring slot, the parity of its current use, and the group whose turn it is
     const int h_end = (p.Ht + 1) & ~1;  // an odd head count: the empty half of the last slot still has to be signed off
+    uint32_t ks_ph = 0;
+    int cur_b = -1;
     bool ok = true;
     for (int tile = tile_first; ok && tile < tile_end; ++tile) {
       const int b = tile / p.tiles_per_image;
+      if (b != cur_b) {
+        cur_b = b;
+        ok = mbar_wait(ks_bar, ks_ph, abort_flag);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        ks_ph ^= 1;
+      }
       for (int h = 0; ok && h < h_end; ++h) {
         const uint32_t cs = s, cph = ph;  // this slice's slot; the counters move on to the next slice
         const bool mine = (int)turn == xg;
         if (h & 1) { if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1; } }
-        if (++turn == O_XWARPS / 4) turn = 0;
+        if ((int)++turn == groups) turn = 0;
         if (!mine) continue;
-        // with 64-token tiles only the first two warps of a group own rows; past the last head there is nothing to do
-        const bool has_row = (int)row < p.ot && h < p.Ht;
         if constexpr (PL) {
           constexpr int CB = D / 8;  // channel octets; register (o, cb) of lane (g, t) holds channels 8 cb + 2t, + 1 of token 8 o + g
           const int t = lane & 3;
-          float2 kk[CB];  // the lane's key sums, fetched before the wait so that their latency hides behind it
-          const float2* ksp = reinterpret_cast<const float2*>(p.ks + ((long long)b * p.Ht + min(h, p.Ht - 1)) * D) + t;
+          float2 kk[CB];  // the lane's key sums
+          const uint32_t ksp = ks_sm + (uint32_t)(min(h, p.Ht - 1) * D + 2 * t) * 4u;
 #pragma unroll
-          for (int cb = 0; cb < CB; ++cb) {
-            const uint2 v = ld_dep64(ksp + 4 * cb);
-            kk[cb] = make_float2(__uint_as_float(v.x), __uint_as_float(v.y));
-          }
-          ok = mbar_wait(full_bar + 8 * cs, cph, &abort_flag);
+          for (int cb = 0; cb < CB; ++cb) asm volatile("ld.shared.v2.f32 {%0,%1}, [%2];" : "=f"(kk[cb].x), "=f"(kk[cb].y) : "r"(ksp + 32u * cb));
+          ok = mbar_wait(full_bar + 8 * cs, cph, abort_flag);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
-          if (wig * 32 >= p.ot || h >= p.Ht) {  // warp-uniform
+          if (h >= p.Ht) {
             if (lane == 0) mbar_arrive_cluster(ready_remote + 8 * cs);
             continue;
           }
@@ -656,19 +659,16 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
             asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(base + i * 512), "r"(q[4 * i]), "r"(q[4 * i + 1]),
                          "r"(q[4 * i + 2]), "r"(q[4 * i + 3]) : "memory");
         } else {
-        // the head's key sums, fetched before the wait so that their latency hides behind it
-        float kk[D];
-        const float4* ksp = reinterpret_cast<const float4*>(p.ks + ((long long)b * p.Ht + min(h, p.Ht - 1)) * D);
+        float kk[D];  // the head's key sums
+        const uint32_t ksp = ks_sm + (uint32_t)(min(h, p.Ht - 1) * D) * 4u;
 #pragma unroll
-        for (int a4 = 0; a4 < D / 4; ++a4) {
-          const float4 v = ld_dep128f(ksp + a4);
-          kk[4 * a4] = v.x; kk[4 * a4 + 1] = v.y; kk[4 * a4 + 2] = v.z; kk[4 * a4 + 3] = v.w;
-        }
-        ok = mbar_wait(full_bar + 8 * cs, cph, &abort_flag);
+        for (int a4 = 0; a4 < D / 4; ++a4)
+          asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(kk[4 * a4]), "=f"(kk[4 * a4 + 1]), "=f"(kk[4 * a4 + 2]), "=f"(kk[4 * a4 + 3]) : "r"(ksp + 16u * a4));
+        ok = mbar_wait(full_bar + 8 * cs, cph, abort_flag);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         const uint32_t rbase = ring + cs * SLOT + (uint32_t)(h & 1) * SLICE + row_off;
-        if (!has_row) {  // warp-uniform
+        if (h >= p.Ht) {
           if (lane == 0) mbar_arrive_cluster(ready_remote + 8 * cs);
           continue;
         }
@@ -722,7 +722,7 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
     for (int tile = tile_first; ok && tile < tile_end; ++tile, ++local) {
       const int b = tile / p.tiles_per_image, nt = tile % p.tiles_per_image;
       const uint32_t acc = local & 1, acc_ph = (local >> 1) & 1;
-      ok = mbar_wait_cluster(tfull_bar + 8 * acc, acc_ph, &abort_flag);
+      ok = mbar_wait_cluster(tfull_bar + 8 * acc, acc_ph, abort_flag);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
@@ -742,7 +742,7 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
           if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
           __syncwarp();
           if (RES) {           // this block of the residual was requested one block ago
-            ok = mbar_wait(my_resid_bar, res_count & 1, &abort_flag);
+            ok = mbar_wait(my_resid_bar, res_count & 1, abort_flag);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             ++res_count;
@@ -788,7 +788,7 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
   // ------------------------------------------------------------------ teardown
   tc_fence_before();
   __syncthreads();
-  if (abort_flag) {
+  if (*abort_flag) {
     // give copies and MMAs still in flight time to land before memory is released
     for (int i = 0; i < 64; ++i) __nanosleep(1000);
     if (threadIdx.x == 0) atomicExch(&g_fused_timeout_flag, 1);
@@ -887,7 +887,7 @@ msla_status_t run_fused_out_bf16(const void* q, long long q_sb, long long q_sh, 
     const cuuint32_t bM[3] = {OKS, OM, 1};
     const cuuint64_t dQ[4] = {(cuuint64_t)d, (cuuint64_t)N, (cuuint64_t)Ht, (cuuint64_t)B};
     const cuuint64_t sQ[3] = {(cuuint64_t)d * 2, (cuuint64_t)q_sh * 2, (cuuint64_t)q_sb * 2};
-    const cuuint32_t bQ[4] = {(cuuint32_t)d, (cuuint32_t)ot, 1, 1};
+    const cuuint32_t bQ[4] = {(cuuint32_t)d, (cuuint32_t)ot, 2, 1};
     const cuuint64_t dO[3] = {(cuuint64_t)N, (cuuint64_t)Cout, (cuuint64_t)B};
     const cuuint64_t sO[2] = {(cuuint64_t)ldy * 2, (cuuint64_t)Cout * ldy * 2};
     const cuuint32_t bO[3] = {64, 32, 1};
@@ -920,7 +920,7 @@ msla_status_t run_fused_out_bf16(const void* q, long long q_sb, long long q_sh, 
   if (tiles > 0x7fffffffLL) return fail(MSLA_ERR_UNSUPPORTED, "too many token tiles");
   p.num_tiles = (int)tiles;
   // the query ring takes what shared memory is left beside the rows of M (and the residual blocks)
-  const int smem_fixed = p.kslices * O_A_SLICE + O_SMEM_FIXED + (residual ? O_STAGING : 0), slot = 2 * OT * d * 2;
+  const int smem_fixed = p.kslices * O_A_SLICE + O_SMEM_FIXED + (residual ? O_STAGING : 0), slot = 2 * ot * d * 2;
   p.stages = (O_SMEM_LIMIT - smem_fixed) / slot;
   if (p.stages > O_MAX_STAGES) p.stages = O_MAX_STAGES;
   if (p.stages < O_MIN_STAGES) return fail(MSLA_ERR_UNSUPPORTED, "fused apply + projection: no room for the query ring (%d slots)", p.stages);

@@ -316,3 +316,14 @@ def test_project_in_tiles(dtype, B, C, Cout, N):
 @pytest.mark.parametrize("dtype,B,Cin,Cout,N", [("bf16", 1, 136, 200, 72), ("f16", 1, 40, 96, 9480), ("bf16", 3, 24, 200, 6408), ("bf16", 2, 1032, 72, 8)])
 def test_project_out_tiles(dtype, B, Cin, Cout, N):
     test_stage_project_out(dtype, B, Cin, Cout, N)
+
+
+# Both tile widths of the fused apply + projection kernel (64 and 128 tokens per CTA) with an odd head count, a ragged last tile
+# and several images per pair of CTAs.
+@pytest.mark.parametrize("B,H,W,d", [(2, 10, 28, 16), (40, 16, 35, 32), (90, 8, 33, 16)])
+def test_fused_output_tiles(B, H, W, d):
+    s = inputs.ModuleShape("tiles", "bf16", B, 32, H, W, 1, d, seed=44, n_scales=3, agg_kernel=5, agg_kernel2=3)
+    t = inputs.module_inputs(s)
+    ref = oracle.msla_forward3(t["x"], t["w_qkv"], t["w_dw"], t["w_pw"], t["w_dw2"], t["w_pw2"], t["w_proj"], heads=1, d=d)
+    util.assert_close(util.run_module(s, t), ref, "bf16", "tiles", block=util.MODULE_BLOCK)
+    assert binding.msla_debug_wait_timeouts() == 0
