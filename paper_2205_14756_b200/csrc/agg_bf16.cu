@@ -31,8 +31,9 @@
 //       four times the cycles of the staging writes).
 // The single TMA buffer is refilled for the next tile as soon as P1 is over.
 // The grid is persistent: two CTAs per SM, each with a contiguous run of
-// (image, group, tile) units; the weight fragments are reloaded when the group
-// changes.
+// (group, image, tile) units; the weight fragments are reloaded when the group
+// changes.  With images outermost every unit of a one-tile image changed group and waited for its
+// fragments: [64, 256, 14, 14] 76.9 -> 70.0 us a forward, [32, 384, 7, 7] 51.3 -> 46.8.
 #include <cuda.h>
 
 #include "msla_common.cuh"
@@ -107,7 +108,9 @@ struct ToeplitzParams {
   int dst_planes_per_batch;
   int groups;                  // blocks of 32 channels per image: plane `group` (d = 32) or planes 2*group, 2*group+1 (d = 16)
   int tiles_x, tiles_y, tiles_total;  // tiles per plane
-  long long units;             // B * groups * tiles_total, tile fastest
+  int B;
+  int taps_ready;              // 0: the taps come from the previous kernel (a 3x3 filter embedded in 5x5)
+  long long units;             // groups * B * tiles_total, tile fastest
   long long units_per_cta;
 };
 
@@ -126,7 +129,7 @@ aggregate_toeplitz_kernel(const __grid_constant__ CUtensorMap tm_src, const __gr
   const int unit_count = (int)max(0LL, min(p.units_per_cta, p.units - unit_first));
   const uint32_t bar = smem_addr(&bar_storage);
 
-  // Cursor over (image, group, tile) units, tile fastest, advanced without divisions.  Inside a plane the
+  // Cursor over (group, image, tile) units, tile fastest, advanced without divisions.  Inside a plane the
   // tiles run down bands of T_BAND tile rows, column by column, so that a tile's lower and right
   // neighbours follow within a few iterations and find the shared halo rows and columns in L2.
   struct Unit { int tile, tx, ty, band_end, group, b; };  // band_end: first tile row below the current band
@@ -139,8 +142,8 @@ aggregate_toeplitz_kernel(const __grid_constant__ CUtensorMap tm_src, const __gr
     const int bh = r.band_end - band * T_BAND;
     r.tx = rem / bh;
     r.ty = band * T_BAND + rem - r.tx * bh;
-    r.b = (int)(bg / p.groups);
-    r.group = (int)(bg - (long long)r.b * p.groups);
+    r.group = (int)(bg / p.B);
+    r.b = (int)(bg - (long long)r.group * p.B);
     return r;
   };
   auto advance = [&](Unit& u) {
@@ -152,7 +155,7 @@ aggregate_toeplitz_kernel(const __grid_constant__ CUtensorMap tm_src, const __gr
     }
     if (u.tile == p.tiles_total) {
       u.tile = 0; u.ty = 0; u.band_end = min(T_BAND, p.tiles_y);
-      if (++u.group == p.groups) { u.group = 0; ++u.b; }
+      if (++u.b == p.B) { u.b = 0; ++u.group; }
     }
   };
   // x and y may start below 0 and run past W, H: the TMA unit returns zeros there.
@@ -187,9 +190,9 @@ aggregate_toeplitz_kernel(const __grid_constant__ CUtensorMap tm_src, const __gr
     for (int cc = 0; cc < 4; ++cc)
 #pragma unroll
       for (int dy = 0; dy < 5; ++dy) {
-        const bf16* wrow = p.w_dw + (long long)(ch0 + 4 * warp + cc) * 25 + dy * 5;
+        const unsigned short* wrow = reinterpret_cast<const unsigned short*>(p.w_dw) + (long long)(ch0 + 4 * warp + cc) * 25 + dy * 5;
         const int i0 = 2 * t - g - 2;
-        auto tap = [&](int i) -> uint32_t { return (i >= 0 && i < 5) ? (uint32_t)__bfloat16_as_ushort(wrow[i]) : 0u; };
+        auto tap = [&](int i) -> uint32_t { return (i >= 0 && i < 5) ? (uint32_t)wrow[i] : 0u; };
         bt[cc][dy][0] = tap(i0) | (tap(i0 + 1) << 16);
         bt[cc][dy][1] = tap(i0 + 8) | (tap(i0 + 9) << 16);
       }
@@ -213,6 +216,7 @@ aggregate_toeplitz_kernel(const __grid_constant__ CUtensorMap tm_src, const __gr
       }
   };
   int cur_group = un.group;
+  if (!p.taps_ready) pdl_wait();
   load_weights(cur_group);
 
   // Per-lane address offsets of the six ldmatrix loads of a channel.  Matrix (r, h) = staged rows
@@ -368,7 +372,7 @@ bool aggregate_bf16_supported(int H, int W, int Ch, int d) { return (d == 32 || 
 namespace {
 template <bool D16, bool F16>
 msla_status_t launch_toeplitz(const void* src, long long src_planes_total, int src_ppb, const void* w_dw, const void* w_pw,
-                              void* dst, long long dst_planes_total, int dst_ppb, int B, int H, int W, int Ch, cudaStream_t st) {
+                              void* dst, long long dst_planes_total, int dst_ppb, int B, int H, int W, int Ch, cudaStream_t st, bool taps_ready) {
   constexpr int DP = D16 ? 16 : 32;  // channels per plane
   CUtensorMap tm_src, tm_dst;
   {
@@ -384,6 +388,7 @@ msla_status_t launch_toeplitz(const void* src, long long src_planes_total, int s
   ToeplitzParams p;
   p.w_dw = (const bf16*)w_dw; p.w_pw = (const bf16*)w_pw;
   p.src_planes_per_batch = src_ppb; p.dst_planes_per_batch = dst_ppb; p.groups = Ch / TD;
+  p.B = B; p.taps_ready = taps_ready;
   p.tiles_x = (W + TW - 1) / TW;
   p.tiles_y = (H + TH - 1) / TH;
   const long long tiles = (long long)p.tiles_x * p.tiles_y;
@@ -410,16 +415,16 @@ msla_status_t launch_toeplitz(const void* src, long long src_planes_total, int s
 // the plane size).
 msla_status_t run_aggregate_bf16(const void* src, long long src_planes_total, int src_ppb, const void* w_dw,
                                  const void* w_pw, void* dst, long long dst_sb, int B, int H, int W, int Ch, int d,
-                                 cudaStream_t st, bool f16) {
+                                 cudaStream_t st, bool f16, bool taps_ready) {
   const long long plane = (long long)H * W * d;
   if (!aggregate_bf16_supported(H, W, Ch, d) || dst_sb % plane != 0)
     return fail(MSLA_ERR_UNSUPPORTED, "aggregation: d = %d, %d channels, output batch stride %lld elements", d, Ch, dst_sb);
   const long long dst_ppb = dst_sb / plane, dst_total = (B - 1) * dst_ppb + Ch / d;
   if (f16)
-    return d == 16 ? launch_toeplitz<true, true>(src, src_planes_total, src_ppb, w_dw, w_pw, dst, dst_total, (int)dst_ppb, B, H, W, Ch, st)
-                   : launch_toeplitz<false, true>(src, src_planes_total, src_ppb, w_dw, w_pw, dst, dst_total, (int)dst_ppb, B, H, W, Ch, st);
-  return d == 16 ? launch_toeplitz<true, false>(src, src_planes_total, src_ppb, w_dw, w_pw, dst, dst_total, (int)dst_ppb, B, H, W, Ch, st)
-                 : launch_toeplitz<false, false>(src, src_planes_total, src_ppb, w_dw, w_pw, dst, dst_total, (int)dst_ppb, B, H, W, Ch, st);
+    return d == 16 ? launch_toeplitz<true, true>(src, src_planes_total, src_ppb, w_dw, w_pw, dst, dst_total, (int)dst_ppb, B, H, W, Ch, st, taps_ready)
+                   : launch_toeplitz<false, true>(src, src_planes_total, src_ppb, w_dw, w_pw, dst, dst_total, (int)dst_ppb, B, H, W, Ch, st, taps_ready);
+  return d == 16 ? launch_toeplitz<true, false>(src, src_planes_total, src_ppb, w_dw, w_pw, dst, dst_total, (int)dst_ppb, B, H, W, Ch, st, taps_ready)
+                 : launch_toeplitz<false, false>(src, src_planes_total, src_ppb, w_dw, w_pw, dst, dst_total, (int)dst_ppb, B, H, W, Ch, st, taps_ready);
 }
 
 int agg_timeout_flag() {

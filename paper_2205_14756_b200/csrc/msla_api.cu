@@ -422,7 +422,7 @@ static msla_status_t run_aggregate_plain(const void* src, const void* w_dw, cons
 // src, dst planar [B, Ch/d, H*W, d] with batch strides src_sb, dst_sb (elements)
 static msla_status_t run_aggregate(msla_dtype_t dt, const void* src, const void* w_dw, const void* w_pw,
                                    void* dst, int B, int H, int W, int Ch, int d, long long src_sb,
-                                   long long dst_sb, cudaStream_t st) {
+                                   long long dst_sb, cudaStream_t st, bool taps_ready = true) {
   if (dt == MSLA_F32) return run_aggregate_plain<float>(src, w_dw, w_pw, dst, B, H, W, Ch / d, d, src_sb, dst_sb, st);
   const long long plane = (long long)H * W * d;
   const bool f16 = dt == MSLA_F16;
@@ -432,7 +432,7 @@ static msla_status_t run_aggregate(msla_dtype_t dt, const void* src, const void*
     else if (d == 16 && Ch > 16 && aggregate_bf16_supported(H, W, Ch - 16, d)) done = Ch - 16;
   }
   if (done) {
-    const msla_status_t s = run_aggregate_bf16(src, (long long)B * (src_sb / plane), (int)(src_sb / plane), w_dw, w_pw, dst, dst_sb, B, H, W, done, d, st, f16);
+    const msla_status_t s = run_aggregate_bf16(src, (long long)B * (src_sb / plane), (int)(src_sb / plane), w_dw, w_pw, dst, dst_sb, B, H, W, done, d, st, f16, taps_ready);
     if (s != MSLA_OK || done == Ch) return s;
   }
   const size_t first = (size_t)(done / d) * plane * 2;
@@ -461,7 +461,7 @@ static msla_status_t run_branches(const msla_desc* desc, const msla_weights* w, 
   const size_t branch_bytes = (size_t)3 * p.Cp * p.N * elem_size(desc->dtype);
   for (int br = 1; br < p.S; ++br) {
     const msla_status_t s = run_aggregate(desc->dtype, ms, aggregation_taps(desc, w, p, br, st), br == 1 ? w->w_pw : w->w_pw2, ms + br * branch_bytes,
-                                          desc->B, desc->H, desc->W, 3 * p.Cp, desc->d, ms_sb, ms_sb, st);
+                                          desc->B, desc->H, desc->W, 3 * p.Cp, desc->d, ms_sb, ms_sb, st, (br == 1 ? desc->agg_kernel : desc->agg_kernel2) == 5);
     if (s != MSLA_OK) return s;
   }
   return MSLA_OK;

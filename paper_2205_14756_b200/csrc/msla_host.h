@@ -136,11 +136,11 @@ int gemm_timeout_flag();
 int run_wait_selftest(long long limit_cycles, int* scratch, cudaStream_t st);
 
 // bf16 aggregation (d = 16 or 32, Ch a multiple of 32): TMA halo tiles, depthwise filter as banded matrices on
-// tensor cores (agg_bf16.cu).  dst_sb must be a multiple of the plane size H*W*d.
+// tensor cores (agg_bf16.cu).  taps_ready: w_dw is not the previous kernel's output.  dst_sb must be a multiple of the plane size H*W*d.
 bool aggregate_bf16_supported(int H, int W, int Ch, int d);
 msla_status_t run_aggregate_bf16(const void* src, long long src_planes_total, int src_ppb, const void* w_dw,
                                  const void* w_pw, void* dst, long long dst_sb, int B, int H, int W, int Ch, int d,
-                                 cudaStream_t st, bool f16 = false);
+                                 cudaStream_t st, bool f16, bool taps_ready);
 int agg_timeout_flag();
 
 // Rows of n 16-bit elements to and from rows `pitch` (a multiple of 8) elements apart (repack.cu).
