@@ -29,20 +29,26 @@
 // head; d = 16: of two heads), then of blocks of queries.  Tiles run down bands of four tile rows, column by column, so that the
 // halo rows and columns shared with the neighbours are still in L2.  Warps are specialised, so that the phases of neighbouring
 // tiles overlap (all warps taking the phases in turn, 16 of them, kept the tensor pipe 43 % busy):
-//   copies       (one lane of warp 16) 20 rows x 3 (queries: 4) octets per block by TMA, even and odd image rows apart (two tensor maps), so that
-//                the rows of an ldmatrix matrix (2g + r, g = 0 .. 7) are neighbours: a box of 8 channels x 8 pixels (128 bytes, 128B
-//                swizzle) x 10 rows x octets x channel groups lands as [group][octet][row][128 bytes], and eight consecutive rows
-//                fall on different banks.  Rows and octets outside the image are zero-filled = the padding.  Two buffers (queries: four)
 //   warps 0-15   depthwise step of four channels each (queries: two), Toeplitz fragments in registers while the head lasts; fp32
 //                sums rounded once into a [channel][pixel] tile, double buffered
 //   warps 16-23  keys and values: 16 key channels x 4 image rows of both states each, accumulators in registers while the (head,
 //                image) lasts: the un-aggregated scale from the staged rows, the aggregated one from the depthwise tile, keys
 //                through their grouped 1x1 first (transposed: channels x pixels, whose accumulator layout is the A-fragment
 //                layout of the state's MMA)
-//                queries: grouped 1x1 of two image rows each, staged and written by bulk copies
-// Shared-memory wavefronts and the MMA rate bound it about equally (per 16 x 16 tile of a head's K, V and Q: about 3400
-// wavefronts and 1540 MMAs of two cycles).  [1, 256, 512, 512]: 205 us,
-// where the token-major aggregation (209 us) and the state kernel (98 us) took 307.
+//                queries: grouped 1x1 of two image rows each, staged
+//   warp 24      requests the tiles: 20 rows x 3 (queries: 4) octets per block by TMA, even and odd image rows apart (two tensor maps), so that
+//                the rows of an ldmatrix matrix (2g + r, g = 0 .. 7) are neighbours: a box of 8 channels x 8 pixels (128 bytes, 128B
+//                swizzle) x 10 rows x octets x channel groups lands as [group][octet][row][128 bytes], and eight consecutive rows
+//                fall on different banks.  Rows and octets outside the image are zero-filled = the padding.  Two buffers (queries: four)
+//   warp 25      writes the staged query tiles, one TMA store each
+// Issuing a copy takes a thread about 0.14 us.  With the copies issued by the summing warps (per tile of queries two loads by one of
+// them and two row copies by each) a tile of queries took 1.32 us against 1.12 now: the warps wait for one another in turn.
+// In each role the next operands are fetched before the stores that wait for the current products.
+// Shared-memory wavefronts, the MMA rate and issue slots bound it together (per 16 x 16 tile of a head's K, V and Q: about 3400
+// wavefronts and 1540 MMAs of two cycles; leaving out the depthwise MMAs, the state of either scale or the loads takes 16, 12, 12
+// or 3 % off the keys and values).  [1, 256, 512, 512]: 192 us (212 before the copies had warps of their own), where the
+// token-major aggregation (209 us) and the state kernel (98 us) took 307; [1, 128, 512, 512] d = 16: 97 (119); whole
+// forward 415 -> 393, 251 -> 229, [16, 256, 64, 64] 141.5 -> 136, building block [1, 256, 128, 256] / 1024 160.5 -> 157.
 // All waits are bounded; on time-out every warp leaves its loop and a flag is raised.
 #include <cuda.h>
 
@@ -56,11 +62,16 @@ namespace {
 
 using bf16 = __nv_bfloat16;
 
-constexpr int AS_DW_WARPS = 16, AS_SUM_WARPS = 8, AS_THREADS = 32 * (AS_DW_WARPS + AS_SUM_WARPS);
+constexpr int AS_DW_WARPS = 16, AS_SUM_WARPS = 8, AS_COPY_WARPS = 4;  // of the last four one requests loads and one stores
+constexpr int AS_THREADS = 32 * (AS_DW_WARPS + AS_SUM_WARPS + AS_COPY_WARPS);
+constexpr int AS_LOAD_WARP = AS_DW_WARPS + AS_SUM_WARPS, AS_STORE_WARP = AS_LOAD_WARP + 1;
+// Registers a thread: the launch's 72, shared out (80 for 24 warps alike spilled in both computing roles)
+constexpr int AS_DW_REGS = 64, AS_SUM_REGS = 104, AS_COPY_REGS = 40;
+static_assert(AS_DW_WARPS * AS_DW_REGS + AS_SUM_WARPS * AS_SUM_REGS + AS_COPY_WARPS * AS_COPY_REGS == AS_THREADS / 32 * 72, "shares of the launch's registers");
 constexpr int AS_TW = 16, AS_TH = 16, AS_ROWS = AS_TH + 4;
 constexpr int AS_DWO_CH = AS_TW * AS_TH * 2 + 16;   // depthwise output: bytes per channel (33 * 16)
 constexpr int AS_DWO_SIDE = 32 * AS_DWO_CH;          // of one block
-constexpr int AS_STAGE = 2048, AS_STAGE_WARP = 2 * AS_STAGE;  // query output of a warp: 2 rows x 16 pixels x 32 channels, double buffered
+constexpr int AS_STAGE = AS_TH * 1024;              // staged query output: 16 rows x 16 pixels x 32 channels, double buffered
 constexpr int AS_BAND = 4;                          // tile rows per band of the traversal
 // Staged tile of the two roles: SIDES blocks of OCT octets per row; [block][row parity][channel group of 8][octet][row / 2][128 bytes].
 template <int SIDES_, int OCT_, int BUFS_> struct AsStage {
@@ -72,7 +83,7 @@ template <int SIDES_, int OCT_, int BUFS_> struct AsStage {
 using AsKv = AsStage<2, 3, 2>;
 using AsQ = AsStage<1, 4, 4>;
 constexpr int AS_RED = 2 * AS_SUM_WARPS * 16 * 33 * 4;  // the warps' states on their way to the partial sums
-constexpr int AS_SMEM_KV = AsKv::BUFS * AsKv::BUF + 2 * AsKv::DWO + AS_RED, AS_SMEM_Q = AsQ::BUFS * AsQ::BUF + 2 * AsQ::DWO + AS_SUM_WARPS * AS_STAGE_WARP;
+constexpr int AS_SMEM_KV = AsKv::BUFS * AsKv::BUF + 2 * AsKv::DWO + AS_RED, AS_SMEM_Q = AsQ::BUFS * AsQ::BUF + 2 * AsQ::DWO + 2 * AS_STAGE;
 constexpr int AS_SMEM = (AS_SMEM_KV > AS_SMEM_Q ? AS_SMEM_KV : AS_SMEM_Q) + 1024;  // + slack to align the base (the swizzle is a function of the address)
 static_assert(AsKv::PAR % 1024 == 0 && AsQ::PAR % 1024 == 0 && (AS_DWO_CH / 16) % 2 == 1, "swizzle atoms; conflict-free pitch");
 static_assert(AS_SMEM + 256 <= 227 * 1024, "dynamic and static shared memory of a CTA");
@@ -80,7 +91,6 @@ static_assert(AS_SMEM + 256 <= 227 * 1024, "dynamic and static shared memory of 
 __device__ int g_aggstate_timeout_flag = 0;
 
 struct AggStateParams {
-  unsigned char* q1;         // [B][heads] planes of aggregated queries
   float* partial;            // slots of 2 states per head of the block: [.., un-aggregated, aggregated][d][d + 1]
   const bf16* w_dw;          // [3 * heads * d][5][5]
   const bf16* w_pw;          // [3 * heads * d][d]
@@ -156,8 +166,9 @@ __device__ __forceinline__ void as_tma_load(uint32_t dst, const CUtensorMap* map
       "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], [%2];"
       ::"r"(dst), "l"(map), "r"(bar), "r"(0), "r"(row2), "r"(oct), "r"(0), "r"(plane) : "memory");
 }
-__device__ __forceinline__ void as_bulk_store(void* dst, uint32_t src, uint32_t bytes) {
-  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(src), "r"(bytes) : "memory");
+__device__ __forceinline__ void as_tma_store(const CUtensorMap* map, uint32_t src, int piece, int row, int plane) {
+  asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];"
+               ::"l"(map), "r"(src), "r"(0), "r"(piece), "r"(row), "r"(plane) : "memory");
 }
 
 // A tile of the run: pair of blocks, image, position.  Advanced without divisions.
@@ -190,21 +201,20 @@ __device__ __forceinline__ void as_advance(const AggStateParams& p, AsUnit& u, i
   u.band_end = min(u.ty + AS_BAND, p.tiles_y);
 }
 
-// Toeplitz B fragments of N channels from `ch` on: the lane's two words of filter row dy are taps i0, i0 + 1 and i1, i1 + 1 (zero
-// outside the five).  No branches: all loads of a thread are in flight together.
+// Words of Toeplitz B fragments of N channels from `ch` on: taps i, i + 1 of every filter row (zero outside the five).  No branches: all
+// loads of a thread are in flight together.
 template <int N>
-__device__ __forceinline__ void as_load_taps(const bf16* w_dw, int ch, int i0, int i1, uint32_t (&bt)[N][5][2]) {
+__device__ __forceinline__ void as_load_taps(const bf16* w_dw, int ch, int i, uint32_t (&bt)[N][5]) {
 #pragma unroll
   for (int cc = 0; cc < N; ++cc)
 #pragma unroll
     for (int dy = 0; dy < 5; ++dy) {
       const unsigned short* row = reinterpret_cast<const unsigned short*>(w_dw) + (long long)(ch + cc) * 25 + dy * 5;
-      auto tap = [&](int i) -> uint32_t {
-        const uint32_t v = ld_dep16(row + min(max(i, 0), 4));
-        return i >= 0 && i < 5 ? v : 0u;
+      auto tap = [&](int j) -> uint32_t {
+        const uint32_t v = ld_dep16(row + min(max(j, 0), 4));
+        return j >= 0 && j < 5 ? v : 0u;
       };
-      bt[cc][dy][0] = tap(i0) | (tap(i0 + 1) << 16);
-      bt[cc][dy][1] = tap(i1) | (tap(i1 + 1) << 16);
+      bt[cc][dy] = tap(i) | (tap(i + 1) << 16);
     }
 }
 // Pixel pair (row 2g + half, columns 8nb + 2t, + 1): word t of octet (2nb + half) * 8 + g of the channel.
@@ -219,15 +229,14 @@ __device__ __forceinline__ void as_put_depthwise(uint32_t dst, const float (&acc
 template <int D, bool F16>
 __global__ void __launch_bounds__(AS_THREADS, 1)
 agg_state_kernel(const __grid_constant__ CUtensorMap kv_even, const __grid_constant__ CUtensorMap kv_odd, const __grid_constant__ CUtensorMap q_even,
-                 const __grid_constant__ CUtensorMap q_odd, AggStateParams p) {
+                 const __grid_constant__ CUtensorMap q_odd, const __grid_constant__ CUtensorMap q_out, AggStateParams p) {
   constexpr bool D16 = D == 16;
-  constexpr int BLK = D * 16;        // bytes of a pixel octet of one plane
   constexpr int NE = D * (D + 1);
   constexpr int HPB = 32 / D;        // heads per 32-channel block
   constexpr int NJ = D / 8;          // 8-channel column blocks of a state
   extern __shared__ unsigned char smem_raw[];
   const uint32_t box = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  __shared__ __align__(8) unsigned long long bar_storage[20];
+  __shared__ __align__(8) unsigned long long bar_storage[24];
   __shared__ int abort_flag;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
@@ -253,6 +262,8 @@ agg_state_kernel(const __grid_constant__ CUtensorMap kv_even, const __grid_const
   auto freed = [&](int role, uint32_t buf) { return bars + 64 * role + (role ? 32 : 16) + 8 * buf; };
   auto dwo_full = [&](int role, uint32_t buf) { return bars + 64 * role + (role ? 64 : 32) + 8 * buf; };
   auto dwo_freed = [&](int role, uint32_t buf) { return bars + 64 * role + (role ? 80 : 48) + 8 * buf; };
+  auto staged = [&](uint32_t buf) { return bars + 160 + 8 * buf; };       // queries: the output tile is staged / has been copied out
+  auto staging_freed = [&](uint32_t buf) { return bars + 176 + 8 * buf; };
   pdl_launch_dependents();
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -265,6 +276,10 @@ agg_state_kernel(const __grid_constant__ CUtensorMap kv_even, const __grid_const
         mbar_init(dwo_full(r, i), AS_DW_WARPS);
         mbar_init(dwo_freed(r, i), AS_SUM_WARPS);
       }
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(staged(i), AS_SUM_WARPS);
+      mbar_init(staging_freed(i), 1);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -279,7 +294,7 @@ agg_state_kernel(const __grid_constant__ CUtensorMap kv_even, const __grid_const
     __syncwarp();
     if (lane == 0) mbar_arrive(bar);
   };
-  // Requests tile `un` of keys and values / of queries and moves the cursor on; one lane of the first of the summing warps.
+  // Requests tile `un` of keys and values / of queries and moves the cursor on.
   auto request_kv = [&](AsUnit& un, uint32_t buf) {
     if (lane == 0) {
       mbar_expect_tx(full(0, buf), AsKv::BUF);
@@ -312,332 +327,390 @@ agg_state_kernel(const __grid_constant__ CUtensorMap kv_even, const __grid_const
   };
   pdl_wait();  // the planes are the previous kernel's output; q1 and the partial states may still be read by an earlier one
 
-  // 16 depthwise warps of 72 registers and 8 summing warps of 96: together the 24 * 80 of the launch.  With 80 for all both
-  // spilled (keys and values of 512 x 512 tokens: 217 -> 182 us).
-  if (warp < AS_DW_WARPS) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
-  else asm volatile("setmaxnreg.inc.sync.aligned.u32 96;");
+  // Roles.  Each branch ends the keys and values at the same barrier, after which the queries' tiles take over the shared memory (in
+  // one piece of code per role: where branches with different register counts meet, the compiler allows the smallest).
+  auto end_of_kv = [&]() -> bool {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("bar.sync 2, %0;" ::"n"(AS_THREADS) : "memory");
+    ok = ok && !*(volatile int*)&abort_flag;
+    return ok && q_count > 0;
+  };
   if (warp < AS_DW_WARPS) {
-    // ---------------------------------------------------------------- depthwise: keys and values
-    using ST = AsKv;
-    const int side = warp >> 3, c0 = 4 * (warp & 7);
-    const uint32_t dwo = box + 2 * ST::BUF + (uint32_t)(side * AS_DWO_SIDE + c0 * AS_DWO_CH + lane * 4);
-    // matrix (r, o) = staged rows 2g' + r, octet o of channel c0; lane l supplies row l % 8 of matrix l / 8.  Channel c0 + cc: XOR
-    // cc << 4 (the swizzle permutes the 16-byte pieces of a row by XOR).
-    auto mat = [&](int r, int o) { return box + at(ST{}, side, 2 * (lane & 7) + r, o, c0); };
-    const int mi = lane >> 3;
-    const uint32_t a0 = mi < 3 ? mat(0, mi) : mat(1, 0), a1 = mi < 2 ? mat(1, 1 + mi) : mat(2, mi - 2), a2 = mi == 0 ? mat(2, 2) : mat(3, mi - 1),
-                   a3 = mi < 3 ? mat(4, mi) : mat(5, 0), a4 = mat(5, 1 + (mi & 1));
-    uint32_t bt[4][5][2];  // Toeplitz B fragments: window pixel k, output pixel n: tap k - n - 4
-    int change = 0;        // tile at which the pair of blocks changes
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(AS_DW_REGS));
+    {
+      // ---------------------------------------------------------------- depthwise: keys and values
+      using ST = AsKv;
+      const int side = warp >> 3, c0 = 4 * (warp & 7);
+      const uint32_t dwo = box + 2 * ST::BUF + (uint32_t)(side * AS_DWO_SIDE + c0 * AS_DWO_CH + lane * 4);
+      // matrix (r, o) = staged rows 2g' + r, octet o of channel c0; lane l supplies row l % 8 of matrix l / 8.  Channel c0 + cc: XOR
+      // cc << 4 (the swizzle permutes the 16-byte pieces of a row by XOR).
+      auto mat = [&](int r, int o) { return box + at(ST{}, side, 2 * (lane & 7) + r, o, c0); };
+      const int mi = lane >> 3;
+      const uint32_t a0 = mi < 3 ? mat(0, mi) : mat(1, 0), a1 = mi < 2 ? mat(1, 1 + mi) : mat(2, mi - 2), a2 = mi == 0 ? mat(2, 2) : mat(3, mi - 1),
+                     a3 = mi < 3 ? mat(4, mi) : mat(5, 0), a4 = mat(5, 1 + (mi & 1));
+      // Toeplitz B fragments: window pixel k, output pixel n: tap k - n - 4.  Of a lane's two words (k = 2t, + 1 and 2t + 8, + 9) one at
+      // most meets the five taps, the same one throughout.
+      uint32_t bt[4][5];
+      const bool low = 2 * t - g - 4 >= -1;
+      int change = 0;        // tile at which the pair of blocks changes
 #pragma unroll 1
-    for (int i = 0; i < kv_count; ++i) {
-      const uint32_t buf = i & 1, ph = (i >> 1) & 1;
-      if (i == change) {
-        const long long per_pair = (long long)p.kv_tiles * p.B;
-        const int pr = (int)((u_first + i) / per_pair);
-        change = (int)min((pr + 1) * per_pair - u_first, (long long)kv_count);
-        as_load_taps<4>(p.w_dw, plane_of(1 + side, pr, D16 ? c0 >> 4 : 0) * D + (c0 & (D - 1)), 2 * t - g - 4, 2 * t - g + 4, bt);
-      }
-      if (!wait(full(0, buf), ph)) break;
-      if (!wait(dwo_freed(0, buf), ph ^ 1)) break;
-      const uint32_t ro = buf * ST::BUF, dw = dwo + buf * ST::DWO;
-#pragma unroll
-      for (int cc = 0; cc < 4; ++cc) {
+      for (int i = 0; i < kv_count; ++i) {
+        const uint32_t buf = i & 1, ph = (i >> 1) & 1;
+        if (i == change) {
+          const long long per_pair = (long long)p.kv_tiles * p.B;
+          const int pr = (int)((u_first + i) / per_pair);
+          change = (int)min((pr + 1) * per_pair - u_first, (long long)kv_count);
+          as_load_taps<4>(p.w_dw, plane_of(1 + side, pr, D16 ? c0 >> 4 : 0) * D + (c0 & (D - 1)), low ? 2 * t - g - 4 : 2 * t - g + 4, bt);
+        }
+        if (!wait(full(0, buf), ph)) break;
+        if (!wait(dwo_freed(0, buf), ph ^ 1)) break;
+        const uint32_t ro = buf * ST::BUF, dw = dwo + buf * ST::DWO;
         uint32_t R[6][3];
-        as_ldsm4(R[0][0], R[0][1], R[0][2], R[1][0], (a0 + ro) ^ (uint32_t)(cc << 4));
-        as_ldsm4(R[1][1], R[1][2], R[2][0], R[2][1], (a1 + ro) ^ (uint32_t)(cc << 4));
-        as_ldsm4(R[2][2], R[3][0], R[3][1], R[3][2], (a2 + ro) ^ (uint32_t)(cc << 4));
-        as_ldsm4(R[4][0], R[4][1], R[4][2], R[5][0], (a3 + ro) ^ (uint32_t)(cc << 4));
-        as_ldsm2(R[5][1], R[5][2], (a4 + ro) ^ (uint32_t)(cc << 4));
-        if (cc == 3) arrive(freed(0, buf));
-        float acc[2][4];
+        auto load = [&](int cc) {
+          as_ldsm4(R[0][0], R[0][1], R[0][2], R[1][0], (a0 + ro) ^ (uint32_t)(cc << 4));
+          as_ldsm4(R[1][1], R[1][2], R[2][0], R[2][1], (a1 + ro) ^ (uint32_t)(cc << 4));
+          as_ldsm4(R[2][2], R[3][0], R[3][1], R[3][2], (a2 + ro) ^ (uint32_t)(cc << 4));
+          as_ldsm4(R[4][0], R[4][1], R[4][2], R[5][0], (a3 + ro) ^ (uint32_t)(cc << 4));
+          as_ldsm2(R[5][1], R[5][2], (a4 + ro) ^ (uint32_t)(cc << 4));
+        };
+        load(0);
 #pragma unroll
-        for (int nb = 0; nb < 2; ++nb) as_mma_first<F16>(acc[nb], R[0][nb], R[1][nb], R[0][nb + 1], R[1][nb + 1], bt[cc][0][0], bt[cc][0][1]);
+        for (int cc = 0; cc < 4; ++cc) {
+          float acc[2][4];
 #pragma unroll
-        for (int dy = 1; dy < 5; ++dy)
+          for (int nb = 0; nb < 2; ++nb) as_mma_first<F16>(acc[nb], R[0][nb], R[1][nb], R[0][nb + 1], R[1][nb + 1], low ? bt[cc][0] : 0u, low ? 0u : bt[cc][0]);
 #pragma unroll
-          for (int nb = 0; nb < 2; ++nb) as_mma<F16>(acc[nb], R[dy][nb], R[dy + 1][nb], R[dy][nb + 1], R[dy + 1][nb + 1], bt[cc][dy][0], bt[cc][dy][1]);
-        as_put_depthwise<F16>(dw + cc * AS_DWO_CH, acc);
+          for (int dy = 1; dy < 5; ++dy)
+#pragma unroll
+            for (int nb = 0; nb < 2; ++nb) as_mma<F16>(acc[nb], R[dy][nb], R[dy + 1][nb], R[dy][nb + 1], R[dy + 1][nb + 1], low ? bt[cc][dy] : 0u, low ? 0u : bt[cc][dy]);
+          if (cc < 3) load(cc + 1);  // ahead of the stores below, which wait for the products
+          if (cc == 2) arrive(freed(0, buf));
+          as_put_depthwise<F16>(dw + cc * AS_DWO_CH, acc);
+        }
+        arrive(dwo_full(0, buf));
       }
-      arrive(dwo_full(0, buf));
     }
-  } else if (kv_count > 0) {
-    // ---------------------------------------------------------------- states
-    using ST = AsKv;
-    const int sw = warp - AS_DW_WARPS, mh = sw >> 2, rg = sw & 3;  // key channels 16 mh .. + 15 of the block (d = 16: head mh of the pair), image rows 4 rg .. + 3
-    const uint32_t dwo = box + 2 * ST::BUF;
-    AsUnit un = as_locate(p, u_first, p.kv_tiles_x, p.kv_tiles), nxt = un;  // nxt: the tile requested next (first warp only)
-    if (sw == 0) {
-      request_kv(nxt, 0);
-      if (kv_count > 1) request_kv(nxt, 1);
-    }
-    const uint32_t ONES = F16 ? 0x3C003C00u : 0x3F803F80u;
-    const uint32_t ones0 = (g & 1) ? 0u : ONES, ones1 = (g & 1) ? ONES : 0u;  // even columns count scale 0, odd ones the aggregated scale
-    float acc0[NJ][4], acc1[NJ][4], accs[4];
-    auto clear = [&] {
+    if (end_of_kv()) {
+      // ---------------------------------------------------------------- depthwise
+      using ST = AsQ;
+      const int c0 = 2 * warp;
+      const uint32_t dwo = box + ST::BUFS * ST::BUF + (uint32_t)(c0 * AS_DWO_CH + lane * 4);
+      uint32_t main_off[3], edge_off[3];  // octets 1, 2 of staged rows 2g + r (r = 2k + lane bit 3), and the neighbours' pixel pairs
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        accs[e] = 0.f;
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) acc0[j][e] = acc1[j][e] = 0.f;
+      for (int k = 0; k < 3; ++k) {
+        main_off[k] = box + at(ST{}, 0, 2 * (lane & 7) + 2 * k + ((lane >> 3) & 1), 1 + (lane >> 4), c0);
+        edge_off[k] = box + at(ST{}, 0, 2 * g + 2 * k, t >= 2 ? 0 : 3, c0) + (t >= 2 ? 12 : 0);
       }
-    };
-    clear();
-    uint32_t wk[D / 16][4];  // A fragments of the keys' grouped 1x1, rows 16 mh .. + 15
-    int cur_p = -1;
-    // depthwise tile: row 2g' + half of column block nb is octet (2nb + half) * 8 + g'; this warp's rows are g' = 2 rg, 2 rg + 1
-    const uint32_t k1_off = dwo + (uint32_t)((D16 ? 16 * mh + (lane & 15) : lane) * AS_DWO_CH + rg * 32);
-    const uint32_t v1_off = dwo + AS_DWO_SIDE + (uint32_t)(((D16 ? 16 * mh : 0) + 8 * (lane >> 4) + (lane & 7)) * AS_DWO_CH + ((lane >> 3) & 1) * 256 + rg * 32);
-    // staged row of image row 4 rg (+ PAR: 4 rg + 1; + 128 and another swizzle phase: 4 rg + 2), octets 1 and 2; keys: channels
-    // 16 mh + .., values: from channel 0 (d = 16: 16 mh) on
-    uint32_t k0_off[2], v0_off[2];
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      k0_off[e] = box + at(ST{}, 0, 4 * rg + 2 * e + 2, 1 + (lane >> 4), 16 * mh + (lane & 15));
-      v0_off[e] = box + at(ST{}, 1, 4 * rg + 2 * e + 2, 1 + ((lane >> 3) & 1), (D16 ? 16 * mh : 0) + 8 * (lane >> 4) + (lane & 7));
-    }
-    // two channel groups further on: 60 rows of 128 bytes, i.e. the swizzle phase changes by 4
-    static_assert(2 * ST::OCT * ST::ROWS2 % 8 == 4, "phase of the second pair of channel groups");
-    constexpr uint32_t V0_STEP = 2 * ST::OCT * ST::ROWS2 * 128;
+      // Toeplitz B fragments: [0] the octet itself, tap k - n + 2; [1] the mixed octet: left neighbour's pixel 6 (= -2) in lane t = 3,
+      // right neighbour's pixel 0 (= 8) in lane t = 0
+      uint32_t b0[2][5], b1[2][5];
+      int change = 0;
 #pragma unroll 1
-    for (int i = 0; i < kv_count; ++i) {
-      const uint32_t buf = i & 1, ph = (i >> 1) & 1;
-      if (un.p != cur_p) {
-        cur_p = un.p;
-        const uint32_t* wp = reinterpret_cast<const uint32_t*>(p.w_pw + ((long long)plane_of(1, cur_p, D16 ? mh : 0) * D + (D16 ? 0 : 16 * mh)) * D);
-#pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-          const uint32_t* a = wp + (g * D + 16 * ks) / 2 + t;
-          wk[ks][0] = __ldg(a); wk[ks][1] = __ldg(a + 4 * D); wk[ks][2] = __ldg(a + 4); wk[ks][3] = __ldg(a + 4 * D + 4);
+      for (int i = 0; i < q_count; ++i) {
+        const uint32_t buf = i & 1, ph = (i >> 1) & 1;
+        if (i == change) {
+          const long long per_block = (long long)p.q_tiles * p.B;
+          const int pr = (int)((q_first + i) / per_block);
+          change = (int)min((pr + 1) * per_block - q_first, (long long)q_count);
+          as_load_taps<2>(p.w_dw, plane_of(0, pr, D16 ? c0 >> 4 : 0) * D + (c0 & (D - 1)), 2 * t - g + 2, b0);
+          as_load_taps<2>(p.w_dw, plane_of(0, pr, D16 ? c0 >> 4 : 0) * D + (c0 & (D - 1)), t == 3 ? -g : t == 0 ? 10 - g : -8, b1);
         }
-      }
-      const int y = un.ty * AS_TH + 4 * rg, x0 = un.tx * AS_TW - 2;
-      const bool edge_y = un.ty * AS_TH < p.row_lo || un.ty * AS_TH + AS_TH > p.row_hi;
-      const bool edge = edge_y || x0 < 0 || x0 + AS_TW > p.W;
-      // ---- un-aggregated scale: octets 2 tx, 2 tx + 1 of the staged rows
-      if (!wait(full(0, buf), ph)) break;
-      if (p.with_scale0) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const uint32_t ro = buf * ST::BUF + (r & 1) * ST::PAR;
-          uint32_t a[4];
-          as_ldsm4(a[0], a[1], a[2], a[3], k0_off[r >> 1] + ro);
-#pragma unroll
-          for (int e = 0; e < 4; ++e) a[e] = as_relu<F16>(a[e]);
-          if (edge_y) {
-            const bool in = y + r >= p.row_lo && y + r < p.row_hi;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) a[e] = in ? a[e] : 0u;
-          }
-          as_mma<F16>(accs, a[0], a[1], a[2], a[3], ones0, ones0);
-#pragma unroll
-          for (int j = 0; j < NJ; j += 2) {
-            uint32_t v[4];
-            as_ldsm4(v[0], v[1], v[2], v[3], j == 0 ? v0_off[r >> 1] + ro : (v0_off[r >> 1] + ro + V0_STEP) ^ 64u);
-            as_mma<F16>(acc0[j], a[0], a[1], a[2], a[3], v[0], v[1]);
-            as_mma<F16>(acc0[j + 1], a[0], a[1], a[2], a[3], v[2], v[3]);
-          }
-        }
-      }
-      arrive(freed(0, buf));
-      if (sw == 0 && i + 2 < kv_count) {  // once the others are through with the staged tile too (the depthwise warps are ahead)
-        if (!wait(freed(0, buf), ph)) break;
-        request_kv(nxt, buf);
-      }
-      // ---- aggregated scale
-      if (!wait(dwo_full(0, buf), ph)) break;
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const uint32_t ro = buf * ST::DWO + (r >> 1) * 16 + (r & 1) * 128;
-        uint32_t a[4];
-#pragma unroll
-        for (int nb = 0; nb < 2; ++nb) {
-          float c[4];
-          if constexpr (D16) {
-            uint32_t b0, b1;
-            as_ldsm2t(b0, b1, k1_off + ro + nb * 256);
-            as_mma_first<F16>(c, wk[0][0], wk[0][1], wk[0][2], wk[0][3], b0, b1);
-          } else {
-            uint32_t b[4];
-            as_ldsm4t(b, k1_off + ro + nb * 256);
-            as_mma_first<F16>(c, wk[0][0], wk[0][1], wk[0][2], wk[0][3], b[0], b[1]);
-            as_mma<F16>(c, wk[D / 16 - 1][0], wk[D / 16 - 1][1], wk[D / 16 - 1][2], wk[D / 16 - 1][3], b[2], b[3]);
-          }
-          a[2 * nb] = as_pack_relu<F16>(c[0], c[1]);
-          a[2 * nb + 1] = as_pack_relu<F16>(c[2], c[3]);
-          if (edge) {  // outputs that do not exist or do not count
-            const int x = x0 + 8 * nb + 2 * t;
-            const bool in = y + r >= p.row_lo && y + r < p.row_hi;
-            const uint32_t m = in ? (x >= 0 && x < p.W ? 0xFFFFu : 0u) | (x + 1 >= 0 && x + 1 < p.W ? 0xFFFF0000u : 0u) : 0u;
-            a[2 * nb] &= m; a[2 * nb + 1] &= m;
-          }
-        }
-        as_mma<F16>(accs, a[0], a[1], a[2], a[3], ones1, ones1);
-#pragma unroll
-        for (int j = 0; j < NJ; j += 2) {
-          uint32_t v[4];
-          as_ldsm4(v[0], v[1], v[2], v[3], v1_off + ro + (uint32_t)(j * 8 * AS_DWO_CH));
-          as_mma<F16>(acc1[j], a[0], a[1], a[2], a[3], v[0], v[1]);
-          as_mma<F16>(acc1[j + 1], a[0], a[1], a[2], a[3], v[2], v[3]);
-        }
-      }
-      arrive(dwo_freed(0, buf));
-
-      const int pb = un.p * p.B + un.b;
-      as_advance(p, un, p.kv_tiles_x);
-      if (i + 1 < kv_count && un.p * p.B + un.b == pb) continue;
-      // The run leaves this (head, image): add the warps' sums in warp order and write them to this CTA's slot.
-      float* red = reinterpret_cast<float*>(smem_raw + (dwo + 2 * ST::DWO - smem_u32(smem_raw)));  // [state][warp][16][D + 1]
-      float* mine = red + sw * 16 * (D + 1);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int r = g + 8 * (e >> 1);
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) {
-          mine[r * (D + 1) + 8 * j + 2 * t + (e & 1)] = acc0[j][e];
-          mine[AS_SUM_WARPS * 16 * (D + 1) + r * (D + 1) + 8 * j + 2 * t + (e & 1)] = acc1[j][e];
-        }
-        if (t == 0) mine[(e & 1) * AS_SUM_WARPS * 16 * (D + 1) + r * (D + 1) + D] = accs[e];
-      }
-      clear();
-      asm volatile("bar.sync 1, %0;" ::"n"(32 * AS_SUM_WARPS) : "memory");
-      // [state][mh][r][c] of the block: d = 32: rows 16 mh + r of one head's states; d = 16: rows r of head mh's
-      float* out = p.partial + ((long long)pb + blockIdx.x) * (HPB * 2 * NE);
-      for (int e = threadIdx.x - 32 * AS_DW_WARPS; e < HPB * 2 * NE; e += 32 * AS_SUM_WARPS) {
-        const int s = D16 ? (e / NE) & 1 : e / NE, r = e - (e / NE) * NE;
-        const int half = D16 ? e / (2 * NE) : r / (16 * (D + 1)), rr = D16 ? r : r - half * 16 * (D + 1);
-        const float* src = red + (s * AS_SUM_WARPS + half * 4) * 16 * (D + 1) + rr;
-        float sum = src[0];
-#pragma unroll
-        for (int w = 1; w < 4; ++w) sum += src[w * 16 * (D + 1)];
-        out[e] = sum;
-      }
-      asm volatile("bar.sync 1, %0;" ::"n"(32 * AS_SUM_WARPS) : "memory");
-    }
-  }
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  ok = __syncthreads_and(ok);  // every warp is out of the loop: the queries' tiles take over the shared memory
-
-  // ------------------------------------------------------------------ queries
-  if (!ok || q_count <= 0) {
-  } else if (warp < AS_DW_WARPS) {
-    // ---------------------------------------------------------------- depthwise
-    using ST = AsQ;
-    const int c0 = 2 * warp;
-    const uint32_t dwo = box + ST::BUFS * ST::BUF + (uint32_t)(c0 * AS_DWO_CH + lane * 4);
-    uint32_t main_off[3], edge_off[3];  // octets 1, 2 of staged rows 2g + r (r = 2k + lane bit 3), and the neighbours' pixel pairs
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      main_off[k] = box + at(ST{}, 0, 2 * (lane & 7) + 2 * k + ((lane >> 3) & 1), 1 + (lane >> 4), c0);
-      edge_off[k] = box + at(ST{}, 0, 2 * g + 2 * k, t >= 2 ? 0 : 3, c0) + (t >= 2 ? 12 : 0);
-    }
-    // Toeplitz B fragments: [0] the octet itself, tap k - n + 2; [1] the mixed octet: left neighbour's pixel 6 (= -2) in lane t = 3,
-    // right neighbour's pixel 0 (= 8) in lane t = 0
-    uint32_t bt[2][5][2];
-    int change = 0;
-#pragma unroll 1
-    for (int i = 0; i < q_count; ++i) {
-      const uint32_t buf = i & 1, ph = (i >> 1) & 1;
-      if (i == change) {
-        const long long per_block = (long long)p.q_tiles * p.B;
-        const int pr = (int)((q_first + i) / per_block);
-        change = (int)min((pr + 1) * per_block - q_first, (long long)q_count);
-        as_load_taps<2>(p.w_dw, plane_of(0, pr, D16 ? c0 >> 4 : 0) * D + (c0 & (D - 1)), 2 * t - g + 2, t == 3 ? -g : t == 0 ? 10 - g : -8, bt);
-      }
-      const uint32_t sbuf = i % ST::BUFS;
-      if (!wait(full(1, sbuf), (i / ST::BUFS) & 1)) break;
-      if (!wait(dwo_freed(1, buf), ph ^ 1)) break;
-      const uint32_t ro = sbuf * ST::BUF, dw = dwo + buf * ST::DWO;
-#pragma unroll
-      for (int cc = 0; cc < 2; ++cc) {
+        const uint32_t sbuf = i % ST::BUFS;
+        if (!wait(full(1, sbuf), (i / ST::BUFS) & 1)) break;
+        if (!wait(dwo_freed(1, buf), ph ^ 1)) break;
+        const uint32_t ro = sbuf * ST::BUF, dw = dwo + buf * ST::DWO;
         uint32_t R[6][2], E[6];
+        auto load = [&](int cc) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) as_ldsm4(R[2 * k][0], R[2 * k + 1][0], R[2 * k][1], R[2 * k + 1][1], (main_off[k] + ro) ^ (uint32_t)(cc << 4));
+          for (int k = 0; k < 3; ++k) as_ldsm4(R[2 * k][0], R[2 * k + 1][0], R[2 * k][1], R[2 * k + 1][1], (main_off[k] + ro) ^ (uint32_t)(cc << 4));
 #pragma unroll
-        for (int r = 0; r < 6; ++r) E[r] = as_lds32(((edge_off[r >> 1] + ro) ^ (uint32_t)(cc << 4)) + (r & 1) * ST::PAR);
-        if (cc == 1) arrive(freed(1, sbuf));
-        float acc[2][4];
+          for (int r = 0; r < 6; ++r) E[r] = as_lds32(((edge_off[r >> 1] + ro) ^ (uint32_t)(cc << 4)) + (r & 1) * ST::PAR);
+        };
+        load(0);
 #pragma unroll
-        for (int nb = 0; nb < 2; ++nb) {
-          uint32_t X[6];  // the mixed octet: left neighbour in lanes t >= 2, right neighbour in lanes t < 2
+        for (int cc = 0; cc < 2; ++cc) {
+          float acc[2][4];
 #pragma unroll
-          for (int r = 0; r < 6; ++r) X[r] = nb == 0 ? (t >= 2 ? E[r] : R[r][1]) : (t >= 2 ? R[r][0] : E[r]);
-          as_mma_first<F16>(acc[nb], R[0][nb], R[1][nb], X[0], X[1], bt[cc][0][0], bt[cc][0][1]);
+          for (int nb = 0; nb < 2; ++nb) {
+            uint32_t X[6];  // the mixed octet: left neighbour in lanes t >= 2, right neighbour in lanes t < 2
 #pragma unroll
-          for (int dy = 1; dy < 5; ++dy) as_mma<F16>(acc[nb], R[dy][nb], R[dy + 1][nb], X[dy], X[dy + 1], bt[cc][dy][0], bt[cc][dy][1]);
+            for (int r = 0; r < 6; ++r) X[r] = nb == 0 ? (t >= 2 ? E[r] : R[r][1]) : (t >= 2 ? R[r][0] : E[r]);
+            as_mma_first<F16>(acc[nb], R[0][nb], R[1][nb], X[0], X[1], b0[cc][0], b1[cc][0]);
+#pragma unroll
+            for (int dy = 1; dy < 5; ++dy) as_mma<F16>(acc[nb], R[dy][nb], R[dy + 1][nb], X[dy], X[dy + 1], b0[cc][dy], b1[cc][dy]);
+          }
+          if (cc == 0) {  // ahead of the stores below, which wait for the products
+            load(1);
+            arrive(freed(1, sbuf));
+          }
+          as_put_depthwise<F16>(dw + cc * AS_DWO_CH, acc);
         }
-        as_put_depthwise<F16>(dw + cc * AS_DWO_CH, acc);
+        arrive(dwo_full(1, buf));
       }
-      arrive(dwo_full(1, buf));
+    }
+  } else if (warp >= AS_LOAD_WARP) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(AS_COPY_REGS));
+    // ---------------------------------------------------------------- copies
+    if (warp == AS_LOAD_WARP && kv_count > 0) {
+      AsUnit nxt = as_locate(p, u_first, p.kv_tiles_x, p.kv_tiles);
+#pragma unroll 1
+      for (int i = 0; i < kv_count; ++i) {
+        if (i >= 2 && !wait(freed(0, i & 1), ((i - 2) >> 1) & 1)) break;
+        request_kv(nxt, i & 1);
+      }
+    }
+    const bool more = end_of_kv();
+    if (more && warp == AS_LOAD_WARP) {
+      // ---------------------------------------------------------------- copies: staged tiles
+      AsUnit nxt = as_locate(p, q_first, p.q_tiles_x, p.q_tiles);
+#pragma unroll 1
+      for (int i = 0; i < q_count; ++i) {
+        if (i >= AsQ::BUFS && !wait(freed(1, i % AsQ::BUFS), (i / AsQ::BUFS - 1) & 1)) break;
+        request_q(nxt, i % AsQ::BUFS);
+      }
+    } else if (more && warp == AS_STORE_WARP) {
+      // ---------------------------------------------------------------- copies: output tiles (rows and octets outside the image are clipped)
+      const uint32_t stage0 = box + AsQ::BUFS * AsQ::BUF + 2 * AsQ::DWO;
+      AsUnit un = as_locate(p, q_first, p.q_tiles_x, p.q_tiles);
+#pragma unroll 1
+      for (int i = 0; i < q_count; ++i, as_advance(p, un, p.q_tiles_x)) {
+        const uint32_t buf = i & 1;
+        if (!wait(staged(buf), (i >> 1) & 1)) break;
+        if (lane == 0) {
+#pragma unroll
+          for (int sub = 0; sub < HPB; ++sub) {
+            const int h = HPB * un.p + sub;
+            if (h < p.heads) as_tma_store(&q_out, stage0 + buf * AS_STAGE + sub * (AS_STAGE / HPB), un.tx * (D / 4), un.ty * AS_TH, un.b * p.heads + h);
+          }
+          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+          asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+          mbar_arrive(staging_freed(buf));
+        }
+      }
+      if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");  // stores done before the CTA retires
     }
   } else {
-    // ---------------------------------------------------------------- grouped 1x1 of image rows 2 sw, 2 sw + 1 of the tile
-    using ST = AsQ;
-    const int sw = warp - AS_DW_WARPS;
-    const uint32_t q_off = box + ST::BUFS * ST::BUF + (uint32_t)(lane * AS_DWO_CH + sw * 16);
-    const uint32_t stage0 = box + ST::BUFS * ST::BUF + 2 * ST::DWO + (uint32_t)(sw * AS_STAGE_WARP);
-    uint32_t wq[2][D / 16][4];  // A fragments of the queries' grouped 1x1: 16-row block m, contraction step ks (d = 16: only ks = m exists)
-    int cur_p = -1;
-    AsUnit un = as_locate(p, q_first, p.q_tiles_x, p.q_tiles), nxt = un;
-    if (sw == 0) {
-      for (int i = 0; i < min(q_count, ST::BUFS); ++i) request_q(nxt, i);
-    }
-#pragma unroll 1
-    for (int i = 0; i < q_count; ++i, as_advance(p, un, p.q_tiles_x)) {
-      const uint32_t buf = i & 1, ph = (i >> 1) & 1;
-      if (sw == 0 && i > 0 && i - 1 + ST::BUFS < q_count) {  // the depthwise warps are through with the staged tile before this one
-        const uint32_t sbuf = (i - 1) % ST::BUFS;
-        if (!wait(freed(1, sbuf), ((i - 1) / ST::BUFS) & 1)) break;
-        request_q(nxt, sbuf);
-      }
-      if (un.p != cur_p) {
-        cur_p = un.p;
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(AS_SUM_REGS));
+    if (kv_count > 0) {
+      // ---------------------------------------------------------------- states
+      using ST = AsKv;
+      const int sw = warp - AS_DW_WARPS, mh = sw >> 2, rg = sw & 3;  // key channels 16 mh .. + 15 of the block (d = 16: head mh of the pair), image rows 4 rg .. + 3
+      const uint32_t dwo = box + 2 * ST::BUF;
+      AsUnit un = as_locate(p, u_first, p.kv_tiles_x, p.kv_tiles);
+      const uint32_t ONES = F16 ? 0x3C003C00u : 0x3F803F80u;
+      const uint32_t ones0 = (g & 1) ? 0u : ONES, ones1 = (g & 1) ? ONES : 0u;  // even columns count scale 0, odd ones the aggregated scale
+      float acc0[NJ][4], acc1[NJ][4], accs[4];
+      auto clear = [&] {
 #pragma unroll
-        for (int m = 0; m < 2; ++m) {
-          const uint32_t* wp = reinterpret_cast<const uint32_t*>(p.w_pw + ((long long)plane_of(0, cur_p, D16 ? m : 0) * D + (D16 ? 0 : 16 * m)) * D);
+        for (int e = 0; e < 4; ++e) {
+          accs[e] = 0.f;
+#pragma unroll
+          for (int j = 0; j < NJ; ++j) acc0[j][e] = acc1[j][e] = 0.f;
+        }
+      };
+      clear();
+      uint32_t wk[D / 16][4];  // A fragments of the keys' grouped 1x1, rows 16 mh .. + 15
+      int cur_p = -1;
+      // depthwise tile: row 2g' + half of column block nb is octet (2nb + half) * 8 + g'; this warp's rows are g' = 2 rg, 2 rg + 1
+      const uint32_t k1_off = dwo + (uint32_t)((D16 ? 16 * mh + (lane & 15) : lane) * AS_DWO_CH + rg * 32);
+      const uint32_t v1_off = dwo + AS_DWO_SIDE + (uint32_t)(((D16 ? 16 * mh : 0) + 8 * (lane >> 4) + (lane & 7)) * AS_DWO_CH + ((lane >> 3) & 1) * 256 + rg * 32);
+      // staged row of image row 4 rg (+ PAR: 4 rg + 1; + 128 and another swizzle phase: 4 rg + 2), octets 1 and 2; keys: channels
+      // 16 mh + .., values: from channel 0 (d = 16: 16 mh) on
+      uint32_t k0_off[2], v0_off[2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        k0_off[e] = box + at(ST{}, 0, 4 * rg + 2 * e + 2, 1 + (lane >> 4), 16 * mh + (lane & 15));
+        v0_off[e] = box + at(ST{}, 1, 4 * rg + 2 * e + 2, 1 + ((lane >> 3) & 1), (D16 ? 16 * mh : 0) + 8 * (lane >> 4) + (lane & 7));
+      }
+      // two channel groups further on: 60 rows of 128 bytes, i.e. the swizzle phase changes by 4
+      static_assert(2 * ST::OCT * ST::ROWS2 % 8 == 4, "phase of the second pair of channel groups");
+      constexpr uint32_t V0_STEP = 2 * ST::OCT * ST::ROWS2 * 128;
+#pragma unroll 1
+      for (int i = 0; i < kv_count; ++i) {
+        const uint32_t buf = i & 1, ph = (i >> 1) & 1;
+        if (un.p != cur_p) {
+          cur_p = un.p;
+          const uint32_t* wp = reinterpret_cast<const uint32_t*>(p.w_pw + ((long long)plane_of(1, cur_p, D16 ? mh : 0) * D + (D16 ? 0 : 16 * mh)) * D);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks) {
             const uint32_t* a = wp + (g * D + 16 * ks) / 2 + t;
-            wq[m][ks][0] = __ldg(a); wq[m][ks][1] = __ldg(a + 4 * D); wq[m][ks][2] = __ldg(a + 4); wq[m][ks][3] = __ldg(a + 4 * D + 4);
+            wk[ks][0] = __ldg(a); wk[ks][1] = __ldg(a + 4 * D); wk[ks][2] = __ldg(a + 4); wk[ks][3] = __ldg(a + 4 * D + 4);
           }
         }
-      }
-      if (lane < 2 * HPB) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");  // the copies of the tile before last have read the staging
-      if (!wait(dwo_full(1, buf), ph)) break;
-      const uint32_t my_stage = stage0 + buf * AS_STAGE;
+        const int y = un.ty * AS_TH + 4 * rg, x0 = un.tx * AS_TW - 2;
+        const bool edge_y = un.ty * AS_TH < p.row_lo || un.ty * AS_TH + AS_TH > p.row_hi;
+        const bool edge = edge_y || x0 < 0 || x0 + AS_TW > p.W;
+        // ---- un-aggregated scale: octets 2 tx, 2 tx + 1 of the staged rows
+        if (!wait(full(0, buf), ph)) break;
+        if (p.with_scale0) {
+          uint32_t k[4], v[NJ / 2][4];  // one image row's operands, fetched while the row before is multiplied
+          auto load = [&](int r) {
+            const uint32_t ro = buf * ST::BUF + (r & 1) * ST::PAR;
+            as_ldsm4(k[0], k[1], k[2], k[3], k0_off[r >> 1] + ro);
 #pragma unroll
-      for (int half = 0; half < 2; ++half)
+            for (int j = 0; j < NJ / 2; ++j) as_ldsm4(v[j][0], v[j][1], v[j][2], v[j][3], j == 0 ? v0_off[r >> 1] + ro : (v0_off[r >> 1] + ro + V0_STEP) ^ 64u);
+          };
+          load(0);
 #pragma unroll
-        for (int nb = 0; nb < 2; ++nb) {
-          uint32_t b[4];
-          as_ldsm4t(b, q_off + buf * ST::DWO + (uint32_t)((2 * nb + half) * 128));
+          for (int r = 0; r < 4; ++r) {
+            uint32_t a[4];
 #pragma unroll
-          for (int m = 0; m < 2; ++m) {
-            float c[4];
-            if constexpr (D16) {
-              as_mma_first<F16>(c, wq[m][0][0], wq[m][0][1], wq[m][0][2], wq[m][0][3], b[2 * m], b[2 * m + 1]);
-            } else {
-              as_mma_first<F16>(c, wq[m][0][0], wq[m][0][1], wq[m][0][2], wq[m][0][3], b[0], b[1]);
-              as_mma<F16>(c, wq[m][D / 16 - 1][0], wq[m][D / 16 - 1][1], wq[m][D / 16 - 1][2], wq[m][D / 16 - 1][3], b[2], b[3]);
+            for (int e = 0; e < 4; ++e) a[e] = as_relu<F16>(k[e]);
+            if (edge_y) {
+              const bool in = y + r >= p.row_lo && y + r < p.row_hi;
+#pragma unroll
+              for (int e = 0; e < 4; ++e) a[e] = in ? a[e] : 0u;
             }
-            // staging: [row][octet][32 channels][8 pixels] (d = 16: [head][row][octet][16 channels][8 pixels])
-            const uint32_t o = my_stage + (uint32_t)((D16 ? m * 1024 + half * 512 + nb * 256 : half * 1024 + nb * 512 + m * 256) + g * 16 + t * 4);
-            as_sts32(o, as_pack<F16>(c[0], c[1]));
-            as_sts32(o + 128, as_pack<F16>(c[2], c[3]));
+            as_mma<F16>(accs, a[0], a[1], a[2], a[3], ones0, ones0);
+#pragma unroll
+            for (int j = 0; j < NJ / 2; ++j) {
+              as_mma<F16>(acc0[2 * j], a[0], a[1], a[2], a[3], v[j][0], v[j][1]);
+              as_mma<F16>(acc0[2 * j + 1], a[0], a[1], a[2], a[3], v[j][2], v[j][3]);
+            }
+            if (r < 3) load(r + 1);
           }
         }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      arrive(dwo_freed(1, buf));
-      if (lane < 2 * HPB) {  // lane: row of the pair (and head of the block)
-        const int half = lane & 1, sub = lane >> 1, h = HPB * un.p + sub;
-        const int y = un.ty * AS_TH + 2 * sw + half;
-        if (h < p.heads && y < p.H)
-          as_bulk_store(p.q1 + ((((long long)un.b * p.heads + h) * p.H + y) * p.Wb + 2 * un.tx) * BLK, my_stage + (uint32_t)(sub * 1024 + half * 2 * BLK),
-                        (uint32_t)(min(2, p.Wb - 2 * un.tx) * BLK));
-        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        arrive(freed(0, buf));
+        // ---- aggregated scale
+        if (!wait(dwo_full(0, buf), ph)) break;
+        uint32_t kb[2][4];  // one image row of keys, both column blocks, fetched a row ahead
+        auto load_keys = [&](int r) {
+          const uint32_t ro = buf * ST::DWO + (r >> 1) * 16 + (r & 1) * 128;
+#pragma unroll
+          for (int nb = 0; nb < 2; ++nb) {
+            if constexpr (D16) as_ldsm2t(kb[nb][0], kb[nb][1], k1_off + ro + nb * 256);
+            else as_ldsm4t(kb[nb], k1_off + ro + nb * 256);
+          }
+        };
+        load_keys(0);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const uint32_t ro = buf * ST::DWO + (r >> 1) * 16 + (r & 1) * 128;
+          uint32_t v[NJ / 2][4];
+#pragma unroll
+          for (int j = 0; j < NJ / 2; ++j) as_ldsm4(v[j][0], v[j][1], v[j][2], v[j][3], v1_off + ro + (uint32_t)(j * 16 * AS_DWO_CH));
+          float c[2][4];
+#pragma unroll
+          for (int nb = 0; nb < 2; ++nb) as_mma_first<F16>(c[nb], wk[0][0], wk[0][1], wk[0][2], wk[0][3], kb[nb][0], kb[nb][1]);
+          if constexpr (!D16) {
+#pragma unroll
+            for (int nb = 0; nb < 2; ++nb)
+              as_mma<F16>(c[nb], wk[D / 16 - 1][0], wk[D / 16 - 1][1], wk[D / 16 - 1][2], wk[D / 16 - 1][3], kb[nb][2], kb[nb][3]);
+          }
+          if (r < 3) load_keys(r + 1);
+          uint32_t a[4];
+#pragma unroll
+          for (int nb = 0; nb < 2; ++nb) {
+            a[2 * nb] = as_pack_relu<F16>(c[nb][0], c[nb][1]);
+            a[2 * nb + 1] = as_pack_relu<F16>(c[nb][2], c[nb][3]);
+            if (edge) {  // outputs that do not exist or do not count
+              const int x = x0 + 8 * nb + 2 * t;
+              const bool in = y + r >= p.row_lo && y + r < p.row_hi;
+              const uint32_t m = in ? (x >= 0 && x < p.W ? 0xFFFFu : 0u) | (x + 1 >= 0 && x + 1 < p.W ? 0xFFFF0000u : 0u) : 0u;
+              a[2 * nb] &= m; a[2 * nb + 1] &= m;
+            }
+          }
+          as_mma<F16>(accs, a[0], a[1], a[2], a[3], ones1, ones1);
+#pragma unroll
+          for (int j = 0; j < NJ / 2; ++j) {
+            as_mma<F16>(acc1[2 * j], a[0], a[1], a[2], a[3], v[j][0], v[j][1]);
+            as_mma<F16>(acc1[2 * j + 1], a[0], a[1], a[2], a[3], v[j][2], v[j][3]);
+          }
+        }
+        arrive(dwo_freed(0, buf));
+
+        const int pb = un.p * p.B + un.b;
+        as_advance(p, un, p.kv_tiles_x);
+        if (i + 1 < kv_count && un.p * p.B + un.b == pb) continue;
+        // The run leaves this (head, image): add the warps' sums in warp order and write them to this CTA's slot.
+        float* red = reinterpret_cast<float*>(smem_raw + (dwo + 2 * ST::DWO - smem_u32(smem_raw)));  // [state][warp][16][D + 1]
+        float* mine = red + sw * 16 * (D + 1);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int r = g + 8 * (e >> 1);
+#pragma unroll
+          for (int j = 0; j < NJ; ++j) {
+            mine[r * (D + 1) + 8 * j + 2 * t + (e & 1)] = acc0[j][e];
+            mine[AS_SUM_WARPS * 16 * (D + 1) + r * (D + 1) + 8 * j + 2 * t + (e & 1)] = acc1[j][e];
+          }
+          if (t == 0) mine[(e & 1) * AS_SUM_WARPS * 16 * (D + 1) + r * (D + 1) + D] = accs[e];
+        }
+        clear();
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * AS_SUM_WARPS) : "memory");
+        // [state][mh][r][c] of the block: d = 32: rows 16 mh + r of one head's states; d = 16: rows r of head mh's
+        float* out = p.partial + ((long long)pb + blockIdx.x) * (HPB * 2 * NE);
+        for (int e = threadIdx.x - 32 * AS_DW_WARPS; e < HPB * 2 * NE; e += 32 * AS_SUM_WARPS) {
+          const int s = D16 ? (e / NE) & 1 : e / NE, r = e - (e / NE) * NE;
+          const int half = D16 ? e / (2 * NE) : r / (16 * (D + 1)), rr = D16 ? r : r - half * 16 * (D + 1);
+          const float* src = red + (s * AS_SUM_WARPS + half * 4) * 16 * (D + 1) + rr;
+          float sum = src[0];
+#pragma unroll
+          for (int w = 1; w < 4; ++w) sum += src[w * 16 * (D + 1)];
+          out[e] = sum;
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * AS_SUM_WARPS) : "memory");
       }
     }
-    if (lane < 2 * HPB) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");  // stores done before the CTA retires
+    if (end_of_kv()) {
+      // ---------------------------------------------------------------- grouped 1x1 of image rows 2 sw, 2 sw + 1 of the tile
+      using ST = AsQ;
+      const int sw = warp - AS_DW_WARPS;
+      const uint32_t q_off = box + ST::BUFS * ST::BUF + (uint32_t)(lane * AS_DWO_CH + sw * 16);
+      // staging: [row][octet][32 channels][8 pixels] (d = 16: [head][row][octet][16 channels][8 pixels])
+      const uint32_t stage0 = box + ST::BUFS * ST::BUF + 2 * ST::DWO + (uint32_t)(sw * 2 * (D16 ? 512 : 1024) + g * 16 + t * 4);
+      uint32_t wq[2][D / 16][4];  // A fragments of the queries' grouped 1x1: 16-row block m, contraction step ks (d = 16: only ks = m exists)
+      int cur_p = -1;
+      AsUnit un = as_locate(p, q_first, p.q_tiles_x, p.q_tiles);
+#pragma unroll 1
+      for (int i = 0; i < q_count; ++i, as_advance(p, un, p.q_tiles_x)) {
+        const uint32_t buf = i & 1, ph = (i >> 1) & 1;
+        if (un.p != cur_p) {
+          cur_p = un.p;
+#pragma unroll
+          for (int m = 0; m < 2; ++m) {
+            const uint32_t* wp = reinterpret_cast<const uint32_t*>(p.w_pw + ((long long)plane_of(0, cur_p, D16 ? m : 0) * D + (D16 ? 0 : 16 * m)) * D);
+#pragma unroll
+            for (int ks = 0; ks < D / 16; ++ks) {
+              const uint32_t* a = wp + (g * D + 16 * ks) / 2 + t;
+              wq[m][ks][0] = __ldg(a); wq[m][ks][1] = __ldg(a + 4 * D); wq[m][ks][2] = __ldg(a + 4); wq[m][ks][3] = __ldg(a + 4 * D + 4);
+            }
+          }
+        }
+        if (!wait(dwo_full(1, buf), ph)) break;
+        const uint32_t my_stage = stage0 + buf * AS_STAGE;
+        uint32_t b[4][4];  // block q = 2 nb + half: image row `half`, pixels 8 nb .. + 7
+#pragma unroll
+        for (int q = 0; q < 4; ++q) as_ldsm4t(b[q], q_off + buf * ST::DWO + (uint32_t)(q * 128));
+        float c[4][2][4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int m = 0; m < 2; ++m) {
+            if constexpr (D16) as_mma_first<F16>(c[q][m], wq[m][0][0], wq[m][0][1], wq[m][0][2], wq[m][0][3], b[q][2 * m], b[q][2 * m + 1]);
+            else as_mma_first<F16>(c[q][m], wq[m][0][0], wq[m][0][1], wq[m][0][2], wq[m][0][3], b[q][0], b[q][1]);
+          }
+        if constexpr (!D16) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+              as_mma<F16>(c[q][m], wq[m][D / 16 - 1][0], wq[m][D / 16 - 1][1], wq[m][D / 16 - 1][2], wq[m][D / 16 - 1][3], b[q][2], b[q][3]);
+        }
+        if (!wait(staging_freed(buf), ph ^ 1)) break;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int m = 0; m < 2; ++m) {
+            const int half = q & 1, nb = q >> 1;
+            const uint32_t o = my_stage + (uint32_t)(D16 ? m * (AS_STAGE / 2) + half * 512 + nb * 256 : half * 1024 + nb * 512 + m * 256);
+            as_sts32(o, as_pack<F16>(c[q][m][0], c[q][m][1]));
+            as_sts32(o + 128, as_pack<F16>(c[q][m][2], c[q][m][3]));
+          }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        arrive(dwo_freed(1, buf));
+        arrive(staged(buf));
+      }
+    }
   }
   if (!ok && lane == 0) {
     for (int k = 0; k < 64; ++k) __nanosleep(1000);  // copies still in flight land before the CTA retires
@@ -646,11 +719,11 @@ agg_state_kernel(const __grid_constant__ CUtensorMap kv_even, const __grid_const
 }
 
 template <int D, bool F16>
-msla_status_t launch_agg_state(int grid, const CUtensorMap (&m)[4], const AggStateParams& p, cudaStream_t st) {
+msla_status_t launch_agg_state(int grid, const CUtensorMap (&m)[5], const AggStateParams& p, cudaStream_t st) {
   static std::atomic<unsigned long long> attr_done{0};
   const msla_status_t s = ensure_smem_attr(attr_done, agg_state_kernel<D, F16>, AS_SMEM);
   if (s != MSLA_OK) return s;
-  launch_pdl(agg_state_kernel<D, F16>, dim3((unsigned)grid), dim3(AS_THREADS), AS_SMEM, st, m[0], m[1], m[2], m[3], p);
+  launch_pdl(agg_state_kernel<D, F16>, dim3((unsigned)grid), dim3(AS_THREADS), AS_SMEM, st, m[0], m[1], m[2], m[3], m[4], p);
   count_launches(1);
   return check_launch(F16 ? "token aggregation and states (fp16)" : "token aggregation and states (bf16)");
 }
@@ -669,9 +742,9 @@ AggStatePlan make_agg_state_plan(int B, int heads, int H, int W, int d) {
   pl.kv_units = pl.segments * pl.kv_tiles;
   const long long q_units = blocks * B * pl.q_tiles_x * pl.tiles_y, units = pl.kv_units + q_units;
   pl.grid = (int)(units < AGG_STATE_CTAS ? units : AGG_STATE_CTAS);
-  // a tile of keys and values takes about 1.8 times one of queries; counted alike where a CTA has few (each must get one)
-  pl.kv_cost = units >= 8 * pl.grid ? 9 : 1;
-  pl.q_cost = units >= 8 * pl.grid ? 5 : 1;
+  // a tile of keys and values takes about 1.85 times one of queries; counted alike where a CTA has few (each must get one)
+  pl.kv_cost = units >= 8 * pl.grid ? 37 : 1;
+  pl.q_cost = units >= 8 * pl.grid ? 20 : 1;
   pl.cost = pl.kv_cost * pl.kv_units + pl.q_cost * q_units;
   pl.slot_floats = hpb * 2 * d * (d + 1);
   pl.partial_bytes = (size_t)(pl.segments + pl.grid) * pl.slot_floats * sizeof(float);
@@ -683,7 +756,7 @@ msla_status_t run_agg_state(const void* ms0, void* q1, float* partial, const voi
   if (H < 2) return fail(MSLA_ERR_UNSUPPORTED, "aggregation on channel-blocked planes: one row");  // no odd rows to map
   if (pl.kv_tiles > 0x7fffffffLL || pl.cost / pl.grid >= 0x7fffffffLL) return fail(MSLA_ERR_UNSUPPORTED, "too many aggregation tiles");
   AggStateParams p{};
-  p.q1 = (unsigned char*)q1; p.partial = partial;
+  p.partial = partial;
   p.w_dw = (const bf16*)w_dw; p.w_pw = (const bf16*)w_pw;
   p.heads = heads; p.B = B; p.H = H; p.W = W; p.Wb = W / 8;
   p.tiles_y = pl.tiles_y; p.kv_tiles_x = pl.kv_tiles_x; p.q_tiles_x = pl.q_tiles_x;
@@ -691,7 +764,7 @@ msla_status_t run_agg_state(const void* ms0, void* q1, float* partial, const voi
   p.row_lo = row_lo; p.row_hi = row_hi; p.with_scale0 = with_scale0 ? 1 : 0;
   p.kv_units = pl.kv_units; p.cost = pl.cost; p.kv_cost = pl.kv_cost; p.q_cost = pl.q_cost;
   // [plane][8-channel group][octet][row of this parity][64 elements]
-  CUtensorMap maps[4];
+  CUtensorMap maps[5];
   const cuuint64_t row = (cuuint64_t)p.Wb * d * 16;
   for (int i = 0; i < 4; ++i) {
     const int odd = i & 1;
@@ -700,6 +773,13 @@ msla_status_t run_agg_state(const void* ms0, void* q1, float* partial, const voi
     const cuuint32_t bx[5] = {64, AS_ROWS / 2, (cuuint32_t)(i < 2 ? 3 : 4), (cuuint32_t)(d / 8), 1};
     if (!tma_make_map_bf16(&maps[i], (const char*)ms0 + odd * row, 5, dims, strides, bx, CU_TENSOR_MAP_SWIZZLE_128B))
       return fail(MSLA_ERR_CUDA, "cuTensorMapEncodeTiled failed for the aggregation");
+  }
+  {  // output of the queries: [plane][row][piece of 64 elements]
+    const cuuint64_t dims[4] = {64, (cuuint64_t)p.Wb * d / 8, (cuuint64_t)H, (cuuint64_t)B * heads};
+    const cuuint64_t strides[3] = {128, row, row * H};
+    const cuuint32_t bx[4] = {64, (cuuint32_t)d / 4, AS_TH, 1};
+    if (!tma_make_map_bf16(&maps[4], q1, 4, dims, strides, bx, CU_TENSOR_MAP_SWIZZLE_NONE))
+      return fail(MSLA_ERR_CUDA, "cuTensorMapEncodeTiled failed for the aggregation's output");
   }
   if (d == 32) return f16 ? launch_agg_state<32, true>(pl.grid, maps, p, st) : launch_agg_state<32, false>(pl.grid, maps, p, st);
   return f16 ? launch_agg_state<16, true>(pl.grid, maps, p, st) : launch_agg_state<16, false>(pl.grid, maps, p, st);

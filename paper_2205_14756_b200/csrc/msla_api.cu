@@ -289,9 +289,9 @@ struct ForwardPlan {
 // channel-blocked planes (msla_host.h) with steps 2 and 3 in one kernel.  The second moves less (the aggregated keys and values
 // are never written) and spends half the shared-memory cycles on step 2, but its kernel has one CTA per SM and a longer
 // start-up, and rows that are no whole number of pixel octets would have to be padded in copies.  Whole forward, us, old / new
-// layout: [1, 256, 512, 512] 491 / 417, [1, 128, 512, 512] d = 16 309 / 254, [16, 256, 64, 64] 147 / 142, [1, 256, 128, 256] 81 / 75,
-// [8, 128, 128, 40] 63 / 61; below the line [1, 256, 128, 128] 51 / 52, [4, 256, 64, 64] 53 / 54, [64, 256, 14, 14] 79 / 80; ragged rows
-// [12, 128, 220, 134] 369 / 396.
+// layout: [1, 256, 512, 512] 489 / 391, [1, 128, 512, 512] d = 16 298 / 228, [16, 256, 64, 64] 144 / 136, [1, 256, 128, 256] 79 / 72,
+// [8, 128, 128, 40] 60 / 56; below the line [1, 256, 128, 128] 50 / 51, [4, 256, 64, 64] 51 / 52, f16 [8, 128, 48, 80] d = 16 50 / 52,
+// [16, 256, 32, 32] 54 / 59, [64, 256, 14, 14] 79 / 80; ragged rows [12, 128, 220, 134] 369 / 396.
 static bool planes_path(const msla_desc* d) {
   return d->dtype != MSLA_F32 && d->W % 8 == 0 && d->H >= 2 && (long long)d->B * d->H * d->W * d->heads * d->d >= (5LL << 20);
 }
