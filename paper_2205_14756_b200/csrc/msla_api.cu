@@ -291,9 +291,13 @@ struct ForwardPlan {
 // start-up, and rows that are no whole number of pixel octets would have to be padded in copies.  Whole forward, us, old / new
 // layout: [1, 256, 512, 512] 489 / 391, [1, 128, 512, 512] d = 16 298 / 228, [16, 256, 64, 64] 144 / 136, [1, 256, 128, 256] 79 / 72,
 // [8, 128, 128, 40] 60 / 56; below the line [1, 256, 128, 128] 50 / 51, [4, 256, 64, 64] 51 / 52, f16 [8, 128, 48, 80] d = 16 50 / 52,
-// [16, 256, 32, 32] 54 / 59, [64, 256, 14, 14] 79 / 80; ragged rows [12, 128, 220, 134] 369 / 396.
+// [64, 256, 14, 14] 79 / 80; ragged rows [12, 128, 220, 134] 369 / 396.  Its tiles of keys and values are 16 pixels wide and begin two
+// pixels to the left of the image, so narrow images leave much of them empty: of 16 pixels half, [64, 384, 16, 16] 91 / 102; of 32 a
+// third, [64, 256, 32, 32] 151 / 154; of 24 or 48 a quarter, [64, 256, 24, 24] 123 / 122, [64, 128, 48, 48] 155 / 151; [64, 192, 40, 40] d = 16
+// 220 / 187.
 static bool planes_path(const msla_desc* d) {
-  return d->dtype != MSLA_F32 && d->W % 8 == 0 && d->H >= 2 && (long long)d->B * d->H * d->W * d->heads * d->d >= (5LL << 20);
+  return d->dtype != MSLA_F32 && d->W % 8 == 0 && d->H >= 2 && (long long)d->B * d->H * d->W * d->heads * d->d >= (5LL << 20) &&
+         3LL * d->W > 32LL * ((d->W + 17) / 16);
 }
 
 // core_B: images the split of the token reduction is planned for, where a call is a part of a batch (0: desc->B); its sums

@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 # half-empty blocks); runs of tiles that cross images and heads; 2C' > 512 (apply and projection apart); C_out != C with a bias
 @pytest.mark.parametrize("dtype,B,C,H,W,heads,d,c_out", [("bf16", 1, 32, 2, 81920, 1, 32, 32), ("bf16", 320, 32, 66, 8, 1, 32, 32), ("f16", 2, 48, 235, 232, 3, 16, 48),
                                                          ("bf16", 1, 96, 239, 248, 3, 32, 40), ("bf16", 3, 64, 112, 256, 4, 16, 264), ("f16", 40, 288, 15, 32, 9, 32, 288),
-                                                         ("f16", 21, 64, 66, 64, 2, 32, 64)])
+                                                         ("f16", 21, 64, 66, 64, 2, 32, 64), ("bf16", 52, 288, 15, 24, 9, 32, 288)])
 def test_planes_module(dtype, B, C, H, W, heads, d, c_out):
     s = inputs.ModuleShape("planes", dtype, B, C, H, W, heads, d, seed=81)
     t = inputs.module_inputs(s)
