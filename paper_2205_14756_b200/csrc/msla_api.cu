@@ -92,7 +92,10 @@ CorePlan make_core_plan(long long BH, int N, int d) {
   CorePlan p;
   p.ne = d * (d + 1);
   const long long s_max = ceil_div_ll(N, 256);
-  const long long s_want = ceil_div_ll(592, BH);
+  // d = 32: the ring of a CTA of the reduction is 64 KB, three to an SM, and no more CTAs than are resident at once (d = 16: half that).
+  // Core, us, with CTAs for 592 rounded up / 444 rounded down: [8, 16, 4096, 32] 36.5 / 34.3, [32, 8, 784, 32] 17.2 / 15.6,
+  // [1, 10, 70844, 32] 49.0 / 47.0, [20, 24, 1500, 32] 51.4 / 49.0; module [2, 384, 100, 40] 56.5 / 53.6.  296: 34.7, 15.4, 46.0, 49.3, 55.0.
+  const long long s_want = d == 32 ? 444 / BH : ceil_div_ll(592, BH);
   long long S = s_max < s_want ? s_max : s_want;
   if (S > 64) S = 64;
   if (S < 1) S = 1;
