@@ -451,21 +451,31 @@ apply_mma_kernel(const bf16* __restrict__ q, const float* __restrict__ state, in
   cp_async_wait<0>();
 }
 
+template <int D, int STAGES, bool F16>
+msla_status_t launch_kv_state(const bf16* k, const bf16* v, float* partial, HeadView in, long long BH, int heads, int N, const CorePlan& p, cudaStream_t st) {
+  constexpr int WARPS = 4, smem = WARPS * STAGES * 2 * 32 * D * 2;
+  static std::atomic<unsigned long long> attr_done{0};
+  const msla_status_t as = ensure_smem_attr(attr_done, kv_state_mma_kernel<D, WARPS, STAGES, F16>, smem);
+  if (as != MSLA_OK) return as;
+  launch_pdl(kv_state_mma_kernel<D, WARPS, STAGES, F16>, dim3((unsigned)BH, p.S), dim3(WARPS * 32), smem, st, k, v, partial, in, heads, N, p.S, p.chunk);
+  return MSLA_OK;
+}
+
 template <int D, bool F16>
 msla_status_t launch_core(const bf16* q, const bf16* k, const bf16* v, bf16* out, HeadView in, HeadView ov, int B,
                           int heads, int N, float eps, const CorePlan& p, char* ws, cudaStream_t st, cudaEvent_t mid, int phases) {
-  // 4 warps per CTA and 4-deep rings in both kernels; two 16-token MMA tiles per FIFO stage of the apply step
-  constexpr int KV_WARPS = 4, KV_STAGES = 4, AP_WARPS = 4, AP_STAGES = 4, AP_U = 2;
+  // 4 warps per CTA and (mostly) 4-deep rings in both kernels; two 16-token MMA tiles per FIFO stage of the apply step
+  constexpr int AP_WARPS = 4, AP_STAGES = 4, AP_U = 2;
   const long long BH = (long long)B * heads;
   float* partial = reinterpret_cast<float*>(ws + p.partial_off);
   float* state = reinterpret_cast<float*>(ws + p.state_off);
-  constexpr int kv_smem = KV_WARPS * KV_STAGES * 2 * 32 * D * 2;
-  static std::atomic<unsigned long long> attr_done{0};
-  const msla_status_t as = ensure_smem_attr(attr_done, kv_state_mma_kernel<D, KV_WARPS, KV_STAGES, F16>, kv_smem);
-  if (as != MSLA_OK) return as;
   int launches = 0;
   if (phases & CORE_STATE) {
-    launch_pdl(kv_state_mma_kernel<D, KV_WARPS, KV_STAGES, F16>, dim3((unsigned)BH, p.S), dim3(KV_WARPS * 32), kv_smem, st, k, v, partial, in, heads, N, p.S, p.chunk);
+    // Many heads of few tokens: no warp has more than two groups, and rings of two stages put twice the CTAs on an SM.  Module, us:
+    // [64, 256, 14, 14] (1024 CTAs) 69.6 -> 68.6, [64, 256, 16, 16] 62.1 -> 60.9, [32, 384, 7, 7] (768) 45.9 -> 45.2; core [64, 8, 196, 32] (512) 11.65 -> 11.9.
+    const bool many = p.chunk <= 256 && BH * p.S > (D == 32 ? 4 : 8) * device_sm_count();
+    const msla_status_t as = many ? launch_kv_state<D, 2, F16>(k, v, partial, in, BH, heads, N, p, st) : launch_kv_state<D, 4, F16>(k, v, partial, in, BH, heads, N, p, st);
+    if (as != MSLA_OK) return as;
     ++launches;
   }
   // A few partial states are added by every CTA of the apply step (S of 4 KB each, from L2); a kernel of its own adds them where

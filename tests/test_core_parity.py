@@ -94,3 +94,12 @@ def test_core_runtime_argument_errors():
     # the context is still usable afterwards
     binding.msla_linattn_relu(q, q, q, out, 1, 1, 8, 32)
     torch.cuda.synchronize()
+
+
+# Many heads of few tokens (short rings in the state reduction), on both sides of the longest chunk that takes them, and one wave
+# of longer ones.
+@pytest.mark.parametrize("dtype,B,heads,N,d", [("bf16", 75, 10, 196, 32), ("f16", 90, 14, 33, 16), ("bf16", 60, 10, 256, 32), ("bf16", 60, 10, 257, 32),
+                                               ("bf16", 37, 12, 300, 32)])
+def test_core_many_heads(dtype, B, heads, N, d):
+    t, ref = _case(dtype, B, heads, N, d, seed=300 + N)
+    util.assert_close(util.run_core(t, dtype), ref, dtype, f"core {dtype} {B}x{heads}x{N}x{d}", block=util.CORE_BLOCK)
