@@ -835,10 +835,11 @@ msla_status_t launch_fused_for(int d, bool res, dim3 grid, int smem, cudaStream_
 
 template <int D, bool F16, bool SLOTS>
 msla_status_t launch_fold(const FoldParams& p, cudaStream_t st) {
-  // few heads: a head's key channels are shared out, to about one CTA per SM
+  // few heads: a head's key channels are shared out, to one or two CTAs per SM (two: [8, 256, 64, 64] 84.0 -> 80.2 us a forward, f16
+  // [8, 128, 45, 80] 49.4 -> 48.6; four are slower, [16, 192, 30, 30] 46.6 -> 49.5)
   const int heads = p.B * p.Ht, sms = device_sm_count();
   if (D == 32 && 4 * heads <= sms) launch_pdl(state_fold_kernel<D, 8, F16, SLOTS>, dim3(heads, D / 8), dim3(FoldShape<D, 8>::THREADS), 0, st, p);
-  else if (2 * heads <= sms) launch_pdl(state_fold_kernel<D, D / 2, F16, SLOTS>, dim3(heads, 2), dim3(FoldShape<D, D / 2>::THREADS), 0, st, p);
+  else if (heads <= sms) launch_pdl(state_fold_kernel<D, D / 2, F16, SLOTS>, dim3(heads, 2), dim3(FoldShape<D, D / 2>::THREADS), 0, st, p);
   else launch_pdl(state_fold_kernel<D, D, F16, SLOTS>, dim3(heads), dim3(FoldShape<D, D>::THREADS), 0, st, p);
   count_launches(1);
   return check_launch("sum of the partial states");
