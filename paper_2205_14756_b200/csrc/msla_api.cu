@@ -298,14 +298,14 @@ struct ForwardPlan {
 // pixels to the left of the image, so narrow images leave much of them empty: of 16 pixels half, [64, 384, 16, 16] 91 / 102; of 32 a
 // third, [64, 256, 32, 32] 151 / 154; of 24 or 48 a quarter, [64, 256, 24, 24] 123 / 122, [64, 128, 48, 48] 155 / 151; [64, 192, 40, 40] d = 16
 // 220 / 187.
-static bool planes_path(const msla_desc* d) {
-  return d->dtype != MSLA_F32 && d->W % 8 == 0 && d->H >= 2 && (long long)d->B * d->H * d->W * d->heads * d->d >= (5LL << 20) &&
+static bool planes_path(const msla_desc* d, int B) {
+  return d->dtype != MSLA_F32 && d->W % 8 == 0 && d->H >= 2 && (long long)B * d->H * d->W * d->heads * d->d >= (5LL << 20) &&
          3LL * d->W > 32LL * ((d->W + 17) / 16);
 }
 
-// core_B: images the split of the token reduction is planned for, where a call is a part of a batch (0: desc->B); its sums
-// are then those of the whole batch, bit for bit.
-static msla_status_t validate_desc(const msla_desc* d, ForwardPlan* plan, int core_B = 0) {
+// whole_B: images of the batch that the call is a part of (0: desc->B).  It decides the layout and the split of the token
+// reduction, so that a part never needs more than the whole batch.
+static msla_status_t validate_desc(const msla_desc* d, ForwardPlan* plan, int whole_B = 0) {
   if (!d) return fail(MSLA_ERR_INVALID_ARG, "null descriptor");
   if (d->struct_size != sizeof(msla_desc)) return fail(MSLA_ERR_INVALID_ARG, "desc.struct_size = %u, expected %zu", d->struct_size, sizeof(msla_desc));
   if (!known_dtype(d->dtype)) return fail(MSLA_ERR_INVALID_ARG, "unknown dtype %d", (int)d->dtype);
@@ -321,20 +321,21 @@ static msla_status_t validate_desc(const msla_desc* d, ForwardPlan* plan, int co
   if ((long long)d->H * d->W > 0x7ffffff8LL) return fail(MSLA_ERR_UNSUPPORTED, "H*W exceeds 2^31-8");
   if (d->C % 8 != 0 || d->C_out % 8 != 0) return fail(MSLA_ERR_UNSUPPORTED, "C and C_out must be multiples of 8");
   const int S = d->n_scales;
+  if (!whole_B) whole_B = d->B;
   if ((long long)d->B * S * d->heads > 65535 || d->B > 65535) return fail(MSLA_ERR_UNSUPPORTED, "B*n_scales*heads exceeds 65535");
   plan->S = S;
   plan->Cp = d->heads * d->d;
   plan->N = d->H * d->W;
   const size_t e = elem_size(d->dtype);
   const size_t tokens = (size_t)d->B * plan->N;
-  plan->core = make_core_plan((long long)(core_B ? core_B : d->B) * S * d->heads, plan->N, d->d);
+  plan->core = make_core_plan((long long)whole_B * S * d->heads, plan->N, d->d);
   plan->ms_off = 0;
   plan->att_off = align_up(tokens * 3 * S * plan->Cp * e, 256);
   // the attention output's region doubles as scratch of the fused apply + projection kernel, which writes no attention output
   size_t att_bytes = tokens * S * plan->Cp * e;
   const size_t fused_scratch = fused_out_bf16_supported(S * d->heads, d->d, d->C_out) ? fused_out_scratch_bytes(d->B, S * d->heads, d->d, d->C_out) : 0;
   if (att_bytes < fused_scratch) att_bytes = fused_scratch;
-  plan->planes = planes_path(d);
+  plan->planes = planes_path(d, whole_B);
   plan->pitch = d->dtype == MSLA_F32 ? plan->N : (int)align_up((size_t)plan->N, 8);
   size_t core_bytes = plan->core.bytes;
   if (plan->planes) {
@@ -549,9 +550,9 @@ static msla_status_t record(void* const* events, int i, cudaStream_t st) {
 // add_x: the output projection adds x (the block's first residual connection; C_out == C).
 // out_padded: receives the address of the padded copy of out where there is one (else of out itself).
 static msla_status_t forward_impl(const msla_desc* desc, const void* x, const msla_weights* w, void* out,
-                                  cudaStream_t st, void* const* events, bool add_x = false, const void** out_padded = nullptr, int core_B = 0) {
+                                  cudaStream_t st, void* const* events, bool add_x = false, const void** out_padded = nullptr, int whole_B = 0) {
   ForwardPlan p;
-  msla_status_t s = validate_desc(desc, &p, core_B);
+  msla_status_t s = validate_desc(desc, &p, whole_B);
   if (s != MSLA_OK) return s;
   if (!x || !out || !w) return fail(MSLA_ERR_INVALID_ARG, "null x, out or weights");
   if (!w->w_qkv || !w->w_dw || !w->w_pw || !w->w_proj) return fail(MSLA_ERR_INVALID_ARG, "null weight pointer");
@@ -674,11 +675,28 @@ static msla_status_t forward_host_impl(const msla_desc* desc, const void* x, con
   ForwardPlan p;
   msla_status_t s = validate_desc(desc, &p);
   if (s != MSLA_OK) return s;
-  if (!x || !out || !w) return fail(MSLA_ERR_INVALID_ARG, "null x, out or weights");
-  if (desc->workspace && !aligned16(desc->workspace)) return fail(MSLA_ERR_ALIGNMENT, "all device pointers must be 16-byte aligned");
   const size_t e = elem_size(desc->dtype);
   const size_t xi = (size_t)desc->C * p.N * e, oi = (size_t)desc->C_out * p.N * e;  // bytes per image
   const size_t xb = desc->B * xi, ob = desc->B * oi;
+  // images per part: whole multiples of 16 bytes, so that every part of the staging buffers is aligned
+  int step = (int)((HOST_PART_BYTES + (xi < oi ? oi : xi) - 1) / (xi < oi ? oi : xi));
+  while (step < desc->B && ((step * xi) % 16 || (step * oi) % 16)) ++step;
+  auto images = [&](int left, int before) {                             // of the next part:
+    int n = before + step;                                              // one step more than the part before,
+    if (n > 4 * step) n = 4 * step;                                     // up to four steps,
+    if (n > (left + 1) / 2) n = ((left + 1) / 2 + step - 1) / step * step;  // and at most half of what is left
+    return n > left ? left : n;
+  };
+  msla_desc part = *desc;
+  part.B = 0;
+  for (int b = 0; b < desc->B; b += part.B) {  // every part fits what the whole batch reserved; known before the first copy
+    part.B = images(desc->B - b, part.B);
+    ForwardPlan pp;
+    if ((s = validate_desc(&part, &pp, desc->B)) != MSLA_OK) return s;
+    if (pp.bytes > p.bytes) return fail(MSLA_ERR_WORKSPACE, "%d of %d images need %zu bytes of scratch, the whole batch %zu", part.B, desc->B, pp.bytes, p.bytes);
+  }
+  if (!x || !out || !w) return fail(MSLA_ERR_INVALID_ARG, "null x, out or weights");
+  if (desc->workspace && !aligned16(desc->workspace)) return fail(MSLA_ERR_ALIGNMENT, "all device pointers must be 16-byte aligned");
   const size_t need = p.bytes + align_up(xb, 256) + align_up(ob, 256);
   if (!desc->workspace || desc->workspace_bytes < need)
     return fail(MSLA_ERR_WORKSPACE, "workspace of %zu bytes needed, %zu given", need, desc->workspace ? desc->workspace_bytes : (size_t)0);
@@ -687,9 +705,6 @@ static msla_status_t forward_host_impl(const msla_desc* desc, const void* x, con
   char* x_dev = (char*)desc->workspace + p.bytes;
   char* out_dev = x_dev + align_up(xb, 256);
 
-  // images per part: whole multiples of 16 bytes, so that every part of the staging buffers is aligned
-  int step = (int)((HOST_PART_BYTES + (xi < oi ? oi : xi) - 1) / (xi < oi ? oi : xi));
-  while (step < desc->B && ((step * xi) % 16 || (step * oi) % 16)) ++step;
   thread_local CopyLanes lanes;
   int dev = -1;
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
@@ -702,14 +717,9 @@ static msla_status_t forward_host_impl(const msla_desc* desc, const void* x, con
     return ce == cudaSuccess;
   };
   if (overlap && ok(cudaEventRecord(lanes.done, st))) ok(cudaStreamWaitEvent(lanes.in, lanes.done, 0));  // the staging buffers are free by then
-  msla_desc part = *desc;
   part.B = 0;
   for (int b = 0; b < desc->B && ce == cudaSuccess; b += part.B) {
-    const int left = desc->B - b;
-    int n = part.B + step;                                              // one step more than the part before,
-    if (n > 4 * step) n = 4 * step;                                     // up to four steps,
-    if (n > (left + 1) / 2) n = ((left + 1) / 2 + step - 1) / step * step;  // and at most half of what is left
-    part.B = !overlap || n > left ? left : n;
+    part.B = overlap ? images(desc->B - b, part.B) : desc->B;
     const char* xs = (const char*)x + b * xi;
     if (!ok(cudaMemcpyAsync(x_dev + b * xi, xs, part.B * xi, cudaMemcpyHostToDevice, overlap ? lanes.in : st))) break;
     if (overlap && (!ok(cudaEventRecord(lanes.arrived, lanes.in)) || !ok(cudaStreamWaitEvent(st, lanes.arrived, 0)))) break;

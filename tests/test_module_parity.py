@@ -305,6 +305,28 @@ def test_forward_host_in_parts(dtype, B, C, H, W, heads, d):
         assert torch.equal(ho[i], refs[i])
 
 
+# Host buffers whose batch lies above the size from which the channel-blocked planes are taken, with parts below it; three branches.
+@pytest.mark.parametrize("dtype,B,C,H,W,d,n_scales", [("bf16", 2, 128, 128, 256, 32, 2), ("bf16", 3, 256, 64, 112, 32, 2), ("f16", 2, 64, 256, 256, 16, 2),
+                                                      ("bf16", 5, 64, 96, 184, 32, 3)])
+def test_forward_host_above_the_planes_line(dtype, B, C, H, W, d, n_scales):
+    dt = util.TORCH_DTYPE[dtype]
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    rnd = lambda *shape: (torch.randn(*shape, generator=gen, device="cuda") * shape[-1] ** -0.5).to(dt)
+    weights = [rnd(3 * C, C), rnd(3 * C, 5, 5), rnd(3 * C, d), rnd(C, n_scales * C), None] + ([rnd(3 * C, 3, 3), rnd(3 * C, d)] if n_scales == 3 else [])
+    w = binding.make_weights(*weights)
+    make = lambda ws=None: binding.make_desc(B, C, H, W, C // d, d, C, util.CODE[dtype], n_scales=n_scales, agg_kernel2=3, workspace=ws)
+    desc = make(torch.empty(binding.msla_forward_host_workspace_bytes(make()), dtype=torch.uint8, device="cuda"))
+    x = torch.randn(B, C, H, W, generator=gen, device="cuda").to(dt)
+    ref = torch.empty_like(x)
+    binding.msla_forward(desc, x, w, ref)
+    hx, ho = x.cpu().pin_memory(), torch.empty(B, C, H, W, dtype=dt, pin_memory=True)
+    for _ in range(2):
+        binding.msla_forward_host(desc, hx, w, ho)
+    torch.cuda.synchronize()
+    util.assert_close(util.host(ho), util.host(ref), dtype, "host call")
+    assert binding.msla_debug_wait_timeouts() == 0
+
+
 # The projections' kernels take 64 to 256 output columns per tile by problem size: each width, with remainders on both sides, rows
 # of up to 512 channels in the kernel that keeps its weights and longer ones in the one that streams them.
 @pytest.mark.parametrize("dtype,B,C,Cout,N", [("bf16", 1, 64, 176, 136), ("f16", 1, 72, 384, 5112), ("bf16", 1, 128, 352, 8952), ("bf16", 5, 40, 464, 7096),

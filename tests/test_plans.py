@@ -1,0 +1,36 @@
+"""What the library reserves and how it cuts a call, checked on the host: every call here is refused for a null pointer before
+anything is launched, and the status says whether the planning before that check found anything wrong."""
+import ctypes
+import random
+
+import __graft_entry__  # noqa: F401
+from paper_2205_14756_b200 import binding
+
+FAKE = 1 << 20            # an aligned address that nothing reads
+NULL_POINTER = 1          # MSLA_ERR_INVALID_ARG; a plan that does not fit answers 4
+
+
+def _desc(dtype, B, C, H, W, d, n_scales=2, nbytes=None):
+    desc = binding.make_desc(B, C, H, W, C // d, d, C, dtype, n_scales=n_scales, agg_kernel2=3)
+    desc.workspace, desc.workspace_bytes = FAKE, nbytes or 0
+    return desc
+
+
+def test_parts_of_a_host_call_fit_the_reservation_of_the_batch():
+    """msla_forward_host runs a batch in parts; each must fit what msla_forward_host_workspace_bytes reserved for the whole."""
+    lib, rng = binding.lib(), random.Random(1)
+    shapes = [(2, 128, 128, 256, 32), (3, 256, 64, 112, 32), (2, 64, 256, 256, 32), (2, 64, 128, 384, 32), (16, 256, 64, 64, 32)]
+    shapes += [(rng.randint(2, 64), 32 * rng.randint(2, 12), rng.randint(7, 512), rng.choice([rng.randint(7, 512), 16 * rng.randint(1, 32)]),
+                rng.choice([16, 32])) for _ in range(4000)]
+    w = binding.msla_weights()
+    for B, C, H, W, d in shapes:
+        if B * C * H * W > 40 << 20:
+            continue
+        for dtype in (binding.MSLA_BF16, binding.MSLA_F32):
+            for n_scales in (2, 3):
+                desc = _desc(dtype, B, C, H, W, d, n_scales)
+                need = lib.msla_forward_host_workspace_bytes(ctypes.byref(desc))
+                assert need > 0
+                desc.workspace_bytes = need
+                st = lib.msla_forward_host(ctypes.byref(desc), None, ctypes.byref(w), None, None)
+                assert st == NULL_POINTER, (B, C, H, W, d, dtype, n_scales, lib.msla_last_error())
