@@ -98,7 +98,8 @@ struct AggStateParams {
   int tiles_y, kv_tiles_x, q_tiles_x, kv_tiles, q_tiles;  // tiles per plane
   int row_lo, row_hi;           // image rows that count in the states
   int with_scale0;
-  long long kv_units;           // (block, image, tile), tile fastest; keys and values first, then queries
+  int batch, first;             // see AggStatePlan
+  long long kv_units;           // of the batch: (block, image, tile), tile fastest; keys and values first, then queries
   long long cost;               // of all units, and of one
   int kv_cost, q_cost;
 };
@@ -241,10 +242,17 @@ agg_state_kernel(const __grid_constant__ CUtensorMap kv_even, const __grid_const
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
 
-  const long long u_first = agg_state_first_unit(p.cost, p.kv_cost, p.q_cost, p.kv_units, blockIdx.x, gridDim.x),
-                  u_end = agg_state_first_unit(p.cost, p.kv_cost, p.q_cost, p.kv_units, blockIdx.x + 1, gridDim.x);
-  const int kv_count = (int)(max(u_first, min(u_end, p.kv_units)) - u_first), q_count = (int)(u_end - u_first) - kv_count;
-  const long long q_first = max(u_first, p.kv_units) - p.kv_units;
+  const long long run_first = agg_state_first_unit(p.cost, p.kv_cost, p.q_cost, p.kv_units, blockIdx.x, gridDim.x),
+                  run_end = agg_state_first_unit(p.cost, p.kv_cost, p.q_cost, p.kv_units, blockIdx.x + 1, gridDim.x);
+  long long u_first = min(run_first, p.kv_units), u_end = min(run_end, p.kv_units);
+  long long q_first = max(run_first, p.kv_units) - p.kv_units, q_end = max(run_end, p.kv_units) - p.kv_units;
+  if (p.batch != p.B) {  // this call's tiles of the run are a run of its own list
+    u_first = agg_state_part_units(u_first, p.kv_tiles, p.batch, p.first, p.B);
+    u_end = agg_state_part_units(u_end, p.kv_tiles, p.batch, p.first, p.B);
+    q_first = agg_state_part_units(q_first, p.q_tiles, p.batch, p.first, p.B);
+    q_end = agg_state_part_units(q_end, p.q_tiles, p.batch, p.first, p.B);
+  }
+  const int kv_count = (int)(u_end - u_first), q_count = (int)(q_end - q_first);
 
   // Plane (inside an image's 3 * heads): block `pr` of queries (s = 0), keys (1) or values (2), sub-block `sub`; an absent head
   // (odd counts, d = 16) repeats the last.
@@ -730,24 +738,25 @@ msla_status_t launch_agg_state(int grid, const CUtensorMap (&m)[5], const AggSta
 
 }  // namespace
 
-AggStatePlan make_agg_state_plan(int B, int heads, int H, int W, int d) {
+AggStatePlan make_agg_state_plan(int B, int heads, int H, int W, int d, int batch, int first) {
   AggStatePlan pl;
+  pl.batch = batch;
+  pl.first = first;
   const int hpb = 32 / d;
   pl.kv_tiles_x = (W + 2 + AS_TW - 1) / AS_TW;
   pl.q_tiles_x = (W + AS_TW - 1) / AS_TW;
   pl.tiles_y = (H + AS_TH - 1) / AS_TH;
   pl.kv_tiles = (long long)pl.kv_tiles_x * pl.tiles_y;
   const long long blocks = (heads + hpb - 1) / hpb;  // of 32 channels
-  pl.segments = blocks * B;
-  pl.kv_units = pl.segments * pl.kv_tiles;
-  const long long q_units = blocks * B * pl.q_tiles_x * pl.tiles_y, units = pl.kv_units + q_units;
+  pl.kv_units = blocks * batch * pl.kv_tiles;
+  const long long q_units = blocks * batch * pl.q_tiles_x * pl.tiles_y, units = pl.kv_units + q_units;
   pl.grid = (int)(units < AGG_STATE_CTAS ? units : AGG_STATE_CTAS);
   // a tile of keys and values takes about 1.85 times one of queries; counted alike where a CTA has few (each must get one)
   pl.kv_cost = units >= 8 * pl.grid ? 37 : 1;
   pl.q_cost = units >= 8 * pl.grid ? 20 : 1;
   pl.cost = pl.kv_cost * pl.kv_units + pl.q_cost * q_units;
   pl.slot_floats = hpb * 2 * d * (d + 1);
-  pl.partial_bytes = (size_t)(pl.segments + pl.grid) * pl.slot_floats * sizeof(float);
+  pl.partial_bytes = (size_t)(blocks * B + pl.grid) * pl.slot_floats * sizeof(float);
   return pl;
 }
 
@@ -762,6 +771,7 @@ msla_status_t run_agg_state(const void* ms0, void* q1, float* partial, const voi
   p.tiles_y = pl.tiles_y; p.kv_tiles_x = pl.kv_tiles_x; p.q_tiles_x = pl.q_tiles_x;
   p.kv_tiles = (int)pl.kv_tiles; p.q_tiles = pl.q_tiles_x * pl.tiles_y;
   p.row_lo = row_lo; p.row_hi = row_hi; p.with_scale0 = with_scale0 ? 1 : 0;
+  p.batch = pl.batch; p.first = pl.first;
   p.kv_units = pl.kv_units; p.cost = pl.cost; p.kv_cost = pl.kv_cost; p.q_cost = pl.q_cost;
   // [plane][8-channel group][octet][row of this parity][64 elements]
   CUtensorMap maps[5];

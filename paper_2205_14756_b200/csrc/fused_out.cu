@@ -223,7 +223,7 @@ struct FoldParams {
   int S;
   const float* slots[2];     // SLOTS: per aggregated branch (the first also carries scale 0)
   const bf16* w_pw[2];       // SLOTS: the branches' grouped 1x1 weights
-  int slot_floats, grid, kv_cost;  // SLOTS: of the aggregation
+  int slot_floats, grid, kv_cost, batch, first_image;  // SLOTS: of the aggregation
   long long tiles, cost;
   const bf16* w;             // projection weights [Cout][K]
   bf16* M;
@@ -281,8 +281,8 @@ state_fold_kernel(FoldParams p) {
   const float* first = p.partial + (long long)bh * S * (D * D1);
   if constexpr (SLOTS) {
     constexpr int HPB = 32 / D;  // heads per slot
-    const long long seg = (long long)(h / HPB) * p.B + b;
-    const long long c0 = agg_state_cta_of(p.cost, p.kv_cost, seg * p.tiles, p.grid), c1 = agg_state_cta_of(p.cost, p.kv_cost, (seg + 1) * p.tiles - 1, p.grid);
+    const long long seg = (long long)(h / HPB) * p.B + b, of_batch = (long long)(h / HPB) * p.batch + p.first_image + b;
+    const long long c0 = agg_state_cta_of(p.cost, p.kv_cost, of_batch * p.tiles, p.grid), c1 = agg_state_cta_of(p.cost, p.kv_cost, (of_batch + 1) * p.tiles - 1, p.grid);
     S = (int)(c1 - c0) + 1;
     stride4 = p.slot_floats / 4;
     first = (branch == 2 ? p.slots[1] : p.slots[0]) + (seg + c0) * p.slot_floats + ((h % HPB) * 2 + (branch > 0 ? 1 : 0)) * (D * D1);
@@ -849,6 +849,7 @@ msla_status_t run_fold(const FoldStates& in, FoldParams& f, int d, cudaStream_t 
   const bool slots = in.plan.grid > 0;
   for (int i = 0; i < 2; ++i) { f.slots[i] = in.slots[i]; f.w_pw[i] = (const bf16*)in.w_pw[i]; }
   f.slot_floats = in.plan.slot_floats; f.grid = in.plan.grid; f.kv_cost = in.plan.kv_cost; f.tiles = in.plan.kv_tiles; f.cost = in.plan.cost;
+  f.batch = in.plan.batch; f.first_image = in.plan.first;
   if (!slots && f.S < 1) return fail(MSLA_ERR_UNSUPPORTED, "fused apply + projection: %d partial states per head", f.S);
   if (d == 32) {
     if (slots) return f16 ? launch_fold<32, true, true>(f, st) : launch_fold<32, false, true>(f, st);

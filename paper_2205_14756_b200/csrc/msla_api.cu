@@ -303,9 +303,11 @@ static bool planes_path(const msla_desc* d, int B) {
          3LL * d->W > 32LL * ((d->W + 17) / 16);
 }
 
-// whole_B: images of the batch that the call is a part of (0: desc->B).  It decides the layout and the split of the token
-// reduction, so that a part never needs more than the whole batch.
-static msla_status_t validate_desc(const msla_desc* d, ForwardPlan* plan, int whole_B = 0) {
+// A call that is a part of a batch: images first .. of whole_B (0: the call is the batch).  The whole decides the layout and
+// where the sums over tokens are cut, so that a part never needs more than the whole batch and gives its results bit for bit.
+struct BatchPart { int whole_B = 0, first = 0; };
+
+static msla_status_t validate_desc(const msla_desc* d, ForwardPlan* plan, BatchPart of = {}) {
   if (!d) return fail(MSLA_ERR_INVALID_ARG, "null descriptor");
   if (d->struct_size != sizeof(msla_desc)) return fail(MSLA_ERR_INVALID_ARG, "desc.struct_size = %u, expected %zu", d->struct_size, sizeof(msla_desc));
   if (!known_dtype(d->dtype)) return fail(MSLA_ERR_INVALID_ARG, "unknown dtype %d", (int)d->dtype);
@@ -321,7 +323,7 @@ static msla_status_t validate_desc(const msla_desc* d, ForwardPlan* plan, int wh
   if ((long long)d->H * d->W > 0x7ffffff8LL) return fail(MSLA_ERR_UNSUPPORTED, "H*W exceeds 2^31-8");
   if (d->C % 8 != 0 || d->C_out % 8 != 0) return fail(MSLA_ERR_UNSUPPORTED, "C and C_out must be multiples of 8");
   const int S = d->n_scales;
-  if (!whole_B) whole_B = d->B;
+  const int whole_B = of.whole_B ? of.whole_B : d->B;
   if ((long long)d->B * S * d->heads > 65535 || d->B > 65535) return fail(MSLA_ERR_UNSUPPORTED, "B*n_scales*heads exceeds 65535");
   plan->S = S;
   plan->Cp = d->heads * d->d;
@@ -339,7 +341,7 @@ static msla_status_t validate_desc(const msla_desc* d, ForwardPlan* plan, int wh
   plan->pitch = d->dtype == MSLA_F32 ? plan->N : (int)align_up((size_t)plan->N, 8);
   size_t core_bytes = plan->core.bytes;
   if (plan->planes) {
-    plan->agg = make_agg_state_plan(d->B, d->heads, d->H, d->W, d->d);
+    plan->agg = make_agg_state_plan(d->B, d->heads, d->H, d->W, d->d, whole_B, of.first);
     plan->q1_off = align_up(tokens * 3 * plan->Cp * e, 256);
     plan->att_off = plan->q1_off + align_up(tokens * (S - 1) * plan->Cp * e, 256);
     att_bytes = fused_out_bf16_supported(S * d->heads, d->d, d->C_out) ? fused_scratch : tokens * S * plan->Cp * e;
@@ -550,9 +552,9 @@ static msla_status_t record(void* const* events, int i, cudaStream_t st) {
 // add_x: the output projection adds x (the block's first residual connection; C_out == C).
 // out_padded: receives the address of the padded copy of out where there is one (else of out itself).
 static msla_status_t forward_impl(const msla_desc* desc, const void* x, const msla_weights* w, void* out,
-                                  cudaStream_t st, void* const* events, bool add_x = false, const void** out_padded = nullptr, int whole_B = 0) {
+                                  cudaStream_t st, void* const* events, bool add_x = false, const void** out_padded = nullptr, BatchPart of = {}) {
   ForwardPlan p;
-  msla_status_t s = validate_desc(desc, &p, whole_B);
+  msla_status_t s = validate_desc(desc, &p, of);
   if (s != MSLA_OK) return s;
   if (!x || !out || !w) return fail(MSLA_ERR_INVALID_ARG, "null x, out or weights");
   if (!w->w_qkv || !w->w_dw || !w->w_pw || !w->w_proj) return fail(MSLA_ERR_INVALID_ARG, "null weight pointer");
@@ -666,9 +668,12 @@ struct CopyLanes {
 
 // A batch goes through in parts of whole images: the copy to the device of one part, the forward of the part before it and the
 // copy back of the one before that run at the same time (the link is full duplex, and the copies, not the kernels, are what
-// takes the time).  Nothing flows back before the first part is through, and nothing in after the last, so those are small
-// (HOST_PART_BYTES); a copy has a fixed cost of 5 to 10 us, so the parts between them grow.  [16, 256, 64, 64] bf16, 33.5 MB each way
-// (628 us one way, 724 both at once): 1400 us with all copies on one stream, 1130 us in equal parts of 2 MB, 1010 us so.  On a capturing stream, and for a single part, everything stays on the caller's stream.
+// takes the time).  Nothing flows back before the first part is through, and nothing in after the last, so parts are small; a copy has
+// a fixed cost of 5 to 10 us, and a part's kernels take a while whatever its size (its sums are cut as the batch's are), so not too
+// small.  [16, 256, 64, 64] bf16, 33.5 MB each way (628 us one way, 724 both at once): 1400 us with all copies on one stream, in
+// parts of 2, 4 or 6 MB 1210, 899 or 1049 us, in parts that grow from 4 MB to 16 and shrink again 1055; [40, 128, 56, 56] 1250, 878,
+// 1038 and 1001; [64, 256, 14, 14] 254, 279, 329 and 276; one image of 4.7 MB per part or growing parts, [4, 256, 96, 96]: 656 and 628.  On a capturing stream, and for a single part, everything stays on the
+// caller's stream.
 constexpr size_t HOST_PART_BYTES = 4 << 20;
 
 static msla_status_t forward_host_impl(const msla_desc* desc, const void* x, const msla_weights* w, void* out, cudaStream_t st) {
@@ -681,18 +686,11 @@ static msla_status_t forward_host_impl(const msla_desc* desc, const void* x, con
   // images per part: whole multiples of 16 bytes, so that every part of the staging buffers is aligned
   int step = (int)((HOST_PART_BYTES + (xi < oi ? oi : xi) - 1) / (xi < oi ? oi : xi));
   while (step < desc->B && ((step * xi) % 16 || (step * oi) % 16)) ++step;
-  auto images = [&](int left, int before) {                             // of the next part:
-    int n = before + step;                                              // one step more than the part before,
-    if (n > 4 * step) n = 4 * step;                                     // up to four steps,
-    if (n > (left + 1) / 2) n = ((left + 1) / 2 + step - 1) / step * step;  // and at most half of what is left
-    return n > left ? left : n;
-  };
   msla_desc part = *desc;
-  part.B = 0;
   for (int b = 0; b < desc->B; b += part.B) {  // every part fits what the whole batch reserved; known before the first copy
-    part.B = images(desc->B - b, part.B);
+    part.B = step < desc->B - b ? step : desc->B - b;
     ForwardPlan pp;
-    if ((s = validate_desc(&part, &pp, desc->B)) != MSLA_OK) return s;
+    if ((s = validate_desc(&part, &pp, {desc->B, b})) != MSLA_OK) return s;
     if (pp.bytes > p.bytes) return fail(MSLA_ERR_WORKSPACE, "%d of %d images need %zu bytes of scratch, the whole batch %zu", part.B, desc->B, pp.bytes, p.bytes);
   }
   if (!x || !out || !w) return fail(MSLA_ERR_INVALID_ARG, "null x, out or weights");
@@ -717,13 +715,12 @@ static msla_status_t forward_host_impl(const msla_desc* desc, const void* x, con
     return ce == cudaSuccess;
   };
   if (overlap && ok(cudaEventRecord(lanes.done, st))) ok(cudaStreamWaitEvent(lanes.in, lanes.done, 0));  // the staging buffers are free by then
-  part.B = 0;
   for (int b = 0; b < desc->B && ce == cudaSuccess; b += part.B) {
-    part.B = overlap ? images(desc->B - b, part.B) : desc->B;
+    part.B = overlap && step < desc->B - b ? step : desc->B - b;
     const char* xs = (const char*)x + b * xi;
     if (!ok(cudaMemcpyAsync(x_dev + b * xi, xs, part.B * xi, cudaMemcpyHostToDevice, overlap ? lanes.in : st))) break;
     if (overlap && (!ok(cudaEventRecord(lanes.arrived, lanes.in)) || !ok(cudaStreamWaitEvent(st, lanes.arrived, 0)))) break;
-    if ((s = forward_impl(&part, x_dev + b * xi, w, out_dev + b * oi, st, nullptr, false, nullptr, desc->B)) != MSLA_OK) break;
+    if ((s = forward_impl(&part, x_dev + b * xi, w, out_dev + b * oi, st, nullptr, false, nullptr, {desc->B, b})) != MSLA_OK) break;
     if (overlap && (!ok(cudaEventRecord(lanes.done, st)) || !ok(cudaStreamWaitEvent(lanes.out, lanes.done, 0)))) break;
     ok(cudaMemcpyAsync((char*)out + b * oi, out_dev + b * oi, part.B * oi, cudaMemcpyDeviceToHost, overlap ? lanes.out : st));
   }

@@ -152,20 +152,26 @@ msla_status_t run_unpad_rows(const void* src, void* dst, long long rows, int n, 
 //
 // Aggregation and state sums (agg_state.cu).  The grid's CTAs take contiguous runs of tiles, of equal cost; CTA c writes the
 // part of segment s (a pair of blocks of one image: s = pair * B + image) that it summed to slot s + c (unique, because both
-// grow along the list of tiles).
+// grow along the list of tiles).  The runs are cut for `batch` images; a call that has images first .. first + B - 1 of them takes
+// those tiles of every run, so that its sums are added as the whole batch adds them.
 constexpr int AGG_STATE_CTAS = 148;
 struct AggStatePlan {
-  int kv_tiles_x, q_tiles_x, tiles_y, grid, slot_floats, kv_cost, q_cost;
-  long long kv_tiles, segments, kv_units, cost;
+  int kv_tiles_x, q_tiles_x, tiles_y, grid, slot_floats, kv_cost, q_cost, batch, first;
+  long long kv_tiles, kv_units, cost;  // kv_units, cost: of the batch
   size_t partial_bytes;
 };
-AggStatePlan make_agg_state_plan(int B, int heads, int H, int W, int d);
+AggStatePlan make_agg_state_plan(int B, int heads, int H, int W, int d, int batch, int first);
 // First tile of CTA c; the CTA that has key/value tile u.
 __host__ __device__ inline long long agg_state_first_unit(long long cost, int kv_cost, int q_cost, long long kv_units, long long c, long long grid) {
   const long long at = cost * c / grid, kv = kv_cost * kv_units;
   return at < kv ? (at + kv_cost - 1) / kv_cost : kv_units + (at - kv + q_cost - 1) / q_cost;
 }
 __host__ __device__ inline long long agg_state_cta_of(long long cost, int kv_cost, long long u, long long grid) { return (grid * (kv_cost * u + 1) - 1) / cost; }
+// Tiles of the batch's list before `u` (`tiles` per plane; pair of blocks, image, tile) that belong to images first .. first + B - 1.
+__host__ __device__ inline long long agg_state_part_units(long long u, long long tiles, int batch, int first, int B) {
+  const long long pb = u / tiles, pair = pb / batch, b = pb - pair * batch - first;
+  return b < 0 ? pair * B * tiles : b >= B ? (pair + 1) * B * tiles : (pair * B + b) * tiles + (u - pb * tiles);
+}
 // ms0: [B][3*heads] planes; q1: [B][heads] planes; rows [row_lo, row_hi) count in the states.
 msla_status_t run_agg_state(const void* ms0, void* q1, float* partial, const void* w_dw, const void* w_pw, const AggStatePlan& plan, int B,
                             int heads, int H, int W, int d, int row_lo, int row_hi, bool with_scale0, cudaStream_t st, bool f16);
