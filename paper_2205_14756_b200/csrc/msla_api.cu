@@ -549,13 +549,8 @@ static msla_status_t record(void* const* events, int i, cudaStream_t st) {
   return MSLA_OK;
 }
 
-// add_x: the output projection adds x (the block's first residual connection; C_out == C).
-// out_padded: receives the address of the padded copy of out where there is one (else of out itself).
-static msla_status_t forward_impl(const msla_desc* desc, const void* x, const msla_weights* w, void* out,
-                                  cudaStream_t st, void* const* events, bool add_x = false, const void** out_padded = nullptr, BatchPart of = {}) {
-  ForwardPlan p;
-  msla_status_t s = validate_desc(desc, &p, of);
-  if (s != MSLA_OK) return s;
+// What msla_forward refuses beyond the descriptor.
+static msla_status_t check_forward_args(const msla_desc* desc, const ForwardPlan& p, const void* x, const msla_weights* w, const void* out) {
   if (!x || !out || !w) return fail(MSLA_ERR_INVALID_ARG, "null x, out or weights");
   if (!w->w_qkv || !w->w_dw || !w->w_pw || !w->w_proj) return fail(MSLA_ERR_INVALID_ARG, "null weight pointer");
   if (p.S == 3 && (!w->w_dw2 || !w->w_pw2)) return fail(MSLA_ERR_INVALID_ARG, "three branches need w_dw2 and w_pw2");
@@ -570,9 +565,21 @@ static msla_status_t forward_impl(const msla_desc* desc, const void* x, const ms
   if (overlaps(out, ob, x, xb)) return fail(MSLA_ERR_INVALID_ARG, "out overlaps x");
   if (overlaps(out, ob, desc->workspace, p.bytes) || overlaps(x, xb, desc->workspace, p.bytes))
     return fail(MSLA_ERR_INVALID_ARG, "workspace overlaps x or out");
+  return MSLA_OK;
+}
+
+// add_x: the output projection adds x (the block's first residual connection; C_out == C).
+// out_padded: receives the address of the padded copy of out where there is one (else of out itself).
+static msla_status_t forward_impl(const msla_desc* desc, const void* x, const msla_weights* w, void* out,
+                                  cudaStream_t st, void* const* events, bool add_x = false, const void** out_padded = nullptr, BatchPart of = {}) {
+  ForwardPlan p;
+  msla_status_t s = validate_desc(desc, &p, of);
+  if (s != MSLA_OK) return s;
+  if ((s = check_forward_args(desc, p, x, w, out)) != MSLA_OK) return s;
   s = check_arch();
   if (s != MSLA_OK) return s;
 
+  const size_t e = elem_size(desc->dtype);
   char* ws = (char*)desc->workspace;
   const void* x_dev = x;
   void* out_dev = out;
@@ -699,9 +706,10 @@ static msla_status_t forward_host_impl(const msla_desc* desc, const void* x, con
   if (!desc->workspace || desc->workspace_bytes < need)
     return fail(MSLA_ERR_WORKSPACE, "workspace of %zu bytes needed, %zu given", need, desc->workspace ? desc->workspace_bytes : (size_t)0);
   if (overlaps(out, ob, x, xb)) return fail(MSLA_ERR_INVALID_ARG, "out overlaps x");
-  if ((s = check_arch()) != MSLA_OK) return s;
   char* x_dev = (char*)desc->workspace + p.bytes;
   char* out_dev = x_dev + align_up(xb, 256);
+  if ((s = check_forward_args(desc, p, x_dev, w, out_dev)) != MSLA_OK) return s;  // nothing is copied for a call that the parts would refuse
+  if ((s = check_arch()) != MSLA_OK) return s;
 
   thread_local CopyLanes lanes;
   int dev = -1;

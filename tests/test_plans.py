@@ -34,3 +34,28 @@ def test_parts_of_a_host_call_fit_the_reservation_of_the_batch():
                 desc.workspace_bytes = need
                 st = lib.msla_forward_host(ctypes.byref(desc), None, ctypes.byref(w), None, None)
                 assert st == NULL_POINTER, (B, C, H, W, d, dtype, n_scales, lib.msla_last_error())
+
+
+def test_a_host_call_that_its_parts_would_refuse_copies_nothing():
+    """A null or misaligned weight is found before the first copy (on a machine without a GPU: before the device is looked for)."""
+    import torch
+    lib = binding.lib()
+    B, C, H, W, d = 6, 64, 64, 96, 32
+    x, out = torch.zeros(B, C, H, W, dtype=torch.bfloat16), torch.zeros(B, C, H, W, dtype=torch.bfloat16)
+    need = binding.msla_forward_host_workspace_bytes(_desc(binding.MSLA_BF16, B, C, H, W, d))
+    # real buffers: a GPU's where there is one (the call is refused all the same)
+    device = "cuda" if torch.cuda.is_available() else "cpu"
+    ws = torch.full((need + 256,), 0xA5, dtype=torch.uint8, device=device)
+    wt = torch.zeros(1 << 20, dtype=torch.bfloat16, device=device)
+    desc = _desc(binding.MSLA_BF16, B, C, H, W, d, nbytes=need)
+    desc.workspace = (ws.data_ptr() + 255) // 256 * 256
+    fields = ("w_qkv", "w_dw", "w_pw", "w_proj")
+    for field, value, status in [("w_dw", None, 1), ("w_proj", None, 1), ("w_pw", wt.data_ptr() + 2, 3), ("b_proj", wt.data_ptr() + 8, 3)]:
+        w = binding.msla_weights()
+        for f in fields:
+            setattr(w, f, wt.data_ptr())
+        setattr(w, field, value)
+        assert lib.msla_forward_host(ctypes.byref(desc), x.data_ptr(), ctypes.byref(w), out.data_ptr(), None) == status, field
+    if device == "cuda":
+        torch.cuda.synchronize()
+    assert bool((ws == 0xA5).all())
