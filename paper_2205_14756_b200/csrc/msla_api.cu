@@ -113,6 +113,15 @@ CorePlan make_core_plan(long long BH, int N, int d) {
   return p;
 }
 
+// Bytes that hold the partial states and their sum for any number of heads up to BH and of tokens up to N.  A plan's own need is not
+// monotone: a chunk is a multiple of 64 tokens, so a longer sequence may have fewer chunks than a shorter one.
+static size_t core_bytes_bound(long long BH, int N, int d) {
+  const long long by_tokens = ceil_div_ll(N, 256), split = BH * (by_tokens < 64 ? by_tokens : 64);
+  const long long by_heads = d == 32 ? (BH > 444 ? BH : 444) : 591 + BH;  // BH * max(1, 444 / BH); BH * ceil(592 / BH)
+  const size_t state = (size_t)d * (d + 1) * sizeof(float);
+  return align_up((size_t)(split < by_heads ? split : by_heads) * state, 256) + align_up((size_t)BH * state, 256);
+}
+
 static bool core_shape_ok(int B, int heads, int N, int d) {
   return B >= 1 && heads >= 1 && N >= 1 && (d == 16 || d == 32) && (long long)B * heads <= 65535;
 }
@@ -339,7 +348,7 @@ static msla_status_t validate_desc(const msla_desc* d, ForwardPlan* plan, BatchP
   if (att_bytes < fused_scratch) att_bytes = fused_scratch;
   plan->planes = planes_path(d, whole_B);
   plan->pitch = d->dtype == MSLA_F32 ? plan->N : (int)align_up((size_t)plan->N, 8);
-  size_t core_bytes = plan->core.bytes;
+  size_t core_bytes = core_bytes_bound((long long)whole_B * S * d->heads, plan->N, d->d);  // a band of the image is split by itself
   if (plan->planes) {
     plan->agg = make_agg_state_plan(d->B, d->heads, d->H, d->W, d->d, whole_B, of.first);
     plan->q1_off = align_up(tokens * 3 * plan->Cp * e, 256);
@@ -764,7 +773,6 @@ static msla_status_t validate_band(const msla_desc* desc, int halo_top, int halo
   b->Nb = (desc->H - halo_top - halo_bottom) * desc->W;
   b->tok_off = (long long)halo_top * desc->W;
   b->core = make_core_plan((long long)desc->B * b->f.S * desc->heads, b->Nb, desc->d);
-  if (!b->f.planes && b->core.bytes > b->f.core.bytes) return fail(MSLA_ERR_WORKSPACE, "band plan exceeds the forward plan");
   if (!desc->workspace || desc->workspace_bytes < b->f.bytes)
     return fail(MSLA_ERR_WORKSPACE, "workspace of %zu bytes needed, %zu given", b->f.bytes, desc->workspace ? desc->workspace_bytes : (size_t)0);
   if (!aligned16(desc->workspace)) return fail(MSLA_ERR_ALIGNMENT, "workspace must be 16-byte aligned");

@@ -59,3 +59,18 @@ def test_a_host_call_that_its_parts_would_refuse_copies_nothing():
     if device == "cuda":
         torch.cuda.synchronize()
     assert bool((ws == 0xA5).all())
+
+
+def test_bands_fit_the_reservation_of_the_band_with_its_halo():
+    """msla_band_states splits the band's own tokens, whose number of chunks may exceed that of the band with its halo."""
+    lib, rng = binding.lib(), random.Random(2)
+    shapes = [(2, 256, 54, 64, 32, 2, 0), (2, 256, 56, 64, 32, 2, 2), (1, 32, 9, 57, 32, 2, 2)]
+    shapes += [(rng.randint(1, 40), 32 * rng.randint(1, 12), rng.randint(5, 300), rng.randint(1, 300), rng.choice([16, 32]), rng.choice([0, 2]),
+                rng.choice([0, 2])) for _ in range(20000)]
+    w = binding.msla_weights()
+    for B, C, H, W, d, top, bottom in shapes:
+        for dtype in (binding.MSLA_BF16, binding.MSLA_F32):
+            desc = _desc(dtype, B, C, H, W, d)
+            desc.workspace_bytes = lib.msla_forward_workspace_bytes(ctypes.byref(desc))
+            st = lib.msla_band_states(ctypes.byref(desc), None, ctypes.byref(w), top, bottom, None, None)
+            assert st == NULL_POINTER, (B, C, H, W, d, top, bottom, lib.msla_last_error())

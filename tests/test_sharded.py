@@ -217,3 +217,17 @@ def test_band_calls_reject_bad_halos():
         binding.msla_band_states(desc, x, binding.make_weights(*w), 2, 2, st)     # no row left
     with pytest.raises(binding.MslaError):
         binding.msla_band_states(desc, x, binding.make_weights(*w), -1, 0, st)
+
+
+# a band with more chunks of tokens than the band with its halo (52 + 2 rows of 64 tokens: 13 against 11), on both sides of the split
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_bands_split_finer_than_the_image(dtype):
+    import oracle
+    import util
+    from paper_2205_14756_b200 import inputs
+    s = inputs.ModuleShape("bands_split", dtype, 2, 64, 104, 64, 8, 32, seed=25)
+    t = inputs.module_inputs(s)
+    ref = oracle.msla_forward(t["x"], t["w_qkv"], t["w_dw"], t["w_pw"], t["w_proj"], heads=s.heads, d=s.d)
+    got, _ = _run_bands(t, s, 2, dtype)
+    util.assert_close(got, ref, dtype, block=util.MODULE_BLOCK)
