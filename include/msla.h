@@ -165,7 +165,10 @@ typedef struct {
 } msla_weights;
 
 /* Scratch bytes msla_forward needs for this descriptor (workspace fields are
- * ignored); 0 if the descriptor is invalid or unsupported. */
+ * ignored); 0 if the descriptor is invalid or unsupported.  The answer does
+ * not fall when B, H or W grows and the rest stays, so a workspace for the
+ * largest of several feature maps serves them all (as do the answers of
+ * msla_forward_host_workspace_bytes and msla_ffn_workspace_bytes). */
 size_t msla_forward_workspace_bytes(const msla_desc* desc);
 
 /* x: device [B, C, H, W]; out: device [B, C_out, H, W]; both of desc->dtype.

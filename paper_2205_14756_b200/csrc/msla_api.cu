@@ -338,33 +338,40 @@ static msla_status_t validate_desc(const msla_desc* d, ForwardPlan* plan, BatchP
   plan->Cp = d->heads * d->d;
   plan->N = d->H * d->W;
   const size_t e = elem_size(d->dtype);
-  const size_t tokens = (size_t)d->B * plan->N;
+  const size_t tokens = (size_t)d->B * plan->N, state = (size_t)d->d * (d->d + 1) * sizeof(float);
+  const bool tuned = d->dtype != MSLA_F32, fused = tuned && fused_out_bf16_supported(S * d->heads, d->d, d->C_out);
   plan->core = make_core_plan((long long)whole_B * S * d->heads, plan->N, d->d);
-  plan->ms_off = 0;
-  plan->att_off = align_up(tokens * 3 * S * plan->Cp * e, 256);
-  // the attention output's region doubles as scratch of the fused apply + projection kernel, which writes no attention output
-  size_t att_bytes = tokens * S * plan->Cp * e;
-  const size_t fused_scratch = fused_out_bf16_supported(S * d->heads, d->d, d->C_out) ? fused_out_scratch_bytes(d->B, S * d->heads, d->d, d->C_out) : 0;
-  if (att_bytes < fused_scratch) att_bytes = fused_scratch;
   plan->planes = planes_path(d, whole_B);
-  plan->pitch = d->dtype == MSLA_F32 ? plan->N : (int)align_up((size_t)plan->N, 8);
-  size_t core_bytes = core_bytes_bound((long long)whole_B * S * d->heads, plan->N, d->d);  // a band of the image is split by itself
+  plan->pitch = tuned ? (int)align_up((size_t)plan->N, 8) : plan->N;
+  plan->ms_off = 0;
+  // the fused apply + projection kernel writes no attention output, and the region is its scratch
+  const size_t att_bytes = align_up(fused ? fused_out_scratch_bytes(d->B, S * d->heads, d->d, d->C_out) : tokens * S * plan->Cp * e, 256);
+  const size_t taps = align_up((size_t)3 * plan->Cp * 25 * e, 256), embedded = (d->agg_kernel == 3 ? taps : 0) + (S == 3 && d->agg_kernel2 == 3 ? taps : 0);
+  const size_t xpad = align_up((size_t)d->B * d->C * plan->pitch * e, 256), ypad = align_up((size_t)d->B * d->C_out * plan->pitch * e, 256);
+  const size_t ms_bytes = align_up(tokens * 3 * S * plan->Cp * e, 256);
+  const size_t core_bytes = core_bytes_bound((long long)whole_B * S * d->heads, plan->N, d->d);  // a band of the image is split by itself
+  size_t sums_bytes = core_bytes;
+  plan->att_off = ms_bytes;
   if (plan->planes) {
     plan->agg = make_agg_state_plan(d->B, d->heads, d->H, d->W, d->d, whole_B, of.first);
     plan->q1_off = align_up(tokens * 3 * plan->Cp * e, 256);
     plan->att_off = plan->q1_off + align_up(tokens * (S - 1) * plan->Cp * e, 256);
-    att_bytes = fused_out_bf16_supported(S * d->heads, d->d, d->C_out) ? fused_scratch : tokens * S * plan->Cp * e;
     plan->partial_bytes = align_up(plan->agg.partial_bytes, 256);
     plan->state_off = (S - 1) * plan->partial_bytes;
-    core_bytes = plan->state_off + align_up((size_t)d->B * S * d->heads * d->d * (d->d + 1) * sizeof(float), 256);
+    sums_bytes = plan->state_off + align_up((size_t)d->B * S * d->heads * state, 256);
   }
-  plan->core_off = plan->att_off + align_up(att_bytes, 256);
-  plan->wpad_off = plan->core_off + core_bytes;
-  plan->wpad2_off = plan->wpad_off + (d->agg_kernel == 3 ? align_up((size_t)3 * plan->Cp * 25 * e, 256) : 0);
-  plan->xpad_off = plan->wpad2_off + (S == 3 && d->agg_kernel2 == 3 ? align_up((size_t)3 * plan->Cp * 25 * e, 256) : 0);
-  plan->ypad_off = plan->xpad_off + (plan->padded() ? align_up((size_t)d->B * d->C * plan->pitch * e, 256) : 0);
+  plan->core_off = plan->att_off + att_bytes;
+  plan->wpad_off = plan->core_off + sums_bytes;
+  plan->wpad2_off = plan->wpad_off + (d->agg_kernel == 3 ? taps : 0);
+  plan->xpad_off = plan->wpad_off + embedded;
+  plan->ypad_off = plan->xpad_off + (plan->padded() ? xpad : 0);
   // (bands of such an image may be ragged where the whole is not, so the output's copy depends on the row length)
-  plan->bytes = plan->ypad_off + (d->dtype != MSLA_F32 && d->W % 8 != 0 ? align_up((size_t)d->B * d->C_out * plan->pitch * e, 256) : 0);
+  const size_t used = plan->ypad_off + (tuned && d->W % 8 != 0 ? ypad : 0);
+  // What is reserved is what token rows and padded copies would take, whether this shape has them or not, and so does not fall
+  // when B, H or W grows.  Planes take less: 4 C' elements per token for the 6 C' of the rows, and partial states whose number grows
+  // with the images and heads.
+  plan->bytes = ms_bytes + att_bytes + core_bytes + embedded + (tuned ? xpad + ypad : 0);
+  if (plan->bytes < used) plan->bytes = used;
   return MSLA_OK;
 }
 
@@ -883,7 +890,7 @@ static msla_status_t band_output_impl(const msla_desc* desc, const msla_weights*
 
 // ---------------------------------------------------------- FFN with a depthwise convolution
 struct FfnPlan {
-  size_t h_off, g_off, bytes;
+  size_t h_off, g_off, bytes;  // the second layer's padded output takes the place of the first one's output
   int N;
   bool tuned;  // bf16 / fp16 tensor-core path with the hidden tensor as planes of 64 channels
   int pitch;   // tuned: elements between rows of x and out; padded copies in the workspace where that is not H*W
@@ -908,12 +915,15 @@ static msla_status_t validate_ffn(const msla_ffn_desc* d, FfnPlan* plan) {
   plan->tuned = d->dtype != MSLA_F32 && ffn_bf16_supported(d->C, d->C_hidden, d->C_out) &&
                 (long long)d->B * (d->C_hidden / 64) <= 65535;
   const size_t hid = align_up((size_t)d->B * d->C_hidden * plan->N * elem_size(d->dtype), 256);
-  plan->h_off = 0;
-  plan->g_off = hid;
-  plan->pitch = plan->tuned ? (int)align_up((size_t)plan->N, 8) : plan->N;
-  plan->xpad_off = 2 * hid;
-  plan->ypad_off = plan->xpad_off + (plan->padded() ? align_up((size_t)d->B * d->C * plan->pitch * 2, 256) : 0);
-  plan->bytes = plan->ypad_off + (plan->padded() ? align_up((size_t)d->B * d->C_out * plan->pitch * 2, 256) : 0);
+  const size_t row = align_up((size_t)plan->N, 8);
+  plan->pitch = plan->tuned ? (int)row : plan->N;
+  // padded copies are reserved where any H and W has them, so that the answer does not fall when B, H or W grows
+  const bool pads = d->dtype != MSLA_F32 && ffn_bf16_supported(d->C, d->C_hidden, d->C_out);
+  const size_t xpad = pads ? align_up((size_t)d->B * d->C * row * 2, 256) : 0, ypad = pads ? align_up((size_t)d->B * d->C_out * row * 2, 256) : 0;
+  plan->h_off = plan->ypad_off = 0;
+  plan->g_off = hid < ypad ? ypad : hid;
+  plan->xpad_off = plan->g_off + hid;
+  plan->bytes = plan->xpad_off + xpad;
   return MSLA_OK;
 }
 

@@ -74,3 +74,25 @@ def test_bands_fit_the_reservation_of_the_band_with_its_halo():
             desc.workspace_bytes = lib.msla_forward_workspace_bytes(ctypes.byref(desc))
             st = lib.msla_band_states(ctypes.byref(desc), None, ctypes.byref(w), top, bottom, None, None)
             assert st == NULL_POINTER, (B, C, H, W, d, top, bottom, lib.msla_last_error())
+
+
+def test_workspaces_do_not_shrink_as_feature_maps_grow():
+    """A workspace sized for the largest batch, height and width serves every smaller one: whole forward, host call and FFN."""
+    lib, rng = binding.lib(), random.Random(3)
+    widths = [(256, 32, 2), (128, 16, 2), (384, 32, 2), (64, 32, 3), (96, 16, 3)]  # the third: apply and projection apart
+    shapes = [(1, 128, 152, 1, 128, 160), (64, 14, 14, 64, 14, 16), (64, 7, 7, 64, 7, 8), (1, 250, 255, 1, 250, 256), (21, 66, 64, 22, 66, 64)]
+    for _ in range(4000):
+        B, H, W = rng.randint(1, 40), rng.randint(1, 260), rng.randint(1, 260)
+        i, by = rng.randrange(3), rng.choice([1, 1, 2, 7, 8, 30])
+        shapes.append((B, H, W) + tuple(v + (by if j == i else 0) for j, v in enumerate((B, H, W))))
+
+    def answers(dtype, C, d, S, B, H, W):
+        desc, ffn = _desc(dtype, B, C, H, W, d, S), binding.make_ffn_desc(B, C, H, W, C + 64, C, dtype)
+        return [lib.msla_forward_workspace_bytes(ctypes.byref(desc)), lib.msla_forward_host_workspace_bytes(ctypes.byref(desc)),
+                lib.msla_ffn_workspace_bytes(ctypes.byref(ffn))]
+
+    for B0, H0, W0, B1, H1, W1 in shapes:
+        for C, d, S in widths:
+            for dtype in (binding.MSLA_BF16, binding.MSLA_F32):
+                small, large = answers(dtype, C, d, S, B0, H0, W0), answers(dtype, C, d, S, B1, H1, W1)
+                assert min(small) > 0 and all(a <= b for a, b in zip(small, large)), (B0, H0, W0, B1, H1, W1, C, d, S, dtype, small, large)
