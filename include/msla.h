@@ -292,7 +292,8 @@ msla_status_t msla_ffn_dwconv(const msla_ffn_desc* desc, const void* x, const ms
 /* The building block of Fig. 2 left with its two residual connections:
  *   y = x + MSLA(x)  (msla_forward),   out = y + FFN+DWConv(y)  (msla_ffn_dwconv with residual).
  * attn and ffn describe the same B, H, W and dtype with attn->C == attn->C_out
- * == ffn->C == ffn->C_out; each carries its own workspace; `y`, device
+ * == ffn->C == ffn->C_out; each carries its workspace (the two may be the same
+ * memory, as the halves run one after the other); `y`, device
  * [B, C, H, W], receives the intermediate (caller-owned, no overlap with x,
  * out or the workspaces).  ffn->residual is taken as 1. */
 msla_status_t msla_evit_block(const msla_desc* attn, const msla_weights* attn_weights, const msla_ffn_desc* ffn,

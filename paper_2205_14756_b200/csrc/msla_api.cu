@@ -1003,7 +1003,9 @@ static msla_status_t block_impl(const msla_desc* attn, const msla_weights* aw, c
   // y = MSLA(x) + x: the output projection's epilogue adds the residual
   const void* y_padded = nullptr;
   if ((s = forward_impl(attn, x, aw, y, st, nullptr, true, &y_padded)) != MSLA_OK) return s;
-  return ffn_impl(ffn, y, fw, out, true, st, ap.padded() ? y_padded : nullptr);
+  // y with padded rows still lies in the attention's workspace, unless the FFN works in the same memory
+  const bool keep = ap.padded() && !overlaps(attn->workspace, ap.bytes, ffn->workspace, fp.bytes);
+  return ffn_impl(ffn, y, fw, out, true, st, keep ? y_padded : nullptr);
 }
 
 }  // namespace msla

@@ -41,3 +41,28 @@ def test_ragged_block(dtype, B, C, H, W, heads, d):
     f = inputs.ffn_inputs(inputs.FfnShape("ragged_block_ffn", dtype, B, C, H, W, 2 * C, C, seed=63))
     ref = oracle.evit_block(t["x"], t, f, heads=heads, d=d, act="hardswish")
     util.assert_close(util.run_block(s, t, f, 2 * C, "hardswish"), ref, dtype, "ragged block", block=util.MODULE_BLOCK)
+
+
+# the two halves of the block on one workspace: the attention's padded output must not be read from memory that the FFN writes
+@pytest.mark.parametrize("dtype,B,C,H,W,heads,d", [("bf16", 2, 64, 7, 9, 2, 32), ("f16", 3, 128, 14, 14, 8, 16), ("bf16", 1, 288, 5, 5, 9, 32),
+                                                   ("bf16", 1, 64, 24, 24, 2, 32)])
+def test_block_on_one_workspace(dtype, B, C, H, W, heads, d):
+    import torch
+    dt, code = util.TORCH_DTYPE[dtype], util.CODE[dtype]
+    gen = torch.Generator(device="cuda").manual_seed(64)
+    rnd = lambda *shape: (torch.randn(*shape, generator=gen, device="cuda") * shape[-1] ** -0.5).to(dt)
+    keep = [rnd(3 * C, C), rnd(3 * C, 5, 5), rnd(3 * C, d), rnd(C, 2 * C)]
+    fkeep = [rnd(4 * C, C), rnd(4 * C, 3, 3), rnd(C, 4 * C)]
+    x = torch.randn(B, C, H, W, generator=gen, device="cuda").to(dt)
+    attn, ffn = (lambda ws=None: binding.make_desc(B, C, H, W, heads, d, C, code, workspace=ws)), \
+                (lambda ws=None: binding.make_ffn_desc(B, C, H, W, 4 * C, C, code, binding.MSLA_ACT_HARDSWISH, True, workspace=ws))
+    na, nf = binding.msla_forward_workspace_bytes(attn()), binding.msla_ffn_workspace_bytes(ffn())
+    scratch = lambda n: torch.zeros(n, dtype=torch.uint8, device="cuda")
+    both = scratch(max(na, nf))
+    outs = []
+    for wa, wf in ((scratch(na), scratch(nf)), (both, both)):
+        y, out = torch.empty_like(x), torch.empty_like(x)
+        binding.msla_evit_block(attn(wa), binding.make_weights(*keep), ffn(wf), binding.make_ffn_weights(*fkeep), x, y, out)
+        torch.cuda.synchronize()
+        outs.append(out)
+    assert torch.equal(outs[0], outs[1])
