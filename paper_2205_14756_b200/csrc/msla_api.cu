@@ -927,12 +927,8 @@ static msla_status_t validate_ffn(const msla_ffn_desc* d, FfnPlan* plan) {
   return MSLA_OK;
 }
 
-// x_padded: a copy of x with rows of the plan's pitch that the caller already has, or nullptr.
-static msla_status_t ffn_impl(const msla_ffn_desc* desc, const void* x, const msla_ffn_weights* w, void* out, bool residual,
-                              cudaStream_t st, const void* x_padded = nullptr) {
-  FfnPlan p;
-  msla_status_t s = validate_ffn(desc, &p);
-  if (s != MSLA_OK) return s;
+// What msla_ffn_dwconv refuses beyond the descriptor.
+static msla_status_t check_ffn_args(const msla_ffn_desc* desc, const FfnPlan& p, const void* x, const msla_ffn_weights* w, const void* out) {
   if (!x || !out || !w) return fail(MSLA_ERR_INVALID_ARG, "null x, out or weights");
   if (!w->w1 || !w->w_dw || !w->w2) return fail(MSLA_ERR_INVALID_ARG, "null weight pointer");
   const void* ptrs[] = {x, out, w->w1, w->b1, w->w_dw, w->b_dw, w->w2, w->b2, desc->workspace};
@@ -940,11 +936,20 @@ static msla_status_t ffn_impl(const msla_ffn_desc* desc, const void* x, const ms
     if (ptr && !aligned16(ptr)) return fail(MSLA_ERR_ALIGNMENT, "all device pointers must be 16-byte aligned");
   if (!desc->workspace || desc->workspace_bytes < p.bytes)
     return fail(MSLA_ERR_WORKSPACE, "workspace of %zu bytes needed, %zu given", p.bytes, desc->workspace ? desc->workspace_bytes : (size_t)0);
-  const size_t e = elem_size(desc->dtype);
-  const int N = p.N, B = desc->B, C = desc->C, Ch = desc->C_hidden, Co = desc->C_out, act = (int)desc->act;
-  const size_t xb = (size_t)B * C * N * e, ob = (size_t)B * Co * N * e;
+  const size_t e = elem_size(desc->dtype), xb = (size_t)desc->B * desc->C * p.N * e, ob = (size_t)desc->B * desc->C_out * p.N * e;
   if (overlaps(out, ob, x, xb) || overlaps(out, ob, desc->workspace, p.bytes) || overlaps(x, xb, desc->workspace, p.bytes))
     return fail(MSLA_ERR_INVALID_ARG, "x, out and the workspace must not overlap");
+  return MSLA_OK;
+}
+
+// x_padded: a copy of x with rows of the plan's pitch that the caller already has, or nullptr.
+static msla_status_t ffn_impl(const msla_ffn_desc* desc, const void* x, const msla_ffn_weights* w, void* out, bool residual,
+                              cudaStream_t st, const void* x_padded = nullptr) {
+  FfnPlan p;
+  msla_status_t s = validate_ffn(desc, &p);
+  if (s != MSLA_OK) return s;
+  if ((s = check_ffn_args(desc, p, x, w, out)) != MSLA_OK) return s;
+  const int N = p.N, B = desc->B, C = desc->C, Ch = desc->C_hidden, Co = desc->C_out, act = (int)desc->act;
   if ((s = check_arch()) != MSLA_OK) return s;
   char* ws = (char*)desc->workspace;
   void* h = ws + p.h_off;
@@ -1000,6 +1005,8 @@ static msla_status_t block_impl(const msla_desc* attn, const msla_weights* aw, c
   if (overlaps(y, bytes, x, bytes) || overlaps(y, bytes, out, bytes) ||
       (attn->workspace && overlaps(y, bytes, attn->workspace, ap.bytes)) || (ffn->workspace && overlaps(y, bytes, ffn->workspace, fp.bytes)))
     return fail(MSLA_ERR_INVALID_ARG, "y overlaps x, out or a workspace");
+  // both halves are checked before either runs
+  if ((s = check_forward_args(attn, ap, x, aw, y)) != MSLA_OK || (s = check_ffn_args(ffn, fp, y, fw, out)) != MSLA_OK) return s;
   // y = MSLA(x) + x: the output projection's epilogue adds the residual
   const void* y_padded = nullptr;
   if ((s = forward_impl(attn, x, aw, y, st, nullptr, true, &y_padded)) != MSLA_OK) return s;

@@ -96,3 +96,30 @@ def test_workspaces_do_not_shrink_as_feature_maps_grow():
             for dtype in (binding.MSLA_BF16, binding.MSLA_F32):
                 small, large = answers(dtype, C, d, S, B0, H0, W0), answers(dtype, C, d, S, B1, H1, W1)
                 assert min(small) > 0 and all(a <= b for a, b in zip(small, large)), (B0, H0, W0, B1, H1, W1, C, d, S, dtype, small, large)
+
+
+def test_a_block_that_its_second_half_would_refuse_runs_nothing():
+    """The FFN's arguments are checked before the attention is launched (without a GPU: before the device is looked for)."""
+    import torch
+    lib = binding.lib()
+    B, C, H, W, d = 1, 64, 8, 8, 32
+    device = "cuda" if torch.cuda.is_available() else "cpu"
+    x, y, out = (torch.zeros(B, C, H, W, dtype=torch.bfloat16, device=device) for _ in range(3))
+    wt = torch.zeros(1 << 20, dtype=torch.bfloat16, device=device)
+    ws = torch.full((8 << 20,), 0xA5, dtype=torch.uint8, device=device)
+    base = (ws.data_ptr() + 255) // 256 * 256
+    desc = _desc(binding.MSLA_BF16, B, C, H, W, d)
+    desc.workspace, desc.workspace_bytes = base, lib.msla_forward_workspace_bytes(ctypes.byref(desc))
+    w, fw = binding.msla_weights(), binding.msla_ffn_weights()
+    w.w_qkv = w.w_dw = w.w_pw = w.w_proj = wt.data_ptr()
+    for w2, short, status in [(None, 0, 1), (wt.data_ptr() + 2, 0, 3), (wt.data_ptr(), 1, 4)]:
+        ffn = binding.make_ffn_desc(B, C, H, W, 4 * C, C, binding.MSLA_BF16, residual=True)
+        need = lib.msla_ffn_workspace_bytes(ctypes.byref(ffn))
+        ffn.workspace, ffn.workspace_bytes = base + (4 << 20), need - short
+        assert need <= 3 << 20
+        fw.w1, fw.w_dw, fw.w2 = wt.data_ptr(), wt.data_ptr(), w2
+        assert lib.msla_evit_block(ctypes.byref(desc), ctypes.byref(w), ctypes.byref(ffn), ctypes.byref(fw), x.data_ptr(), y.data_ptr(),
+                                   out.data_ptr(), None) == status
+    if device == "cuda":
+        torch.cuda.synchronize()
+    assert bool((ws == 0xA5).all())
