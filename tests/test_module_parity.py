@@ -318,7 +318,8 @@ def test_forward_host_above_the_planes_line(dtype, B, C, H, W, d, n_scales):
     weights = [rnd(3 * C, C), rnd(3 * C, 5, 5), rnd(3 * C, d), rnd(C, n_scales * C), None] + ([rnd(3 * C, 3, 3), rnd(3 * C, d)] if n_scales == 3 else [])
     w = binding.make_weights(*weights)
     make = lambda ws=None: binding.make_desc(B, C, H, W, C // d, d, C, util.CODE[dtype], n_scales=n_scales, agg_kernel2=3, workspace=ws)
-    desc = make(torch.empty(binding.msla_forward_host_workspace_bytes(make()), dtype=torch.uint8, device="cuda"))
+    ws = torch.empty(binding.msla_forward_host_workspace_bytes(make()), dtype=torch.uint8, device="cuda")
+    desc = make(ws)
     x = torch.randn(B, C, H, W, generator=gen, device="cuda").to(dt)
     ref = torch.empty_like(x)
     binding.msla_forward(desc, x, w, ref)
