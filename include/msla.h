@@ -12,6 +12,8 @@
  *     kernel was launched by that call (except MSLA_ERR_CUDA raised by a launch
  *     in the middle of a multi-kernel call).  msla_last_error() gives a
  *     thread-local detail string for the most recent failure on this thread.
+ *   - Work that the caller enqueued on `stream` before a call may write any tensor
+ *     passed to it, weights included.
  *   - All buffers are caller-owned.  The library keeps no pointer past the
  *     completion of the work it enqueued.  Outputs must not overlap inputs or
  *     the workspace (overlap is reported as MSLA_ERR_INVALID_ARG).

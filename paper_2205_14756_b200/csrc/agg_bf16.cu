@@ -111,7 +111,7 @@ struct ToeplitzParams {
   int groups;                  // blocks of 32 channels per image: plane `group` (d = 32) or planes 2*group, 2*group+1 (d = 16)
   int tiles_x, tiles_y, tiles_total;  // tiles per plane
   int B;
-  int taps_ready;              // 0: the taps come from the previous kernel (a 3x3 filter embedded in 5x5)
+  int weights_ready;           // 0: the taps come from the previous kernel (a 3x3 filter embedded in 5x5), or this one is the call's first
   long long units;             // groups * B * tiles_total, tile fastest
   long long units_per_cta;
 };
@@ -219,7 +219,7 @@ aggregate_toeplitz_kernel(const __grid_constant__ CUtensorMap tm_src, const __gr
       }
   };
   int cur_group = un.group;
-  if (!p.taps_ready) pdl_wait();
+  if (!p.weights_ready) pdl_wait();
   load_weights(cur_group);
 
   // Per-lane address offsets of the six ldmatrix loads of a channel.  Matrix (r, h) = staged rows
@@ -379,7 +379,7 @@ bool aggregate_bf16_supported(int H, int W, int Ch, int d) { return (d == 32 || 
 namespace {
 template <bool D16, bool F16>
 msla_status_t launch_toeplitz(const void* src, long long src_planes_total, int src_ppb, const void* w_dw, const void* w_pw,
-                              void* dst, long long dst_planes_total, int dst_ppb, int B, int H, int W, int Ch, cudaStream_t st, bool taps_ready) {
+                              void* dst, long long dst_planes_total, int dst_ppb, int B, int H, int W, int Ch, cudaStream_t st, bool weights_ready) {
   constexpr int DP = D16 ? 16 : 32;  // channels per plane
   CUtensorMap tm_src, tm_dst;
   {
@@ -395,7 +395,7 @@ msla_status_t launch_toeplitz(const void* src, long long src_planes_total, int s
   ToeplitzParams p;
   p.w_dw = (const bf16*)w_dw; p.w_pw = (const bf16*)w_pw;
   p.src_planes_per_batch = src_ppb; p.dst_planes_per_batch = dst_ppb; p.groups = Ch / TD;
-  p.B = B; p.taps_ready = taps_ready;
+  p.B = B; p.weights_ready = weights_ready;
   p.tiles_x = (W + TW - 1) / TW;
   p.tiles_y = (H + TH - 1) / TH;
   const long long tiles = (long long)p.tiles_x * p.tiles_y;
@@ -422,16 +422,16 @@ msla_status_t launch_toeplitz(const void* src, long long src_planes_total, int s
 // the plane size).
 msla_status_t run_aggregate_bf16(const void* src, long long src_planes_total, int src_ppb, const void* w_dw,
                                  const void* w_pw, void* dst, long long dst_sb, int B, int H, int W, int Ch, int d,
-                                 cudaStream_t st, bool f16, bool taps_ready) {
+                                 cudaStream_t st, bool f16, bool weights_ready) {
   const long long plane = (long long)H * W * d;
   if (!aggregate_bf16_supported(H, W, Ch, d) || dst_sb % plane != 0)
     return fail(MSLA_ERR_UNSUPPORTED, "aggregation: d = %d, %d channels, output batch stride %lld elements", d, Ch, dst_sb);
   const long long dst_ppb = dst_sb / plane, dst_total = (B - 1) * dst_ppb + Ch / d;
   if (f16)
-    return d == 16 ? launch_toeplitz<true, true>(src, src_planes_total, src_ppb, w_dw, w_pw, dst, dst_total, (int)dst_ppb, B, H, W, Ch, st, taps_ready)
-                   : launch_toeplitz<false, true>(src, src_planes_total, src_ppb, w_dw, w_pw, dst, dst_total, (int)dst_ppb, B, H, W, Ch, st, taps_ready);
-  return d == 16 ? launch_toeplitz<true, false>(src, src_planes_total, src_ppb, w_dw, w_pw, dst, dst_total, (int)dst_ppb, B, H, W, Ch, st, taps_ready)
-                 : launch_toeplitz<false, false>(src, src_planes_total, src_ppb, w_dw, w_pw, dst, dst_total, (int)dst_ppb, B, H, W, Ch, st, taps_ready);
+    return d == 16 ? launch_toeplitz<true, true>(src, src_planes_total, src_ppb, w_dw, w_pw, dst, dst_total, (int)dst_ppb, B, H, W, Ch, st, weights_ready)
+                   : launch_toeplitz<false, true>(src, src_planes_total, src_ppb, w_dw, w_pw, dst, dst_total, (int)dst_ppb, B, H, W, Ch, st, weights_ready);
+  return d == 16 ? launch_toeplitz<true, false>(src, src_planes_total, src_ppb, w_dw, w_pw, dst, dst_total, (int)dst_ppb, B, H, W, Ch, st, weights_ready)
+                 : launch_toeplitz<false, false>(src, src_planes_total, src_ppb, w_dw, w_pw, dst, dst_total, (int)dst_ppb, B, H, W, Ch, st, weights_ready);
 }
 
 int agg_timeout_flag() {

@@ -63,6 +63,7 @@ struct GemmParams {
   int plane_shift;        // log2 of the channels per TMA-stored output plane (5: planes of 32, 6: planes of 64)
   float act_a, act_b;     // EPI 1: act(v) = v * sat(v * act_a + act_b)
   const bf16* residual;   // EPI 2: a tensor laid out like the row-major output, added after the bias
+  int first;              // first kernel of a call: reads no weights before its wait (msla_common.cuh)
 };
 
 __device__ __forceinline__ void tile_coords(const GemmParams& p, int tile, int& b, int& mt, int& nt) {
@@ -239,7 +240,7 @@ gemm_bf16_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
   __shared__ int abort_flag;
   __shared__ uint32_t tmem_base_sh;
 
-  pdl_launch_dependents();
+  if (!p.first) pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int num_tiles = p.batches * p.m_tiles * p.n_tiles;
   const int k_iters = (p.K + BK - 1) / BK;
@@ -273,15 +274,16 @@ gemm_bf16_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         if (A_MN_MAJOR) tma_load_3d(sa + A_STAGE_BYTES, &tmB, bar, kb * BK, nt * TN, 0);
         else            tma_load_3d(sa, &tmA, bar, kb * BK, mt * BM, 0);  // one box of 64 k x 128 rows
       };
-      // the first stages' weights do not come from the previous kernel, the activations do
+      // the first stages' weights do not come from the previous kernel of the call, the activations do
       int b, mt, nt;
-      const int early = min(STAGES, k_iters);
+      const int early = p.first ? 0 : min(STAGES, k_iters);
       tile_coords(p, blockIdx.x, b, mt, nt);
       for (int kb = 0; kb < early; ++kb) {
         mbar_expect_tx(full_bar + 8 * kb, STAGE_BYTES);
         load_weights(smem_base + kb * STAGE_BYTES, full_bar + 8 * kb, kb, mt, nt);
       }
-      pdl_wait();
+      if (p.first) pdl_first_wait();
+      else pdl_wait();
       int it = 0;
       bool ok = true;
       for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x) {
@@ -416,13 +418,14 @@ gemm_bf16_stationary_kernel(const __grid_constant__ CUtensorMap tmA, const __gri
   const uint32_t res_bar = tempty_bar + 16, tmem_slot = res_bar + 8;
   __shared__ int abort_flag;
   __shared__ uint32_t tmem_base_sh;
-  __shared__ __align__(16) float bias_sm[EPI == 1 ? TN : 4];  // the CTA's column biases (weights: not the previous kernel's output)
+  __shared__ __align__(16) float bias_sm[EPI == 1 ? TN : 4];  // the CTA's column biases (weights: not the output of the call's previous kernel)
 
-  pdl_launch_dependents();
+  if (!p.first) pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int k_iters = (p.K + BK - 1) / BK;
   const int blk = blockIdx.x % blocks, worker = blockIdx.x / blocks;
   if (EPI == 1) {
+    if (p.first) pdl_wait();
     for (int i = threadIdx.x; i < TN; i += NUM_THREADS) {
       const int n = blk * TN + i;
       bias_sm[i] = (p.bias && !p.bias_per_row && n < p.N) ? (F16 ? ld16<true>(p.bias + n) : __bfloat162float(p.bias[n])) : 0.f;
@@ -458,10 +461,11 @@ gemm_bf16_stationary_kernel(const __grid_constant__ CUtensorMap tmA, const __gri
     if (lane == 0) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB) : "memory");
+      if (p.first) pdl_first_wait();
       // the resident weight block: all k-slices on one barrier
       mbar_expect_tx(res_bar, (uint32_t)(k_iters * RES_SLICE));
       for (int kb = 0; kb < k_iters; ++kb) tma_load_3d(res_base + kb * RES_SLICE, &tmB, res_bar, kb * BK, blk * TN, 0);
-      pdl_wait();  // the streamed operand may come from the previous kernel; the weights above do not
+      pdl_wait();  // the streamed operand may come from the previous kernel of the call; the weights above do not
       uint32_t it = 0;
       bool ok = true;
       for (int si = worker; ok && si < stream_total; si += workers) {
@@ -657,7 +661,7 @@ bool project_in_bf16_supported(int C, int Cout, int ldx, int d) {
 
 // y[b][o / d][n][o % d] = sum_c w[o][c] * x[b][c][n];  x [B, C, N] with rows ldx elements apart, y planar with batch stride y_sb.
 msla_status_t run_project_in_bf16(const void* x, int ldx, const void* w, void* y, int B, int C, int Cout, int N, int d,
-                                  long long y_sb, cudaStream_t st, bool f16) {
+                                  long long y_sb, cudaStream_t st, bool f16, bool first) {
   const InTile tile = in_tile(C, Cout, N, B);
   CUtensorMap tmA, tmB;
   if (!make_map(&tmA, x, (uint64_t)N, (uint64_t)C, (uint64_t)B, (uint64_t)ldx * 2, (uint64_t)C * ldx * 2, 64, BK) ||
@@ -667,7 +671,7 @@ msla_status_t run_project_in_bf16(const void* x, int ldx, const void* w, void* y
   p.M = N; p.N = Cout; p.K = C; p.batches = B;
   p.m_tiles = (N + BM - 1) / BM; p.n_tiles = (Cout + tile.tn - 1) / tile.tn;
   p.out_batch_stride = y_sb; p.ld_out = 0; p.group = d; p.bias_per_row = 0; p.n_fastest = 1;
-  p.bias = nullptr; p.out = (bf16*)y;
+  p.bias = nullptr; p.out = (bf16*)y; p.first = first;
   // planes of 32 channels are written as 32-token x 32-channel blocks by TMA
   CUtensorMap tmO = tmA;  // placeholder when the direct-store epilogue is used
   const long long plane_elems = (long long)N * 32;
@@ -688,7 +692,7 @@ bool project_out_bf16_supported(int Cin, int Cout, int ldy) { return Cin % 8 == 
 // y[b][m][n] = sum_j w[m][j] * a[b][n][j] + bias[m];  a token-major [B, N, Cin], y (and residual) [B, Cout, N] with rows ldy
 // elements apart.
 msla_status_t run_project_out_bf16(const void* a, const void* w, const void* bias, const void* residual, void* y, int ldy, int B, int Cin,
-                                   int Cout, int N, cudaStream_t st, bool f16) {
+                                   int Cout, int N, cudaStream_t st, bool f16, bool first) {
   const int tn = columns_out(Cout, N, B);
   CUtensorMap tmA, tmB;
   if (!make_map(&tmA, w, (uint64_t)Cin, (uint64_t)Cout, 1, (uint64_t)Cin * 2, (uint64_t)Cin * Cout * 2, BK, BM) ||
@@ -708,7 +712,7 @@ msla_status_t run_project_out_bf16(const void* a, const void* w, const void* bia
     if (!tma_make_map_bf16(&tmO, y, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B))
       return fail(MSLA_ERR_CUDA, "cuTensorMapEncodeTiled failed for the output projection's output");
   }
-  p.residual = (const bf16*)residual;
+  p.residual = (const bf16*)residual; p.first = first;
   if (f16) return residual ? launch_out<false, 2, true>(tmA, tmB, tmO, p, tn, st) : launch_out<false, 0, true>(tmA, tmB, tmO, p, tn, st);
   return residual ? launch_out<false, 2, false>(tmA, tmB, tmO, p, tn, st) : launch_out<false, 0, false>(tmA, tmB, tmO, p, tn, st);
 }
@@ -747,7 +751,7 @@ bool ffn_bf16_supported(int C, int Ch, int Cout) { return C % 8 == 0 && Ch % 64 
 // First layer: h[b][o / 32][n][o % 32] = act(sum_c w1[o][c] * x[b][c][n] + b1[o]); x rows ldx apart, h planes of 32 channels
 // (dense 2 KB per 32 tokens for the epilogue's TMA stores: half-line stores into 64-channel planes cost this GEMM 2x).
 msla_status_t run_ffn_expand_bf16(const void* x, int ldx, const void* w1, const void* b1, void* h, int B, int C, int Ch, int N, int act,
-                                  cudaStream_t st, bool f16) {
+                                  cudaStream_t st, bool f16, bool first) {
   const InTile tile = in_tile(C, Ch, N, B);
   CUtensorMap tmA, tmB, tmO;
   const cuuint64_t dims[3] = {32, (cuuint64_t)N, (cuuint64_t)B * (Ch / 32)};
@@ -765,7 +769,7 @@ msla_status_t run_ffn_expand_bf16(const void* x, int ldx, const void* w1, const 
   p.tma_store = 1; p.planes_per_batch = Ch / 32; p.plane_shift = 5;
   p.act_a = act == 2 ? 1.f / 6.f : (act == 1 ? 1e30f : 0.f);  // act(v) = v * sat(v * act_a + act_b)
   p.act_b = act == 2 ? 0.5f : (act == 1 ? 0.f : 1.f);
-  p.residual = nullptr;
+  p.residual = nullptr; p.first = first;
   return f16 ? launch_in<1, true>(tmA, tmB, tmO, p, tile, st) : launch_in<1, false>(tmA, tmB, tmO, p, tile, st);
 }
 

@@ -46,7 +46,7 @@ template <typename T> __device__ __forceinline__ float4 load4(const T* p) {
     return make_float4(to_f32(e[0]), to_f32(e[1]), to_f32(e[2]), to_f32(e[3]));
   }
 }
-// The same, and one element, of a tensor that an earlier kernel of the stream may have written.
+// The same, and one element, of a tensor that an earlier kernel of the stream may have written (the caller's weights among them).
 template <typename T> __device__ __forceinline__ float4 load4_dep(const T* p) {
   if constexpr (sizeof(T) == 4) {
     return ld_dep128f(p);
@@ -115,7 +115,7 @@ gemm_kernel(const T* __restrict__ A, const T* __restrict__ Wt, const T* __restri
   auto fetch_w = [&](int k0) {  // K is a multiple of 8: a vector exists whole or not at all
 #pragma unroll
     for (int i = 0; i < LW; ++i)
-      *reinterpret_cast<float4*>(rw[i]) = wn + i * (THREADS / KV) < n_left && k0 + wk < g.K ? load4(pw + (long long)i * stepW) : make_float4(0.f, 0.f, 0.f, 0.f);
+      *reinterpret_cast<float4*>(rw[i]) = wn + i * (THREADS / KV) < n_left && k0 + wk < g.K ? load4_dep(pw + (long long)i * stepW) : make_float4(0.f, 0.f, 0.f, 0.f);
     pw += BK;
   };
   auto fetch_a = [&](int k0) {  // FETCH_M4: rows are a multiple of four tokens
@@ -144,8 +144,8 @@ gemm_kernel(const T* __restrict__ A, const T* __restrict__ Wt, const T* __restri
       for (int v = 0; v < 4; ++v) Ws[buf][wk + v][wn + i * (THREADS / KV)] = rw[i][v];
   };
   unsigned long long acc2[TM / 2][TN] = {};  // pairs of tokens
+  pdl_wait();  // this may be the first kernel of a call, whose weights the kernel before it may have written
   fetch_w(0);
-  pdl_wait();  // the weights do not come from the previous kernel
   fetch_a(0);
   put(0);
   __syncthreads();
@@ -188,7 +188,7 @@ gemm_kernel(const T* __restrict__ A, const T* __restrict__ Wt, const T* __restri
     if (n >= g.Nc) continue;
     float bv[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) bv[j] = bias ? to_f32(bias[n + j]) : 0.f;
+    for (int j = 0; j < 4; ++j) bv[j] = bias ? load1_dep(bias + n + j) : 0.f;
     const long long at_n = (long long)(n / g.group) * g.sDg + (long long)(n % g.group) * g.sDn;  // four channels share a plane
 #pragma unroll
     for (int r = 0; r < TM / 4; ++r) {

@@ -398,8 +398,8 @@ static void launch_gemm(const T* A, const T* W, const T* bias, T* D, generic::Ge
 
 // y planar: y[b*y_sb + ((o/d)*N + n)*d + o%d]; rows of x are ldx elements apart (N where the plain kernels run)
 static msla_status_t run_project_in(msla_dtype_t dt, const void* x, int ldx, const void* w, void* y, int B,
-                                    int C, int Cout, int N, int d, long long y_sb, cudaStream_t st) {
-  if (dt != MSLA_F32 && project_in_bf16_supported(C, Cout, ldx, d)) return run_project_in_bf16(x, ldx, w, y, B, C, Cout, N, d, y_sb, st, dt == MSLA_F16);
+                                    int C, int Cout, int N, int d, long long y_sb, cudaStream_t st, bool first) {
+  if (dt != MSLA_F32 && project_in_bf16_supported(C, Cout, ldx, d)) return run_project_in_bf16(x, ldx, w, y, B, C, Cout, N, d, y_sb, st, dt == MSLA_F16, first);
   generic::GemmArgs g{(long long)C * N, 1, N, y_sb, d, 1, (long long)N * d, N, Cout, C, d};
   if (dt == MSLA_F32) launch_gemm<float>((const float*)x, (const float*)w, nullptr, (float*)y, g, B, st);
   else if (dt == MSLA_F16) launch_gemm<__half>((const __half*)x, (const __half*)w, nullptr, (__half*)y, g, B, st);
@@ -408,9 +408,9 @@ static msla_status_t run_project_in(msla_dtype_t dt, const void* x, int ldx, con
 }
 
 static msla_status_t run_project_out(msla_dtype_t dt, const void* a, const void* w, const void* bias,
-                                     void* y, int ldy, int B, int Cin, int Cout, int N, cudaStream_t st, const void* residual = nullptr) {
+                                     void* y, int ldy, int B, int Cin, int Cout, int N, cudaStream_t st, const void* residual = nullptr, bool first = false) {
   if (dt != MSLA_F32 && project_out_bf16_supported(Cin, Cout, ldy))
-    return run_project_out_bf16(a, w, bias, residual, y, ldy, B, Cin, Cout, N, st, dt == MSLA_F16);
+    return run_project_out_bf16(a, w, bias, residual, y, ldy, B, Cin, Cout, N, st, dt == MSLA_F16, first);
   generic::GemmArgs g{(long long)N * Cin, Cin, 1, (long long)Cout * N, 1, N, 0, N, Cout, Cin, Cout, 0, residual};
   if (dt == MSLA_F32) launch_gemm<float>((const float*)a, (const float*)w, (const float*)bias, (float*)y, g, B, st);
   else if (dt == MSLA_F16) launch_gemm<__half>((const __half*)a, (const __half*)w, (const __half*)bias, (__half*)y, g, B, st);
@@ -448,7 +448,7 @@ static msla_status_t run_aggregate_plain(const void* src, const void* w_dw, cons
 // src, dst planar [B, Ch/d, H*W, d] with batch strides src_sb, dst_sb (elements)
 static msla_status_t run_aggregate(msla_dtype_t dt, const void* src, const void* w_dw, const void* w_pw,
                                    void* dst, int B, int H, int W, int Ch, int d, long long src_sb,
-                                   long long dst_sb, cudaStream_t st, bool taps_ready = true) {
+                                   long long dst_sb, cudaStream_t st, bool weights_ready) {
   if (dt == MSLA_F32) return run_aggregate_plain<float>(src, w_dw, w_pw, dst, B, H, W, Ch / d, d, src_sb, dst_sb, st);
   const long long plane = (long long)H * W * d;
   const bool f16 = dt == MSLA_F16;
@@ -458,7 +458,7 @@ static msla_status_t run_aggregate(msla_dtype_t dt, const void* src, const void*
     else if (d == 16 && Ch > 16 && aggregate_bf16_supported(H, W, Ch - 16, d)) done = Ch - 16;
   }
   if (done) {
-    const msla_status_t s = run_aggregate_bf16(src, (long long)B * (src_sb / plane), (int)(src_sb / plane), w_dw, w_pw, dst, dst_sb, B, H, W, done, d, st, f16, taps_ready);
+    const msla_status_t s = run_aggregate_bf16(src, (long long)B * (src_sb / plane), (int)(src_sb / plane), w_dw, w_pw, dst, dst_sb, B, H, W, done, d, st, f16, weights_ready);
     if (s != MSLA_OK || done == Ch) return s;
   }
   const size_t first = (size_t)(done / d) * plane * 2;
@@ -626,7 +626,7 @@ static msla_status_t forward_impl(const msla_desc* desc, const void* x, const ms
     return record(events, 5, st);
   }
   // 1. QKV projection into the scale-0 planes
-  s = run_project_in(desc->dtype, x_dev, p.pitch, w->w_qkv, ms, desc->B, desc->C, 3 * Cp, N, d, ms_sb, st);
+  s = run_project_in(desc->dtype, x_dev, p.pitch, w->w_qkv, ms, desc->B, desc->C, 3 * Cp, N, d, ms_sb, st, !p.padded());
   if (s != MSLA_OK) return s;
   if ((s = record(events, 1, st)) != MSLA_OK) return s;
   // 2. aggregation of every scale-0 plane into the matching scale-1 plane
@@ -818,7 +818,7 @@ static msla_status_t band_states_impl(const msla_desc* desc, const void* x, cons
     if ((s = run_planes_branches(desc, w, p, halo_top, desc->H - halo_bottom, st)) != MSLA_OK) return s;
     return run_sum_states(planes_states(desc, w, p), state_out, desc->B, desc->heads, p.S * desc->heads, d, st, f16);
   }
-  s = run_project_in(desc->dtype, x, p.pitch, w->w_qkv, ms, desc->B, desc->C, 3 * Cp, N, d, ms_sb, st);
+  s = run_project_in(desc->dtype, x, p.pitch, w->w_qkv, ms, desc->B, desc->C, 3 * Cp, N, d, ms_sb, st, !p.padded());
   if (s != MSLA_OK) return s;
   if ((s = run_branches(desc, w, p, ms, ms_sb, st)) != MSLA_OK) return s;
   const HeadView in{ms_sb, 3LL * N * d, d};
@@ -942,9 +942,9 @@ static msla_status_t check_ffn_args(const msla_ffn_desc* desc, const FfnPlan& p,
   return MSLA_OK;
 }
 
-// x_padded: a copy of x with rows of the plan's pitch that the caller already has, or nullptr.
+// first: no kernel of the same call precedes.  x_padded: a copy of x with rows of the plan's pitch that the caller already has, or nullptr.
 static msla_status_t ffn_impl(const msla_ffn_desc* desc, const void* x, const msla_ffn_weights* w, void* out, bool residual,
-                              cudaStream_t st, const void* x_padded = nullptr) {
+                              cudaStream_t st, bool first, const void* x_padded = nullptr) {
   FfnPlan p;
   msla_status_t s = validate_ffn(desc, &p);
   if (s != MSLA_OK) return s;
@@ -965,7 +965,7 @@ static msla_status_t ffn_impl(const msla_ffn_desc* desc, const void* x, const ms
       x = x_padded;
       y = ws + p.ypad_off;
     }
-    if ((s = run_ffn_expand_bf16(x, p.pitch, w->w1, w->b1, h, B, C, Ch, N, act, st, f16)) != MSLA_OK) return s;
+    if ((s = run_ffn_expand_bf16(x, p.pitch, w->w1, w->b1, h, B, C, Ch, N, act, st, f16, first && !p.padded())) != MSLA_OK) return s;
     if ((s = run_ffn_dw3x3_bf16(h, w->w_dw, w->b_dw, g, B, Ch, desc->H, desc->W, act, st, f16)) != MSLA_OK) return s;
     if ((s = run_ffn_project_bf16(g, w->w2, w->b2, residual ? x : nullptr, y, p.pitch, B, Ch, Co, N, st, f16)) != MSLA_OK) return s;
     return p.padded() ? run_unpad_rows(y, out, (long long)B * Co, N, p.pitch, st) : MSLA_OK;
@@ -1012,7 +1012,7 @@ static msla_status_t block_impl(const msla_desc* attn, const msla_weights* aw, c
   if ((s = forward_impl(attn, x, aw, y, st, nullptr, true, &y_padded)) != MSLA_OK) return s;
   // y with padded rows still lies in the attention's workspace, unless the FFN works in the same memory
   const bool keep = ap.padded() && !overlaps(attn->workspace, ap.bytes, ffn->workspace, fp.bytes);
-  return ffn_impl(ffn, y, fw, out, true, st, keep ? y_padded : nullptr);
+  return ffn_impl(ffn, y, fw, out, true, st, false, keep ? y_padded : nullptr);
 }
 
 }  // namespace msla
@@ -1093,7 +1093,7 @@ size_t msla_ffn_workspace_bytes(const msla_ffn_desc* desc) {
 }
 
 msla_status_t msla_ffn_dwconv(const msla_ffn_desc* desc, const void* x, const msla_ffn_weights* w, void* out, void* stream) {
-  return ffn_impl(desc, x, w, out, desc && desc->residual, (cudaStream_t)stream);
+  return ffn_impl(desc, x, w, out, desc && desc->residual, (cudaStream_t)stream, true);
 }
 
 msla_status_t msla_evit_block(const msla_desc* attn, const msla_weights* aw, const msla_ffn_desc* ffn, const msla_ffn_weights* fw,
@@ -1135,7 +1135,7 @@ msla_status_t msla_project_in(msla_dtype_t dtype, const void* x, const void* w, 
   if (!aligned16(x) || !aligned16(w) || !aligned16(y)) return fail(MSLA_ERR_ALIGNMENT, "pointers must be 16-byte aligned");
   msla_status_t s = check_arch();
   if (s != MSLA_OK) return s;
-  return run_project_in(dtype, x, N, w, y, B, C, Cout, N, d, (long long)Cout * N, (cudaStream_t)stream);
+  return run_project_in(dtype, x, N, w, y, B, C, Cout, N, d, (long long)Cout * N, (cudaStream_t)stream, true);
 }
 
 msla_status_t msla_aggregate(msla_dtype_t dtype, const void* t, const void* w_dw, const void* w_pw, void* y, int B, int H, int W, int Ch, int d, void* stream) {
@@ -1151,7 +1151,7 @@ msla_status_t msla_aggregate(msla_dtype_t dtype, const void* t, const void* w_dw
   if (overlaps(t, bytes, y, bytes)) return fail(MSLA_ERR_INVALID_ARG, "y overlaps t");
   msla_status_t s = check_arch();
   if (s != MSLA_OK) return s;
-  return run_aggregate(dtype, t, w_dw, w_pw, y, B, H, W, Ch, d, (long long)Ch * H * W, (long long)Ch * H * W, (cudaStream_t)stream);
+  return run_aggregate(dtype, t, w_dw, w_pw, y, B, H, W, Ch, d, (long long)Ch * H * W, (long long)Ch * H * W, (cudaStream_t)stream, false);
 }
 
 msla_status_t msla_project_out(msla_dtype_t dtype, const void* a, const void* w, const void* bias, void* y, int B, int Cin, int Cout, int N, void* stream) {
@@ -1162,7 +1162,7 @@ msla_status_t msla_project_out(msla_dtype_t dtype, const void* a, const void* w,
   if (!aligned16(a) || !aligned16(w) || !aligned16(y) || (bias && !aligned16(bias))) return fail(MSLA_ERR_ALIGNMENT, "pointers must be 16-byte aligned");
   msla_status_t s = check_arch();
   if (s != MSLA_OK) return s;
-  return run_project_out(dtype, a, w, bias, y, N, B, Cin, Cout, N, (cudaStream_t)stream);
+  return run_project_out(dtype, a, w, bias, y, N, B, Cin, Cout, N, (cudaStream_t)stream, nullptr, true);
 }
 
 const char* msla_status_string(msla_status_t s) {

@@ -40,10 +40,22 @@ template <> __device__ __forceinline__ __half from_f32<__half>(float v) { return
 // memory, tables built from the weights) and then waits here, which returns
 // once the predecessor has finished and its writes are visible.  Every global
 // read of an earlier kernel's output, and every global write, comes after it.
+//
+// The caller's tensors, weights among them, may be written by work that the caller
+// put on the stream just before the call.  So the first kernel of a call reads none of
+// them before its own pdl_wait(), and lets its successor start only after it
+// (pdl_first_wait()): when a later kernel of the call runs at all, the work before
+// the call is complete and visible, and it may fetch weights before it waits.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the next kernel of the stream be scheduled as soon as every CTA of this
 // one has started (it still waits in pdl_wait for this kernel's completion).
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// The wait of a call's first kernel, by one thread of every CTA at least.
+__device__ __forceinline__ void pdl_first_wait() {
+  pdl_wait();
+  pdl_launch_dependents();
+}
 
 // Loads of data that an earlier kernel of the stream wrote, in kernels that may have become resident while it ran.  They are
 // ordered after pdl_wait() (both are volatile) and are plain loads: the read-only path (__ldg, and what the compiler makes of

@@ -106,8 +106,9 @@ msla_status_t run_core_bf16(const void* q, const void* k, const void* v, void* o
 // act: 0 none, 1 ReLU, 2 hard-swish.
 bool ffn_bf16_supported(int C, int Ch, int Cout);
 // ldx, ldy: elements between rows (tokens of one channel) of x, and of y and the residual; multiples of 8, as tensor maps need.
+// first: first kernel of a call (msla_common.cuh).
 msla_status_t run_ffn_expand_bf16(const void* x, int ldx, const void* w1, const void* b1, void* h, int B, int C, int Ch, int N, int act,
-                                  cudaStream_t st, bool f16 = false);
+                                  cudaStream_t st, bool f16, bool first);
 msla_status_t run_ffn_dw3x3_bf16(const void* h, const void* w_dw, const void* b_dw, void* g, int B, int Ch, int H, int W, int act,
                                  cudaStream_t st, bool f16 = false);
 msla_status_t run_ffn_project_bf16(const void* g, const void* w2, const void* b2, const void* residual, void* y, int ldy, int B, int Ch,
@@ -124,11 +125,11 @@ int dw_timeout_flag();
 // bf16 projections on tcgen05 tensor cores (gemm_tcgen05.cu).
 bool project_in_bf16_supported(int C, int Cout, int ldx, int d);
 msla_status_t run_project_in_bf16(const void* x, int ldx, const void* w, void* y, int B, int C, int Cout, int N, int d,
-                                  long long y_batch_stride, cudaStream_t st, bool f16 = false);
+                                  long long y_batch_stride, cudaStream_t st, bool f16, bool first);
 bool project_out_bf16_supported(int Cin, int Cout, int ldy);
 // residual: nullptr, or a tensor shaped like y that is added to it
 msla_status_t run_project_out_bf16(const void* a, const void* w, const void* bias, const void* residual, void* y, int ldy, int B, int Cin,
-                                   int Cout, int N, cudaStream_t st, bool f16 = false);
+                                   int Cout, int N, cudaStream_t st, bool f16, bool first);
 bool project_out_planar_bf16_supported(int Cin, int Cout);
 msla_status_t run_project_out_planar_bf16(const void* a, const void* w, const void* bias, const void* residual, void* y, int ldy, int B,
                                           int Cin, int Cout, int N, cudaStream_t st, bool f16 = false);
@@ -136,11 +137,11 @@ int gemm_timeout_flag();
 int run_wait_selftest(long long limit_cycles, int* scratch, cudaStream_t st);
 
 // bf16 aggregation (d = 16 or 32, Ch a multiple of 32): TMA halo tiles, depthwise filter as banded matrices on
-// tensor cores (agg_bf16.cu).  taps_ready: w_dw is not the previous kernel's output.  dst_sb must be a multiple of the plane size H*W*d.
+// tensor cores (agg_bf16.cu).  weights_ready: an earlier kernel of the call has waited, and none of its wrote w_dw.  dst_sb must be a multiple of the plane size H*W*d.
 bool aggregate_bf16_supported(int H, int W, int Ch, int d);
 msla_status_t run_aggregate_bf16(const void* src, long long src_planes_total, int src_ppb, const void* w_dw,
                                  const void* w_pw, void* dst, long long dst_sb, int B, int H, int W, int Ch, int d,
-                                 cudaStream_t st, bool f16, bool taps_ready);
+                                 cudaStream_t st, bool f16, bool weights_ready);
 int agg_timeout_flag();
 
 // Rows of n 16-bit elements to and from rows `pitch` (a multiple of 8) elements apart (repack.cu).
@@ -177,7 +178,7 @@ msla_status_t run_agg_state(const void* ms0, void* q1, float* partial, const voi
                             int heads, int H, int W, int d, int row_lo, int row_hi, bool with_scale0, cudaStream_t st, bool f16);
 int agg_state_timeout_flag();
 
-// Input projection into scale-0 planes (proj_planes.cu): x [B][C][Np], Np a multiple of 8.
+// Input projection into scale-0 planes (proj_planes.cu), the first kernel of its call: x [B][C][Np], Np a multiple of 8.
 msla_status_t run_project_planes(const void* x, const void* w, void* y, int B, int C, int Cout, int Np, int d, long long y_sb, cudaStream_t st, bool f16);
 int project_planes_timeout_flag();
 

@@ -63,7 +63,6 @@ project_planes_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
   __shared__ int abort_flag;
   __shared__ uint32_t tmem_base_sh;
 
-  pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int blk = blockIdx.x % p.blocks, worker = blockIdx.x / p.blocks;
 
@@ -73,10 +72,6 @@ project_planes_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar + 8 * a, 1); mbar_init(tempty_bar + 8 * a, 8); }
     mbar_init(res_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    if (!STREAM) {  // the resident weights do not come from the previous kernel
-      mbar_expect_tx(res_bar, (uint32_t)(k_iters * HALVES * PP_W_SLICE));
-      for (int kb = 0; kb < k_iters; ++kb) tma_load_3d(smem_base + kb * (HALVES * PP_W_SLICE), &tmW, res_bar, kb * PP_BK, blk * ROWS, 0);
-    }
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tmem_slot), "r"(512) : "memory");
@@ -96,7 +91,11 @@ project_planes_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
   if (warp == 0) {
     // ------------------------------------------------------------ copies
     if (lane == 0) {
-      pdl_wait();  // x may be the previous kernel's output
+      pdl_first_wait();
+      if (!STREAM) {
+        mbar_expect_tx(res_bar, (uint32_t)(k_iters * HALVES * PP_W_SLICE));
+        for (int kb = 0; kb < k_iters; ++kb) tma_load_3d(smem_base + kb * (HALVES * PP_W_SLICE), &tmW, res_bar, kb * PP_BK, blk * ROWS, 0);
+      }
       uint32_t s = 0, ph = 0;
       bool ok = true;
       for (int tile = worker; ok && tile < p.tiles; tile += p.workers) {

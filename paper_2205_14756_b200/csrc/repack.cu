@@ -32,8 +32,7 @@ __device__ __forceinline__ uint4 load8(const unsigned short* __restrict__ src, l
 // dst[row][0 .. pitch) <- src[row][0 .. n); the padding holds elements of the next row (no reader looks at it).
 __global__ void __launch_bounds__(RP_THREADS)
 pad_rows_kernel(const unsigned short* __restrict__ src, uint4* __restrict__ dst, int n, int pieces, long long total, long long count) {
-  pdl_launch_dependents();
-  pdl_wait();
+  pdl_first_wait();  // the first kernel of its call
   const long long i = (long long)blockIdx.x * RP_THREADS + threadIdx.x;
   if (i >= count) return;
   const long long row = count <= 0xffffffffLL ? (uint32_t)i / (uint32_t)pieces : i / pieces;

@@ -331,6 +331,60 @@ def test_forward_host_above_the_planes_line(dtype, B, C, H, W, d, n_scales):
     assert binding.msla_debug_wait_timeouts() == 0
 
 
+# Weights written by the kernel right before the call, one that lets the next kernel start early (the library's own output projection:
+# a product with the identity copies).  Every first kernel: each projection's, ragged rows, planes, fp32; the FFN's; the stages'.
+def _written_on_stream(dtype, w):
+    """w [R, K], K a multiple of 8, through a kernel of the library into memory that held something else."""
+    R, K = w.shape
+    eye, dst = torch.eye(K, device="cuda", dtype=w.dtype), torch.full_like(w, 3.0)
+    torch.cuda.synchronize()
+    return dst, lambda: binding.msla_project_out(util.CODE[dtype], eye, w, None, dst, 1, K, R, K)
+
+
+@pytest.mark.parametrize("dtype,B,C,H,W,heads,d", [("f32", 1, 64, 16, 16, 4, 16), ("bf16", 1, 256, 32, 32, 8, 32), ("bf16", 1, 520, 16, 16, 2, 32), ("f16", 2, 64, 7, 7, 2, 32),
+                                                   ("bf16", 2, 128, 160, 136, 4, 32), ("bf16", 1, 264, 128, 168, 8, 32)])
+@pytest.mark.parametrize("name", ["w_qkv", "w_proj"])
+def test_weights_written_just_before_the_call(dtype, B, C, H, W, heads, d, name):
+    dt, k = util.TORCH_DTYPE[dtype], heads * d
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    rnd = lambda *shape: (torch.randn(*shape, generator=gen, device="cuda") * shape[-1] ** -0.5).to(dt)
+    tensors = {"w_qkv": rnd(3 * k, C), "w_dw": rnd(3 * k, 5, 5), "w_pw": rnd(3 * k, d), "w_proj": rnd(C, 2 * k)}
+    x = torch.randn(B, C, H, W, generator=gen, device="cuda").to(dt)
+    make = lambda ws=None: binding.make_desc(B, C, H, W, heads, d, C, util.CODE[dtype], workspace=ws)
+    ws = torch.empty(binding.msla_forward_workspace_bytes(make()), dtype=torch.uint8, device="cuda")
+    desc = make(ws)
+    ref, out = torch.empty_like(x), torch.empty_like(x)
+    binding.msla_forward(desc, x, binding.make_weights(**tensors), ref)
+    for _ in range(5):
+        late, write = _written_on_stream(dtype, tensors[name])
+        write()
+        binding.msla_forward(desc, x, binding.make_weights(**dict(tensors, **{name: late})), out)
+        torch.cuda.synchronize()
+        assert torch.equal(out, ref)
+
+
+@pytest.mark.parametrize("dtype,C,H,W,Ch", [("bf16", 64, 16, 24, 256), ("f16", 96, 7, 7, 128), ("f32", 32, 8, 8, 64)])
+def test_ffn_weights_written_just_before_the_call(dtype, C, H, W, Ch):
+    dt = util.TORCH_DTYPE[dtype]
+    gen = torch.Generator(device="cuda").manual_seed(10)
+    rnd = lambda *shape: (torch.randn(*shape, generator=gen, device="cuda") * shape[-1] ** -0.5).to(dt)
+    w1, w_dw, w2, b1 = rnd(Ch, C), rnd(Ch, 3, 3), rnd(C, Ch), rnd(8, Ch)
+    x = torch.randn(1, C, H, W, generator=gen, device="cuda").to(dt)
+    make = lambda ws=None: binding.make_ffn_desc(1, C, H, W, Ch, C, util.CODE[dtype], binding.MSLA_ACT_HARDSWISH, True, workspace=ws)
+    ws = torch.empty(binding.msla_ffn_workspace_bytes(make()), dtype=torch.uint8, device="cuda")
+    desc = make(ws)
+    ref, out = torch.empty_like(x), torch.empty_like(x)
+    binding.msla_ffn_dwconv(desc, x, binding.make_ffn_weights(w1, w_dw, w2, b1), ref)
+    for i in range(6):
+        late, write = _written_on_stream(dtype, (w1, w2, b1)[i % 3])
+        write()
+        given = [w1, w_dw, w2, b1]
+        given[(0, 2, 3)[i % 3]] = late
+        binding.msla_ffn_dwconv(desc, x, binding.make_ffn_weights(*given), out)
+        torch.cuda.synchronize()
+        assert torch.equal(out, ref)
+
+
 # The projections' kernels take 64 to 256 output columns per tile by problem size: each width, with remainders on both sides, rows
 # of up to 512 channels in the kernel that keeps its weights and longer ones in the one that streams them.
 @pytest.mark.parametrize("dtype,B,C,Cout,N", [("bf16", 1, 64, 176, 136), ("f16", 1, 72, 384, 5112), ("bf16", 1, 128, 352, 8952), ("bf16", 5, 40, 464, 7096),
