@@ -36,17 +36,8 @@ __device__ __forceinline__ float act_f32(float v, int act) {
   return v;
 }
 
-// Four consecutive elements, aligned to their total size.
-template <typename T> __device__ __forceinline__ float4 load4(const T* p) {
-  if constexpr (sizeof(T) == 4) {
-    return __ldg(reinterpret_cast<const float4*>(p));
-  } else {
-    const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
-    const T* e = reinterpret_cast<const T*>(&v);
-    return make_float4(to_f32(e[0]), to_f32(e[1]), to_f32(e[2]), to_f32(e[3]));
-  }
-}
-// The same, and one element, of a tensor that an earlier kernel of the stream may have written (the caller's weights among them).
+// Four consecutive elements, aligned to their total size, and one element, of a tensor that an earlier kernel of the stream may have
+// written (the caller's weights among them).
 template <typename T> __device__ __forceinline__ float4 load4_dep(const T* p) {
   if constexpr (sizeof(T) == 4) {
     return ld_dep128f(p);
@@ -285,7 +276,7 @@ aggregate_kernel(const T* __restrict__ src, const T* __restrict__ w_dw, const T*
   float taps[25];
   pdl_wait();  // the planes come from the previous kernel, and the taps may (a 3x3 filter embedded in 5x5)
 #pragma unroll
-  for (int i = 0; i < 25; ++i) taps[i] = to_f32(__ldg(w_dw + (long long)(ch0 + c) * 25 + i));
+  for (int i = 0; i < 25; ++i) taps[i] = load1_dep(w_dw + (long long)(ch0 + c) * 25 + i);
   const T* sb = src + (long long)b * src_sb + (long long)blockIdx.y * H * W * D;
 #pragma unroll 8
   for (int e = tid; e < HH * HW_ * CV; e += THREADS) {
@@ -322,7 +313,7 @@ aggregate_kernel(const T* __restrict__ src, const T* __restrict__ w_dw, const T*
   float pw[D];
 #pragma unroll
   for (int i = 0; i < D; i += 4) {
-    const float4 v = load4(w_pw + (long long)(ch0 + c) * D + i);
+    const float4 v = load4_dep(w_pw + (long long)(ch0 + c) * D + i);
     pw[i] = v.x; pw[i + 1] = v.y; pw[i + 2] = v.z; pw[i + 3] = v.w;
   }
   __syncthreads();  // the staged tile has been read

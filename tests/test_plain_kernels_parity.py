@@ -28,3 +28,29 @@ def test_ffn_on_the_plain_kernels(dtype, B, C, H, W, Ch):
     t = inputs.ffn_inputs(s)
     ref = oracle.ffn_dwconv(t["x"], t["w1"], t["w_dw"], t["w2"], t["b1"], t["b_dw"], t["b2"], act="hardswish", residual=True)
     util.assert_close(util.run_ffn(s, t, "hardswish", True), ref, dtype, "FFN on the plain kernels")
+
+
+# 3x3 filters, embedded in 5x5 by the kernel before the aggregation: other filters from call to call on one workspace, fp32 and the
+# 16-bit group that the tensor-core kernel leaves (d = 16, an odd number of groups).  A tap of an earlier call would show.
+@pytest.mark.parametrize("dtype,heads,d", [("f32", 4, 16), ("f32", 2, 32), ("bf16", 1, 16), ("f16", 3, 16)])
+def test_embedded_taps_change_from_call_to_call(dtype, heads, d):
+    import torch
+    from paper_2205_14756_b200 import binding
+    C, k, H, W = 64, heads * d, 24, 20
+    make = lambda ws=None: binding.make_desc(1, C, H, W, heads, d, C, util.CODE[dtype], agg_kernel=3, workspace=ws)
+    ws = torch.zeros(binding.msla_forward_workspace_bytes(make()), dtype=torch.uint8, device="cuda")
+    desc = make(ws)
+    shapes = []
+    for seed in (73, 74):
+        s = inputs.ModuleShape("taps", dtype, 1, C, H, W, heads, d, seed=seed, agg_kernel=3)
+        t = inputs.module_inputs(s)
+        ref = oracle.msla_forward(t["x"], t["w_qkv"], t["w_dw"], t["w_pw"], t["w_proj"], heads=heads, d=d, eps=s.eps)
+        shapes.append(([util.dev(t[n], dtype) for n in ("x", "w_qkv", "w_dw", "w_pw", "w_proj")], ref))
+    outs = []
+    for i in range(20):
+        (x, *w), ref = shapes[i % 2]
+        outs.append((torch.empty_like(x), ref))
+        binding.msla_forward(desc, x, binding.make_weights(*w), outs[-1][0])
+    torch.cuda.synchronize()
+    for out, ref in outs:
+        util.assert_close(util.host(out), ref, dtype, "embedded taps", block=util.MODULE_BLOCK)
