@@ -69,7 +69,7 @@ constexpr int O_BAR_BYTES = 512;
 constexpr int O_KS_BYTES = O_MAX_KS * OKS * 4;  // the image's key sums
 constexpr int O_SMEM_FIXED = O_STAGING + O_BAR_BYTES + O_KS_BYTES;  // besides the rows of M, the ring and the residual blocks
 constexpr int O_SMEM_LIMIT = 227 * 1024;                     // all of it dynamic
-static_assert(24 * O_MAX_STAGES + 16 + 16 + 8 + 8 + 8 + 4 * 8 + 8 + 8 + 8 <= O_BAR_BYTES, "barrier block");
+static_assert(24 * O_MAX_STAGES + 16 + 16 + 8 + 8 + 8 + 4 * 8 + 8 + 8 + 8 + 8 <= O_BAR_BYTES, "barrier block");
 
 __device__ int g_fused_timeout_flag = 0;
 
@@ -433,7 +433,8 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
   const uint32_t mfree_bar = resid_bar + 32;             // the MMAs of an image are complete: its rows of M may be replaced (commit, both CTAs)
   const uint32_t ks_bar = mfree_bar + 8;                 // the image's key sums landed (own CTA)
   const uint32_t ks_sm = bars + O_BAR_BYTES;
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_raw + (ks_bar + 8 - smem_base));
+  const uint32_t kseen_bar = ks_bar + 8;                 // every transform warp has seen the image's key sums land (own CTA)
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_raw + (kseen_bar + 8 - smem_base));
 
   pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -455,6 +456,7 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
     mbar_init(peer_res_bar, 1);
     mbar_init(mfree_bar, 1);
     mbar_init(ks_bar, 1);
+    mbar_init(kseen_bar, O_XWARPS);
     if (RES)
       for (int w = 0; w < 4; ++w) mbar_init(resid_bar + 8 * w, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -528,6 +530,10 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
             // sums).  The accumulators' barriers cannot tell: a parity two phases back looks complete.
             ok = mbar_wait_cluster(mfree_bar, mfree_ph, abort_flag);
             if (!ok) break;
+            // Nor does a group of transform warps that took no slice of that image (two heads, one tile) hold anything back: without its
+            // sign-off it could find ks_bar a phase further on, and wait for good.
+            ok = mbar_wait(kseen_bar, mfree_ph, abort_flag);
+            if (!ok) break;
             mfree_ph ^= 1;
           }
           cur_b = b;
@@ -598,6 +604,7 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         ks_ph ^= 1;
+        if (lane == 0) mbar_arrive(kseen_bar);
       }
       for (int h = 0; ok && h < h_end; ++h) {
         const uint32_t cs = s, cph = ph;  // this slice's slot; the counters move on to the next slice

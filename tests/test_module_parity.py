@@ -277,6 +277,18 @@ def test_many_images_with_few_heads(B, C, H, W, heads, d):
     assert binding.msla_debug_wait_timeouts() == 0
 
 
+# Two heads (one per branch) and one tile per image, several images per pair of CTAs: one of the three transform groups of the fused
+# apply + projection kernel has no slice of an image.
+@pytest.mark.parametrize("dtype,B,C,H,W,d", [("bf16", 128, 32, 14, 14, 32), ("f16", 300, 32, 16, 16, 32), ("bf16", 700, 8, 8, 8, 32)])
+def test_many_images_of_one_tile_with_two_heads(dtype, B, C, H, W, d):
+    s = inputs.ModuleShape("two_heads", dtype, B, C, H, W, 1, d, seed=46)
+    t = inputs.module_inputs(s)
+    ref = _ref(s, t)
+    for _ in range(3):
+        util.assert_close(util.run_module(s, t), ref, dtype, "two heads", block=util.MODULE_BLOCK)
+    assert binding.msla_debug_wait_timeouts() == 0
+
+
 # Host buffers large enough to go through in parts of whole images (copies overlapped with the kernels): equal bit for bit to
 # the call on device tensors, also when calls follow one another on one workspace and when the last part is a small one.
 @pytest.mark.parametrize("dtype,B,C,H,W,heads,d", [("bf16", 7, 64, 64, 96, 2, 32), ("f32", 5, 32, 96, 65, 2, 16), ("f16", 9, 64, 57, 71, 4, 16)])
