@@ -237,7 +237,7 @@ agg_state_kernel(const __grid_constant__ CUtensorMap kv_even, const __grid_const
   constexpr int NJ = D / 8;          // 8-channel column blocks of a state
   extern __shared__ unsigned char smem_raw[];
   const uint32_t box = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  __shared__ __align__(8) unsigned long long bar_storage[24];
+  __shared__ __align__(8) unsigned long long bar_storage[25];
   __shared__ int abort_flag;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
@@ -272,6 +272,7 @@ agg_state_kernel(const __grid_constant__ CUtensorMap kv_even, const __grid_const
   auto dwo_freed = [&](int role, uint32_t buf) { return bars + 64 * role + (role ? 80 : 48) + 8 * buf; };
   auto staged = [&](uint32_t buf) { return bars + 160 + 8 * buf; };       // queries: the output tile is staged / has been copied out
   auto staging_freed = [&](uint32_t buf) { return bars + 176 + 8 * buf; };
+  const uint32_t sums_meet = bars + 192;                                  // the summing warps, twice per (head, image)
   pdl_launch_dependents();
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -289,6 +290,7 @@ agg_state_kernel(const __grid_constant__ CUtensorMap kv_even, const __grid_const
       mbar_init(staged(i), AS_SUM_WARPS);
       mbar_init(staging_freed(i), 1);
     }
+    mbar_init(sums_meet, AS_SUM_WARPS);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
@@ -644,7 +646,8 @@ agg_state_kernel(const __grid_constant__ CUtensorMap kv_even, const __grid_const
           if (t == 0) mine[(e & 1) * AS_SUM_WARPS * 16 * (D + 1) + r * (D + 1) + D] = accs[e];
         }
         clear();
-        asm volatile("bar.sync 1, %0;" ::"n"(32 * AS_SUM_WARPS) : "memory");
+        arrive(sums_meet);  // a bounded wait here too: a warp that has given up does not come
+        if (!wait(sums_meet, 0)) break;
         // [state][mh][r][c] of the block: d = 32: rows 16 mh + r of one head's states; d = 16: rows r of head mh's
         float* out = p.partial + ((long long)pb + blockIdx.x) * (HPB * 2 * NE);
         for (int e = threadIdx.x - 32 * AS_DW_WARPS; e < HPB * 2 * NE; e += 32 * AS_SUM_WARPS) {
@@ -656,7 +659,8 @@ agg_state_kernel(const __grid_constant__ CUtensorMap kv_even, const __grid_const
           for (int w = 1; w < 4; ++w) sum += src[w * 16 * (D + 1)];
           out[e] = sum;
         }
-        asm volatile("bar.sync 1, %0;" ::"n"(32 * AS_SUM_WARPS) : "memory");
+        arrive(sums_meet);
+        if (!wait(sums_meet, 1)) break;
       }
     }
     if (end_of_kv()) {
