@@ -258,7 +258,7 @@ kv_combine_bf16path_kernel(const float* __restrict__ partial, float* __restrict_
 // into 16-bit pieces; the quotient of Eq. 3 does not change.  1 for bf16 (its exponent range is fp32's); for fp16 a
 // power of two near 1/N, so that sums over N tokens fit the format.
 // state: [heads of all images][S][D][D+1], S partial states per head that every CTA adds for itself, in index order (S = 1: the
-// state).  With few of them that costs less than a kernel of its own for the sum: see launch_core.
+// state; PAIR and PLANES: always).  With few of them that costs less than a kernel of its own for the sum: see launch_core.
 // PLANES: the queries lie in channel-blocked planes [token / 8][D][8] (PlanesView); a warp copies them as they lie and
 // ldmatrix.trans makes the fragments.
 struct PlanesView {
@@ -353,34 +353,31 @@ apply_mma_kernel(const bf16* __restrict__ q, const float* __restrict__ state, in
         }
   };
   constexpr int NE = D * (D + 1);
-  if (S == 1) {  // every lane fetches its entries: one round trip
+  if (PAIR || PLANES || S == 1) {  // every lane fetches its entries: one round trip
     const float* src = state + (long long)bh * NE;
     fragments([&](int e) { return __uint_as_float(ld_dep32(src + e)); });
   } else {
     // The sums lie in the warps' last FIFO stage meanwhile, which nothing is copied into yet: with memory of their own an SM would
     // hold a CTA less.
-    constexpr int NV = NE / 4, HPC = PAIR ? 2 : 1, CAP = NWARPS * STAGEB / 16;  // vectors that fit there
-    __shared__ float4 rest[HPC * NV > CAP ? HPC * NV - CAP : 1];
+    constexpr int NV = NE / 4;
+    static_assert(NV <= NWARPS * STAGEB / 16, "the state fits the last stages");
     auto vec = [&](int i) -> float4* {
-      if (HPC * NV > CAP && i >= CAP) return rest + (i - CAP);
       return reinterpret_cast<float4*>(fifo + (i / (STAGEB / 16)) * (STAGES * STAGEB) + (STAGES - 1) * STAGEB) + i % (STAGEB / 16);
     };
-    const float4* src = reinterpret_cast<const float4*>(state) + (long long)(PAIR ? 2 * blockIdx.y : blockIdx.y) * S * NV;
-    for (int i = threadIdx.x; i < HPC * NV; i += NWARPS * 32) {
-      const float4* p = src + (PAIR && i >= NV ? (long long)S * NV + i - NV : i);
+    const float4* src = reinterpret_cast<const float4*>(state) + (long long)bh * S * NV;
+    for (int i = threadIdx.x; i < NV; i += NWARPS * 32) {
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
       for (int s = 0; s < S; s += 4) {
         float4 x[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = s + u < S ? ld_dep128f(p + (s + u) * NV) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int u = 0; u < 4; ++u) x[u] = s + u < S ? ld_dep128f(src + (s + u) * NV + i) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int u = 0; u < 4; ++u) { v.x += x[u].x; v.y += x[u].y; v.z += x[u].z; v.w += x[u].w; }
       }
       *vec(i) = v;
     }
     __syncthreads();
-    const int first = PAIR ? (warp & 1) * NE : 0;
-    fragments([&](int e) { e += first; return reinterpret_cast<const float*>(vec(e >> 2))[e & 3]; });
+    fragments([&](int e) { return reinterpret_cast<const float*>(vec(e >> 2))[e & 3]; });
     __syncthreads();  // every warp has its fragments: the stages may be filled
   }
 
