@@ -40,7 +40,7 @@ from paper_2205_14756_b200 import inputs  # noqa: E402
 METRIC = "msla_fwd_tokens_per_s"
 UNIT = "tokens/s"
 STAGES = ("project_in", "aggregate", "kv_state", "apply", "project_out")
-# when the library runs steps 4 and 5 as one kernel (msla_forward_fuses_apply), they are one stage
+# when the library runs steps 4 and 5 as one kernel (msla_forward_plan), they are one stage
 STAGES_FUSED = ("project_in", "aggregate", "kv_state", "apply_project")
 # 16-bit storage and many tokens: steps 2 and 3 are one kernel (the event between them falls directly after the one that ends it)
 MERGED = {"aggregate": "aggregate_kv_state"}
@@ -53,11 +53,11 @@ def workload_by_name(name: str) -> inputs.ModuleShape:
     return table[name]
 
 
-def plan_stages(s: inputs.ModuleShape, fused: bool, launches: int) -> tuple:
-    """Names of the steps that one forward of `launches` kernels runs as a kernel (or more) each.  A 16-bit forward takes 5
-    launches with steps 4 and 5 fused and 6 without; one fewer means that steps 2 and 3 are fused too."""
-    names = STAGES_FUSED if fused else STAGES
-    if s.dtype != "f32" and launches == (4 if fused else 5):
+def plan_stages(plan: int) -> tuple:
+    """Names of the steps that a forward of this plan (msla_forward_plan) runs as a kernel (or more) each."""
+    from paper_2205_14756_b200 import binding
+    names = STAGES_FUSED if plan & binding.MSLA_PLAN_FUSES_APPLY else STAGES
+    if plan & binding.MSLA_PLAN_FUSES_STATES:
         names = tuple(MERGED.get(n, n) for n in names if n != "kv_state")
     return names
 
@@ -538,20 +538,17 @@ def main() -> None:
         mdesc = binding.make_desc(ms_shape.B, ms_shape.C, ms_shape.H, ms_shape.W, ms_shape.heads, ms_shape.d, ms_shape.C_out, mcode,
                                   ms_shape.eps, workspace=mws)
         call = lambda i: binding.msla_forward(mdesc, mx, mweights, mo, stream)
-        call(0)
-        before = binding.msla_kernel_launches()
-        call(1)
-        launches_m = binding.msla_kernel_launches() - before
-        call(2)
+        for i in range(3):
+            call(i)
         ms = [m / steps for m in timed_blocks(call, blocks=blocks, steps=steps)]
-        fused_m = binding.msla_forward_fuses_apply(mdesc) == 1
+        plan_m = binding.msla_forward_plan(mdesc)
         bpt_m = stage_bytes_per_token(ms_shape)
-        names = plan_stages(ms_shape, fused_m, launches_m)
+        names = plan_stages(plan_m)
         mbytes = sum(bpt_m[n] for n in names) * ms_shape.B * ms_shape.N
         return {"workload": ms_shape.name, "tokens": ms_shape.B * ms_shape.N, "ms": round(med(ms), 5), "ms_min": round(min(ms), 5),
                 "ms_max": round(max(ms), 5), "tokens_per_s": ms_shape.B * ms_shape.N / (med(ms) * 1e-3),
                 "module_GBps": round(mbytes / (med(ms) * 1e-3) / 1e9, 1),
-                "l2": "exceeds L2" if mbytes > 4 * 126e6 else "L2-resident", "steps_4_5_fused": fused_m}
+                "l2": "exceeds L2" if mbytes > 4 * 126e6 else "L2-resident", "steps_4_5_fused": bool(plan_m & binding.MSLA_PLAN_FUSES_APPLY)}
 
     def time_ffn_block(ms_shape: inputs.ModuleShape, c_hidden: int, blocks=5, steps=5):
         """The other half of the building block at this workload's shape: FFN+DWConv alone (hard-swish, biases,
@@ -625,8 +622,9 @@ def main() -> None:
         [ms_total, ms_lo, ms_hi, med(ms_e2e_blocks), med(ms_e2e_serial_blocks), med(ms_plain_blocks)], device="cuda")
 
     if rank == 0:
-        fused = binding.msla_forward_fuses_apply(desc) == 1
-        stage_names = plan_stages(s, fused, launches // K)
+        plan = binding.msla_forward_plan(desc)
+        fused = bool(plan & binding.MSLA_PLAN_FUSES_APPLY)
+        stage_names = plan_stages(plan)
         stage_ms = {name: statistics.mean(v) for name, v in stage_acc.items()}
         if fused:  # the event between steps 4 and 5 falls directly after the one that ends step 3
             stage_ms["apply_project"] = stage_ms.pop("apply") + stage_ms.pop("project_out")

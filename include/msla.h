@@ -183,14 +183,13 @@ msla_status_t msla_forward(const msla_desc* desc, const void* x, const msla_weig
  * array of n_events = 6 cudaEvent_t handles (as void*): events[0] is recorded
  * on `stream` before step 1 and events[i] after step i (1 projection, 2
  * aggregation, 3 KV-state reduction, 4 apply, 5 output projection; Section
- * 3.1).  When msla_forward_fuses_apply(desc) == 1 steps 4 and 5 are one
- * kernel: events[3] is then recorded after the first level of the state
+ * 3.1).  When msla_forward_plan(desc) has MSLA_PLAN_FUSES_APPLY steps 4 and 5 are
+ * one kernel: events[3] is then recorded after the first level of the state
  * reduction (the per-chunk partial states), events[4] directly after it, so
  * the interval of step 4 is empty and events[4]..events[5] covers the second
  * level of the state reduction (fixed-order sum of the partial states, folded
- * into the projection weights) together with apply + projection.  With 16-bit
- * storage, rows of a multiple of 8 pixels and many tokens steps 2 and 3 are
- * one kernel: events[2] is recorded after it and events[3] directly after
+ * into the projection weights) together with apply + projection.  With
+ * MSLA_PLAN_FUSES_STATES steps 2 and 3 are one kernel: events[2] is recorded after it and events[3] directly after
  * events[2].  Everything else is as for msla_forward. */
 msla_status_t msla_forward_profiled(const msla_desc* desc, const void* x, const msla_weights* weights,
                                     void* out, void* stream, void* const* events, int n_events);
@@ -301,11 +300,17 @@ msla_status_t msla_ffn_dwconv(const msla_ffn_desc* desc, const void* x, const ms
 msla_status_t msla_evit_block(const msla_desc* attn, const msla_weights* attn_weights, const msla_ffn_desc* ffn,
                               const msla_ffn_weights* ffn_weights, const void* x, void* y, void* out, void* stream);
 
-/* 1 if msla_forward runs steps 4 and 5 of Section 3.1 (apply and output
- * projection) as one kernel for this descriptor, so that the head concat never
- * goes to device memory; 0 if they run as two kernels; -1 on an invalid
- * descriptor.  A pure function of the descriptor (workspace fields ignored);
- * host only, launches nothing.  Benchmarks use it to attribute time and bytes. */
+/* Which of Section 3.1's steps msla_forward runs as one kernel for this
+ * descriptor, as a sum of the flags below; -1 on an invalid descriptor.  A pure
+ * function of the descriptor (workspace fields ignored); host only, launches
+ * nothing.  Benchmarks use it to attribute time and bytes. */
+#define MSLA_PLAN_FUSES_APPLY 1  /* steps 4 and 5: the head concat never goes to device memory */
+#define MSLA_PLAN_FUSES_STATES 2 /* steps 2 and 3: nor do the aggregated keys and values */
+int msla_forward_plan(const msla_desc* desc);
+
+/* 1 if the storage type is bf16 and msla_forward_plan reports
+ * MSLA_PLAN_FUSES_APPLY, 0 if not, -1 on an invalid descriptor.  (fp16 runs the
+ * same kernels and is answered with 0 here; msla_forward_plan tells.) */
 int msla_forward_fuses_apply(const msla_desc* desc);
 
 /* Number of kernels this library has launched from the calling thread since it

@@ -73,6 +73,7 @@ EXPORTS = {
     "msla_ffn_dwconv": (c_int, [ctypes.POINTER(msla_ffn_desc), c_void_p, ctypes.POINTER(msla_ffn_weights), c_void_p, c_void_p]),
     "msla_evit_block": (c_int, [ctypes.POINTER(msla_desc), ctypes.POINTER(msla_weights), ctypes.POINTER(msla_ffn_desc),
                                 ctypes.POINTER(msla_ffn_weights), c_void_p, c_void_p, c_void_p, c_void_p]),
+    "msla_forward_plan": (c_int, [ctypes.POINTER(msla_desc)]),
     "msla_forward_fuses_apply": (c_int, [ctypes.POINTER(msla_desc)]),
     "msla_kernel_launches": (ctypes.c_ulonglong, []),
     "msla_debug_wait_timeouts": (c_int, []),
@@ -253,6 +254,13 @@ def msla_debug_wait_timeouts() -> int:
 def msla_debug_wait_selftest(limit_cycles: int, scratch, stream=None) -> int:
     """Runs the library's bounded wait on a barrier nobody arrives at; 1 = it gave up at the limit."""
     return lib().msla_debug_wait_selftest(limit_cycles, _ptr(scratch), _stream(stream))
+
+
+MSLA_PLAN_FUSES_APPLY, MSLA_PLAN_FUSES_STATES = 1, 2
+
+
+def msla_forward_plan(desc: msla_desc) -> int:
+    return lib().msla_forward_plan(ctypes.byref(desc))
 
 
 def msla_forward_fuses_apply(desc: msla_desc) -> int:

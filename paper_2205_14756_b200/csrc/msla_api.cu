@@ -290,6 +290,7 @@ struct ForwardPlan {
   int pitch;
   size_t xpad_off, ypad_off;
   bool padded() const { return pitch != N; }
+  bool fused;  // steps 4 and 5 as one kernel: the head concat stays in shared memory
   // Channel-blocked planes (see planes_path): ms holds the 3*heads projected planes per image, then the aggregated query
   // planes branch by branch.
   bool planes;
@@ -339,13 +340,14 @@ static msla_status_t validate_desc(const msla_desc* d, ForwardPlan* plan, BatchP
   plan->N = d->H * d->W;
   const size_t e = elem_size(d->dtype);
   const size_t tokens = (size_t)d->B * plan->N, state = (size_t)d->d * (d->d + 1) * sizeof(float);
-  const bool tuned = d->dtype != MSLA_F32, fused = tuned && fused_out_bf16_supported(S * d->heads, d->d, d->C_out);
+  const bool tuned = d->dtype != MSLA_F32;
+  plan->fused = tuned && fused_out_bf16_supported(S * d->heads, d->d, d->C_out);
   plan->core = make_core_plan((long long)whole_B * S * d->heads, plan->N, d->d);
   plan->planes = planes_path(d, whole_B);
   plan->pitch = tuned ? (int)align_up((size_t)plan->N, 8) : plan->N;
   plan->ms_off = 0;
   // the fused apply + projection kernel writes no attention output, and the region is its scratch
-  const size_t att_bytes = align_up(fused ? fused_out_scratch_bytes(d->B, S * d->heads, d->d, d->C_out) : tokens * S * plan->Cp * e, 256);
+  const size_t att_bytes = align_up(plan->fused ? fused_out_scratch_bytes(d->B, S * d->heads, d->d, d->C_out) : tokens * S * plan->Cp * e, 256);
   const size_t taps = align_up((size_t)3 * plan->Cp * 25 * e, 256), embedded = (d->agg_kernel == 3 ? taps : 0) + (S == 3 && d->agg_kernel2 == 3 ? taps : 0);
   const size_t xpad = align_up((size_t)d->B * d->C * plan->pitch * e, 256), ypad = align_up((size_t)d->B * d->C_out * plan->pitch * e, 256);
   const size_t ms_bytes = align_up(tokens * 3 * S * plan->Cp * e, 256);
@@ -534,7 +536,7 @@ static msla_status_t run_planes_rest(const msla_desc* desc, const msla_weights* 
   char* att = ws + p.att_off;
   const PlanesQueries q{ws + p.ms_off, ws + p.q1_off, desc->heads, p.pitch, first};
   msla_status_t s = MSLA_OK;
-  if (fused_out_bf16_supported(Ht, d, desc->C_out)) {
+  if (p.fused) {
     if (events && ((s = record(events, 3, st)) != MSLA_OK || (s = record(events, 4, st)) != MSLA_OK)) return s;
     return run_fused_out_bf16(nullptr, 0, 0, &q, in, att, w->w_proj, w->b_proj, residual, y, tokens, B, Ht, d, tokens, desc->C_out, desc->eps, st, f16);
   }
@@ -641,14 +643,12 @@ static msla_status_t forward_impl(const msla_desc* desc, const void* x, const ms
   const bool att_planar = desc->dtype != MSLA_F32 && d == 32 && Ht % 2 == 0 && project_out_planar_bf16_supported(S * Cp, desc->C_out);
   const HeadView ov = att_planar ? HeadView{(long long)N * ld_att, (long long)N * 2 * d, 2 * d, 1}
                                  : HeadView{(long long)N * ld_att, d, ld_att, 0};
-  // Steps 4 and 5 run as one kernel when it takes the shape: the head concat then stays in shared memory.
-  const bool fused = desc->dtype != MSLA_F32 && fused_out_bf16_supported(Ht, d, desc->C_out);
   s = run_core(desc->dtype, ms, ms + (size_t)N * d * e, ms + (size_t)2 * N * d * e, att, in, ov, desc->B, Ht, N, d, desc->eps, p.core,
-               ws + p.core_off, st, events ? (cudaEvent_t)events[3] : nullptr, fused ? CORE_STATE : CORE_ALL);
+               ws + p.core_off, st, events ? (cudaEvent_t)events[3] : nullptr, p.fused ? CORE_STATE : CORE_ALL);
   if (s != MSLA_OK) return s;
   if ((s = record(events, 4, st)) != MSLA_OK) return s;
   // 5. output projection back to NCHW
-  if (fused)
+  if (p.fused)
     s = run_fused_out_bf16(ms, ms_sb, 3LL * N * d, nullptr, dense_states(ws + p.core_off + p.core.partial_off, p.core.S), att, w->w_proj, w->b_proj,
                             residual, y_dev, p.pitch, desc->B, Ht, d, N, desc->C_out, desc->eps, st, f16);
   else
@@ -871,7 +871,7 @@ static msla_status_t band_output_impl(const msla_desc* desc, const msla_weights*
   const int pitch = desc->dtype == MSLA_F32 ? Nb : (int)align_up((size_t)Nb, 8);
   const bool padded = pitch != Nb;
   void* y = padded ? ws + p.ypad_off : out;
-  if (desc->dtype != MSLA_F32 && fused_out_bf16_supported(Ht, d, desc->C_out)) {
+  if (p.fused) {
     s = run_fused_out_bf16(q, ms_sb, 3LL * N * d, nullptr, dense_states(state, 1), att, w->w_proj, w->b_proj, nullptr, y, pitch, desc->B, Ht, d, Nb, desc->C_out, desc->eps, st, f16);
   } else {
     const HeadView in{ms_sb, 3LL * N * d, d};
@@ -1101,10 +1101,15 @@ msla_status_t msla_evit_block(const msla_desc* attn, const msla_weights* aw, con
   return block_impl(attn, aw, ffn, fw, x, y, out, (cudaStream_t)stream);
 }
 
-int msla_forward_fuses_apply(const msla_desc* desc) {
+int msla_forward_plan(const msla_desc* desc) {
   ForwardPlan p;
   if (validate_desc(desc, &p) != MSLA_OK) return -1;
-  return desc->dtype == MSLA_BF16 && fused_out_bf16_supported(p.S * desc->heads, desc->d, desc->C_out) ? 1 : 0;
+  return (p.fused ? MSLA_PLAN_FUSES_APPLY : 0) | (p.planes ? MSLA_PLAN_FUSES_STATES : 0);
+}
+
+int msla_forward_fuses_apply(const msla_desc* desc) {
+  const int plan = msla_forward_plan(desc);
+  return plan < 0 ? -1 : desc->dtype == MSLA_BF16 && (plan & MSLA_PLAN_FUSES_APPLY) ? 1 : 0;
 }
 
 unsigned long long msla_kernel_launches(void) { return g_launches; }

@@ -123,3 +123,21 @@ def test_a_block_that_its_second_half_would_refuse_runs_nothing():
     if device == "cuda":
         torch.cuda.synchronize()
     assert bool((ws == 0xA5).all())
+
+
+def test_plan_of_a_forward():
+    """Which steps are one kernel, for every storage type, and the stages that the benchmark counts bytes for."""
+    import bench
+    plan = lambda dtype, C, H, W, heads, d, B=1: binding.msla_forward_plan(binding.make_desc(B, C, H, W, heads, d, C, dtype))
+    apply, states = binding.MSLA_PLAN_FUSES_APPLY, binding.MSLA_PLAN_FUSES_STATES
+    for dtype in (binding.MSLA_BF16, binding.MSLA_F16):
+        assert plan(dtype, 256, 512, 512, 8, 32) == apply | states
+        assert plan(dtype, 256, 512, 511, 8, 32) == apply           # rows of no whole octets
+        assert plan(dtype, 256, 32, 32, 8, 32) == apply             # few tokens
+        assert plan(dtype, 384, 256, 256, 12, 32) == states         # too many channels for the fused output kernel
+        assert plan(dtype, 288, 7, 7, 9, 32) == 0
+    assert plan(binding.MSLA_F32, 256, 512, 512, 8, 32) == 0
+    assert plan(binding.MSLA_BF16, 60, 8, 8, 1, 32) == -1
+    assert bench.plan_stages(0) == bench.STAGES and bench.plan_stages(apply) == bench.STAGES_FUSED
+    assert bench.plan_stages(apply | states) == ("project_in", "aggregate_kv_state", "apply_project")
+    assert bench.plan_stages(states) == ("project_in", "aggregate_kv_state", "apply", "project_out")
