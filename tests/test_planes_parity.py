@@ -41,6 +41,23 @@ def test_planes_three_branches(C, H, W, heads, d, k1, k2):
     util.assert_close(util.run_module(s, t), ref, "bf16", "planes, three branches", block=util.MODULE_BLOCK)
 
 
+# d = 16: three branches and 3x3 filters.  The queries of scale 0 get a positive mean (a constant channel of x), so that no row is without
+# an entry well above zero (see above).
+@pytest.mark.parametrize("dtype,C,H,W,heads,n_scales,k1,k2", [("bf16", 64, 240, 344, 4, 3, 5, 3), ("f16", 96, 240, 232, 6, 3, 3, 5),
+                                                              ("bf16", 80, 240, 280, 5, 2, 3, 5), ("f16", 32, 416, 400, 2, 2, 3, 5)])
+def test_planes_of_narrow_heads(dtype, C, H, W, heads, n_scales, k1, k2):
+    s = inputs.ModuleShape("planes16", dtype, 1, C, H, W, heads, 16, seed=85, n_scales=n_scales, agg_kernel=k1, agg_kernel2=k2)
+    t = inputs.module_inputs(s)
+    t["x"][:, 0] = 4.0
+    t["w_qkv"].reshape(heads, 3, 16, C)[:, 0, :, 0] = 0.5
+    if n_scales == 3:
+        ref = oracle.msla_forward3(t["x"], t["w_qkv"], t["w_dw"], t["w_pw"], t["w_dw2"], t["w_pw2"], t["w_proj"], heads=heads, d=16)
+    else:
+        ref = oracle.msla_forward(t["x"], t["w_qkv"], t["w_dw"], t["w_pw"], t["w_proj"], heads=heads, d=16, eps=s.eps)
+    util.assert_close(util.run_module(s, t), ref, dtype, "planes, d = 16", block=util.MODULE_BLOCK)
+    assert binding.msla_debug_wait_timeouts() == 0
+
+
 def test_planes_block():
     s = inputs.ModuleShape("planes_block", "bf16", 2, 64, 200, 208, 2, 32, seed=83)
     t = inputs.module_inputs(s)
