@@ -87,6 +87,29 @@ static bool known_dtype(msla_dtype_t t) { return t == MSLA_F32 || t == MSLA_BF16
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // ----------------------------------------------------------------- core plan
+// Tokens per CTA of the apply step.  d = 16: all CTAs resident at once, about eight per SM.  d = 32, where the state's fragments cost
+// each CTA more: four to an SM, i.e. waves of 592; of one wave more than 2048 tokens a CTA allow, up to three more, the count whose
+// CTAs, filled evenly, take the shortest (300 tokens: what a CTA costs besides its own).  Core, us, with CTAs for 592 whatever the
+// last wave / this rule / what it was for 1184 CTAs: [8, 16, 4096, 32] 32.8 / 32.8 / 34.7, [15, 10, 10000, 32] 84.3 / 79.7 / 81.6,
+// [37, 4, 20000, 32] 149.6 / 143.1, [64, 6, 3000, 32] 65.9 / 60.3 / 60.2, [37, 16, 3000, 32] 92.6 / 86.1 / 85.7, [22, 20, 4096, 32] 91.1 /
+// 88.3 / 95.1, [6, 10, 5000, 32] 21.8 / 19.0 / 23.2, [1, 10, 70844, 32] 45.2 / 45.1 / 47.9; d = 16 [16, 8, 9000, 16] for 1184 / 592 36.5 / 38.2.
+static int apply_tokens(long long BH, int N, int d) {
+  if (d != 32) {
+    const long long at = ceil_div_ll(ceil_div_ll((long long)N * BH, 1184), 256) * 256;
+    return (int)(at < 256 ? 256 : (at > 2048 ? 2048 : at));
+  }
+  const long long few = ceil_div_ll(N, 2048), many = ceil_div_ll(N, 256), wave = 592, first = ceil_div_ll(BH * few, wave);  // CTAs per head
+  long long best = 0, tokens = 2048;
+  for (long long w = first; w < first + 4; ++w) {
+    const long long n = wave * w / BH < many ? wave * w / BH : many;
+    long long at = ceil_div_ll(ceil_div_ll(N, n), 128) * 128;
+    if (at < 256) at = 256;
+    const long long cost = w * (at + 300);
+    if (w == first || cost < best) { best = cost; tokens = at; }
+  }
+  return (int)tokens;
+}
+
 // The split of the token reduction is a function of the shape only.
 CorePlan make_core_plan(long long BH, int N, int d) {
   CorePlan p;
@@ -103,10 +126,7 @@ CorePlan make_core_plan(long long BH, int N, int d) {
   chunk = ceil_div_ll(chunk, 64) * 64;
   p.chunk = (int)chunk;
   p.S = (int)ceil_div_ll(N, chunk);
-  // tokens per CTA of the apply step: all CTAs resident at once, about eight per SM for d = 16; about four for d = 32, where the
-  // state's fragments cost each CTA more (core [8, 16, 4096, 32], us, with CTAs for 1184 / 592: 39.3 / 37.0; d = 16 [16, 8, 9000, 16] 36.5 / 38.2)
-  long long at = ceil_div_ll(ceil_div_ll((long long)N * BH, d == 32 ? 592 : 1184), 256) * 256;
-  p.apply_tokens = (int)(at < 256 ? 256 : (at > 2048 ? 2048 : at));
+  p.apply_tokens = apply_tokens(BH, N, d);
   p.partial_off = 0;
   p.state_off = align_up((size_t)BH * p.S * p.ne * sizeof(float), 256);
   p.bytes = p.state_off + align_up((size_t)BH * p.ne * sizeof(float), 256);

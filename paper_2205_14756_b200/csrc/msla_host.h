@@ -16,7 +16,7 @@ struct CorePlan {
   int S;       // number of token chunks per (batch, head)
   int chunk;   // tokens per chunk (multiple of 64)
   int ne;      // d*(d+1) state entries
-  int apply_tokens;  // tokens per CTA of the tuned apply kernel (multiple of 256)
+  int apply_tokens;  // tokens per CTA of the tuned apply kernel (multiple of 128)
   size_t partial_off, state_off, bytes;
 };
 
