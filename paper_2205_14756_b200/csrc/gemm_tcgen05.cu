@@ -398,6 +398,8 @@ constexpr int RES_BYTES = 128 * 1024;
 constexpr int WS_RING_BYTES = 80 * 1024;
 constexpr int WS_SMEM_BYTES = RES_BYTES + WS_RING_BYTES + STAGING_BYTES + 256 + 1024;
 constexpr int WS_MAX_STAGES = 6;
+constexpr int WS_MAX_SLICES = RES_BYTES / (128 * BK * 2);  // k-slices of the longest rows (stationary_columns)
+static_assert(16 * WS_MAX_STAGES + 32 + 8 * WS_MAX_SLICES + 8 <= 256, "barrier block");
 
 template <int TN, int EPI, bool F16>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
@@ -415,7 +417,7 @@ gemm_bf16_stationary_kernel(const __grid_constant__ CUtensorMap tmA, const __gri
   const uint32_t bars = staging + NBUF * STAGING_BYTES;
   const uint32_t full_bar = bars, empty_bar = bars + 8 * WS_MAX_STAGES;
   const uint32_t tfull_bar = bars + 16 * WS_MAX_STAGES, tempty_bar = tfull_bar + 16;
-  const uint32_t res_bar = tempty_bar + 16, tmem_slot = res_bar + 8;
+  const uint32_t res_bar = tempty_bar + 16, tmem_slot = res_bar + 8 * WS_MAX_SLICES;  // res_bar: [k-slice]
   __shared__ int abort_flag;
   __shared__ uint32_t tmem_base_sh;
   __shared__ __align__(16) float bias_sm[EPI == 1 ? TN : 4];  // the CTA's column biases (weights: not the output of the call's previous kernel)
@@ -438,7 +440,7 @@ gemm_bf16_stationary_kernel(const __grid_constant__ CUtensorMap tmA, const __gri
     abort_flag = 0;
     for (int s = 0; s < NSTAGE; ++s) { mbar_init(full_bar + 8 * s, 1); mbar_init(empty_bar + 8 * s, 1); }
     for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar + 8 * a, 1); mbar_init(tempty_bar + 8 * a, 8); }
-    mbar_init(res_bar, 1);
+    for (int kb = 0; kb < k_iters; ++kb) mbar_init(res_bar + 8 * kb, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -461,17 +463,25 @@ gemm_bf16_stationary_kernel(const __grid_constant__ CUtensorMap tmA, const __gri
     if (lane == 0) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB) : "memory");
-      if (p.first) pdl_first_wait();
-      // the resident weight block: all k-slices on one barrier
-      mbar_expect_tx(res_bar, (uint32_t)(k_iters * RES_SLICE));
-      for (int kb = 0; kb < k_iters; ++kb) tma_load_3d(res_base + kb * RES_SLICE, &tmB, res_bar, kb * BK, blk * TN, 0);
-      pdl_wait();  // the streamed operand may come from the previous kernel of the call; the weights above do not
+      const auto load_weights = [&](int kb) {
+        mbar_expect_tx(res_bar + 8 * kb, RES_SLICE);
+        tma_load_3d(res_base + kb * RES_SLICE, &tmB, res_bar + 8 * kb, kb * BK, blk * TN, 0);
+      };
+      // The weights do not come from the previous kernel of the call, the streamed operand may.  In a call's first kernel both are
+      // fetched after the wait, slice by slice in turn, so that the first products need not wait for the whole block.
+      if (p.first) {
+        pdl_first_wait();
+      } else {
+        for (int kb = 0; kb < k_iters; ++kb) load_weights(kb);
+        pdl_wait();
+      }
       uint32_t it = 0;
       bool ok = true;
       for (int si = worker; ok && si < stream_total; si += workers) {
         const int b = si / stream_per_batch, st = si % stream_per_batch;
         for (int kb = 0; ok && kb < k_iters; ++kb, ++it) {
           const uint32_t s = it % NSTAGE, ph = (it / NSTAGE) & 1;
+          if (p.first && si == worker) load_weights(kb);
           ok = mbar_wait(empty_bar + 8 * s, ph ^ 1, &abort_flag);
           if (!ok) break;
           const uint32_t dst = ring_base + s * STREAM_BYTES;
@@ -488,7 +498,7 @@ gemm_bf16_stationary_kernel(const __grid_constant__ CUtensorMap tmA, const __gri
       const uint32_t idesc = (1u << 4) | operand_format_bits<F16>() | (1u << 15) |
                              ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
       uint32_t it = 0, local = 0;
-      bool ok = mbar_wait(res_bar, 0, &abort_flag);
+      bool ok = true;
       for (int si = worker; ok && si < stream_total; si += workers, ++local) {
         const uint32_t acc = local & 1, acc_ph = (local >> 1) & 1;
         ok = mbar_wait(tempty_bar + 8 * acc, acc_ph ^ 1, &abort_flag);
@@ -497,7 +507,7 @@ gemm_bf16_stationary_kernel(const __grid_constant__ CUtensorMap tmA, const __gri
         const uint32_t d_tmem = tmem_base + acc * BN;
         for (int kb = 0; ok && kb < k_iters; ++kb, ++it) {
           const uint32_t s = it % NSTAGE, ph = (it / NSTAGE) & 1;
-          ok = mbar_wait(full_bar + 8 * s, ph, &abort_flag);
+          ok = (local > 0 || mbar_wait(res_bar + 8 * kb, 0, &abort_flag)) && mbar_wait(full_bar + 8 * s, ph, &abort_flag);
           if (!ok) break;
           tc_fence_after();
           const uint32_t stream = ring_base + s * STREAM_BYTES, res = res_base + kb * RES_SLICE;
