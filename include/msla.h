@@ -189,8 +189,9 @@ msla_status_t msla_forward(const msla_desc* desc, const void* x, const msla_weig
  * the interval of step 4 is empty and events[4]..events[5] covers the second
  * level of the state reduction (fixed-order sum of the partial states, folded
  * into the projection weights) together with apply + projection.  With
- * MSLA_PLAN_FUSES_STATES steps 2 and 3 are one kernel: events[2] is recorded after it and events[3] directly after
- * events[2].  Everything else is as for msla_forward. */
+ * MSLA_PLAN_FUSES_STATES steps 2 and 3 are one kernel: events[2] is recorded
+ * after it and events[3] directly after events[2].  Everything else is as for
+ * msla_forward. */
 msla_status_t msla_forward_profiled(const msla_desc* desc, const void* x, const msla_weights* weights,
                                     void* out, void* stream, void* const* events, int n_events);
 
@@ -199,7 +200,11 @@ msla_status_t msla_forward_profiled(const msla_desc* desc, const void* x, const 
  * out_host are host pointers (pinned memory if the copies are to be
  * asynchronous); weights stay device pointers.  The call enqueues a
  * host-to-device copy of x, the five steps and a device-to-host copy of the
- * result on `stream`.  desc->workspace must hold
+ * result; a large batch goes through in parts of whole images, so that the
+ * copies overlap one another and the kernels, with the copies on two streams
+ * that the calling thread's first such call creates.  Work enqueued on `stream`
+ * before the call precedes all of it, and work enqueued after the call follows
+ * all of it.  The result is that of msla_forward, bit for bit.  desc->workspace must hold
  * msla_forward_host_workspace_bytes(desc) bytes: the forward scratch plus
  * device staging for x and out. */
 size_t msla_forward_host_workspace_bytes(const msla_desc* desc);
