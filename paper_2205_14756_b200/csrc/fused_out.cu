@@ -216,8 +216,10 @@ __device__ __forceinline__ void fold_mma(float (&c)[4], const uint32_t (&a)[4], 
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// F16: M and ks are multiplied by `scale`, a power of two near 1 / N (the output kernel scales eps alike, so Eq. 3's quotient is
-// unchanged): sums over N tokens then stay inside binary16's range.
+// F16: row a of the state is divided by its key sum (0 where that is 0), and the output kernel multiplies its queries by it,
+//   M[m][hd + a] = sum_c w[m][hd + c] S_h[a][c] / ks_h[a],   qt[hd + a][n] = relu(q_h[n][a]) ks_h[a] / den_h[n] <= 1,
+// so that both stay inside binary16's range whatever N and the key sums are.  relu(q) / den alone does not: where the keys have nothing
+// above zero in the channels that a query has, den is eps, and infinity times the zero column of M is not a number.
 struct FoldParams {
   const float* partial;      // [B*Ht][S][D][D+1]
   int S;
@@ -229,7 +231,6 @@ struct FoldParams {
   bf16* M;
   float *ks, *state_out;
   int B, heads, Ht, Cout, K;
-  float scale;
 };
 template <int D, int DA, bool F16, bool SLOTS>
 __global__ void __launch_bounds__(FoldShape<D, DA>::THREADS, DA == D ? 4 : 1)
@@ -243,7 +244,6 @@ state_fold_kernel(FoldParams p) {
   float* st = reinterpret_cast<float*>(run_sum[0]);
   pdl_launch_dependents();
   const int Ht = p.Ht, Cout = p.Cout, K = p.K;
-  const float scale = p.scale;
   const bf16* w = p.w;
   const int bh = blockIdx.x, b = bh / Ht, hh = bh % Ht, a0 = blockIdx.y * DA;
   const int branch = SLOTS ? hh / p.heads : 0, h = SLOTS ? hh - branch * p.heads : 0;
@@ -351,11 +351,14 @@ state_fold_kernel(FoldParams p) {
     for (int i = tid; i < DA * D1; i += THREADS) p.state_out[(long long)bh * (D * D1) + a0 * D1 + i] = st[i];
     return;
   }
-  if (tid < DA) p.ks[(long long)bh * D + a0 + tid] = F16 ? st[tid * D1 + D] * scale : st[tid * D1 + D];
+  if (tid < DA) p.ks[(long long)bh * D + a0 + tid] = st[tid * D1 + D];
   for (int i = tid; i < DA * D / 2; i += THREADS) {
     const int al = i / (D / 2), c2 = i - al * (D / 2);
     float v0 = st[al * D1 + 2 * c2], v1 = st[al * D1 + 2 * c2 + 1];
-    if (F16) { v0 *= scale; v1 *= scale; }
+    if (F16) {
+      const float sum = st[al * D1 + D], r = sum > 0.f ? 1.f / sum : 0.f;
+      v0 *= r; v1 *= r;
+    }
 #pragma unroll
     for (int k = 0; k < PIECES; ++k) {
       const uint32_t word = pack16<F16>(v0, v1);
@@ -658,7 +661,7 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
 #pragma unroll
             for (int cb = 0; cb < CB; ++cb) {
               uint32_t& w = q[o * CB + cb];
-              w = pack16<F16>(lo16<F16>(w) * io, hi16<F16>(w) * io);
+              w = F16 ? pack16<F16>(lo16<F16>(w) * kk[cb].x * io, hi16<F16>(w) * kk[cb].y * io) : pack16<F16>(lo16<F16>(w) * io, hi16<F16>(w) * io);
             }
           }
 #pragma unroll
@@ -694,7 +697,8 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
         }
         const float inv = __frcp_rn((den[0] + den[1]) + (den[2] + den[3]) + p.eps);
 #pragma unroll
-        for (int w = 0; w < D / 2; ++w) q[w] = pack16<F16>(lo16<F16>(q[w]) * inv, hi16<F16>(q[w]) * inv);
+        for (int w = 0; w < D / 2; ++w)
+          q[w] = F16 ? pack16<F16>(lo16<F16>(q[w]) * kk[2 * w] * inv, hi16<F16>(q[w]) * kk[2 * w + 1] * inv) : pack16<F16>(lo16<F16>(q[w]) * inv, hi16<F16>(q[w]) * inv);
 #pragma unroll
         for (int c = 0; c < PCS; ++c)
           asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(rbase + (((uint32_t)c ^ swz) << 4)), "r"(q[4 * c]), "r"(q[4 * c + 1]),
@@ -870,12 +874,11 @@ msla_status_t run_fold(const FoldStates& in, FoldParams& f, int d, cudaStream_t 
 msla_status_t run_sum_states(const FoldStates& in, float* state_out, int B, int heads, int Ht, int d, cudaStream_t st, bool f16) {
   FoldParams f{};
   f.state_out = state_out;
-  f.B = B; f.heads = heads; f.Ht = Ht; f.scale = 1.f;
+  f.B = B; f.heads = heads; f.Ht = Ht;
   return run_fold(in, f, d, st, f16);
 }
 
-// f16: queries, weights, bias, residual and output are IEEE binary16 instead of bfloat16; M, the key sums and eps are
-// scaled by the power of two just above 1 / N (N tokens' sums would leave binary16's range otherwise).
+// f16: queries, weights, bias, residual and output are IEEE binary16 instead of bfloat16 (see FoldParams).
 // planes: nullptr, or the channel-blocked query planes that take the place of q.
 msla_status_t run_fused_out_bf16(const void* q, long long q_sb, long long q_sh, const PlanesQueries* planes, const FoldStates& states, void* scratch,
                                  const void* w, const void* bias, const void* residual, void* y, int ldy, int B, int Ht, int d, int N, int Cout,
@@ -907,12 +910,9 @@ msla_status_t run_fused_out_bf16(const void* q, long long q_sb, long long q_sh, 
       return fail(MSLA_ERR_CUDA, "cuTensorMapEncodeTiled failed for the fused apply + output projection");
     if (planes) tmQ = tmM;  // not read
   }
-  float scale = 1.f;
-  if (f16)
-    for (long long n = 1; n < N; n <<= 1) scale *= 0.5f;
   FoldParams f{};
   f.w = (const bf16*)w; f.M = M; f.ks = ks;
-  f.B = B; f.heads = planes ? planes->heads : Ht; f.Ht = Ht; f.Cout = Cout; f.K = K; f.scale = scale;
+  f.B = B; f.heads = planes ? planes->heads : Ht; f.Ht = Ht; f.Cout = Cout; f.K = K;
   msla_status_t s = run_fold(states, f, d, st, f16);
   if (s != MSLA_OK) return s;
   OutParams p{};
@@ -921,7 +921,7 @@ msla_status_t run_fused_out_bf16(const void* q, long long q_sb, long long q_sh, 
     p.plane_bytes = planes->plane_tokens * d * 2; p.tok_bytes = planes->first_token * d * 2;
   }
   p.ks = ks; p.bias = (const bf16*)bias; p.residual = (const bf16*)residual;
-  p.B = B; p.N = N; p.Cout = Cout; p.Ht = Ht; p.d = d; p.eps = eps * scale;
+  p.B = B; p.N = N; p.Cout = Cout; p.Ht = Ht; p.d = d; p.eps = eps;
   p.kslices = (K + OKS - 1) / OKS;
   p.ot = ot;
   p.tiles_per_image = (N + 2 * ot - 1) / (2 * ot);

@@ -75,3 +75,24 @@ def test_ffn_f16_tensor_core_shapes(B, C, H, W, Ch, act, residual):
     ft = inputs.ffn_inputs(fs)
     ref = oracle.ffn_dwconv(ft["x"], ft["w1"], ft["w_dw"], ft["w2"], ft["b1"], ft["b_dw"], ft["b2"], act=act, residual=residual)
     util.assert_close(util.run_ffn(fs, ft, act, residual), ref, "f16", "FFN fp16 (tensor cores)", block=util.MODULE_BLOCK)
+
+
+# Rows of queries that have nothing above zero in the channels where the keys have: Eq. 3 gives 0 / (0 + eps) there, a zero row.  Single tokens,
+# and key channels that are negative in every token (a constant channel of x), in the fused steps 4 + 5: planes of token rows,
+# channel-blocked planes, and rows padded to 8 tokens; bf16 beside fp16.
+@pytest.mark.parametrize("dtype,B,C,H,W,heads,d,dead", [("f16", 60, 64, 1, 1, 4, 16, 0), ("bf16", 60, 64, 1, 1, 4, 16, 0), ("f16", 2, 64, 16, 24, 4, 16, 12), ("f16", 2, 64, 15, 9, 2, 32, 27),
+                                                        ("f16", 1, 64, 240, 344, 2, 32, 26), ("f16", 1, 64, 240, 344, 4, 16, 11), ("bf16", 2, 64, 16, 24, 4, 16, 12)])
+def test_queries_that_meet_no_key(dtype, B, C, H, W, heads, d, dead):
+    s = inputs.ModuleShape("no_key", dtype, B, C, H, W, heads, d, seed=57)
+    t = inputs.module_inputs(s)
+    if dead:
+        # no aggregation (one tap, the identity as 1x1), so that the scales agree on which channels are dead
+        t["w_dw"][:] = 0.0
+        t["w_dw"][:, 2, 2] = 1.0
+        t["w_pw"][:] = np.tile(np.eye(d), (3 * heads, 1))
+        t["x"][:, 0] = 4.0
+        keys = t["w_qkv"].reshape(heads, 3, d, C)[:, 1]
+        keys[:, :dead] = 0.0
+        keys[:, :dead, 0] = -1.0
+    ref = oracle.msla_forward(t["x"], t["w_qkv"], t["w_dw"], t["w_pw"], t["w_proj"], heads=heads, d=d, eps=s.eps)
+    util.assert_close(util.run_module(s, t), ref, dtype, "queries that meet no key", block=util.MODULE_BLOCK)
