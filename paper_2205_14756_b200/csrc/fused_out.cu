@@ -179,6 +179,14 @@ template <bool F16> __device__ __forceinline__ uint32_t pack16(float lo, float h
   }
 }
 
+// F16: two queries times their key sums and the reciprocal of the normaliser, the products of both in one instruction each.
+__device__ __forceinline__ uint32_t scale_pair(uint32_t w, float k0, float k1, float inv) {
+  float lo = lo16<true>(w), hi = hi16<true>(w);
+  asm("{\n\t.reg .b64 q, k, i;\n\tmov.b64 q, {%0, %1};\n\tmov.b64 k, {%2, %3};\n\tmov.b64 i, {%4, %4};\n\t"
+      "mul.rn.f32x2 q, q, k;\n\tmul.rn.f32x2 q, q, i;\n\tmov.b64 {%0, %1}, q;\n\t}" : "+f"(lo), "+f"(hi) : "f"(k0), "f"(k1), "f"(inv));
+  return pack16<true>(lo, hi);
+}
+
 // ---------------------------------------------------------------------------
 // Second level of the state reduction (Eq. 3) and the fold of the state into the projection weights.
 // Grid (B * Ht, D / DA): a CTA takes one head and DA of its key channels a, i.e. DA consecutive rows of the head's state.
@@ -661,7 +669,7 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
 #pragma unroll
             for (int cb = 0; cb < CB; ++cb) {
               uint32_t& w = q[o * CB + cb];
-              w = F16 ? pack16<F16>(lo16<F16>(w) * kk[cb].x * io, hi16<F16>(w) * kk[cb].y * io) : pack16<F16>(lo16<F16>(w) * io, hi16<F16>(w) * io);
+              w = F16 ? scale_pair(w, kk[cb].x, kk[cb].y, io) : pack16<F16>(lo16<F16>(w) * io, hi16<F16>(w) * io);
             }
           }
 #pragma unroll
@@ -698,7 +706,7 @@ fused_out_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant_
         const float inv = __frcp_rn((den[0] + den[1]) + (den[2] + den[3]) + p.eps);
 #pragma unroll
         for (int w = 0; w < D / 2; ++w)
-          q[w] = F16 ? pack16<F16>(lo16<F16>(q[w]) * kk[2 * w] * inv, hi16<F16>(q[w]) * kk[2 * w + 1] * inv) : pack16<F16>(lo16<F16>(q[w]) * inv, hi16<F16>(q[w]) * inv);
+          q[w] = F16 ? scale_pair(q[w], kk[2 * w], kk[2 * w + 1], inv) : pack16<F16>(lo16<F16>(q[w]) * inv, hi16<F16>(q[w]) * inv);
 #pragma unroll
         for (int c = 0; c < PCS; ++c)
           asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(rbase + (((uint32_t)c ^ swz) << 4)), "r"(q[4 * c]), "r"(q[4 * c + 1]),
