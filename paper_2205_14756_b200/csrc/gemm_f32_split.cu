@@ -1,0 +1,398 @@
+// fp32 GEMM of the 1x1 projections (Section 3.1) and of the FFN's two layers on the 5th-generation tensor cores.
+//
+//   D[m][n] = sum_k A[m][k] * B[n][k]  (+ bias[n], activation, + residual)
+//
+// Every fp32 operand is cut into three bf16 pieces, x = x0 + x1 + x2 (x0 by truncation, so that no finite value becomes infinite,
+// the others rounded: at most 2^-25 of x is lost), and six of the nine products are formed, each exact in the tensor core's fp32
+// accumulator:
+//   main  A0 B0        X  A0 B1 + A1 B0        Y  A0 B2 + A1 B1 + A2 B0
+// (the other three are below 2^-23 of |A||B| at worst, of either sign and 2^-26 on average).  The tensor core's additions to an accumulator
+// truncate, where the fp32 pipes round, so an accumulator takes CHUNK k-slices at most and the chunks are added on the fp32 pipes.
+//
+// The pieces of B lie side by side in shared memory, so that one instruction takes A0 to [main | X | Y] (192 columns), one A1 to
+// [X | Y] and one A2 to [Y]: three instructions per 16 k.
+//
+// Against the packed multiply-adds of the fp32 pipes (generic::gemm_kernel), [1, 192, 8192] -> 576 channels: 43.8 -> 22.7 us, error (2-norm,
+// against 64 bits) 2.5e-7 -> 1.1e-7; 384 -> 192, token-major: 61.9 -> 19.0 us, 2.6e-7 -> 1.0e-7; 768 -> 384: 121 -> 43.3 us, 5.0e-7 -> 1.3e-7.
+// Chunks of one k-slice: 8e-8, 23.2 us for the first; of four: 1.8e-7, 21.8 us.  What bounds it is the cutting: a slice takes a group
+// of warps about 4000 cycles, two of which overlap, where its MMAs take 768 (ncu, the first shape: issue 55 %, ALU 46 %, tensor 27 % of
+// active cycles; the cutting warps wait on their own chains of two-cycle conversions, and registers allow no more of them).
+//
+// Roles of the persistent CTA (one per SM, tiles of 128 x 64):
+//   warps 0-15   fetch and cut: two groups of eight warps take the 64-wide k-slices in turn, a thread holds six runs of eight
+//                elements of its group's next slice in registers while it cuts the present one, so that two slices are in flight
+//   warp 16      issues the MMAs (17-19 only give their registers away)
+//   warps 20-27  add up the accumulators and write the tile; a lane is a row m, which is the index that is contiguous in the
+//                output, so that a warp's store of one column is a line
+#include <cuda.h>
+
+#include "msla_common.cuh"
+#include "msla_host.h"
+#include "tcgen05_util.cuh"
+
+namespace msla {
+namespace {
+
+constexpr int SG_M = 128, SG_N = 64, SG_K = 64;
+constexpr int SG_PIECES = 3;
+constexpr int SG_A_PIECE = SG_M * SG_K * 2, SG_B_PIECE = SG_N * SG_K * 2;
+constexpr int SG_STAGE = SG_PIECES * (SG_A_PIECE + SG_B_PIECE), SG_STAGES = 3;
+constexpr int SG_GROUPS = 2, SG_GROUP_WARPS = 8, SG_GROUP_THREADS = 32 * SG_GROUP_WARPS;
+constexpr int SG_CUT_WARPS = SG_GROUPS * SG_GROUP_WARPS, SG_MMA_WARPS = 4, SG_SUM_WARPS = 8;
+constexpr int SG_THREADS = 32 * (SG_CUT_WARPS + SG_MMA_WARPS + SG_SUM_WARPS);
+constexpr int SG_CUT_REGS = 80, SG_MMA_REGS = 40, SG_SUM_REGS = 72;  // registers a thread: the launch's 72, shared out
+static_assert(SG_CUT_WARPS * SG_CUT_REGS + SG_MMA_WARPS * SG_MMA_REGS + SG_SUM_WARPS * SG_SUM_REGS == SG_THREADS / 32 * 72, "shares of the launch's registers");
+constexpr int SG_A_RUNS = SG_M * SG_K / 8 / SG_GROUP_THREADS, SG_B_RUNS = SG_N * SG_K / 8 / SG_GROUP_THREADS;  // runs of eight elements per thread
+constexpr int SG_SMEM = SG_STAGES * SG_STAGE + 1024;
+constexpr int SG_ACC_PITCH = 256;  // columns from one accumulator (three times SG_N of them) to the other
+constexpr int SG_CHUNK = 2;  // k-slices per accumulator
+static_assert(SG_SMEM + 512 <= 227 * 1024, "shared memory of a CTA");
+
+__device__ int g_split_timeout_flag = 0;
+
+struct SplitParams {
+  const float *A, *B;        // A: [M][K] or, MN kernels, [K][M]; B likewise
+  long long sAb, sBb, sDb;   // batch strides
+  int ldA, ldB;
+  int M, N, K, batches;
+  int group;                 // D(m, n) = D[b * sDb + m / group * sDg + m % group + n * sDn]
+  long long sDg, sDn;
+  float* D;
+  const float *bias, *residual;  // of column n; laid out like D
+  int act;                   // see act_f32
+  int m_tiles, n_tiles;
+  int first;                 // first kernel of a call
+};
+
+// How an operand is fetched: k contiguous, runs of eight 32- or 16-byte aligned; rows (m or n) contiguous, runs 32- or 16-byte aligned or not at all.
+// (With two 16-byte loads a warp touches every line twice: 8192 x 576 x 192 23.5 us against 21.9.)
+enum SplitFetch { SPLIT_K, SPLIT_K4, SPLIT_MN, SPLIT_MN4, SPLIT_MN1 };
+__host__ __device__ constexpr bool sg_k_contiguous(SplitFetch f) { return f == SPLIT_K || f == SPLIT_K4; }
+
+// Loads that a predicate leaves out (zeros), without branches: the cutting of one run overlaps the fetch of another.  Eight consecutive
+// floats, 32-byte aligned; four, 16-byte aligned; one.
+__device__ __forceinline__ void sg_load8(float* v, const float* p, bool ok) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %9, 0;\n\t@q ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n\t}"
+               : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]) : "l"(p), "r"((int)ok));
+}
+__device__ __forceinline__ void sg_load4(float* v, const float* p, bool ok) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t@q ld.global.v4.f32 {%0,%1,%2,%3}, [%4];\n\t}"
+               : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]) : "l"(p), "r"((int)ok));
+}
+__device__ __forceinline__ void sg_load1(float* v, const float* p, bool ok) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t@q ld.global.f32 %0, [%1];\n\t}" : "+f"(v[0]) : "l"(p), "r"((int)ok));
+}
+
+// Eight elements of an operand: `run` of a slice of ROWS x 64 that begins at row r0, k = k0.  K-contiguous: k 8c .. + 7 of a row;
+// otherwise rows 8c .. + 7 of one k.
+template <int ROWS, SplitFetch F>
+__device__ __forceinline__ void sg_fetch(float (&v)[8], const float* base, int ld, int rows, int K, int r0, int k0, int run) {
+  constexpr int PER_K = ROWS / 8;
+  const int r = sg_k_contiguous(F) ? r0 + run / 8 : r0 + run % PER_K * 8, k = sg_k_contiguous(F) ? k0 + run % 8 * 8 : k0 + run / PER_K;
+  const float* p = base + (sg_k_contiguous(F) ? (long long)r * ld + k : (long long)k * ld + r);
+#pragma unroll
+  for (int e = 0; e < 8; ++e) v[e] = 0.f;
+  const bool ok = k < K && r < rows;  // K is a multiple of eight, and the rows are one of eight (SPLIT_MN) or four (SPLIT_MN4)
+  if constexpr (F == SPLIT_K || F == SPLIT_MN) {
+    sg_load8(v, p, ok);
+  } else if constexpr (F == SPLIT_MN1) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) sg_load1(v + e, p + e, ok && r + e < rows);
+  } else {
+    sg_load4(v, p, ok);
+    sg_load4(v + 4, p + 4, ok && (F == SPLIT_K4 || r + 4 < rows));
+  }
+}
+// The pieces of a run go to the same 16 bytes of the three piece tiles: rows of 64 elements (128 bytes, 128B swizzle), k-contiguous
+// operands a row per m or n, the others a row per k in blocks of 64 rows.
+template <int ROWS, SplitFetch F, int PIECE>
+__device__ __forceinline__ void sg_put(uint32_t tile, const float (&v)[8], int run) {
+  constexpr int PER_K = ROWS / 8;
+  const int row = sg_k_contiguous(F) ? run / 8 : run / PER_K, c = sg_k_contiguous(F) ? run % 8 : run % PER_K;
+  const uint32_t at = tile + (uint32_t)((c >> 3) * (64 * 128) + row * 128 + (((c & 7) ^ (row & 7)) << 4));
+  uint32_t w[SG_PIECES][4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    float a = v[2 * e], b = v[2 * e + 1];
+    w[0][e] = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+    a -= __uint_as_float(__float_as_uint(a) & 0xffff0000u);
+    b -= __uint_as_float(__float_as_uint(b) & 0xffff0000u);
+    w[1][e] = pack2(a, b);
+    a -= __uint_as_float(w[1][e] << 16);
+    b -= __uint_as_float(w[1][e] & 0xffff0000u);
+    w[2][e] = pack2(a, b);
+  }
+#pragma unroll
+  for (int i = 0; i < SG_PIECES; ++i)
+    asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(at + i * PIECE), "r"(w[i][0]), "r"(w[i][1]), "r"(w[i][2]), "r"(w[i][3]) : "memory");
+}
+
+__device__ __forceinline__ void sg_tmem_ld8(uint32_t taddr, float (&f)[8]) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) f[i] = __uint_as_float(r[i]);
+}
+
+template <SplitFetch FA, SplitFetch FB, bool FULL>
+__global__ void __launch_bounds__(SG_THREADS, 1)
+split_gemm_kernel(SplitParams p) {
+  extern __shared__ unsigned char smem_raw[];
+  const uint32_t ring = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  __shared__ __align__(8) unsigned long long bar_storage[2 * SG_STAGES + 4];
+  __shared__ uint32_t tmem_slot;
+  __shared__ int abort_flag;
+  const uint32_t bars = smem_u32(bar_storage);
+  const uint32_t full_bar = bars, empty_bar = bars + 8 * SG_STAGES, afull_bar = bars + 16 * SG_STAGES, aempty_bar = afull_bar + 16;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int tiles = p.batches * p.m_tiles * p.n_tiles, k_iters = (p.K + SG_K - 1) / SG_K;
+  if (!p.first) pdl_launch_dependents();
+  if (threadIdx.x == 0) {
+    abort_flag = 0;
+    for (int s = 0; s < SG_STAGES; ++s) { mbar_init(full_bar + 8 * s, SG_GROUP_WARPS); mbar_init(empty_bar + 8 * s, 1); }
+    for (int a = 0; a < 2; ++a) { mbar_init(afull_bar + 8 * a, 1); mbar_init(aempty_bar + 8 * a, SG_SUM_WARPS); }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == SG_CUT_WARPS) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *(volatile uint32_t*)&tmem_slot;
+  if (p.first) pdl_first_wait();
+  else pdl_wait();
+  bool ok = true;
+  auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
+    ok = mbar_wait(bar, parity, &abort_flag);
+    ok = __all_sync(0xffffffffu, ok);
+    return ok;
+  };
+  // tiles that share columns (the larger part of the bytes to fetch is A's) run side by side
+  auto locate = [&](int tile, int& b, int& m0, int& n0) {
+    const int per = p.m_tiles * p.n_tiles;
+    b = tile / per;
+    const int r = tile - b * per;
+    n0 = r / p.m_tiles * SG_N;
+    m0 = r % p.m_tiles * SG_M;
+  };
+
+  if (warp < SG_CUT_WARPS) {
+    // ------------------------------------------------------------ fetch and cut
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(SG_CUT_REGS));
+    const int group = warp / SG_GROUP_WARPS, tid = threadIdx.x - group * SG_GROUP_THREADS;
+    float ra[SG_A_RUNS][8], rb[SG_B_RUNS][8];
+    const int slices = tiles > (int)blockIdx.x ? ((tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1) * k_iters : 0;  // of all tiles of this CTA
+    int tile = blockIdx.x, kb = 0;  // of the group's next slice to fetch
+    const float *pa = nullptr, *pb = nullptr;
+    int m0 = 0, n0 = 0;
+    auto seek = [&] {
+      int b;
+      locate(tile, b, m0, n0);
+      pa = p.A + (long long)b * p.sAb;
+      pb = p.B + (long long)b * p.sBb;
+    };
+    auto advance = [&](int by) {
+      kb += by;
+      bool moved = false;
+      while (kb >= k_iters) { kb -= k_iters; tile += gridDim.x; moved = true; }
+      if (moved && tile < tiles) seek();
+    };
+    if (slices > 0) seek();
+    advance(group);
+    if (group < slices) {
+#pragma unroll
+      for (int i = 0; i < SG_A_RUNS; ++i) sg_fetch<SG_M, FA>(ra[i], pa, p.ldA, p.M, p.K, m0, kb * SG_K, tid + i * SG_GROUP_THREADS);
+#pragma unroll
+      for (int i = 0; i < SG_B_RUNS; ++i) sg_fetch<SG_N, FB>(rb[i], pb, p.ldB, p.N, p.K, n0, kb * SG_K, tid + i * SG_GROUP_THREADS);
+    }
+#pragma unroll 1
+    for (int it = group; it < slices; it += SG_GROUPS) {
+      const uint32_t s = (uint32_t)it % SG_STAGES, ph = ((uint32_t)it / SG_STAGES) & 1;
+      if (!wait(empty_bar + 8 * s, ph ^ 1)) break;
+      advance(SG_GROUPS);
+      const bool more = it + SG_GROUPS < slices;
+      const uint32_t sa = ring + s * SG_STAGE, sb = sa + SG_PIECES * SG_A_PIECE;
+#pragma unroll
+      for (int i = 0; i < SG_A_RUNS; ++i) {
+        sg_put<SG_M, FA, SG_A_PIECE>(sa, ra[i], tid + i * SG_GROUP_THREADS);
+        if (more) sg_fetch<SG_M, FA>(ra[i], pa, p.ldA, p.M, p.K, m0, kb * SG_K, tid + i * SG_GROUP_THREADS);
+      }
+#pragma unroll
+      for (int i = 0; i < SG_B_RUNS; ++i) {
+        sg_put<SG_N, FB, SG_B_PIECE>(sb, rb[i], tid + i * SG_GROUP_THREADS);
+        if (more) sg_fetch<SG_N, FB>(rb[i], pb, p.ldB, p.N, p.K, n0, kb * SG_K, tid + i * SG_GROUP_THREADS);
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the tensor cores read what was just written
+      __syncwarp();
+      if (lane == 0) mbar_arrive(full_bar + 8 * s);
+    }
+  } else if (warp < SG_CUT_WARPS + SG_MMA_WARPS) {
+    // ------------------------------------------------------------ MMA issuer
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SG_MMA_REGS));
+    if (warp == SG_CUT_WARPS && lane == 0) {
+      // D = f32, A = B = bf16; bits 15 and 16: A, B are row-contiguous; N >> 3 at 17, M >> 4 at 24
+      constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (sg_k_contiguous(FA) ? 0u : 1u << 15) | (sg_k_contiguous(FB) ? 0u : 1u << 16) | ((uint32_t)(SG_M >> 4) << 24);
+      constexpr uint32_t a_step = sg_k_contiguous(FA) ? 32 : 2048, b_step = sg_k_contiguous(FB) ? 32 : 2048;  // bytes per 16 k
+      uint32_t it = 0, chunk = 0;
+      for (int tile = blockIdx.x; ok && tile < tiles; tile += gridDim.x) {
+        for (int kb = 0; ok && kb < k_iters; ++kb, ++it) {
+          const uint32_t acc = chunk & 1, d = tmem_base + acc * SG_ACC_PITCH;
+          const bool start = kb % SG_CHUNK == 0, end = kb % SG_CHUNK == SG_CHUNK - 1 || kb == k_iters - 1;
+          if (start) {
+            ok = mbar_wait(aempty_bar + 8 * acc, ((chunk >> 1) & 1) ^ 1, &abort_flag);
+            if (!ok) break;
+          }
+          const uint32_t s = it % SG_STAGES, ph = (it / SG_STAGES) & 1;
+          ok = mbar_wait(full_bar + 8 * s, ph, &abort_flag);
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t sa = ring + s * SG_STAGE, sb = sa + SG_PIECES * SG_A_PIECE;
+#pragma unroll
+          for (int kk = 0; kk < SG_K / 16; ++kk) {
+            const uint32_t more = start && kk == 0 ? 0u : 1u;
+            const uint64_t bd = make_desc(sb + kk * b_step, sg_k_contiguous(FB) ? 1 : SG_B_PIECE >> 4, 1024 >> 4);
+#pragma unroll
+            for (int i = 0; i < SG_PIECES; ++i)  // piece i of A meets the first 3 - i pieces of B
+              umma_bf16(d + i * SG_N, make_desc(sa + i * SG_A_PIECE + kk * a_step, sg_k_contiguous(FA) ? 1 : (SG_A_PIECE / 2) >> 4, 1024 >> 4), bd,
+                        idesc | ((uint32_t)((SG_PIECES - i) * SG_N >> 3) << 17), i == 0 ? more : 1u);
+          }
+          umma_commit(empty_bar + 8 * s);
+          if (end) { umma_commit(afull_bar + 8 * acc); ++chunk; }
+        }
+      }
+    }
+  } else {
+    // ------------------------------------------------------------ sums and output
+    const int quarter = warp & 3, half = (warp - SG_CUT_WARPS - SG_MMA_WARPS) >> 2;  // TMEM lanes 32 * quarter .. (a hardware rule), columns 32 * half ..
+    const uint32_t taddr = tmem_base + (uint32_t)(half * 32) + ((uint32_t)(quarter * 32) << 16);
+    const int chunks = (k_iters + SG_CHUNK - 1) / SG_CHUNK;
+    uint32_t chunk = 0;
+#pragma unroll 1
+    for (int tile = blockIdx.x; ok && tile < tiles; tile += gridDim.x) {
+      int b, m0, n0;
+      locate(tile, b, m0, n0);
+      const float bias = FULL && p.bias && n0 + half * 32 + lane < p.N ? __uint_as_float(ld_dep32(p.bias + n0 + half * 32 + lane)) : 0.f;
+      float sum[32];
+#pragma unroll
+      for (int c = 0; c < 32; ++c) sum[c] = 0.f;
+#pragma unroll 1
+      for (int i = 0; i < chunks; ++i, ++chunk) {
+        const uint32_t acc = chunk & 1;
+        if (!wait(afull_bar + 8 * acc, (chunk >> 1) & 1)) break;
+        tc_fence_after();
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          const uint32_t at = taddr + acc * SG_ACC_PITCH + h * 8;
+          float x[8], y[8], z[8];
+          sg_tmem_ld8(at, x);
+          sg_tmem_ld8(at + SG_N, y);
+          sg_tmem_ld8(at + 2 * SG_N, z);
+          tmem_ld_wait();
+#pragma unroll
+          for (int c = 0; c < 8; ++c) sum[8 * h + c] += x[c] + (y[c] + z[c]);
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(aempty_bar + 8 * acc);
+      }
+      if (!ok) break;
+      const int m = m0 + quarter * 32 + lane;
+      const int n = n0 + half * 32, cols = m < p.M ? min(32, p.N - n) : 0;
+      const long long at = (long long)b * p.sDb + (long long)(m / p.group) * p.sDg + m % p.group + n * p.sDn;
+      float* out = p.D + at;
+      if constexpr (!FULL) {
+#pragma unroll
+        for (int c = 0; c < 32; ++c, out += p.sDn)
+          if (c < cols) *out = sum[c];
+      } else {
+        // bias: a column per lane, fetched before the sums are waited for; residual: eight columns at a time
+        const float* res = p.residual + at;
+#pragma unroll
+        for (int c8 = 0; c8 < 32; c8 += 8) {
+          float x[8];
+#pragma unroll
+          for (int c = 0; c < 8; ++c, res += p.sDn) x[c] = p.residual && c8 + c < cols ? __uint_as_float(ld_dep32(res)) : 0.f;
+#pragma unroll
+          for (int c = 0; c < 8; ++c, out += p.sDn) {
+            float v = sum[c8 + c] + __shfl_sync(0xffffffffu, bias, c8 + c);
+            if (p.act) v = p.act == 1 ? fmaxf(v, 0.f) : v * __saturatef(fmaf(v, 1.f / 6.f, 0.5f));
+            if (c8 + c < cols) *out = v + x[c];
+          }
+        }
+      }
+      __syncwarp();
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (abort_flag) {
+    for (int i = 0; i < 64; ++i) __nanosleep(1000);  // MMAs still in flight end before memory is released
+    if (threadIdx.x == 0) atomicExch(&g_split_timeout_flag, 1);
+    __syncthreads();
+  }
+  if (warp == SG_CUT_WARPS) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
+  }
+}
+
+bool aligned32(const void* p) { return reinterpret_cast<uintptr_t>(p) % 32 == 0; }
+
+template <SplitFetch FA, SplitFetch FB, bool FULL>
+msla_status_t launch_split(SplitParams p, cudaStream_t st) {
+  static std::atomic<unsigned long long> attr_done{0};
+  const msla_status_t s = ensure_smem_attr(attr_done, split_gemm_kernel<FA, FB, FULL>, SG_SMEM);
+  if (s != MSLA_OK) return s;
+  p.m_tiles = (p.M + SG_M - 1) / SG_M;
+  p.n_tiles = (p.N + SG_N - 1) / SG_N;
+  const long long tiles = (long long)p.batches * p.m_tiles * p.n_tiles;
+  if (tiles * ((p.K + SG_K - 1) / SG_K) > 0x7fffffffLL) return fail(MSLA_ERR_UNSUPPORTED, "too many tiles");
+  const int grid = (int)(tiles < device_sm_count() ? tiles : device_sm_count());
+  launch_pdl(split_gemm_kernel<FA, FB, FULL>, dim3((unsigned)grid), dim3(SG_THREADS), SG_SMEM, st, p);
+  count_launches(1);
+  return check_launch("fp32 GEMM on tensor cores");
+}
+
+}  // namespace
+
+// y planar [B][Cout / d][N][d] = w [Cout][C] times x [B][C][N].
+msla_status_t run_project_in_split(const float* x, const float* w, float* y, int B, int C, int Cout, int N, int d, long long y_sb, cudaStream_t st, bool first) {
+  SplitParams p{};
+  p.A = w; p.ldA = C;
+  p.B = x; p.ldB = N; p.sBb = (long long)C * N;
+  p.M = Cout; p.N = N; p.K = C; p.batches = B;
+  p.D = y; p.sDb = y_sb; p.group = d; p.sDg = (long long)N * d; p.sDn = d;
+  p.first = first;
+  if (N % 8 == 0 && aligned32(x) && aligned32(w)) return launch_split<SPLIT_K, SPLIT_MN, false>(p, st);
+  return N % 4 == 0 ? launch_split<SPLIT_K4, SPLIT_MN4, false>(p, st) : launch_split<SPLIT_K4, SPLIT_MN1, false>(p, st);
+}
+
+// y [B][Cout][N] = act(w [Cout][K] times a + bias) + residual; a: [B][N][K] (token_major) or [B][K][N].
+msla_status_t run_project_out_split(const float* a, bool token_major, const float* w, const float* bias, int act, const float* residual, float* y, int B, int K,
+                                    int Cout, int N, cudaStream_t st, bool first) {
+  SplitParams p{};
+  p.A = a; p.ldA = token_major ? K : N; p.sAb = (long long)K * N;
+  p.B = w; p.ldB = K;
+  p.M = N; p.N = Cout; p.K = K; p.batches = B;
+  p.D = y; p.sDb = (long long)Cout * N; p.group = N; p.sDg = 0; p.sDn = N;
+  p.bias = bias; p.act = act; p.residual = residual; p.first = first;
+  const bool wide = aligned32(a) && aligned32(w);
+  if (token_major) return wide ? launch_split<SPLIT_K, SPLIT_K, true>(p, st) : launch_split<SPLIT_K4, SPLIT_K4, true>(p, st);
+  if (N % 8 == 0 && wide) return launch_split<SPLIT_MN, SPLIT_K, true>(p, st);
+  return N % 4 == 0 ? launch_split<SPLIT_MN4, SPLIT_K4, true>(p, st) : launch_split<SPLIT_MN1, SPLIT_K4, true>(p, st);
+}
+
+int split_gemm_timeout_flag() {
+  int v = 0;
+  if (cudaMemcpyFromSymbol(&v, g_split_timeout_flag, sizeof(int)) != cudaSuccess) {
+    cudaGetLastError();
+    return -1;
+  }
+  return v;
+}
+
+}  // namespace msla

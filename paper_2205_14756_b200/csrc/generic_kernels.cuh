@@ -1,7 +1,7 @@
 // Kernels on the fp32 pipes for every stage of the module, templated on the storage
-// type.  They are the fp32 path (a TF32 tensor-core product would not meet the
-// fp32 accuracy bound) and the fallback for 16-bit shapes the tensor-core kernels do
-// not cover.  All accumulate in fp32 and are deterministic.
+// type.  They are the fp32 path (but for large projections, which run on tensor cores in
+// gemm_f32_split.cu; a TF32 product would not meet the fp32 accuracy bound) and the fallback for 16-bit
+// shapes the tensor-core kernels do not cover.  All accumulate in fp32 and are deterministic.
 //
 // What bounds them is how many multiply-adds a shared-memory access feeds: every inner loop works on a register tile
 // (4 x 4 to 8 x 4 outputs) read in 16-byte pieces.  Module [1, 192, 64, 128], d = 32, fp32: 333 us per forward with one or
@@ -29,12 +29,6 @@ struct GemmArgs {
   int act;       // applied to the sum + bias: 0 none, 1 ReLU, 2 hard-swish
   const void* residual;  // nullptr, or a tensor laid out like D, added after the activation
 };
-
-__device__ __forceinline__ float act_f32(float v, int act) {
-  if (act == 1) return fmaxf(v, 0.f);
-  if (act == 2) return v * fminf(fmaxf(v + 3.f, 0.f), 6.f) / 6.f;
-  return v;
-}
 
 // Four consecutive elements, aligned to their total size, and one element, of a tensor that an earlier kernel of the stream may have
 // written (the caller's weights among them).

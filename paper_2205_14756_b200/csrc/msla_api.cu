@@ -418,10 +418,28 @@ static void launch_gemm(const T* A, const T* W, const T* bias, T* D, generic::Ge
   else launch_gemm_tile<T, 32, 32, 32, 4, 4>(A, W, bias, D, g, B, vec, st);
 }
 
+// fp32 products on tensor cores (gemm_f32_split.cu) or on the fp32 pipes.  One call of B x N tokens, us, pipes / tensor cores: 8192 tokens 192 -> 576
+// 43.8 / 22.7, 384 -> 192 (token-major) 61.9 / 19.0, 4096 tokens 1024 -> 256 124 / 21.8, 784 tokens 128 -> 384 14.7 / 6.4, 2 x 196 128 -> 384
+// 7.2 / 6.6, 196 512 -> 256 13.2 / 12.1; below the line, where a few CTAs run the longer chain, 784 128 -> 128 5.0 / 6.3, 512 128 -> 128 4.9 / 6.2,
+// 1024 64 -> 192 4.8 / 5.0, 2 x 196 256 -> 128 7.7 / 8.4.
+static bool split_gemm_pays(int B, int N, int Cout, int K) { return (long long)B * N * Cout * K >= 1LL << 24; }
+
+// A layer of the FFN, activations [B][channels][tokens].
+template <typename T>
+static msla_status_t launch_nchw_gemm(const T* x, const T* w, const T* bias, T* y, const generic::GemmArgs& g, int B, bool first, cudaStream_t st) {
+  if constexpr (sizeof(T) == 4) {
+    if (split_gemm_pays(B, g.M, g.Nc, g.K))
+      return run_project_out_split(x, false, w, bias, g.act, (const float*)g.residual, y, B, g.K, g.Nc, g.M, st, first);
+  }
+  launch_gemm<T>(x, w, bias, y, g, B, st);
+  return MSLA_OK;
+}
+
 // y planar: y[b*y_sb + ((o/d)*N + n)*d + o%d]; rows of x are ldx elements apart (N where the plain kernels run)
 static msla_status_t run_project_in(msla_dtype_t dt, const void* x, int ldx, const void* w, void* y, int B,
                                     int C, int Cout, int N, int d, long long y_sb, cudaStream_t st, bool first) {
   if (dt != MSLA_F32 && project_in_bf16_supported(C, Cout, ldx, d)) return run_project_in_bf16(x, ldx, w, y, B, C, Cout, N, d, y_sb, st, dt == MSLA_F16, first);
+  if (dt == MSLA_F32 && split_gemm_pays(B, N, Cout, C)) return run_project_in_split((const float*)x, (const float*)w, (float*)y, B, C, Cout, N, d, y_sb, st, first);
   generic::GemmArgs g{(long long)C * N, 1, N, y_sb, d, 1, (long long)N * d, N, Cout, C, d};
   if (dt == MSLA_F32) launch_gemm<float>((const float*)x, (const float*)w, nullptr, (float*)y, g, B, st);
   else if (dt == MSLA_F16) launch_gemm<__half>((const __half*)x, (const __half*)w, nullptr, (__half*)y, g, B, st);
@@ -433,6 +451,8 @@ static msla_status_t run_project_out(msla_dtype_t dt, const void* a, const void*
                                      void* y, int ldy, int B, int Cin, int Cout, int N, cudaStream_t st, const void* residual = nullptr, bool first = false) {
   if (dt != MSLA_F32 && project_out_bf16_supported(Cin, Cout, ldy))
     return run_project_out_bf16(a, w, bias, residual, y, ldy, B, Cin, Cout, N, st, dt == MSLA_F16, first);
+  if (dt == MSLA_F32 && split_gemm_pays(B, N, Cout, Cin))
+    return run_project_out_split((const float*)a, true, (const float*)w, (const float*)bias, 0, (const float*)residual, (float*)y, B, Cin, Cout, N, st, first);
   generic::GemmArgs g{(long long)N * Cin, Cin, 1, (long long)Cout * N, 1, N, 0, N, Cout, Cin, Cout, 0, residual};
   if (dt == MSLA_F32) launch_gemm<float>((const float*)a, (const float*)w, (const float*)bias, (float*)y, g, B, st);
   else if (dt == MSLA_F16) launch_gemm<__half>((const __half*)a, (const __half*)w, (const __half*)bias, (__half*)y, g, B, st);
@@ -996,14 +1016,15 @@ static msla_status_t ffn_impl(const msla_ffn_desc* desc, const void* x, const ms
   const long long total = (long long)B * Ch * N;
   auto plain = [&](auto* tag) {
     using T = std::remove_pointer_t<decltype(tag)>;
-    launch_gemm<T>((const T*)x, (const T*)w->w1, (const T*)w->b1, (T*)h, g1, B, st);
+    if ((s = launch_nchw_gemm<T>((const T*)x, (const T*)w->w1, (const T*)w->b1, (T*)h, g1, B, first, st)) != MSLA_OK) return;
     generic::ffn_dw3x3_nchw_kernel<T><<<(unsigned)ceil_div_ll(total, 256), 256, 0, st>>>((const T*)h, (const T*)w->w_dw, (const T*)w->b_dw, (T*)g, Ch,
                                                                                         desc->H, desc->W, act, total);
-    launch_gemm<T>((const T*)g, (const T*)w->w2, (const T*)w->b2, (T*)out, g2, B, st);
+    s = launch_nchw_gemm<T>((const T*)g, (const T*)w->w2, (const T*)w->b2, (T*)out, g2, B, false, st);
   };
   if (desc->dtype == MSLA_F32) plain((float*)nullptr);
   else if (desc->dtype == MSLA_F16) plain((__half*)nullptr);
   else plain((__nv_bfloat16*)nullptr);
+  if (s != MSLA_OK) return s;
   count_launches(1);
   return check_launch("FFN with a depthwise convolution");
 }
@@ -1136,7 +1157,7 @@ unsigned long long msla_kernel_launches(void) { return g_launches; }
 
 int msla_debug_wait_timeouts(void) {
   int all = 0;
-  for (int (*flag)() : {gemm_timeout_flag, agg_timeout_flag, fused_timeout_flag, dw_timeout_flag, agg_state_timeout_flag, project_planes_timeout_flag}) {
+  for (int (*flag)() : {gemm_timeout_flag, agg_timeout_flag, fused_timeout_flag, dw_timeout_flag, agg_state_timeout_flag, project_planes_timeout_flag, split_gemm_timeout_flag}) {
     const int v = flag();
     if (v < 0) return -1;
     all |= v;

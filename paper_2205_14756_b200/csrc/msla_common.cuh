@@ -34,6 +34,13 @@ template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(flo
 }
 template <> __device__ __forceinline__ __half from_f32<__half>(float v) { return __float2half_rn(v); }
 
+// The activations of the fp32 kernels: 0 none, 1 ReLU, 2 hard-swish.
+__device__ __forceinline__ float act_f32(float v, int act) {
+  if (act == 1) return fmaxf(v, 0.f);
+  if (act == 2) return v * fminf(fmaxf(v + 3.f, 0.f), 6.f) / 6.f;
+  return v;
+}
+
 // Programmatic dependent launch.  The tuned kernels are launched so that a
 // kernel may become resident while its predecessor in the stream is still
 // running: it sets up what depends on no earlier kernel (barriers, tensor

@@ -134,6 +134,12 @@ bool project_out_planar_bf16_supported(int Cin, int Cout);
 msla_status_t run_project_out_planar_bf16(const void* a, const void* w, const void* bias, const void* residual, void* y, int ldy, int B,
                                           int Cin, int Cout, int N, cudaStream_t st, bool f16 = false);
 int gemm_timeout_flag();
+
+// fp32 projections on tensor cores (gemm_f32_split.cu); K a multiple of 8, 16-byte aligned tensors.
+msla_status_t run_project_in_split(const float* x, const float* w, float* y, int B, int C, int Cout, int N, int d, long long y_sb, cudaStream_t st, bool first);
+msla_status_t run_project_out_split(const float* a, bool token_major, const float* w, const float* bias, int act, const float* residual, float* y, int B, int K,
+                                    int Cout, int N, cudaStream_t st, bool first);
+int split_gemm_timeout_flag();
 int run_wait_selftest(long long limit_cycles, int* scratch, cudaStream_t st);
 
 // bf16 aggregation (d = 16 or 32, Ch a multiple of 32): TMA halo tiles, depthwise filter as banded matrices on
