@@ -96,7 +96,7 @@ __device__ __forceinline__ void lds64(uint32_t (&r)[2], uint32_t addr) {
 // occupancy); no block-wide barrier is taken inside the loop.  An extra B tile
 // of bf16 ones yields sum relu(k).
 // ---------------------------------------------------------------------------
-template <int D, int NWARPS, int STAGES, bool F16>
+template <int D, int NWARPS, int STAGES, bool F16, bool HOLD>
 __global__ void __launch_bounds__(NWARPS * 32)
 kv_state_mma_kernel(const bf16* __restrict__ k, const bf16* __restrict__ v, float* __restrict__ partial,
                     HeadView kv, int heads, int N, int S, int chunk) {
@@ -113,8 +113,11 @@ kv_state_mma_kernel(const bf16* __restrict__ k, const bf16* __restrict__ v, floa
   extern __shared__ __align__(128) unsigned char smem[];
   static_assert(NWARPS * STAGES * 2 * TILEB >= NWARPS * NE * 4, "reduction buffer must fit in the stage ring");
 
-  pdl_launch_dependents();
-  pdl_wait();  // k and v come from the previous kernel
+  // k and v may come from the previous kernel.  HOLD: the apply step fetches queries before its own wait, so it may only run once what
+  // came before this kernel is complete.
+  if (!HOLD) pdl_launch_dependents();
+  pdl_wait();
+  if (HOLD) pdl_launch_dependents();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
   const int bh = blockIdx.x, s = blockIdx.y;
@@ -269,7 +272,7 @@ struct PlanesView {
 template <int D, int NWARPS, int STAGES, int U, bool PAIR, bool F16, bool PLANES = false>
 __global__ void __launch_bounds__(NWARPS * 32)
 apply_mma_kernel(const bf16* __restrict__ q, const float* __restrict__ state, int S, bf16* __restrict__ out,
-                 HeadView qv, HeadView ov, int heads, int N, float eps, int tok_per_cta, float state_scale, PlanesView pv) {
+                 HeadView qv, HeadView ov, int heads, int N, float eps, int tok_per_cta, float state_scale, PlanesView pv, bool early) {
   constexpr int KS = D / 16;   // MMA steps over the channel contraction
   constexpr int NT = D / 8;    // output tiles, + 1 for the denominator
   constexpr int CPT = D / 4;   // channels per lane per token
@@ -281,7 +284,7 @@ apply_mma_kernel(const bf16* __restrict__ q, const float* __restrict__ state, in
   // the MMAs without holding registers and without any cross-lane hand-off.
   __shared__ __align__(16) unsigned char fifo[NWARPS * STAGES * STAGEB];
   pdl_launch_dependents();
-  pdl_wait();  // the state comes from the previous kernel
+  if (!early) pdl_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
   constexpr int NW = PAIR ? NWARPS / 2 : NWARPS;  // warps sharing one head's tokens
@@ -336,6 +339,7 @@ apply_mma_kernel(const bf16* __restrict__ q, const float* __restrict__ state, in
     cp_async_commit();
   }
 
+  if (early) pdl_wait();  // the state comes from the previous kernel, the queries from before the reduction
   // The state's B fragments (bf16 hi + lo), overlapping the first copies
   uint32_t bhi[KS][NT + 1][2], blo[KS][NT + 1][2];
   auto fragments = [&](auto st) {  // st(e): entry e of the head's state
@@ -448,13 +452,13 @@ apply_mma_kernel(const bf16* __restrict__ q, const float* __restrict__ state, in
   cp_async_wait<0>();
 }
 
-template <int D, int STAGES, bool F16>
+template <int D, int STAGES, bool F16, bool HOLD>
 msla_status_t launch_kv_state(const bf16* k, const bf16* v, float* partial, HeadView in, long long BH, int heads, int N, const CorePlan& p, cudaStream_t st) {
   constexpr int WARPS = 4, smem = WARPS * STAGES * 2 * 32 * D * 2;
   static std::atomic<unsigned long long> attr_done{0};
-  const msla_status_t as = ensure_smem_attr(attr_done, kv_state_mma_kernel<D, WARPS, STAGES, F16>, smem);
+  const msla_status_t as = ensure_smem_attr(attr_done, kv_state_mma_kernel<D, WARPS, STAGES, F16, HOLD>, smem);
   if (as != MSLA_OK) return as;
-  launch_pdl(kv_state_mma_kernel<D, WARPS, STAGES, F16>, dim3((unsigned)BH, p.S), dim3(WARPS * 32), smem, st, k, v, partial, in, heads, N, p.S, p.chunk);
+  launch_pdl(kv_state_mma_kernel<D, WARPS, STAGES, F16, HOLD>, dim3((unsigned)BH, p.S), dim3(WARPS * 32), smem, st, k, v, partial, in, heads, N, p.S, p.chunk);
   return MSLA_OK;
 }
 
@@ -467,11 +471,18 @@ msla_status_t launch_core(const bf16* q, const bf16* k, const bf16* v, bf16* out
   float* partial = reinterpret_cast<float*>(ws + p.partial_off);
   float* state = reinterpret_cast<float*>(ws + p.state_off);
   int launches = 0;
+  // The apply step's first queries are fetched while the reduction ends, where both run.  Core, us, without / with: [8, 16, 4096, 32] 32.7 / 30.9,
+  // [2, 24, 12000, 32] 36.3 / 34.3, [6, 10, 5000, 32] 23.4 / 22.0, [16, 8, 9000, 16] 35.1 / 33.0, [4, 24, 1600, 32] 15.7 / 14.6, [1, 8, 16384, 32]
+  // 17.4 / 16.2.  Not for small problems, where the later launch costs as much ([1, 16, 4096, 32] 11.2 to 11.8 / 11.7), nor where the reduction
+  // takes more than a wave and its last CTAs start late ([37, 16, 3000, 32] 85.1 / 85.9).
+  const bool early = (phases & CORE_STATE) && (phases & CORE_APPLY) && BH * N * D >= 3LL << 20 && BH * p.S <= (D == 32 ? 3 : 6) * device_sm_count();
   if (phases & CORE_STATE) {
-    // Many heads of few tokens: no warp has more than two groups, and rings of two stages put twice the CTAs on an SM.  Module, us:
+    // (never together with `early`, which excludes more than a wave) Many heads of few tokens: no warp has more than two groups, and rings of two stages put twice the CTAs on an SM.  Module, us:
     // [64, 256, 14, 14] (1024 CTAs) 69.6 -> 68.6, [64, 256, 16, 16] 62.1 -> 60.9, [32, 384, 7, 7] (768) 45.9 -> 45.2; core [64, 8, 196, 32] (512) 11.65 -> 11.9.
     const bool many = p.chunk <= 256 && BH * p.S > (D == 32 ? 4 : 8) * device_sm_count();
-    const msla_status_t as = many ? launch_kv_state<D, 2, F16>(k, v, partial, in, BH, heads, N, p, st) : launch_kv_state<D, 4, F16>(k, v, partial, in, BH, heads, N, p, st);
+    const msla_status_t as = many    ? launch_kv_state<D, 2, F16, false>(k, v, partial, in, BH, heads, N, p, st)
+                             : early ? launch_kv_state<D, 4, F16, true>(k, v, partial, in, BH, heads, N, p, st)
+                                     : launch_kv_state<D, 4, F16, false>(k, v, partial, in, BH, heads, N, p, st);
     if (as != MSLA_OK) return as;
     ++launches;
   }
@@ -496,11 +507,11 @@ msla_status_t launch_core(const bf16* q, const bf16* k, const bf16* v, bf16* out
     if (ov.pair) {  // heads is even here, so a pair never straddles two images
       const int tok_per_cta = p.apply_tokens / 2;
       launch_pdl(apply_mma_kernel<D, AP_WARPS, AP_STAGES, AP_U, true, F16>, dim3((unsigned)ceil_div_ll(N, tok_per_cta), (unsigned)(BH / 2)),
-                 dim3(AP_WARPS * 32), 0, st, q, sums, S, out, in, ov, heads, N, eps, tok_per_cta, state_scale, PlanesView{});
+                 dim3(AP_WARPS * 32), 0, st, q, sums, S, out, in, ov, heads, N, eps, tok_per_cta, state_scale, PlanesView{}, early);
     } else {
       const int tok_per_cta = p.apply_tokens;
       launch_pdl(apply_mma_kernel<D, AP_WARPS, AP_STAGES, AP_U, false, F16>, dim3((unsigned)ceil_div_ll(N, tok_per_cta), (unsigned)BH),
-                 dim3(AP_WARPS * 32), 0, st, q, sums, S, out, in, ov, heads, N, eps, tok_per_cta, state_scale, PlanesView{});
+                 dim3(AP_WARPS * 32), 0, st, q, sums, S, out, in, ov, heads, N, eps, tok_per_cta, state_scale, PlanesView{}, early);
     }
     ++launches;
   }
@@ -515,10 +526,10 @@ msla_status_t launch_apply_planes(const PlanesView& pv, const float* state, bf16
   const int tok = make_core_plan(BH, N, D).apply_tokens;
   if (ov.pair)
     launch_pdl(apply_mma_kernel<D, AP_WARPS, AP_STAGES, AP_U, true, F16, true>, dim3((unsigned)ceil_div_ll(N, tok / 2), (unsigned)(BH / 2)), dim3(AP_WARPS * 32), 0, st,
-               nullptr, state, 1, out, HeadView{}, ov, Ht, N, eps, tok / 2, state_scale, pv);
+               nullptr, state, 1, out, HeadView{}, ov, Ht, N, eps, tok / 2, state_scale, pv, false);
   else
     launch_pdl(apply_mma_kernel<D, AP_WARPS, AP_STAGES, AP_U, false, F16, true>, dim3((unsigned)ceil_div_ll(N, tok), (unsigned)BH), dim3(AP_WARPS * 32), 0, st,
-               nullptr, state, 1, out, HeadView{}, ov, Ht, N, eps, tok, state_scale, pv);
+               nullptr, state, 1, out, HeadView{}, ov, Ht, N, eps, tok, state_scale, pv, false);
   count_launches(1);
   return check_launch("apply step on channel-blocked planes");
 }

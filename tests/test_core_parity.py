@@ -103,3 +103,33 @@ def test_core_runtime_argument_errors():
 def test_core_many_heads(dtype, B, heads, N, d):
     t, ref = _case(dtype, B, heads, N, d, seed=300 + N)
     util.assert_close(util.run_core(t, dtype), ref, dtype, f"core {dtype} {B}x{heads}x{N}x{d}", block=util.CORE_BLOCK)
+
+
+# Sizes at which the apply step fetches queries before the reduction is over (3 * 2^20 values and more, one wave of CTAs): tensors that a
+# kernel writes on the same stream just before the call are the ones that it reads, call after call.
+@pytest.mark.parametrize("B,heads,N,d", [(2, 24, 2187, 32), (3, 7, 9363, 16), (1, 1, 98304, 32), (4, 111, 225, 32)])
+def test_queries_written_just_before_the_call(B, heads, N, d):
+    assert B * heads * N * d >= 3 << 20
+    g = torch.Generator(device="cuda").manual_seed(5)
+    draws = [[torch.randn(B, heads, N, d, generator=g, device="cuda").to(torch.bfloat16) for _ in range(3)] for _ in range(2)]
+    nbytes = binding.msla_linattn_relu_workspace_bytes(B, heads, N, d)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    run = lambda t, out: binding.msla_linattn_relu_ws(binding.MSLA_BF16, *t, out, B, heads, N, d, 1e-15, ws, nbytes)
+    refs = []
+    for t in draws:
+        refs.append(torch.empty_like(t[0]))
+        run(t, refs[-1])
+        torch.cuda.synchronize()
+        q, k, v = (x.double() for x in t)
+        q, k = q.relu(), k.relu()
+        want = q @ (k.transpose(-1, -2) @ v) / (q @ k.sum(-2).unsqueeze(-1) + 1e-15)
+        util.assert_close(util.host(refs[-1]), util.host(want), "bf16", "core", block=util.CORE_BLOCK)
+    bufs, outs = [torch.empty_like(x) for x in draws[0]], []
+    for i in range(20):
+        for b, x in zip(bufs, draws[i % 2]):
+            b.copy_(x)
+        outs.append(torch.empty_like(bufs[0]))
+        run(bufs, outs[-1])
+    torch.cuda.synchronize()
+    for i, out in enumerate(outs):
+        assert torch.equal(out, refs[i % 2]), i
