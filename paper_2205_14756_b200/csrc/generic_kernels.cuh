@@ -5,7 +5,7 @@
 //
 // What bounds them is how many multiply-adds a shared-memory access feeds: every inner loop works on a register tile
 // (4 x 4 to 8 x 4 outputs) read in 16-byte pieces.  Module [1, 192, 64, 128], d = 32, fp32: 333 us per forward with one or
-// two shared-memory loads per multiply-add, 176 us now; [1, 64, 16, 16], d = 16 (all latency): 71 -> 21 us.
+// two shared-memory loads per multiply-add, 176 us with register tiles (92.7 with the projections on tensor cores); [1, 64, 16, 16], d = 16 (all latency): 71 -> 21 us.
 #pragma once
 
 #include "msla_common.cuh"
@@ -247,9 +247,12 @@ embed_taps_kernel(const T* __restrict__ w3, T* __restrict__ w5, long long total)
 // on planar activations [B, groups, H*W, D].  One CTA = one tile of TH x TW pixels of
 // one group.  src(b, g, n, i) = src[b*src_sb + (g*H*W + n)*D + i]; dst likewise with dst_sb.
 // A lane keeps one channel (D = 16: the half-warps take different pixels): the depthwise step slides down a strip of
-// four pixel columns and SH rows with five rows of sums in registers (8 shared-memory loads per 100 multiply-adds), the
-// 1x1 step holds the channel's D weights in registers and reads the depthwise results, which replace the staged tile in
-// shared memory, as broadcast 16-byte pieces.
+// four pixel columns and SH rows with five rows of sums in registers (8 shared-memory loads per 100 multiply-adds).  The depthwise
+// results replace the staged tile in shared memory, and the 1x1 step forms 4 x 8 outputs per thread from 16-byte pieces of them
+// and of the weights (12 loads per 128 multiply-adds; a 16-byte load takes four cycles of the path to the registers also where all
+// lanes read the same: a channel per lane with its weights in registers, 8 loads per 32 multiply-adds, was bound by that).  fp32 tiles
+// come by asynchronous copies.  576 channels of 64 x 128 tokens, d = 32: 27.7 -> 21.0 us, 384 of 45 x 80, d = 16: 14.6 -> 8.0, 8 x 768 of 14 x 14:
+// 19.2 -> 10.5 (copies alone 27.2, 8.8, 13.6).  Tiles of 8 x 16, 16 x 8 and 8 x 8 pixels re-read more halo: 30 to 32 us for the first.
 // ---------------------------------------------------------------------------
 template <typename T, int D, int TH, int TW, int SH>
 __global__ void __launch_bounds__(TH * TW * D / (4 * SH))
@@ -259,7 +262,10 @@ aggregate_kernel(const T* __restrict__ src, const T* __restrict__ w_dw, const T*
   constexpr int HW_ = TW + 4, HH = TH + 4, CV = D / 4;
   static_assert(TH % SH == 0 && TW % 4 == 0, "strips of 4 x SH pixels");
   extern __shared__ __align__(16) float agg_smem[];
-  float* tile = agg_smem;  // [HH][HW_][D], then the depthwise results [TH * TW][D]
+  float* tile = agg_smem;  // [HH][HW_][D], then the depthwise results [TH * TW][P]
+  constexpr int P = D + 4;  // pitch of rows of which eight lanes read a 16-byte piece each
+  static_assert(TH * TW * P <= HH * HW_ * D, "the results fit the staged tile");
+  __shared__ __align__(16) float wt[D * P];  // 1x1 weights: output channel 8 g + j in row j * (D / 8) + g
   pdl_launch_dependents();
   const int tid = threadIdx.x;
   const int tiles_x = (W + TW - 1) / TW;
@@ -269,9 +275,28 @@ aggregate_kernel(const T* __restrict__ src, const T* __restrict__ w_dw, const T*
   const int c = tid % D, strip = tid / D;  // strips: row-major over (TH / SH) x (TW / 4)
   float taps[25];
   pdl_wait();  // the planes come from the previous kernel, and the taps may (a 3x3 filter embedded in 5x5)
+  const T* sb = src + (long long)b * src_sb + (long long)blockIdx.y * H * W * D;
+  if constexpr (sizeof(T) == 4) {  // as they are: all copies in flight at once, no registers
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(tile);
+#pragma unroll 4
+    for (int e = tid; e < HH * HW_ * CV; e += THREADS) {
+      const int cv = e % CV, p = e / CV;
+      const int yy = y0 + p / HW_ - 2, xx = x0 + p % HW_ - 2;
+      const bool in = yy >= 0 && yy < H && xx >= 0 && xx < W;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + (uint32_t)(p * D + cv * 4) * 4u), "l"(sb + (in ? ((long long)yy * W + xx) * D + cv * 4 : 0)),
+                   "r"(in ? 16 : 0) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
 #pragma unroll
   for (int i = 0; i < 25; ++i) taps[i] = load1_dep(w_dw + (long long)(ch0 + c) * 25 + i);
-  const T* sb = src + (long long)b * src_sb + (long long)blockIdx.y * H * W * D;
+  for (int e = tid; e < D * CV; e += THREADS) {
+    const int oc = e / CV, k = e % CV * 4;
+    *reinterpret_cast<float4*>(wt + ((oc & 7) * (D / 8) + (oc >> 3)) * P + k) = load4_dep(w_pw + (long long)(ch0 + oc) * D + k);
+  }
+  if constexpr (sizeof(T) == 4) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+  } else {
 #pragma unroll 8
   for (int e = tid; e < HH * HW_ * CV; e += THREADS) {
     const int cv = e % CV, p = e / CV;
@@ -279,6 +304,7 @@ aggregate_kernel(const T* __restrict__ src, const T* __restrict__ w_dw, const T*
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     if (yy >= 0 && yy < H && xx >= 0 && xx < W) v = load4_dep(sb + ((long long)yy * W + xx) * D + cv * 4);
     *reinterpret_cast<float4*>(tile + p * D + cv * 4) = v;
+  }
   }
   __syncthreads();
   const int sx = (strip % (TW / 4)) * 4, sy = strip / (TW / 4) * SH;
@@ -304,30 +330,46 @@ aggregate_kernel(const T* __restrict__ src, const T* __restrict__ w_dw, const T*
       }
     }
   }
-  float pw[D];
-#pragma unroll
-  for (int i = 0; i < D; i += 4) {
-    const float4 v = load4_dep(w_pw + (long long)(ch0 + c) * D + i);
-    pw[i] = v.x; pw[i + 1] = v.y; pw[i + 2] = v.z; pw[i + 3] = v.w;
-  }
   __syncthreads();  // the staged tile has been read
 #pragma unroll
   for (int o = 0; o < SH; ++o)
 #pragma unroll
-    for (int x = 0; x < 4; ++x) tile[((sy + o) * TW + sx + x) * D + c] = acc[o][x];
+    for (int x = 0; x < 4; ++x) tile[((sy + o) * TW + sx + x) * P + c] = acc[o][x];
   __syncthreads();
-  T* db = dst + (long long)b * dst_sb + (long long)blockIdx.y * H * W * D;
-#pragma unroll 2
-  for (int i = 0; i < PX; ++i) {
-    const int p = strip + i * (THREADS / D);
-    const int yy = y0 + p / TW, xx = x0 + p % TW;
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+  // 1x1: a thread forms PT pixels x 8 output channels, the even and the odd input channels in the halves of a packed sum
+  constexpr int OG = D / 8, PG = 32 / OG, PT = PX / 8;
+  const int og = tid % OG, p0 = tid / 32 * (PG * PT) + tid % 32 / OG;
+  unsigned long long sum[PT][8] = {};
 #pragma unroll
-    for (int k = 0; k < D; k += 4) {
-      const float4 v = *reinterpret_cast<const float4*>(tile + p * D + k);
-      a0 = fmaf(pw[k], v.x, a0); a1 = fmaf(pw[k + 1], v.y, a1); a2 = fmaf(pw[k + 2], v.z, a2); a3 = fmaf(pw[k + 3], v.w, a3);
+  for (int k = 0; k < D; k += 4) {
+    ulonglong2 v[PT];
+#pragma unroll
+    for (int i = 0; i < PT; ++i) v[i] = *reinterpret_cast<const ulonglong2*>(tile + (p0 + i * PG) * P + k);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(wt + (j * OG + og) * P + k);
+#pragma unroll
+      for (int i = 0; i < PT; ++i) {
+        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(sum[i][j]) : "l"(v[i].x), "l"(w.x));
+        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(sum[i][j]) : "l"(v[i].y), "l"(w.y));
+      }
     }
-    if (yy < H && xx < W) db[((long long)yy * W + xx) * D + c] = from_f32<T>((a0 + a1) + (a2 + a3));
+  }
+  T* db = dst + (long long)b * dst_sb + (long long)blockIdx.y * H * W * D + og * 8;
+#pragma unroll
+  for (int i = 0; i < PT; ++i) {
+    const int p = p0 + i * PG, yy = y0 + p / TW, xx = x0 + p % TW;
+    if (yy >= H || xx >= W) continue;
+    float lo[4], hi[4];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      float even, odd;
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(even), "=f"(odd) : "l"(sum[i][j]));
+      (j < 4 ? lo : hi)[j & 3] = even + odd;
+    }
+    T* o = db + ((long long)yy * W + xx) * D;
+    store4(o, lo);
+    store4(o + 4, hi);
   }
 }
 template <int D, int TH, int TW> constexpr int aggregate_smem() { return (TH + 4) * (TW + 4) * D * 4; }
