@@ -261,7 +261,7 @@ kv_combine_bf16path_kernel(const float* __restrict__ partial, float* __restrict_
 // into 16-bit pieces; the quotient of Eq. 3 does not change.  1 for bf16 (its exponent range is fp32's); for fp16 a
 // power of two near 1/N, so that sums over N tokens fit the format.
 // state: [heads of all images][S][D][D+1], S partial states per head that every CTA adds for itself, in index order (S = 1: the
-// state; PAIR and PLANES: always).  With few of them that costs less than a kernel of its own for the sum: see launch_core.
+// state; PLANES: always).  With few of them that costs less than a kernel of its own for the sum: see launch_core.
 // PLANES: the queries lie in channel-blocked planes [token / 8][D][8] (PlanesView); a warp copies them as they lie and
 // ldmatrix.trans makes the fragments.
 struct PlanesView {
@@ -356,30 +356,36 @@ apply_mma_kernel(const bf16* __restrict__ q, const float* __restrict__ state, in
           blo[ks][j][r] = pack16<F16>(v0 - round16<F16>(v0), v1 - round16<F16>(v1));
         }
   };
-  constexpr int NE = D * (D + 1);
-  if (PAIR || PLANES || S == 1) {  // every lane fetches its entries: one round trip
+  constexpr int NE = D * (D + 1), NV = NE / 4;
+  const float4* partial4 = reinterpret_cast<const float4*>(state);
+  auto sum_of = [&](long long head, int i) -> float4 {  // vector i of the sum of a head's partial states
+    const float4* src = partial4 + head * S * NV + i;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s = 0; s < S; s += 4) {
+      float4 x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[u] = s + u < S ? ld_dep128f(src + (s + u) * NV) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) { v.x += x[u].x; v.y += x[u].y; v.z += x[u].z; v.w += x[u].w; }
+    }
+    return v;
+  };
+  if (PLANES || S == 1) {  // every lane fetches its entries: one round trip
     const float* src = state + (long long)bh * NE;
     fragments([&](int e) { return __uint_as_float(ld_dep32(src + e)); });
+  } else if constexpr (PAIR) {  // both heads' sums
+    __shared__ float4 sums[2][NV];
+    for (int i = threadIdx.x; i < 2 * NV; i += NWARPS * 32) sums[i / NV][i % NV] = sum_of(2 * blockIdx.y + i / NV, i % NV);
+    __syncthreads();
+    fragments([&](int e) { return reinterpret_cast<const float*>(sums[warp & 1])[e]; });
   } else {
     // The sums lie in the warps' last FIFO stage meanwhile, which nothing is copied into yet: with memory of their own an SM would
     // hold a CTA less.
-    constexpr int NV = NE / 4;
     static_assert(NV <= NWARPS * STAGEB / 16, "the state fits the last stages");
     auto vec = [&](int i) -> float4* {
       return reinterpret_cast<float4*>(fifo + (i / (STAGEB / 16)) * (STAGES * STAGEB) + (STAGES - 1) * STAGEB) + i % (STAGEB / 16);
     };
-    const float4* src = reinterpret_cast<const float4*>(state) + (long long)bh * S * NV;
-    for (int i = threadIdx.x; i < NV; i += NWARPS * 32) {
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int s = 0; s < S; s += 4) {
-        float4 x[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = s + u < S ? ld_dep128f(src + (s + u) * NV + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) { v.x += x[u].x; v.y += x[u].y; v.z += x[u].z; v.w += x[u].w; }
-      }
-      *vec(i) = v;
-    }
+    for (int i = threadIdx.x; i < NV; i += NWARPS * 32) *vec(i) = sum_of(bh, i);
     __syncthreads();
     fragments([&](int e) { return reinterpret_cast<const float*>(vec(e >> 2))[e & 3]; });
     __syncthreads();  // every warp has its fragments: the stages may be filled
@@ -487,10 +493,10 @@ msla_status_t launch_core(const bf16* q, const bf16* k, const bf16* v, bf16* out
     ++launches;
   }
   // A few partial states are added by every CTA of the apply step (S of 4 KB each, from L2); a kernel of its own adds them where
-  // there are more (few heads, many chunks), where the caller wants the sum, and for paired planes, whose CTAs serve two heads with
-  // half the tokens each.  Core, us, with / without that kernel: [1, 16, 4096, 32] (S = 16) 19.4 / 16.1, [32, 8, 784, 32] (S = 3) 19.0 /
+  // there are more (few heads, many chunks), where the caller wants the sum, and for paired planes of many tokens, whose CTAs serve two
+  // heads with half the tokens each (up to 1024 tokens they are few, and the launch counts for more: module [16, 384, 7, 7] 32.9 / 32.3).  Core, us, with / without that kernel: [1, 16, 4096, 32] (S = 16) 19.4 / 16.1, [32, 8, 784, 32] (S = 3) 19.0 /
   // 17.1, [2, 24, 12000, 32] 39.3 / 38.0; [1, 10, 70844, 32] (S = 60) 52 / 61; module [2, 384, 100, 40] (paired) 58 / 60.
-  const bool direct = (phases & CORE_STATE) && (phases & CORE_APPLY) && !ov.pair && p.S <= 16;
+  const bool direct = (phases & CORE_STATE) && (phases & CORE_APPLY) && (!ov.pair || N <= 1024) && p.S <= 16;
   if ((phases & CORE_COMBINE) && !direct) {
     const long long total = BH * p.ne;
     launch_pdl(kv_combine_bf16path_kernel, dim3((unsigned)ceil_div_ll(total, 256)), dim3(256), 0, st, partial, state, p.S, p.ne, total);
