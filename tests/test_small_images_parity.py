@@ -1,0 +1,54 @@
+"""Batches of small images, whose apply step and output projection run as kernels of their own: the edges of that rule, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import __graft_entry__  # noqa: F401
+import oracle
+import util
+from paper_2205_14756_b200 import binding, inputs
+
+pytestmark = pytest.mark.gpu
+
+
+# the smallest and the largest images of the rule and their neighbours on the other side (tokens, octets, output channels, images, d), an
+# odd number of heads, and three branches' worth of channels that leave no room for the attention output
+@pytest.mark.parametrize("dtype,B,C,H,W,heads,d,apart", [("f16", 4, 128, 28, 28, 8, 16, True), ("bf16", 4, 64, 16, 16, 4, 16, False), ("bf16", 5, 64, 24, 11, 4, 16, True),
+                                                        ("f16", 4, 96, 21, 24, 5, 16, True), ("bf16", 4, 64, 64, 64, 4, 16, True), ("bf16", 4, 64, 65, 64, 4, 16, False),
+                                                        ("bf16", 4, 192, 32, 64, 12, 16, True), ("bf16", 4, 192, 33, 64, 12, 16, False), ("f16", 4, 96, 21, 23, 6, 16, False),
+                                                        ("bf16", 3, 128, 28, 28, 8, 16, False), ("bf16", 4, 64, 28, 28, 8, 16, False), ("bf16", 4, 128, 28, 28, 4, 32, False)])
+def test_small_images(dtype, B, C, H, W, heads, d, apart):
+    s = inputs.ModuleShape("small", dtype, B, C, H, W, heads, d, seed=61)
+    t = inputs.module_inputs(s)
+    plan = binding.msla_forward_plan(binding.make_desc(B, C, H, W, heads, d, C, util.CODE[dtype]))
+    assert bool(plan & binding.MSLA_PLAN_FUSES_APPLY) != apart
+    ref = oracle.msla_forward(t["x"], t["w_qkv"], t["w_dw"], t["w_pw"], t["w_proj"], heads=heads, d=d, eps=s.eps)
+    util.assert_close(util.run_module(s, t), ref, dtype, "small images", block=util.MODULE_BLOCK)
+    assert binding.msla_debug_wait_timeouts() == 0
+
+
+# the host call runs the batch in parts of fewer images than the rule asks for: the batch decides, bit for bit
+def test_small_images_from_host_memory():
+    B, C, H, W, heads, d = 45, 128, 28, 20, 8, 16
+    g = torch.Generator(device="cuda").manual_seed(3)
+    r = lambda *shape, std=1.0: (torch.randn(*shape, generator=g, device="cuda") * std).to(torch.bfloat16)
+    x, keep = r(B, C, H, W), [r(3 * C, C, std=C ** -0.5), r(3 * C, 5, 5, std=0.2), r(3 * C, d, std=d ** -0.5), r(C, 2 * C, std=(2 * C) ** -0.5)]
+    w = binding.make_weights(*keep)
+    make = lambda ws=None: binding.make_desc(B, C, H, W, heads, d, C, binding.MSLA_BF16, workspace=ws)
+    desc = make(torch.empty(binding.msla_forward_host_workspace_bytes(make()), dtype=torch.uint8, device="cuda"))
+    out, host_out = torch.empty_like(x), torch.empty(B, C, H, W, dtype=torch.bfloat16, pin_memory=True)
+    binding.msla_forward(desc, x, w, out)
+    binding.msla_forward_host(desc, x.cpu().pin_memory(), w, host_out)
+    torch.cuda.synchronize()
+    assert np.array_equal(util.host(out), util.host(host_out))
+
+
+# apply step on paired planes that adds several partial states per head itself (heads that the fused kernel does not take), and the size from
+# which a kernel of its own adds them
+@pytest.mark.parametrize("dtype,B,C,H,W,heads", [("bf16", 2, 320, 32, 32, 10), ("f16", 1, 288, 25, 41, 10), ("bf16", 7, 384, 13, 24, 12)])
+def test_sums_of_paired_heads(dtype, B, C, H, W, heads):
+    s = inputs.ModuleShape("pairs", dtype, B, C, H, W, heads, 32, seed=62)
+    t = inputs.module_inputs(s)
+    assert binding.msla_forward_plan(binding.make_desc(B, C, H, W, heads, 32, C, util.CODE[dtype])) == 0
+    ref = oracle.msla_forward(t["x"], t["w_qkv"], t["w_dw"], t["w_pw"], t["w_proj"], heads=heads, d=32, eps=s.eps)
+    util.assert_close(util.run_module(s, t), ref, dtype, "paired heads", block=util.MODULE_BLOCK)
